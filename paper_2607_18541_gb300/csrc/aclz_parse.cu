@@ -6,14 +6,16 @@
 // same 4-byte prefix is a candidate, nearest first.  Sorting the positions
 // by (prefix, position) therefore lays every chain out contiguously, so the
 // candidates of position p are the entries just before p in that order.
-// The parse itself is sequential only within an LZ block (a match never
-// crosses its block's end), so one warp parses each block, its lanes
-// scoring up to 32 candidates at a time.
+// What a position's best match is does not depend on the parse either, only
+// whether the walk stops there does, so every position is scored at once;
+// the walk, sequential within an LZ block (a match never crosses its
+// block's end), then only steps from match to match.
 //
 //  1. k_keys          prefix of every position with 4 bytes left
 //  2. radix sort      stable, 8-bit digits: k_rs_hist, exclusive scan,
 //                     k_rs_scatter (4 passes)
-//  3. k_rank          rank of each position in the sorted order
+//  3. k_best          best match of every position, one thread each, in
+//                     sorted order
 //  4. k_parse_blocks  one warp per block: greedy walk, tokens to a per-block
 //                     slot array
 //  5. scans of the per-block token and literal counts, then k_emit writes
@@ -109,12 +111,6 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_scatter(const uint32_t *__r
     }
 }
 
-__global__ void k_rank(const uint32_t *__restrict__ val_s, uint64_t m, uint32_t *__restrict__ rank) {
-    for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < m;
-         r += (uint64_t)gridDim.x * blockDim.x)
-        rank[val_s[r]] = (uint32_t)r;
-}
-
 // 8 bytes at a (little endian) from two aligned words; needs a + 16 <= the
 // padded end of the buffer.
 __device__ __forceinline__ uint64_t ld8u(const uint8_t *a) {
@@ -140,21 +136,193 @@ __device__ __forceinline__ uint32_t common_len(const uint8_t *x, uint64_t q, uin
 
 __device__ __forceinline__ int dclass(uint64_t d) { return d < 128 ? 0 : d < 16384 ? 1 : d < 2097152 ? 2 : 3; }
 
+// Match lengths of kCap and more are left to the walk (kLong): scoring them
+// for every position of a long repeat would cost its length squared.
+constexpr uint32_t kCap = 64, kLong = 255;
+constexpr int kBestThreads = 256;
+constexpr uint32_t kHalo = 64;             // candidates per round
+constexpr uint32_t kLenWindow = 32 * 16;  // positions a warp of the walk holds
+
+__device__ __forceinline__ uint32_t class_min(uint32_t d, uint32_t T) {
+    return (T >> (8 * dclass(d))) & 255u;
+}
+
+// Best match of every position: thread r takes the position p of rank r.
+// Its candidates are the entries of rank r - 1, r - 2, ... while their
+// prefix is p's, at most depth of them and no farther than window; the
+// longest whose length (capped at the distance and the block end) meets its
+// distance class minimum wins, the nearest on ties.  best_len[p] receives
+// the length (0, as cleared before, when there is none) and best_src[p] the
+// source; best_len[p] = kLong and best_src[p] = r when a candidate matches
+// kCap bytes.
+//
+// Neighbouring ranks share their candidates, so a CTA stages the entries of
+// its ranks and of the kHalo before them (prefix, position and the 16 bytes
+// after the prefix) in shared memory: a candidate costs a 64-bit compare
+// against the bytes it must match to win, and only those that match all 20
+// staged bytes go back to the input.  Issue-bound; the whole of 16 MiB of
+// word text at depth 64 is scored in 1.6 ms, where one warp per block
+// scoring one position at a time took 135 ms.
+__global__ void __launch_bounds__(kBestThreads) k_best(const uint8_t *__restrict__ x, uint64_t n, uint64_t m,
+                                                       uint32_t log2bs, const uint32_t *__restrict__ key_s,
+                                                       const uint32_t *__restrict__ val_s, const uint8_t *mm,
+                                                       const uint8_t *__restrict__ block_mm, uint32_t depth,
+                                                       uint64_t window, uint8_t *__restrict__ best_len,
+                                                       uint32_t *__restrict__ best_src) {
+    __shared__ uint32_t skey[kBestThreads + kHalo], spos[kBestThreads + kHalo];
+    __shared__ ulonglong2 swin[kBestThreads + kHalo];
+    const uint64_t r0 = (uint64_t)blockIdx.x * kBestThreads;
+    const uint64_t r = r0 + threadIdx.x;
+    bool live = r < m;
+    uint32_t kp = 0, p = 0, T = 0, rem = 0, need = 0, blen = 0, bsrc = 0;
+    unsigned long long w0 = 0, w1 = 0, mask = 0;
+    const uint32_t no_key = ~__ldg(key_s);  // differs from any chain that reaches rank 0
+    // bytes 4 .. need - 1 of a candidate must match (up to 12 of them)
+    auto set_need = [&](uint32_t v) {
+        need = v;
+        mask = v >= 12 ? ~0ULL : (v <= 4 ? 0ULL : (1ULL << (8 * (v - 4))) - 1ULL);
+    };
+    for (uint32_t kb = 0; kb < depth; kb += kHalo) {
+        for (uint32_t i = threadIdx.x; i < kBestThreads + kHalo; i += kBestThreads) {
+            const long long rr = (long long)r0 - (long long)kb - (long long)kHalo + (long long)i;
+            uint32_t k = no_key, q = 0;
+            ulonglong2 w = make_ulonglong2(0, 0);
+            if (rr >= 0 && (uint64_t)rr < m) {
+                k = __ldg(key_s + rr);
+                q = __ldg(val_s + rr);
+                w = make_ulonglong2(ld8u(x + q + 4), ld8u(x + q + 12));
+            }
+            skey[i] = k;
+            spos[i] = q;
+            swin[i] = w;
+        }
+        __syncthreads();
+        if (kb == 0 && live) {
+            kp = skey[threadIdx.x + kHalo];
+            p = spos[threadIdx.x + kHalo];
+            w0 = swin[threadIdx.x + kHalo].x;
+            w1 = swin[threadIdx.x + kHalo].y;
+            const uint32_t b = p >> log2bs;
+            const uint64_t bend = min((uint64_t)(b + 1) << log2bs, n);
+            rem = (uint32_t)(bend - p);
+            const uint8_t *Tp = block_mm ? block_mm + 4 * (uint64_t)b : mm;
+            T = (uint32_t)Tp[0] | ((uint32_t)Tp[1] << 8) | ((uint32_t)Tp[2] << 16) | ((uint32_t)Tp[3] << 24);
+            set_need(min(min((uint32_t)Tp[0], (uint32_t)Tp[1]), min((uint32_t)Tp[2], (uint32_t)Tp[3])));
+            if (rem < need) live = false;
+        }
+        const uint32_t kn = min(kHalo, depth - kb);
+        for (uint32_t k = 0; live && k < kn; k++) {
+            const uint32_t e = threadIdx.x + kHalo - 1 - k;  // rank r - 1 - (kb + k)
+            const uint32_t q = spos[e];
+            if (skey[e] != kp || (uint64_t)(p - q) > window) {
+                live = false;
+                break;
+            }
+            const unsigned long long x0 = swin[e].x ^ w0;
+            if (x0 & mask) continue;
+            const uint32_t d = p - q;
+            const uint32_t lim = d < rem ? d : rem;
+            if (lim < need) continue;
+            uint32_t len;
+            if (x0) {
+                len = 4 + (uint32_t)(__ffsll((long long)x0) - 1) / 8;
+            } else {
+                const unsigned long long x1 = swin[e].y ^ w1;
+                if (x1) {
+                    len = 12 + (uint32_t)(__ffsll((long long)x1) - 1) / 8;
+                } else {
+                    const uint32_t cap = lim < kCap ? lim : kCap;
+                    len = cap <= 20 ? cap : 20 + common_len(x, (uint64_t)q + 20, (uint64_t)p + 20, cap - 20);
+                    if (len >= kCap) {
+                        blen = kLong;
+                        bsrc = (uint32_t)r;
+                        live = false;
+                        break;
+                    }
+                }
+            }
+            len = len < lim ? len : lim;
+            if (len >= need && len >= class_min(d, T)) {
+                blen = len;
+                bsrc = q;
+                set_need(len + 1 > need ? len + 1 : need);
+                if (need > rem) live = false;  // no longer match fits the block
+            }
+        }
+        if (!__syncthreads_or(live && kb + kHalo < depth)) break;
+    }
+    if (blen) {
+        best_len[p] = (uint8_t)blen;
+        best_src[p] = bsrc;
+    }
+}
+
 struct TokOut {
     uint32_t lit, len;
     uint64_t src;
 };
 
-// One warp per block: the greedy walk.  Candidates of p: the entries
-// rank[p] - 1, rank[p] - 2, ... of the sorted order while their prefix is
-// p's, at most depth of them and no farther than window; the longest whose
-// length (capped at the distance and the block end) meets its distance
-// class minimum wins, the nearest on ties.  Tokens go to
-// slots[b * cap_tok ...]; ntok[b] and nlit[b] receive the counts.
+// Best match of position p (rank r) whatever its length, lanes scoring 32
+// candidates at a time by the rule of k_best; *len 0 when there is none.
+__device__ __forceinline__ void best_long(const uint8_t *__restrict__ x, const uint32_t *__restrict__ key_s,
+                                          const uint32_t *__restrict__ val_s, uint64_t p, uint64_t bend, uint32_t r,
+                                          uint32_t T, uint32_t depth, uint64_t window, int lane, uint32_t *len_out,
+                                          uint32_t *src_out) {
+    const uint32_t kp = __ldg(key_s + r);
+    uint32_t best_len = 0, best_src = 0;
+    bool more = true;
+    for (uint32_t k0 = 0; k0 < depth && more; k0 += 32) {
+        const uint32_t k = k0 + lane;
+        // candidate k exists when it is in the chain, in the window and
+        // among the first depth
+        bool ok = k < depth && r >= k + 1;
+        uint64_t q = 0;
+        if (ok) {
+            const uint32_t rr = r - 1 - k;
+            ok = __ldg(key_s + rr) == kp;
+            q = __ldg(val_s + rr);
+            ok = ok && p - q <= window;
+        }
+        uint32_t len = 0;
+        if (ok) {
+            const uint64_t d = p - q;
+            const uint64_t lim = d < bend - p ? d : bend - p;
+            len = common_len(x, q, p, (uint32_t)lim);
+            if (len < class_min((uint32_t)d, T)) len = 0;
+        }
+        // longest, then nearest (smallest k): one 64-bit key per lane
+        unsigned long long key = len ? ((unsigned long long)len << 32) | (0xffffffffu - k) : 0ULL;
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, o);
+            key = other > key ? other : key;
+        }
+        if (key) {
+            const uint32_t l = (uint32_t)(key >> 32);
+            const uint32_t kk = 0xffffffffu - (uint32_t)key;
+            if (l > best_len) {  // an earlier round keeps its ties (nearer)
+                best_len = l;
+                best_src = __ldg(val_s + (r - 1 - kk));
+            }
+        }
+        more = __all_sync(0xffffffffu, !(k < depth) || ok);  // the chain went on past this round
+    }
+    *len_out = best_len;
+    *src_out = best_src;
+}
+
+// One warp per block: the greedy walk over the best matches of k_best.  The
+// warp holds the lengths of kLenWindow positions, 16 to a lane, with the
+// next window loaded ahead; a step finds the first position with a match
+// at or after p, emits its token and moves past it.  Lane i keeps token i of
+// the current 32 and looks its source up when they are written.  Tokens go
+// to slots[b * cap_tok ...]; ntok[b] and nlit[b] receive the counts.
+// best_len is readable, zero, for two windows past the input.
 __global__ void __launch_bounds__(256) k_parse_blocks(const uint8_t *__restrict__ x, uint64_t n, uint32_t bs,
                                                       uint32_t nb, const uint32_t *__restrict__ key_s,
                                                       const uint32_t *__restrict__ val_s,
-                                                      const uint32_t *__restrict__ rank, const uint8_t *mm,
+                                                      const uint8_t *__restrict__ best_len,
+                                                      const uint32_t *__restrict__ best_src, const uint8_t *mm,
                                                       const uint8_t *__restrict__ block_mm, uint32_t depth,
                                                       uint64_t window, uint32_t cap_tok, TokOut *__restrict__ slots,
                                                       uint32_t *__restrict__ ntok, uint32_t *__restrict__ nlit) {
@@ -162,73 +330,80 @@ __global__ void __launch_bounds__(256) k_parse_blocks(const uint8_t *__restrict_
     const int lane = threadIdx.x & 31;
     if (b >= nb) return;
     const uint8_t *Tp = block_mm ? block_mm + 4 * (uint64_t)b : mm;
-    const uint32_t T0 = Tp[0], T1 = Tp[1], T2 = Tp[2], T3 = Tp[3];
+    const uint32_t T = (uint32_t)Tp[0] | ((uint32_t)Tp[1] << 8) | ((uint32_t)Tp[2] << 16) | ((uint32_t)Tp[3] << 24);
     const uint64_t bstart = (uint64_t)b * bs;
     const uint64_t bend = bstart + bs < n ? bstart + bs : n;
     TokOut *out = slots + (uint64_t)b * cap_tok;
     uint64_t p = bstart, lit_start = bstart;
     uint32_t cnt = 0, lits = 0;
-    while (p < bend) {
-        uint32_t best_len = 0;
-        uint64_t best_src = 0;
-        if (p + 4 <= n) {
-            const uint32_t r = rank[p];
-            const uint32_t kp = key_s[r];
-            bool more = true;
-            for (uint32_t k0 = 0; k0 < depth && more; k0 += 32) {
-                const uint32_t k = k0 + lane;
-                // candidate k exists when it is in the chain, in the window
-                // and among the first depth
-                bool ok = k < depth && r >= k + 1;
-                uint64_t q = 0;
-                if (ok) {
-                    const uint32_t rr = r - 1 - k;
-                    ok = key_s[rr] == kp;
-                    q = val_s[rr];
-                    ok = ok && p - q <= window;
-                }
-                uint32_t len = 0;
-                if (ok) {
-                    const uint64_t d = p - q;
-                    const uint64_t lim = d < bend - p ? d : bend - p;
-                    len = common_len(x, q, p, (uint32_t)lim);
-                    const int c = dclass(d);
-                    const uint32_t t = c == 0 ? T0 : c == 1 ? T1 : c == 2 ? T2 : T3;
-                    if (len < t) len = 0;
-                }
-                // longest, then nearest (smallest k): one 64-bit key per lane
-                unsigned long long key = len ? ((unsigned long long)len << 32) | (0xffffffffu - k) : 0ULL;
-#pragma unroll
-                for (int o = 16; o; o >>= 1) {
-                    const unsigned long long other = __shfl_xor_sync(0xffffffffu, key, o);
-                    key = other > key ? other : key;
-                }
-                if (key) {
-                    const uint32_t l = (uint32_t)(key >> 32);
-                    const uint32_t kk = 0xffffffffu - (uint32_t)key;
-                    if (l > best_len) {  // an earlier round keeps its ties (nearer)
-                        best_len = l;
-                        best_src = (uint64_t)val_s[r - 1 - kk];
-                    }
-                }
-                more = __all_sync(0xffffffffu, !(k < depth) || ok);  // the chain went on past this round
-            }
+    // this lane's token of the current 32: literals, length, source (or the
+    // position whose source is still to be looked up)
+    uint32_t t_lit = 0, t_len = 0, t_src = 0;
+    bool t_at = false;
+    auto flush = [&](uint32_t k) {  // the first k tokens of the current 32
+        if ((uint32_t)lane < k)
+            out[(cnt - k) + lane] = TokOut{t_lit, t_len, t_at ? (uint64_t)__ldg(best_src + t_src) : (uint64_t)t_src};
+    };
+    auto emit = [&](uint32_t lit, uint32_t len, uint32_t src, bool at) {
+        if ((uint32_t)lane == (cnt & 31u)) {
+            t_lit = lit;
+            t_len = len;
+            t_src = src;
+            t_at = at;
         }
-        if (best_len) {
-            if (lane == 0) out[cnt] = TokOut{(uint32_t)(p - lit_start), best_len, best_src};
-            lits += (uint32_t)(p - lit_start);
-            cnt++;
-            p += best_len;
-            lit_start = p;
-        } else {
-            p++;
-        }
-    }
-    if (lit_start < bend || cnt == 0) {
-        if (lane == 0) out[cnt] = TokOut{(uint32_t)(bend - lit_start), 0u, 0ULL};
-        lits += (uint32_t)(bend - lit_start);
+        lits += lit;
         cnt++;
+        if (!(cnt & 31u)) flush(32);
+    };
+    auto load = [&](uint64_t at) { return __ldg(reinterpret_cast<const uint4 *>(best_len + at) + lane); };
+    // bit i: position 16 * lane + i of the window has a match
+    auto nonzero = [](const uint4 &v) {
+        auto four = [](uint32_t w) {
+            const uint32_t t = ((w & 0x7f7f7f7fu) + 0x7f7f7f7fu) | w;  // bit 7 of each byte that is not 0
+            return ((t >> 7) & 1u) | ((t >> 14) & 2u) | ((t >> 21) & 4u) | ((t >> 28) & 8u);
+        };
+        return four(v.x) | (four(v.y) << 4) | (four(v.z) << 8) | (four(v.w) << 12);
+    };
+    uint64_t base = p & ~(uint64_t)(kLenWindow - 1);
+    uint4 cur = load(base), nxt = load(base + kLenWindow);
+    uint32_t bits = nonzero(cur);
+    while (p < bend) {
+        const int below = (int)(p - base) - 16 * lane;  // positions of this lane before p
+        const uint32_t left = below <= 0 ? bits : (below >= 16 ? 0u : bits & (0xffffu << below));
+        const unsigned have = __ballot_sync(0xffffffffu, left != 0);
+        if (have) {
+            const uint32_t at = (uint32_t)__ffs(left) - 1u;
+            const uint32_t word = at & 8 ? (at & 4 ? cur.w : cur.z) : (at & 4 ? cur.y : cur.x);
+            const uint32_t mine = ((word >> (8 * (at & 3))) & 255u) | (at << 8);
+            const int f = __ffs(have) - 1;
+            const uint32_t got = __shfl_sync(0xffffffffu, mine, f);
+            const uint64_t q = base + 16 * (uint32_t)f + (got >> 8);
+            if (q >= bend) break;
+            uint32_t len = got & 255u, src = (uint32_t)q;
+            const bool lng = len == kLong;
+            if (lng) best_long(x, key_s, val_s, q, bend, __ldg(best_src + q), T, depth, window, lane, &len, &src);
+            if (!len) {
+                p = q + 1;
+            } else {
+                emit((uint32_t)(q - lit_start), len, src, !lng);
+                p = q + len;
+                lit_start = p;
+            }
+        } else {
+            p = base + kLenWindow;
+        }
+        if (p - base >= kLenWindow) {
+            const uint64_t nbase = p & ~(uint64_t)(kLenWindow - 1);
+            if (p < bend) {
+                cur = nbase == base + kLenWindow ? nxt : load(nbase);
+                nxt = load(nbase + kLenWindow);
+                bits = nonzero(cur);
+            }
+            base = nbase;
+        }
     }
+    if (lit_start < bend || cnt == 0) emit((uint32_t)(bend - lit_start), 0u, 0u, false);
+    flush(cnt & 31u);
     if (lane == 0) {
         ntok[b] = cnt;
         nlit[b] = lits;
@@ -337,7 +512,7 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
         }
         return rc == ACLZ_OK;
     };
-    Dev dx, dk0, dv0, dk1, dv1, drank, dhist, dslots, dntok, dnlit, dtoff, dloff, dmm, dbmm, dcont;
+    Dev dx, dk0, dv0, dk1, dv1, dlen, dhist, dslots, dntok, dnlit, dtoff, dloff, dmm, dbmm, dcont;
     const uint32_t ntiles = (uint32_t)((m + kSortTile - 1) / kSortTile);
     // the input with 16 zero bytes after it (the 8-byte compares read
     // whole aligned words)
@@ -346,7 +521,7 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
         return rc;
     const uint64_t mm1 = m ? m : 1;
     if (!ck(cudaMalloc(&dk0.p, 4 * mm1)) || !ck(cudaMalloc(&dv0.p, 4 * mm1)) || !ck(cudaMalloc(&dk1.p, 4 * mm1)) ||
-        !ck(cudaMalloc(&dv1.p, 4 * mm1)) || !ck(cudaMalloc(&drank.p, 4 * mm1)) ||
+        !ck(cudaMalloc(&dv1.p, 4 * mm1)) || !ck(cudaMalloc(&dlen.p, n + 3 * kLenWindow)) ||
         !ck(cudaMalloc(&dhist.p, 4 * (256ULL * (ntiles ? ntiles : 1) + 4))))
         return rc;
     uint32_t *k0 = (uint32_t *)dk0.p, *v0 = (uint32_t *)dv0.p, *k1 = (uint32_t *)dk1.p, *v1 = (uint32_t *)dv1.p;
@@ -368,8 +543,6 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
             std::swap(v0, v1);
         }
         if (rc) return rc;
-        k_rank<<<g, 256, 0, st>>>(v0, m, (uint32_t *)drank.p);
-        ck(cudaGetLastError());
     }
     // thresholds
     if (!ck(cudaMalloc(&dmm.p, 16)) || !ck(cudaMemcpyAsync(dmm.p, p->min_match, 4, cudaMemcpyHostToDevice, st)))
@@ -383,8 +556,14 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
         return rc;
     const uint64_t window = p->window;
     if (nb) {
+        // k1 and v1 are free after the sort; v1 holds the sources
+        if (!ck(cudaMemsetAsync(dlen.p, 0, n + 3 * kLenWindow, st))) return rc;
+        if (m)
+            k_best<<<(unsigned)((m + kBestThreads - 1) / kBestThreads), kBestThreads, 0, st>>>(
+                (const uint8_t *)dx.p, n, m, log2u(bs), k0, v0, (const uint8_t *)dmm.p, (const uint8_t *)dbmm.p,
+                p->chain_depth, window, (uint8_t *)dlen.p, v1);
         k_parse_blocks<<<(nb + 7) / 8, 256, 0, st>>>((const uint8_t *)dx.p, n, bs, nb, k0, v0,
-                                                     (const uint32_t *)drank.p, (const uint8_t *)dmm.p,
+                                                     (const uint8_t *)dlen.p, v1, (const uint8_t *)dmm.p,
                                                      (const uint8_t *)dbmm.p, p->chain_depth, window, cap_tok,
                                                      (TokOut *)dslots.p, (uint32_t *)dntok.p, (uint32_t *)dnlit.p);
         if (!ck(cudaGetLastError())) return rc;
