@@ -47,9 +47,6 @@ constexpr int kUnrollRanges = 4; // the same in the persistent schedule's regist
 constexpr uint32_t kTmaMin = 192;
 constexpr uint32_t kPiece = 2048;
 constexpr uint32_t kSmemPerSm = 220u * 1024u;  // stage memory shared by the CTAs of one SM
-// per-wave copies put full chunks first when deferred matches average
-// at least this many bytes
-constexpr double kFullFirstMin = 48.0;
 // per-wave kernels are launched with programmatic stream serialization
 constexpr int kWavePdl = 1;
 // wave 0 reads literals through the non-coherent L1 path; before
@@ -175,7 +172,7 @@ __device__ __forceinline__ void block_wave0(const Group<G> &g, uint32_t b, const
             const uint64_t nt2 = w + 2 * G + 8 * (g.lane - 4);
             if (g.lane >= 4 && g.lane < 8 && nt2 < t1) asm volatile("prefetch.global.L2 [%0];" ::"l"(tok + nt2));
         }
-        group_copy<G, UW, false, kWave0Ro>(g, out, dl, lit + (lbase + lincl - ll), ll);
+        group_copy<G, UW, kWave0Ro>(g, out, dl, lit + (lbase + lincl - ll), ll);
         g.sync();
         // in-order matches, batched so no batch reads what it writes: each
         // batch takes the lanes whose sources overlap no output of a lane
@@ -391,10 +388,8 @@ __global__ void __launch_bounds__(kThreads, STAGED ? 2 : 3)
 
 // Copy one wave's worklist.  Group k owns the segments (runs of one block)
 // that start in [k*T, (k+1)*T); a segment crossing the range end is
-// finished by the group that started it.  FULL_FIRST: the matches' full
-// 16-byte chunks are copied before their partial ones (for matches of
-// several chunks); otherwise chunks go in match order.
-template <int G, int ITEMS, bool FULL_FIRST>
+// finished by the group that started it.
+template <int G, int ITEMS>
 __global__ void __launch_bounds__(kWaveThreads, kWaveMinCtas) k_wave_copy(const uint4 *__restrict__ tri, uint64_t n,
                                                         uint8_t *out, uint32_t log2bs) {
     Group<G> g;
@@ -449,10 +444,7 @@ __global__ void __launch_bounds__(kWaveThreads, kWaveMinCtas) k_wave_copy(const 
         while (rem) {
             const unsigned batch = g.ballot(((rem >> g.lane) & 1u) && (deps & rem) == 0u);
             const bool mine = (batch >> g.lane) & 1u;
-            if (FULL_FIRST)
-                group_copy_full_first<G, kUnrollCopy>(g, out, d, out + sr, mine ? len : 0u);
-            else
-                group_copy<G, kUnrollCopy>(g, out, d, out + sr, mine ? len : 0u);
+            group_copy<G, kUnrollCopy>(g, out, d, out + sr, mine ? len : 0u);
             g.sync();
             rem &= ~batch;
         }
@@ -470,9 +462,6 @@ int launch_waves(aclz_handle *h, uint8_t *out, cudaStream_t st, cudaEvent_t phas
     if (phase) cudaEventRecord(phase, st);
     // one window of G triplets per group: the most resident groups per wave
     constexpr int ITEMS = 1;
-    // deferred matches of three or more 16-byte chunks on average: full
-    // chunks first
-    const bool ff = h->mean_deferred_len >= (double)kFullFirstMin;
     for (uint32_t w = 1; w < h->n_waves; w++) {
         const uint64_t a = h->wave_start[w], n = h->wave_start[w + 1] - a;
         if (!n) continue;
@@ -481,7 +470,7 @@ int launch_waves(aclz_handle *h, uint8_t *out, cudaStream_t st, cudaEvent_t phas
         constexpr int gpcw = kWaveThreads / G;
         const unsigned grid = (unsigned)((groups + gpcw - 1) / gpcw);
         const uint4 *t = (const uint4 *)h->d_tri + a;
-        auto k = ff ? k_wave_copy<G, ITEMS, true> : k_wave_copy<G, ITEMS, false>;
+        auto k = k_wave_copy<G, ITEMS>;
         // programmatic stream serialization: this wave's CTAs may start (and
         // load their worklist) while the previous kernel's last CTAs finish
         cudaLaunchConfig_t lc = {};

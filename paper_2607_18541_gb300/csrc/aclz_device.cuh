@@ -1,8 +1,9 @@
 // Device-side building blocks of the decode kernels: G-lane groups
 // (G in {8, 16, 32} lanes of one warp cooperate on one LZ block, Sec. II),
-// group scans and ballots, and the packed 16-byte-vectorised copy that maps
-// every lane to one aligned 16-byte chunk of output (Sec. III-C: short
-// matches leave lanes idle unless several are packed into one pass).
+// group scans and ballots, and the packed 16-byte-vectorised copy that deals
+// the aligned 16-byte output chunks of several jobs to the group's lanes
+// (Sec. III-C: short matches leave lanes idle unless several are packed into
+// one pass).
 #pragma once
 
 #include <cstdint>
@@ -47,20 +48,17 @@ struct Group {
         return v;
     }
     __device__ __forceinline__ unsigned lanemask_lt() const { return (1u << lane) - 1u; }
+    // bitwise or over the group's lanes
+    __device__ __forceinline__ unsigned or_all(unsigned v) const {
+        if (G == 32) return __reduce_or_sync(0xffffffffu, v);
+#pragma unroll
+        for (int o = 1; o < G; o <<= 1) v |= __shfl_xor_sync(mask, v, o, G);
+        return v;
+    }
 };
-
-__device__ __forceinline__ uint4 ldcg16(const uint8_t *p) {
-    return __ldcg(reinterpret_cast<const uint4 *>(p));
-}
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ uint4 lds16(const uint8_t *p) {
-    uint4 v;
-    asm("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(smem_u32(p)));
-    return v;
 }
 
 __device__ __forceinline__ uint4 lds16_u32(uint32_t a) {
@@ -71,228 +69,185 @@ __device__ __forceinline__ uint4 lds16_u32(uint32_t a) {
 
 // Bytes [r, r + 16) of the 32-byte little-endian concatenation a || b.
 __device__ __forceinline__ uint4 window16(uint4 a, uint4 b, uint32_t r) {
-    uint32_t v0 = a.x, v1 = a.y, v2 = a.z, v3 = a.w, v4 = b.x, v5 = b.y, v6 = b.z, v7 = b.w;
-    const uint32_t q = r >> 2, sh = (r & 3) * 8;
-    uint32_t w0, w1, w2, w3, w4;
-    if (q == 0) { w0 = v0; w1 = v1; w2 = v2; w3 = v3; w4 = v4; }
-    else if (q == 1) { w0 = v1; w1 = v2; w2 = v3; w3 = v4; w4 = v5; }
-    else if (q == 2) { w0 = v2; w1 = v3; w2 = v4; w3 = v5; w4 = v6; }
-    else { w0 = v3; w1 = v4; w2 = v5; w3 = v6; w4 = v7; }
+    const bool two = r & 8, one = r & 4;
+    const uint32_t sh = (r & 3) * 8;
+    const uint32_t y0 = two ? a.z : a.x, y1 = two ? a.w : a.y, y2 = two ? b.x : a.z, y3 = two ? b.y : a.w,
+                   y4 = two ? b.z : b.x, y5 = two ? b.w : b.y;
+    const uint32_t z0 = one ? y1 : y0, z1 = one ? y2 : y1, z2 = one ? y3 : y2, z3 = one ? y4 : y3,
+                   z4 = one ? y5 : y4;
     uint4 o;
-    o.x = __funnelshift_r(w0, w1, sh);
-    o.y = __funnelshift_r(w1, w2, sh);
-    o.z = __funnelshift_r(w2, w3, sh);
-    o.w = __funnelshift_r(w3, w4, sh);
+    o.x = __funnelshift_r(z0, z1, sh);
+    o.y = __funnelshift_r(z1, z2, sh);
+    o.z = __funnelshift_r(z2, z3, sh);
+    o.w = __funnelshift_r(z3, z4, sh);
     return o;
 }
 
-// Store bytes [lo, hi) of the 16-byte word v at the aligned address p,
-// as at most seven naturally aligned 1/2/4/8-byte stores.
-__device__ __forceinline__ void store_partial16(uint8_t *p, uint4 v, uint32_t lo, uint32_t hi) {
-    const unsigned long long q0 = (unsigned long long)v.x | ((unsigned long long)v.y << 32);
-    const unsigned long long q1 = (unsigned long long)v.z | ((unsigned long long)v.w << 32);
-    // byte t of the word, t in [0, 16), and the little-endian field at t
-    auto field = [&](uint32_t t) -> unsigned long long { return t < 8 ? (q0 >> (8 * t)) | (t ? q1 << (64 - 8 * t) : 0ULL) : q1 >> (8 * (t - 8)); };
-    uint32_t t = lo;
-    if ((t & 1) && t + 1 <= hi) { p[t] = (uint8_t)field(t); t += 1; }
-    if ((t & 2) && t + 2 <= hi) { *reinterpret_cast<uint16_t *>(p + t) = (uint16_t)field(t); t += 2; }
-    if ((t & 4) && t + 4 <= hi) { *reinterpret_cast<uint32_t *>(p + t) = (uint32_t)field(t); t += 4; }
-    if ((t & 8) && t + 8 <= hi) { *reinterpret_cast<unsigned long long *>(p + t) = field(t); t += 8; }
-    while (t + 8 <= hi) { *reinterpret_cast<unsigned long long *>(p + t) = field(t); t += 8; }
-    if (t + 4 <= hi) { *reinterpret_cast<uint32_t *>(p + t) = (uint32_t)field(t); t += 4; }
-    if (t + 2 <= hi) { *reinterpret_cast<uint16_t *>(p + t) = (uint16_t)field(t); t += 2; }
-    if (t + 1 <= hi) { p[t] = (uint8_t)field(t); }
+// One aligned source word: L2 (bytes other kernels wrote), or the
+// non-coherent L1 path (RO: bytes nobody writes during the kernel).
+template <bool RO>
+__device__ __forceinline__ uint4 ld_word(uintptr_t a) {
+    return RO ? __ldg(reinterpret_cast<const uint4 *>(a)) : __ldcg(reinterpret_cast<const uint4 *>(a));
 }
 
-// One aligned 16-byte output chunk of a copy job: output bytes
-// [A + lo, A + hi) receive source bytes starting at s (the source of
-// output byte A + lo).  Only the aligned source words holding needed bytes
-// are read, so reads never leave the 16-byte words of the source range.
-// SMEM: the source is a shared-memory staging copy whose addresses are
-// congruent mod 16 to the global source.  RO: the source is global memory
-// that no thread writes during the kernel (the literal array), read through
-// the non-coherent L1 path.
-template <bool SMEM, bool RO = false>
-__device__ __forceinline__ void chunk_load(const uint8_t *s, uint32_t lo, uint32_t hi, uint4 &w0, uint4 &w1,
-                                           uint32_t &r) {
-    const uintptr_t vs = reinterpret_cast<uintptr_t>(s) - lo;
-    const uintptr_t base = vs & ~(uintptr_t)15;
-    r = (uint32_t)(vs & 15);
-    const uintptr_t s0 = reinterpret_cast<uintptr_t>(s);
-    const uintptr_t s1 = s0 + (hi - lo);  // one past the last needed source byte
-    w0 = make_uint4(0, 0, 0, 0);
-    w1 = make_uint4(0, 0, 0, 0);
-    if (SMEM) {
-        if (base + 16 > s0) w0 = lds16(reinterpret_cast<const uint8_t *>(base));
-        if (s1 > base + 16) w1 = lds16(reinterpret_cast<const uint8_t *>(base + 16));
-    } else if (RO) {
-        if (base + 16 > s0) w0 = __ldg(reinterpret_cast<const uint4 *>(base));
-        if (s1 > base + 16) w1 = __ldg(reinterpret_cast<const uint4 *>(base + 16));
-    } else {
-        if (base + 16 > s0) w0 = ldcg16(reinterpret_cast<const uint8_t *>(base));
-        if (s1 > base + 16) w1 = ldcg16(reinterpret_cast<const uint8_t *>(base + 16));
+// The 16 bytes from s on, of which the first n (1 <= n <= 16) are wanted:
+// only the aligned words holding wanted bytes are read.
+template <bool RO>
+__device__ __forceinline__ uint4 load_bytes(uintptr_t s, uint32_t n) {
+    const uint32_t r = (uint32_t)s & 15u;
+    const uintptr_t base = s & ~(uintptr_t)15;
+    uint4 a = ld_word<RO>(base), b = a;
+    if (r + n > 16) b = ld_word<RO>(base + 16);
+    return window16(a, b, r);
+}
+
+// The first n (0 <= n <= 16) bytes of v to p, as naturally aligned stores:
+// 1, 2 and 4 bytes up to the next 8-byte boundary, then 8, 8, 4, 2 and 1 as
+// they fit (what is left after a skipped step is shorter than that step).
+__device__ __forceinline__ void store_bytes(uintptr_t p, uint4 v, uint32_t n) {
+    if ((p & 1) && n) {
+        *reinterpret_cast<uint8_t *>(p) = (uint8_t)v.x;
+        v.x = __funnelshift_r(v.x, v.y, 8);
+        v.y = __funnelshift_r(v.y, v.z, 8);
+        v.z = __funnelshift_r(v.z, v.w, 8);
+        v.w >>= 8;
+        p += 1;
+        n -= 1;
     }
+    if ((p & 2) && n >= 2) {
+        *reinterpret_cast<uint16_t *>(p) = (uint16_t)v.x;
+        v.x = __funnelshift_r(v.x, v.y, 16);
+        v.y = __funnelshift_r(v.y, v.z, 16);
+        v.z = __funnelshift_r(v.z, v.w, 16);
+        v.w >>= 16;
+        p += 2;
+        n -= 2;
+    }
+    if ((p & 4) && n >= 4) {
+        *reinterpret_cast<uint32_t *>(p) = v.x;
+        v.x = v.y;
+        v.y = v.z;
+        v.z = v.w;
+        p += 4;
+        n -= 4;
+    }
+    if (n >= 8) {
+        *reinterpret_cast<uint2 *>(p) = make_uint2(v.x, v.y);
+        v.x = v.z;
+        v.y = v.w;
+        p += 8;
+        n -= 8;
+        if (n >= 8) {
+            *reinterpret_cast<uint2 *>(p) = make_uint2(v.x, v.y);
+            n -= 8;  // 0: n was 16
+        }
+    }
+    if (n >= 4) {
+        *reinterpret_cast<uint32_t *>(p) = v.x;
+        v.x = v.y;
+        p += 4;
+    }
+    if (n & 2) {
+        *reinterpret_cast<uint16_t *>(p) = (uint16_t)v.x;
+        v.x >>= 16;
+        p += 2;
+    }
+    if (n & 1) *reinterpret_cast<uint8_t *>(p) = (uint8_t)v.x;
 }
 
-__device__ __forceinline__ void chunk_store(uint8_t *dst, uint32_t lo, uint32_t hi, uint4 w0, uint4 w1,
-                                            uint32_t r) {
-    uint4 v = window16(w0, w1, r);
-    if (lo == 0 && hi == 16)
-        *reinterpret_cast<uint4 *>(dst) = v;
-    else
-        store_partial16(dst, v, lo, hi);
-}
-
-// Lane of the group's first job whose inclusive prefix count exceeds k.
+// Lane of the group's o-th set bit of m (o < popc(m)).
 template <int G>
-__device__ __forceinline__ int owner_lane(const Group<G> &g, uint32_t incl, uint32_t k) {
-    int lo = 0, hi = G - 1;
+__device__ __forceinline__ int select_bit(unsigned m, uint32_t o) {
+    int pos = 0;
 #pragma unroll
-    for (int st = G; st > 1; st >>= 1) {
-        const int mid = (lo + hi) >> 1;
-        const uint32_t v = g.shfl(incl, mid);
-        if (v > k) hi = mid; else lo = mid + 1;
-    }
-    return lo;
+    for (int w = G / 2; w; w >>= 1)
+        if ((uint32_t)__popc(m & ((1u << (pos + w)) - 1u)) <= o) pos += w;
+    return pos;
 }
 
-// Packed group copy, chunks in job order: the jobs' aligned 16-byte output
-// chunks (c per lane, inclusive prefix incl, total in all) are numbered in
-// lane order and dealt to the group's lanes, U per lane per round, loads
-// issued before stores.
-template <int G, int U, bool SMEM, bool RO = false>
-__device__ __forceinline__ void copy_chunks_in_order(const Group<G> &g, uint8_t *out, uint64_t d,
-                                                     const uint8_t *s, uint32_t n, uint32_t c,
-                                                     uint32_t incl, uint32_t total) {
-    for (uint32_t base = 0; base < total; base += (uint32_t)G * U) {
-        uint8_t *dst[U];
-        uint32_t lohi[U];
-        uint4 a[U], b[U];
-        uint32_t r[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            lohi[u] = 0u;
-            const uint32_t k0 = base + (uint32_t)u * G;  // the same on every lane
-            if (k0 >= total) continue;
-            const uint32_t k = k0 + (uint32_t)g.lane;
-            const int j = owner_lane<G>(g, incl, k);
-            const uint32_t ej = g.shfl(incl - c, j);
-            const uint64_t dj = g.shfl(d, j);
-            const uint8_t *sj = reinterpret_cast<const uint8_t *>(
-                g.shfl(reinterpret_cast<unsigned long long>(s), j));
-            const uint32_t nj = g.shfl(n, j);
-            const uint64_t A = ((dj >> 4) + (k - ej)) << 4;
-            const uint64_t blo = dj > A ? dj : A;
-            const uint64_t bhi = (dj + nj) < (A + 16) ? (dj + nj) : (A + 16);
-            const uint32_t clo = (uint32_t)(blo - A), chi = (uint32_t)(bhi - A);
-            dst[u] = out + A;
-            if (k < total) {
-                lohi[u] = clo | (chi << 8);
-                chunk_load<SMEM, RO>(sj + (blo - dj), clo, chi, a[u], b[u], r[u]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; u++)
-            if (lohi[u]) chunk_store(dst[u], lohi[u] & 0xff, lohi[u] >> 8, a[u], b[u], r[u]);
+// The full 16-byte output chunks of the group's jobs (P: output address of
+// a job's first full chunk, S: source address of its first byte, c: chunks),
+// numbered in lane order and dealt to the lanes, U per lane per round, loads
+// before stores.  The job of a chunk is found from the starts of the jobs
+// within the slot of G chunks: one bit per start, or-reduced over the group,
+// counted up to the own lane.
+template <int G, int U, bool RO>
+__device__ __forceinline__ void copy_full_chunks(const Group<G> &g, uintptr_t P, uintptr_t S, uint32_t c,
+                                                 unsigned have) {
+    if (have & (have + 1u)) {  // bring the jobs to the lowest lanes
+        const uint32_t nj = __popc(have);
+        const bool v = (uint32_t)g.lane < nj;
+        const int from = v ? select_bit<G>(have, (uint32_t)g.lane) : 0;
+        P = (uintptr_t)g.shfl((unsigned long long)P, from);
+        S = (uintptr_t)g.shfl((unsigned long long)S, from);
+        c = g.shfl(c, from);
+        if (!v) c = 0;
     }
-}
-
-// Packed group copy, full chunks first: every job's full 16-byte chunks
-// (in lane order), then the partial head and tail chunks, dealt as above.
-// A slot of G chunks is then all full 16-byte stores or all narrow partial
-// stores, except the one slot at the boundary, so the narrow-store path
-// runs once per G partial chunks instead of in every slot.
-template <int G, int U, bool SMEM>
-__device__ __forceinline__ void copy_chunks_full_first(const Group<G> &g, uint8_t *out, uint64_t d,
-                                                       const uint8_t *s, uint32_t n, uint32_t c) {
-    const uint64_t e = d + n;
-    // chunk 0 is partial unless it starts at d and is filled; the last
-    // chunk (if another) is partial unless the job ends on a boundary
-    const uint32_t p0 = (n && ((d & 15) || (c == 1 && (e & 15)))) ? 1u : 0u;
-    const uint32_t np = p0 + ((c >= 2 && (e & 15)) ? 1u : 0u);
-    const uint32_t nf = c - np;
-    const uint32_t inclF = g.scan_incl(nf);
-    const uint32_t inclP = g.scan_incl(np);
-    const uint32_t exF = inclF - nf, exP = inclP - np;
-    const uint32_t cf = c | (p0 << 31);  // c < 2^21 (jobs are shorter than 2^25 bytes)
-    const uint32_t F = g.shfl(inclF, G - 1);
-    const uint32_t total = F + g.shfl(inclP, G - 1);
-    for (uint32_t base = 0; base < total; base += (uint32_t)G * U) {
-        uint8_t *dst[U];
-        uint32_t lohi[U];
-        uint4 a[U], b[U];
-        uint32_t r[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            lohi[u] = 0u;
-            const uint32_t k0 = base + (uint32_t)u * G;  // the same on every lane
-            if (k0 >= total) continue;
-            const uint32_t k = k0 + (uint32_t)g.lane;
-            const bool full = k < F;
-            // owner among the full chunks, the partial ones, or both (only
-            // in the slot that straddles the boundary); branches are uniform
-            int j;
-            uint32_t exj;
-            if (k0 + G <= F) {
-                j = owner_lane<G>(g, inclF, k);
-                exj = g.shfl(exF, j);
-            } else if (k0 >= F) {
-                j = owner_lane<G>(g, inclP, k - F);
-                exj = g.shfl(exP, j);
-            } else {
-                const int jf = owner_lane<G>(g, inclF, k);
-                const int jp = owner_lane<G>(g, inclP, k - F);
-                j = full ? jf : jp;
-                const uint32_t xf = g.shfl(exF, j), xp = g.shfl(exP, j);
-                exj = full ? xf : xp;
-            }
-            const uint64_t dj = g.shfl(d, j);
-            const uint8_t *sj = reinterpret_cast<const uint8_t *>(
-                g.shfl(reinterpret_cast<unsigned long long>(s), j));
-            const uint32_t nj = g.shfl(n, j);
-            const uint32_t cfj = g.shfl(cf, j);
-            const uint32_t cj = cfj & 0x7fffffffu, p0j = cfj >> 31;
-            // chunk index within the job: full chunks are [p0j, p0j + nf);
-            // the partial ones are chunk 0 (if p0j) then chunk cj - 1
-            const uint32_t idx = full ? p0j + (k - exj) : ((k - F == exj && p0j) ? 0u : cj - 1u);
-            const uint64_t A = ((dj >> 4) + idx) << 4;
-            const uint64_t blo = dj > A ? dj : A;
-            const uint64_t bhi = (dj + nj) < (A + 16) ? (dj + nj) : (A + 16);
-            const uint32_t clo = (uint32_t)(blo - A), chi = (uint32_t)(bhi - A);
-            dst[u] = out + A;
-            if (k < total) {
-                lohi[u] = clo | (chi << 8);
-                chunk_load<SMEM>(sj + (blo - dj), clo, chi, a[u], b[u], r[u]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; u++)
-            if (lohi[u]) chunk_store(dst[u], lohi[u] & 0xff, lohi[u] >> 8, a[u], b[u], r[u]);
-    }
-}
-
-// Packed group copies.  Each lane holds one job (d: output offset, s:
-// source pointer, n: length; n == 0 for none), cut into aligned 16-byte
-// output chunks.  group_copy deals the chunks in job order and suits short
-// jobs (literal runs, in-block matches of wave 0); group_copy_full_first
-// deals every job's full chunks first, for match copies of a few chunks or
-// more.  Jobs must be independent: no job's source may overlap another
-// job's output in the same call.
-template <int G, int U, bool SMEM = false, bool RO = false>
-__device__ __forceinline__ void group_copy(const Group<G> &g, uint8_t *out, uint64_t d,
-                                           const uint8_t *s, uint32_t n) {
-    const uint32_t c = n ? (uint32_t)(((d + n - 1) >> 4) - (d >> 4) + 1) : 0u;
     const uint32_t incl = g.scan_incl(c);
     const uint32_t total = g.shfl(incl, G - 1);
-    copy_chunks_in_order<G, U, SMEM, RO>(g, out, d, s, n, c, incl, total);
+    const uint32_t ex = incl - c;
+    P -= 16 * (uint64_t)ex;
+    S -= 16 * (uint64_t)ex;
+    uint32_t before = 0;  // jobs that start in earlier slots
+    for (uint32_t base = 0; base < total; base += (uint32_t)G * U) {
+        uintptr_t dst[U];
+        uint4 a[U], b[U];
+        uint32_t r[U];
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const uint32_t k0 = base + (uint32_t)u * G;  // the same on every lane
+            dst[u] = 0;
+            if (k0 >= total) continue;
+            const uint32_t k = k0 + (uint32_t)g.lane;
+            const uint32_t t = ex - k0;
+            const unsigned starts = g.or_all((c && t < (uint32_t)G) ? 1u << t : 0u);
+            const int j = (int)(before + (uint32_t)__popc(starts & ((2u << g.lane) - 1u)) - 1u);
+            before += (uint32_t)__popc(starts);
+            const uintptr_t dj = (uintptr_t)g.shfl((unsigned long long)P, j) + 16 * (uint64_t)k;
+            const uintptr_t sj = (uintptr_t)g.shfl((unsigned long long)S, j) + 16 * (uint64_t)k;
+            if (k < total) {
+                dst[u] = dj;
+                r[u] = (uint32_t)sj & 15u;
+                const uintptr_t w = sj & ~(uintptr_t)15;
+                a[u] = ld_word<RO>(w);
+                if (r[u]) b[u] = ld_word<RO>(w + 16);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; u++)
+            if (dst[u]) *reinterpret_cast<uint4 *>(dst[u]) = window16(a[u], b[u], r[u]);
+    }
 }
 
-template <int G, int U, bool SMEM = false>
-__device__ __forceinline__ void group_copy_full_first(const Group<G> &g, uint8_t *out, uint64_t d,
-                                                      const uint8_t *s, uint32_t n) {
-    const uint32_t c = n ? (uint32_t)(((d + n - 1) >> 4) - (d >> 4) + 1) : 0u;
-    if (!g.ballot(n > 0)) return;
-    copy_chunks_full_first<G, U, SMEM>(g, out, d, s, n, c);
+// Packed group copy.  Each lane holds one job (d: output offset, s: source
+// pointer, n: length; n == 0 for none).  A job of at most 16 bytes is copied
+// by its own lane; of a longer one the lane copies the bytes before the
+// first and after the last 16-byte boundary of the output, and the full
+// chunks between are dealt to the whole group (copy_full_chunks).  Jobs must
+// be independent: no job's source may overlap another job's output in the
+// same call.  RO: the source is global memory that no thread writes during
+// the kernel.
+//
+// The copy is issue-bound, so it is built to take few instructions.  Against
+// a form that searched every chunk's job by shuffles and cut its partial
+// chunks from 64-bit fields (about 235 instructions for 32 chunks), whole
+// decodes on GB300: 32 MiB of word text at 6/8/10/12, flattened (pieces of
+// 3 bytes), 1217 -> 911 us; the 512 MiB copy sweep at L = 128 1096 -> 1038 us;
+// 64 MiB of FASTQ-like text at 12/16/24/32 244 -> 230 us.
+template <int G, int U, bool RO = false>
+__device__ __forceinline__ void group_copy(const Group<G> &g, uint8_t *out, uint64_t d, const uint8_t *s,
+                                           uint32_t n) {
+    const uintptr_t p = reinterpret_cast<uintptr_t>(out) + d, q = reinterpret_cast<uintptr_t>(s);
+    const uint32_t head = n <= 16 ? n : (0u - (uint32_t)p) & 15u;
+    const uint32_t rest = n - head;           // of a job longer than 16 bytes
+    const uint32_t tail = rest & 15u, c = rest >> 4;
+    uint4 hv = make_uint4(0, 0, 0, 0), tv = hv;
+    if (head) hv = load_bytes<RO>(q, head);
+    if (tail) tv = load_bytes<RO>(q + n - tail, tail);
+    const unsigned have = g.ballot(c > 0);
+    if (have) copy_full_chunks<G, U, RO>(g, p + head, q + head, c, have);
+    if (g.ballot(head > 0)) store_bytes(p, hv, head);
+    if (g.ballot(tail > 0)) store_bytes(p + n - tail, tv, tail);
 }
 
 // Bytes [r, r + 16) of a || b for a shift r that is the same on every lane
