@@ -386,45 +386,43 @@ __global__ void __launch_bounds__(kThreads, STAGED ? 2 : 3)
 
 // ------------------------------------------------------ wave schedule
 
-// Copy one wave's worklist.  Group k owns the segments (runs of one block)
-// that start in [k*T, (k+1)*T); a segment crossing the range end is
-// finished by the group that started it.
-template <int G, int ITEMS>
-__global__ void __launch_bounds__(kWaveThreads, kWaveMinCtas) k_wave_copy(const uint4 *__restrict__ tri, uint64_t n,
-                                                        uint8_t *out, uint32_t log2bs) {
-    Group<G> g;
-    constexpr uint64_t T = (uint64_t)G * ITEMS;
-    griddep_launch_dependents();
-    const uint64_t gid = (blockIdx.x * (uint64_t)kWaveThreads + threadIdx.x) / G;
-    const uint64_t a = gid * T;
-    if (a >= n) return;
-    const uint64_t e = a + T < n ? a + T : n;
-    // first cut point in [a, e): a segment start, or any triplet of a
-    // segment without an internal chain
-    uint64_t s = ~0ULL;
-    for (uint64_t w = a; w < e; w += G) {
-        const uint64_t i = w + g.lane;
-        bool st = false;
-        if (i < e) {
-            const uint4 ti = __ldg(tri + i);
-            const uint64_t bi = tri_dst(ti) >> log2bs;
-            st = (i == 0) || tri_cut(ti) || (bi != (tri_dst(__ldg(tri + i - 1)) >> log2bs));
-        }
-        const unsigned m = g.ballot(st);
-        if (m) { s = w + (uint64_t)(__ffs(m) - 1); break; }
+// Copy one window of a wave's worklist (n triplets): the group whose window
+// starts at triplet a.  A window of cuttable triplets (segments without an
+// internal chain, marked at upload) is copied as it stands: no dependency
+// test, no look at its neighbours.  Otherwise the group owns the segments
+// (runs of one block) that start in its window, and cuttable triplets in
+// it; a segment crossing the window's end is finished by the group that
+// started it.  PDL: sources are read after griddep_wait only.
+template <int G, bool PDL>
+__device__ __forceinline__ void wave_window(const Group<G> &g, const uint4 *__restrict__ tri, uint64_t n, uint64_t a,
+                                            uint8_t *out, uint32_t log2bs) {
+    const uint4 z4 = make_uint4(0, 0, 0, 0);
+    const uint4 t0 = a + g.lane < n ? __ldg(tri + a + g.lane) : z4;
+    if (!g.ballot(a + g.lane < n && !tri_cut(t0))) {
+        if (PDL) griddep_wait();
+        group_copy<G, kUnrollCopy>(g, out, tri_dst(t0), out + tri_src(t0), tri_len(t0));
+        return;
     }
-    if (s == ~0ULL) return;
+    const uint64_t e = a + G < n ? a + G : n;
+    // first cut point in [a, e): a segment start, or a cuttable triplet
+    bool st0 = false;
+    if (a + g.lane < e)
+        st0 = a + g.lane == 0 || tri_cut(t0) ||
+              (tri_dst(t0) >> log2bs) != (tri_dst(__ldg(tri + a + g.lane - 1)) >> log2bs);
+    const unsigned m0 = g.ballot(st0);
+    if (!m0) return;
+    const uint64_t s = a + (uint64_t)(__ffs(m0) - 1);
     // the next window's triplets are loaded while the current one is copied;
     // lane 0 takes the block of the triplet before its window from the last
     // lane of the previous window (every lane of which was valid)
-    uint4 nt = s + g.lane < n ? __ldg(tri + s + g.lane) : make_uint4(0, 0, 0, 0);
+    uint4 nt = s + g.lane < n ? __ldg(tri + s + g.lane) : z4;
     uint64_t prev_blk = ~0ULL;
     // the worklist was written at upload; the sources, by earlier waves
-    griddep_wait();
+    if (PDL) griddep_wait();
     for (uint64_t cur = s; cur < n; cur += G) {
         const uint64_t i = cur + g.lane;
         const bool v = i < n;
-        const uint4 t = v ? nt : make_uint4(0, 0, 0, 0);
+        const uint4 t = v ? nt : z4;
         if (cur + G + g.lane < n) nt = __ldg(tri + cur + G + g.lane);
         const uint64_t d = tri_dst(t), sr = tri_src(t);
         const uint32_t len = v ? tri_len(t) : 0u;
@@ -452,6 +450,17 @@ __global__ void __launch_bounds__(kWaveThreads, kWaveMinCtas) k_wave_copy(const 
     }
 }
 
+// One wave's worklist, one window of G triplets per group (the most resident
+// groups: two or four windows each were 2-8% slower).
+template <int G>
+__global__ void __launch_bounds__(kWaveThreads, kWaveMinCtas) k_wave_copy(const uint4 *__restrict__ tri, uint64_t n,
+                                                                          uint8_t *out, uint32_t log2bs) {
+    Group<G> g;
+    griddep_launch_dependents();
+    const uint64_t a = (blockIdx.x * (uint64_t)kWaveThreads + threadIdx.x) / G * G;
+    if (a < n) wave_window<G, true>(g, tri, n, a, out, log2bs);
+}
+
 template <int G>
 int launch_waves(aclz_handle *h, uint8_t *out, cudaStream_t st, cudaEvent_t phase) {
     constexpr int gpc = kThreads / G;  // groups per CTA
@@ -460,17 +469,14 @@ int launch_waves(aclz_handle *h, uint8_t *out, cudaStream_t st, cudaEvent_t phas
                                                               h->d_blk_lit, h->d_slot, nullptr, out,
                                                               h->n_blocks, h->log2_bs, nullptr, nullptr, 0);
     if (phase) cudaEventRecord(phase, st);
-    // one window of G triplets per group: the most resident groups per wave
-    constexpr int ITEMS = 1;
     for (uint32_t w = 1; w < h->n_waves; w++) {
         const uint64_t a = h->wave_start[w], n = h->wave_start[w + 1] - a;
         if (!n) continue;
-        const uint64_t per = (uint64_t)G * ITEMS;
-        const uint64_t groups = (n + per - 1) / per;
+        const uint64_t groups = (n + G - 1) / G;
         constexpr int gpcw = kWaveThreads / G;
         const unsigned grid = (unsigned)((groups + gpcw - 1) / gpcw);
         const uint4 *t = (const uint4 *)h->d_tri + a;
-        auto k = k_wave_copy<G, ITEMS>;
+        auto k = k_wave_copy<G>;
         // programmatic stream serialization: this wave's CTAs may start (and
         // load their worklist) while the previous kernel's last CTAs finish
         cudaLaunchConfig_t lc = {};
