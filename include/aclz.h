@@ -218,7 +218,9 @@ int aclz_acle_encode(const void *host_container, uint64_t n, int threads, void *
  * (its 0/1 tags are not a legal wave tagging). */
 int aclz_export(const aclz_handle *h, void *host_out, uint64_t cap, uint64_t *out_size);
 
-/* Free a handle and its device memory (after its work has completed). */
+/* Free a handle and its device memory (after its work has completed; the
+ * call waits for the device).  The library keeps at most 512 MiB of freed
+ * device memory for its next allocations. */
 int aclz_free(aclz_handle *h);
 
 /* Sizes of the uploaded stream and of its decode schedule: total_len,

@@ -16,6 +16,7 @@
 
 #include "aclz_device.cuh"
 #include "aclz_internal.h"
+#include "aclz_mem.h"
 
 using namespace aclz;
 
@@ -157,9 +158,9 @@ int fill_from_acle(aclz_handle *h, const View &v, const void *ctx, void *stream)
         return rc == ACLZ_OK;
     };
     const uint64_t nt = a.tiles.size();
-    if (ck(cudaMalloc(&d_pay, a.pay_bytes ? a.pay_bytes : 16)) &&
-        ck(cudaMalloc(&d_td, sizeof(TileDesc) * (nt ? nt : 1))) &&
-        ck(cudaMalloc(&d_planes, a.plane_bytes ? a.plane_bytes : 16)) && ck(cudaMalloc(&d_err, 4)) &&
+    if (ck(dev_alloc((void **)&d_pay, a.pay_bytes ? a.pay_bytes : 16, st)) &&
+        ck(dev_alloc((void **)&d_td, sizeof(TileDesc) * (nt ? nt : 1), st)) &&
+        ck(dev_alloc((void **)&d_planes, a.plane_bytes ? a.plane_bytes : 16, st)) && ck(dev_alloc((void **)&d_err, 4, st)) &&
         ck(cudaMemsetAsync(d_err, 0, 4, st)) &&
         (!a.pay_bytes || ck(cudaMemcpyAsync(d_pay, a.pay, a.pay_bytes, cudaMemcpyHostToDevice, st))) &&
         (!nt || ck(cudaMemcpyAsync(d_td, a.tiles.data(), sizeof(TileDesc) * nt, cudaMemcpyHostToDevice, st)))) {
@@ -183,7 +184,7 @@ int fill_from_acle(aclz_handle *h, const View &v, const void *ctx, void *stream)
     }
     cudaStreamSynchronize(st);
     for (void *q : {(void *)d_pay, (void *)d_td, (void *)d_planes, (void *)d_err})
-        if (q) cudaFree(q);
+        dev_free(q, st);
     return rc;
 }
 

@@ -26,6 +26,7 @@
 
 #include "aclz_device.cuh"
 #include "aclz_internal.h"
+#include "aclz_mem.h"
 
 using namespace aclz;
 
@@ -199,17 +200,6 @@ __global__ void k_fl_segs(const uint64_t *__restrict__ blk_tok, const uint32_t *
     }
 }
 
-struct Dev {
-    void *p = nullptr;
-    ~Dev() {
-        if (p) cudaFree(p);
-    }
-    template <class T>
-    T *as() const {
-        return (T *)p;
-    }
-};
-
 int rc_of(cudaError_t e) {
     if (e == cudaSuccess) return ACLZ_OK;
     note_cuda_error((int)e);
@@ -227,7 +217,7 @@ unsigned grid_for(uint64_t n) { return (unsigned)std::min<uint64_t>((n + 255) / 
 // Pieces of every deferred match after up to max_rounds doubling rounds
 // (fewer when no piece overlaps deferred bytes any more: final).
 struct Pieces {
-    Dev defscan, P, owner, off, dmk;
+    Scratch defscan, P, owner, off, dmk;
     uint64_t np = 0, D = 0;
     unsigned long long def_bytes = 0;
     bool final = false;
@@ -237,9 +227,9 @@ int make_pieces(aclz_handle *h, cudaStream_t st, int max_rounds, Pieces &pc) {
     const uint64_t nt = h->n_tokens;
     const uint32_t nb = h->n_blocks;
     // deferred matches in token order: defscan[t] = rank, defscan[nt] = D
-    Dev work;
-    FCK(cudaMalloc(&pc.defscan.p, 4 * (nt + 1)));
-    FCK(cudaMalloc(&work.p, 64));
+    Scratch work;
+    FCK(pc.defscan.alloc(4 * (nt + 1), st));
+    FCK(work.alloc(64, st));
     uint32_t *d_any = work.as<uint32_t>(), *d_total = work.as<uint32_t>() + 1;
     unsigned long long *d_bytes = (unsigned long long *)(work.as<char>() + 8);
     FCK(cudaMemsetAsync(work.p, 0, 64, st));
@@ -254,10 +244,10 @@ int make_pieces(aclz_handle *h, cudaStream_t st, int max_rounds, Pieces &pc) {
     if (D == 0) return ACLZ_OK;
     // round 0: one piece per match
     uint64_t np = D;
-    FCK(cudaMalloc(&pc.P.p, 16 * np));
-    FCK(cudaMalloc(&pc.owner.p, 4 * np));
-    FCK(cudaMalloc(&pc.off.p, 8 * (D + 1)));
-    FCK(cudaMalloc(&pc.dmk.p, 8 * D));
+    FCK(pc.P.alloc(16 * np, st));
+    FCK(pc.owner.alloc(4 * np, st));
+    FCK(pc.off.alloc(8 * (D + 1), st));
+    FCK(pc.dmk.alloc(8 * D, st));
     FCK(cudaMemcpyAsync(pc.off.as<uint64_t>() + D, &np, 8, cudaMemcpyHostToDevice, st));
     k_fl_init<<<(nb + 7) / 8, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst,
                                              pc.defscan.as<uint32_t>(), nb, h->log2_bs, pc.P.as<uint4>(),
@@ -270,8 +260,8 @@ int make_pieces(aclz_handle *h, cudaStream_t st, int max_rounds, Pieces &pc) {
         if (round > 64) return ACLZ_E_UNSUPPORTED;
         FlatIdx ix{(const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, pc.defscan.as<uint32_t>(), pc.P.as<uint4>(),
                    pc.off.as<uint64_t>(), h->log2_bs};
-        Dev cnt;
-        FCK(cudaMalloc(&cnt.p, 4 * np + 4));
+        Scratch cnt;
+        FCK(cnt.alloc(4 * np + 4, st));
         FCK(cudaMemsetAsync(d_any, 0, 4, st));
         k_fl_count<<<grid_for(np), 256, 0, st>>>(ix, np, cnt.as<uint32_t>(), d_any);
         FCK(cudaGetLastError());
@@ -288,10 +278,10 @@ int make_pieces(aclz_handle *h, cudaStream_t st, int max_rounds, Pieces &pc) {
         FCK(cudaMemcpyAsync(&total, d_total, 4, cudaMemcpyDeviceToHost, st));
         FCK(cudaStreamSynchronize(st));
         if (total >= 0xfffffff0u) return ACLZ_E_UNSUPPORTED;
-        Dev P2, owner2, off2;
-        FCK(cudaMalloc(&P2.p, 16 * (uint64_t)total));
-        FCK(cudaMalloc(&owner2.p, 4 * (uint64_t)total));
-        FCK(cudaMalloc(&off2.p, 8 * (D + 1)));
+        Scratch P2, owner2, off2;
+        FCK(P2.alloc(16 * (uint64_t)total, st));
+        FCK(owner2.alloc(4 * (uint64_t)total, st));
+        FCK(off2.alloc(8 * (D + 1), st));
         k_fl_emit<<<grid_for(np), 256, 0, st>>>(ix, np, cnt.as<uint32_t>(), pc.owner.as<uint32_t>(),
                                                  P2.as<uint4>(), owner2.as<uint32_t>());
         k_fl_off<<<grid_for(D + 1), 256, 0, st>>>(pc.off.as<uint64_t>(), D, np, cnt.as<uint32_t>(), d_total,
@@ -325,17 +315,17 @@ extern "C" int aclz_flatten(aclz_handle *h, void *stream) {
         h->flat = true;
         return ACLZ_OK;
     }
-    Dev &defscan = pc.defscan, &P = pc.P, &owner = pc.owner, &off = pc.off, &dmk = pc.dmk;
+    Scratch &defscan = pc.defscan, &P = pc.P, &owner = pc.owner, &off = pc.off, &dmk = pc.dmk;
     const uint64_t np = pc.np;
     const unsigned long long def_bytes = pc.def_bytes;
     // the two-wave schedule: triplets, per-block segments, pending bits
-    Dev tri, bflag, seg, pending, done;
-    FCK(cudaMalloc(&tri.p, 16 * np));
+    Scratch tri, bflag, seg, pending, done;
+    FCK(tri.alloc(16 * np, st));
     k_fl_tri<<<grid_for(np), 256, 0, st>>>(P.as<uint4>(), owner.as<uint32_t>(), dmk.as<uint64_t>(), np,
                                             tri.as<uint4>());
-    FCK(cudaMalloc(&bflag.p, 4 * ((uint64_t)nb + 1)));
-    FCK(cudaMalloc(&pending.p, 8 * (uint64_t)nb));
-    FCK(cudaMalloc(&done.p, 8 * (uint64_t)nb));
+    FCK(bflag.alloc(4 * ((uint64_t)nb + 1), st));
+    FCK(pending.alloc(8 * (uint64_t)nb, st));
+    FCK(done.alloc(8 * (uint64_t)nb, st));
     k_fl_blocks<<<grid_for(nb), 256, 0, st>>>(h->d_blk_tok, defscan.as<uint32_t>(), off.as<uint64_t>(), nb,
                                                bflag.as<uint32_t>(), pending.as<uint64_t>());
     FCK(cudaGetLastError());
@@ -343,16 +333,17 @@ extern "C" int aclz_flatten(aclz_handle *h, void *stream) {
     uint32_t nseg = 0;
     FCK(cudaMemcpyAsync(&nseg, bflag.as<uint32_t>() + nb, 4, cudaMemcpyDeviceToHost, st));
     FCK(cudaStreamSynchronize(st));
-    FCK(cudaMalloc(&seg.p, 16 * (uint64_t)(nseg ? nseg : 1)));
+    FCK(seg.alloc(16 * (uint64_t)(nseg ? nseg : 1), st));
     k_fl_segs<<<grid_for(nb), 256, 0, st>>>(h->d_blk_tok, defscan.as<uint32_t>(), off.as<uint64_t>(),
                                              bflag.as<uint32_t>(), nb, seg.as<uint4>());
     FCK(cudaGetLastError());
     FCK(cudaStreamSynchronize(st));
     // install
-    cudaFree(h->d_tri);
-    cudaFree(h->d_seg);
-    cudaFree(h->d_pending);
-    cudaFree(h->d_done);
+    cudaDeviceSynchronize();
+    dev_free(h->d_tri, st);
+    dev_free(h->d_seg, st);
+    dev_free(h->d_pending, st);
+    dev_free(h->d_done, st);
     h->d_tri = tri.p;
     tri.p = nullptr;
     h->d_seg = seg.p;
@@ -435,8 +426,8 @@ extern "C" int aclz_reshape(aclz_handle *h, uint32_t rounds, void *stream) {
     Pieces pc;
     if (int rc = make_pieces(h, st, (int)rounds, pc)) return rc;
     if (pc.D == 0) return ACLZ_OK;
-    Dev cnt, tok2, blk2;
-    FCK(cudaMalloc(&cnt.p, 4 * (nt + 1)));
+    Scratch cnt, tok2, blk2;
+    FCK(cnt.alloc(4 * (nt + 1), st));
     k_rs_count<<<grid_for(nt), 256, 0, st>>>((const uint4 *)h->d_tok, pc.defscan.as<uint32_t>(), pc.off.as<uint64_t>(),
                                               nt, cnt.as<uint32_t>());
     FCK(cudaGetLastError());
@@ -445,15 +436,15 @@ extern "C" int aclz_reshape(aclz_handle *h, uint32_t rounds, void *stream) {
     FCK(cudaMemcpyAsync(&nt2, cnt.as<uint32_t>() + nt, 4, cudaMemcpyDeviceToHost, st));
     FCK(cudaStreamSynchronize(st));
     if (nt2 >= 0xfffffff0u) return ACLZ_E_UNSUPPORTED;
-    FCK(cudaMalloc(&tok2.p, 16 * (uint64_t)nt2));
-    FCK(cudaMalloc(&blk2.p, 8 * ((uint64_t)nb + 1)));
+    FCK(tok2.alloc(16 * (uint64_t)nt2, st));
+    FCK(blk2.alloc(8 * ((uint64_t)nb + 1), st));
     k_rs_emit<<<grid_for(nt), 256, 0, st>>>((const uint4 *)h->d_tok, pc.defscan.as<uint32_t>(), pc.off.as<uint64_t>(),
                                              pc.P.as<uint4>(), cnt.as<uint32_t>(), nt, tok2.as<uint4>());
     k_rs_blk<<<grid_for(nb + 1), 256, 0, st>>>(h->d_blk_tok, cnt.as<uint32_t>(), nb, nt2, blk2.as<uint64_t>());
     FCK(cudaGetLastError());
-    FCK(cudaStreamSynchronize(st));
-    cudaFree(h->d_tok);
-    cudaFree(h->d_blk_tok);
+    FCK(cudaDeviceSynchronize());
+    dev_free(h->d_tok, st);
+    dev_free(h->d_blk_tok, st);
     h->d_tok = tok2.p;
     tok2.p = nullptr;
     h->d_blk_tok = blk2.as<uint64_t>();

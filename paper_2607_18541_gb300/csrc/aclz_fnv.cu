@@ -25,6 +25,7 @@
 
 #include "aclz_device.cuh"
 #include "aclz_internal.h"
+#include "aclz_mem.h"
 
 using namespace aclz;
 
@@ -274,14 +275,14 @@ extern "C" int aclz_fnv(const void *d_buf, uint64_t n, uint64_t *out_hash, void 
     cudaStream_t st = (cudaStream_t)stream;
     const uint64_t nchunks = (n + kChunk - 1) / kChunk;
     uint64_t *scratch = nullptr;
-    cudaError_t e = cudaMallocAsync((void **)&scratch, 8 * (nchunks + 1), st);
+    cudaError_t e = dev_alloc((void **)&scratch, 8 * (nchunks + 1), st);
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? ACLZ_E_NOMEM : ACLZ_E_CUDA;
     int rc = fnv_enqueue((const uint8_t *)d_buf, n, scratch, st);
     uint64_t hv = 0;
     if (rc == ACLZ_OK &&
         cudaMemcpyAsync(&hv, scratch + nchunks, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         rc = ACLZ_E_CUDA;
-    cudaFreeAsync(scratch, st);
+    dev_free(scratch, st);
     if (cudaStreamSynchronize(st) != cudaSuccess) rc = ACLZ_E_CUDA;
     if (rc == ACLZ_OK) *out_hash = hv;
     return rc;

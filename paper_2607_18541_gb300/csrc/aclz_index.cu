@@ -19,6 +19,7 @@
 
 #include "aclz_device.cuh"
 #include "aclz_internal.h"
+#include "aclz_mem.h"
 
 using namespace aclz;
 
@@ -662,13 +663,6 @@ __global__ void k_gather_starts(const uint32_t *base, uint64_t nb, uint32_t nw1,
 }
 
 // ---------------------------------------------------------- host helpers
-struct DevBuf {
-    void *p = nullptr;
-    ~DevBuf() {
-        if (p) cudaFree(p);
-    }
-};
-
 int cuda_rc(cudaError_t e) {
     if (e == cudaSuccess) return ACLZ_OK;
     return e == cudaErrorMemoryAllocation ? ACLZ_E_NOMEM : ACLZ_E_CUDA;
@@ -688,13 +682,13 @@ int aclz::device_excl_scan(uint32_t *d, uint64_t n, uint32_t *d_total, void *str
     cudaStream_t st = (cudaStream_t)stream;
     const uint64_t ntile = (n + kScanTile - 1) / kScanTile;
     uint32_t *part = nullptr;
-    cudaError_t e = cudaMallocAsync((void **)&part, sizeof(uint32_t) * (ntile + 1), st);
+    cudaError_t e = dev_alloc((void **)&part, sizeof(uint32_t) * (ntile + 1), st);
     if (e != cudaSuccess) return cuda_rc(e);
     if (ntile) k_scan_reduce<<<(unsigned)ntile, kScanThreads, 0, st>>>(d, n, part);
     k_scan_parts<<<1, kScanThreads, 0, st>>>(part, ntile);
     if (ntile) k_scan_apply<<<(unsigned)ntile, kScanThreads, 0, st>>>(d, n, part);
     cudaMemcpyAsync(d_total, part + ntile, sizeof(uint32_t), cudaMemcpyDeviceToDevice, st);
-    cudaFreeAsync(part, st);
+    dev_free(part, st);
     return cuda_rc(cudaGetLastError());
 }
 
@@ -709,8 +703,8 @@ bool relax_tags(aclz_handle *h, uint32_t *d_tags, uint32_t *d_maxtag, cudaStream
     const uint32_t nb = h->n_blocks;
     const uint64_t nt = h->n_tokens;
     if (!nb) return true;
-    DevBuf flags;
-    if (cudaMalloc(&flags.p, 4 * kRelaxBatch) != cudaSuccess) return false;
+    Scratch flags;
+    if (flags.alloc(4 * kRelaxBatch, st) != cudaSuccess) return false;
     uint32_t *changed = (uint32_t *)flags.p;
     if (cudaMemsetAsync(d_tags, 0, 4 * (nt ? nt : 1), st) != cudaSuccess) return false;
     const unsigned wblocks = (nb + 7) / 8;
@@ -746,18 +740,18 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     int rc = ACLZ_OK;
     for (void **pp : {(void **)&h->d_tokdst, (void **)&h->d_toklit, (void **)&h->d_slot, &h->d_tri, &h->d_seg,
                       &h->d_ranges, (void **)&h->d_pending, (void **)&h->d_done}) {
-        if (*pp) cudaFree(*pp);
+        dev_free(*pp, st);
         *pp = nullptr;
     }
     h->n_seg = h->n_ranges = 0;
     h->n_deferred = 0;
-    CK(cudaMalloc((void **)&h->d_tokdst, 4 * (nt ? nt : 1)));
-    CK(cudaMalloc((void **)&h->d_toklit, 4 * (nt ? nt : 1)));
-    CK(cudaMalloc((void **)&h->d_slot, 4 * (nt ? nt : 1)));
+    CK(dev_alloc((void **)&h->d_tokdst, 4 * (nt ? nt : 1), st));
+    CK(dev_alloc((void **)&h->d_toklit, 4 * (nt ? nt : 1), st));
+    CK(dev_alloc((void **)&h->d_slot, 4 * (nt ? nt : 1), st));
     CK(cudaMemsetAsync(h->d_err, 0, 64, st));
     // scratch words: [0] err (handle), work: maxtag, counter, total, first_bad
-    DevBuf work;
-    CK(cudaMalloc(&work.p, 64));
+    Scratch work;
+    CK(work.alloc(64, st));
     uint32_t *d_maxtag = (uint32_t *)work.p, *d_ctr = d_maxtag + 1, *d_total = d_maxtag + 2;
     // words: [0] max tag, [1] counter, [2] deferred total, [3] segment count,
     // [4] range count; bytes 32..39: first bad token
@@ -774,8 +768,8 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     CK(cudaStreamSynchronize(st));
     if (herr) { cleanup(); return ACLZ_E_CORRUPT; }
     // tags
-    DevBuf tags, done;
-    CK(cudaMalloc(&tags.p, 4 * (nt ? nt : 1)));
+    Scratch tags, done;
+    CK(tags.alloc(4 * (nt ? nt : 1), st));
     uint32_t *d_tags = (uint32_t *)tags.p;
     h->local_tags = false;
     if (has_tags) {
@@ -792,7 +786,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         k_store_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_tags, nt);
     } else {
         CK(cudaMemsetAsync(d_maxtag, 0, 4, st));
-        CK(cudaMalloc(&done.p, 4 * nb));
+        CK(done.alloc(4 * nb, st));
         CK(cudaMemsetAsync(done.p, 0, 4 * nb, st));
         int dev_sms = 0;
         cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, h->device);
@@ -825,9 +819,9 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     h->needs_flatten = maxtag > 0 && (uint64_t)maxtag * nb > (1ULL << 28);
     if (maxtag > 0 && !h->needs_flatten) {
         const uint64_t M = (uint64_t)maxtag * nb;
-        DevBuf cnt, starts;
-        CK(cudaMalloc(&cnt.p, 4 * M));
-        CK(cudaMalloc(&starts.p, 8 * (maxtag + 1)));
+        Scratch cnt, starts;
+        CK(cnt.alloc(4 * M, st));
+        CK(starts.alloc(8 * (maxtag + 1), st));
         CK(cudaMemsetAsync(cnt.p, 0, 4 * M, st));
         unsigned long long *d_def_bytes = (unsigned long long *)((char *)work.p + 40);
         CK(cudaMemsetAsync(d_def_bytes, 0, 8, st));
@@ -841,8 +835,8 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         // persistent-mode segments and ranges, from the segment bases
         // (before k_slots turns the bases into cursors)
         {
-            DevBuf flag;
-            CK(cudaMalloc(&flag.p, 4 * M));
+            Scratch flag;
+            CK(flag.alloc(4 * M, st));
             k_seg_flags<<<1024, 256, 0, st>>>((const uint32_t *)cnt.p, M, d_total, (uint32_t *)flag.p);
             uint32_t *d_nseg = d_total + 1;
             rc = device_excl_scan((uint32_t *)flag.p, M, d_nseg, st);
@@ -852,8 +846,8 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
             CK(cudaStreamSynchronize(st));
             h->n_seg = nseg;
             h->n_wave_words = (maxtag + 1 + 63) / 64;
-            CK(cudaMalloc(&h->d_seg, 16 * (size_t)(nseg ? nseg : 1)));
-            CK(cudaMalloc((void **)&h->d_pending, 8 * (size_t)nb * h->n_wave_words));
+            CK(dev_alloc(&h->d_seg, 16 * (size_t)(nseg ? nseg : 1), st));
+            CK(dev_alloc((void **)&h->d_pending, 8 * (size_t)nb * h->n_wave_words, st));
             k_segs_build<<<(nb + 255) / 256, 256, 0, st>>>((const uint32_t *)cnt.p, (const uint32_t *)flag.p,
                                                           d_total, nb, maxtag, h->n_wave_words,
                                                           (uint4 *)h->d_seg,
@@ -871,7 +865,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         CK(cudaStreamSynchronize(st));
         h->n_deferred = h->wave_start[h->n_waves];
         if (h->n_deferred) {
-            CK(cudaMalloc(&h->d_tri, 16 * h->n_deferred));
+            CK(dev_alloc(&h->d_tri, 16 * h->n_deferred, st));
             k_tri_build<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, h->d_slot,
                                                   nb, h->log2_bs, (uint4 *)h->d_tri);
             CK(cudaGetLastError());
@@ -883,10 +877,10 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     if (!h->d_pending) {  // no deferred matches: wave 0 finishes every block
         h->n_wave_words = 1;
         std::vector<uint64_t> ones(nb, 1ULL);
-        CK(cudaMalloc((void **)&h->d_pending, 8 * (size_t)nb));
+        CK(dev_alloc((void **)&h->d_pending, 8 * (size_t)nb, st));
         CK(cudaMemcpyAsync(h->d_pending, ones.data(), 8 * (size_t)nb, cudaMemcpyHostToDevice, st));
     }
-    CK(cudaMalloc((void **)&h->d_done, 8 * (size_t)nb * h->n_wave_words));
+    CK(dev_alloc((void **)&h->d_done, 8 * (size_t)nb * h->n_wave_words, st));
     CK(cudaStreamSynchronize(st));
     return ACLZ_OK;
 }
@@ -937,11 +931,11 @@ int upload_view(const View &v, uint32_t flags, void *stream, FillFn fill, const 
     }
     bt[nb] = nt;
     bl[nb] = v.n_literals;
-    CK(cudaMalloc(&h->d_tok, kTok * (nt ? nt : 1)));
-    CK(cudaMalloc((void **)&h->d_lit, v.n_literals + 32));
-    CK(cudaMalloc((void **)&h->d_blk_tok, 8 * (nb + 1)));
-    CK(cudaMalloc((void **)&h->d_blk_lit, 8 * (nb + 1)));
-    CK(cudaMalloc((void **)&h->d_err, 64));
+    CK(dev_alloc(&h->d_tok, kTok * (nt ? nt : 1), st));
+    CK(dev_alloc((void **)&h->d_lit, v.n_literals + 32, st));
+    CK(dev_alloc((void **)&h->d_blk_tok, 8 * (nb + 1), st));
+    CK(dev_alloc((void **)&h->d_blk_lit, 8 * (nb + 1), st));
+    CK(dev_alloc((void **)&h->d_err, 64, st));
     CK(cudaMemsetAsync(h->d_err, 0, 64, st));
     CK(cudaMemsetAsync(h->d_lit + v.n_literals, 0, 32, st));
     if (int rc = fill(h, v, ctx, stream); rc != ACLZ_OK) {
@@ -984,8 +978,13 @@ extern "C" int aclz_free(aclz_handle *h) {
     void *ps[] = {h->d_tok, h->d_lit,    h->d_blk_tok, h->d_blk_lit,      h->d_slot,      h->d_tokdst,
                   h->d_toklit, h->d_tri, h->d_err,     h->d_seg,          h->d_ranges,    h->d_seg_pieces,
                   h->d_seg_cnt, h->d_pending, h->d_done};
-    for (void *p : ps)
-        if (p) cudaFree(p);
+    // work in flight on any stream may still read them
+    int dev = h->device, cur = h->device;
+    cudaGetDevice(&cur);
+    if (cur != dev) cudaSetDevice(dev);
+    cudaDeviceSynchronize();
+    for (void *p : ps) dev_free(p, nullptr);
+    if (cur != dev) cudaSetDevice(cur);
     delete h;
     return ACLZ_OK;
 }
@@ -1028,8 +1027,9 @@ extern "C" int aclz_set_range_bytes(aclz_handle *h, uint32_t range_bytes, void *
     cudaStream_t st = (cudaStream_t)stream;
     h->range_bytes = range_bytes;
     h->range_T = range_matches(range_bytes, h->mean_deferred_len);
+    if (h->d_ranges) cudaDeviceSynchronize();  // a decode on another stream may still read them
     for (void **pp : {&h->d_ranges, (void **)&h->d_seg_pieces, (void **)&h->d_seg_cnt}) {
-        if (*pp) cudaFree(*pp);
+        dev_free(*pp, st);
         *pp = nullptr;
     }
     h->n_ranges = 0;
@@ -1048,7 +1048,7 @@ extern "C" int aclz_set_range_bytes(aclz_handle *h, uint32_t range_bytes, void *
         const uint64_t nwv = h->wave_start[w + 1] - h->wave_start[w];
         wT[w] = (uint32_t)std::min<uint64_t>(h->range_T, std::max<uint64_t>(1, (nwv + P - 1) / P));
     }
-    DevBuf b_of, b_dep, b_flag, b_ex, b_ws, b_wT;
+    Scratch b_of, b_dep, b_flag, b_ex, b_ws, b_wT;
     int rc = ACLZ_OK;
     auto ck = [&](cudaError_t e) {
         if (e != cudaSuccess && rc == ACLZ_OK) {
@@ -1057,9 +1057,9 @@ extern "C" int aclz_set_range_bytes(aclz_handle *h, uint32_t range_bytes, void *
         }
         return rc == ACLZ_OK;
     };
-    if (!ck(cudaMalloc(&b_of.p, 4 * n)) || !ck(cudaMalloc(&b_dep.p, 4 * nseg)) ||
-        !ck(cudaMalloc(&b_flag.p, 4 * n)) || !ck(cudaMalloc(&b_ex.p, 4 * n + 16)) ||
-        !ck(cudaMalloc(&b_ws.p, 8 * ((size_t)nw + 1))) || !ck(cudaMalloc(&b_wT.p, 4 * (size_t)nw)))
+    if (!ck(b_of.alloc(4 * n, st)) || !ck(b_dep.alloc(4 * nseg, st)) ||
+        !ck(b_flag.alloc(4 * n, st)) || !ck(b_ex.alloc(4 * n + 16, st)) ||
+        !ck(b_ws.alloc(8 * ((size_t)nw + 1), st)) || !ck(b_wT.alloc(4 * (size_t)nw, st)))
         return rc;
     uint32_t *seg_of = (uint32_t *)b_of.p, *segdep = (uint32_t *)b_dep.p, *flag = (uint32_t *)b_flag.p,
              *ex = (uint32_t *)b_ex.p, *d_nr = ex + n;
@@ -1083,8 +1083,8 @@ extern "C" int aclz_set_range_bytes(aclz_handle *h, uint32_t range_bytes, void *
     if (rc == ACLZ_OK) ck(cudaMemcpyAsync(&nr, d_nr, 4, cudaMemcpyDeviceToHost, st));
     if (rc == ACLZ_OK) ck(cudaStreamSynchronize(st));
     if (rc == ACLZ_OK && nr) {
-        if (ck(cudaMalloc(&h->d_ranges, 16 * ((size_t)nr + 1))) && ck(cudaMalloc((void **)&h->d_seg_pieces, 4 * nseg)) &&
-            ck(cudaMalloc((void **)&h->d_seg_cnt, 4 * nseg))) {
+        if (ck(dev_alloc(&h->d_ranges, 16 * ((size_t)nr + 1), st)) && ck(dev_alloc((void **)&h->d_seg_pieces, 4 * nseg, st)) &&
+            ck(dev_alloc((void **)&h->d_seg_cnt, 4 * nseg, st))) {
             k_range_build<<<grid, 256, 0, st>>>(seg, seg_of, flag, ex, n, nr, (uint4 *)h->d_ranges);
             k_seg_pieces<<<gseg, 256, 0, st>>>(seg, flag, ex, nseg, h->d_seg_pieces);
             ck(cudaGetLastError());

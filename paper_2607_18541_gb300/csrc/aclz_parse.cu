@@ -26,6 +26,7 @@
 
 #include "aclz_device.cuh"
 #include "aclz_internal.h"
+#include "aclz_mem.h"
 
 using namespace aclz;
 
@@ -478,13 +479,6 @@ __global__ void __launch_bounds__(256) k_emit(const uint8_t *__restrict__ x, uin
     }
 }
 
-struct Dev {
-    void *p = nullptr;
-    ~Dev() {
-        if (p) cudaFree(p);
-    }
-};
-
 }  // namespace
 
 extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_encode_params *p,
@@ -512,17 +506,17 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
         }
         return rc == ACLZ_OK;
     };
-    Dev dx, dk0, dv0, dk1, dv1, dlen, dhist, dslots, dntok, dnlit, dtoff, dloff, dmm, dbmm, dcont;
+    Scratch dx, dk0, dv0, dk1, dv1, dlen, dhist, dslots, dntok, dnlit, dtoff, dloff, dmm, dbmm, dcont;
     const uint32_t ntiles = (uint32_t)((m + kSortTile - 1) / kSortTile);
     // the input with 16 zero bytes after it (the 8-byte compares read
     // whole aligned words)
-    if (!ck(cudaMalloc(&dx.p, n + 64)) || !ck(cudaMemsetAsync((uint8_t *)dx.p + (n & ~(uint64_t)15), 0, 48, st)) ||
+    if (!ck(dx.alloc(n + 64, st)) || !ck(cudaMemsetAsync((uint8_t *)dx.p + (n & ~(uint64_t)15), 0, 48, st)) ||
         (n && !ck(cudaMemcpyAsync(dx.p, host_src, n, cudaMemcpyHostToDevice, st))))
         return rc;
     const uint64_t mm1 = m ? m : 1;
-    if (!ck(cudaMalloc(&dk0.p, 4 * mm1)) || !ck(cudaMalloc(&dv0.p, 4 * mm1)) || !ck(cudaMalloc(&dk1.p, 4 * mm1)) ||
-        !ck(cudaMalloc(&dv1.p, 4 * mm1)) || !ck(cudaMalloc(&dlen.p, n + 3 * kLenWindow)) ||
-        !ck(cudaMalloc(&dhist.p, 4 * (256ULL * (ntiles ? ntiles : 1) + 4))))
+    if (!ck(dk0.alloc(4 * mm1, st)) || !ck(dv0.alloc(4 * mm1, st)) || !ck(dk1.alloc(4 * mm1, st)) ||
+        !ck(dv1.alloc(4 * mm1, st)) || !ck(dlen.alloc(n + 3 * kLenWindow, st)) ||
+        !ck(dhist.alloc(4 * (256ULL * (ntiles ? ntiles : 1) + 4), st)))
         return rc;
     uint32_t *k0 = (uint32_t *)dk0.p, *v0 = (uint32_t *)dv0.p, *k1 = (uint32_t *)dk1.p, *v1 = (uint32_t *)dv1.p;
     if (m) {
@@ -545,14 +539,14 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
         if (rc) return rc;
     }
     // thresholds
-    if (!ck(cudaMalloc(&dmm.p, 16)) || !ck(cudaMemcpyAsync(dmm.p, p->min_match, 4, cudaMemcpyHostToDevice, st)))
+    if (!ck(dmm.alloc(16, st)) || !ck(cudaMemcpyAsync(dmm.p, p->min_match, 4, cudaMemcpyHostToDevice, st)))
         return rc;
-    if (block_min_match && (!ck(cudaMalloc(&dbmm.p, 4ULL * nb)) ||
+    if (block_min_match && (!ck(dbmm.alloc(4ULL * nb, st)) ||
                             !ck(cudaMemcpyAsync(dbmm.p, block_min_match, 4ULL * nb, cudaMemcpyHostToDevice, st))))
         return rc;
-    if (!ck(cudaMalloc(&dslots.p, sizeof(TokOut) * (uint64_t)cap_tok * (nb ? nb : 1))) ||
-        !ck(cudaMalloc(&dntok.p, 4ULL * nb + 16)) || !ck(cudaMalloc(&dnlit.p, 4ULL * nb + 16)) ||
-        !ck(cudaMalloc(&dtoff.p, 4ULL * nb + 16)) || !ck(cudaMalloc(&dloff.p, 4ULL * nb + 16)))
+    if (!ck(dslots.alloc(sizeof(TokOut) * (uint64_t)cap_tok * (nb ? nb : 1), st)) ||
+        !ck(dntok.alloc(4ULL * nb + 16, st)) || !ck(dnlit.alloc(4ULL * nb + 16, st)) ||
+        !ck(dtoff.alloc(4ULL * nb + 16, st)) || !ck(dloff.alloc(4ULL * nb + 16, st)))
         return rc;
     const uint64_t window = p->window;
     if (nb) {
@@ -585,7 +579,7 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
     *out_size = need;
     if (!host_out) return ACLZ_OK;
     if (cap < need) return ACLZ_E_CAPACITY;
-    if (!ck(cudaMalloc(&dcont.p, need ? need : 16))) return rc;
+    if (!ck(dcont.alloc(need ? need : 16, st))) return rc;
     uint8_t *c = (uint8_t *)dcont.p;
     if (nb) {
         k_emit<<<(nb + 7) / 8, 256, 0, st>>>((const uint8_t *)dx.p, n, bs, nb, (const TokOut *)dslots.p, cap_tok,
