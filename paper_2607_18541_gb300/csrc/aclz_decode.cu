@@ -1,16 +1,20 @@
 // Match-phase decode: the device-resident hot path.
 //
-// Wave 0 (k_wave0): one G-lane group per LZ block (Sec. II) walks the
-// block's tokens G at a time, prefix-sums literal and match lengths into
-// absolute output offsets, copies every literal run and every match whose
-// source is already final in block order (tag 0), and writes each deferred
-// match as a (dst, src, len) triplet into its wave's worklist.
+// Wave 0 copies what needs no other match's output: every literal run
+// (k_lits, over literal units of about equal bytes), then the in-order
+// matches, whose source bytes are literals or in-order match bytes of the
+// same block, level by level (a level's matches are independent; the levels
+// are found at upload).
 //
 // Waves w >= 1 hold the matches whose sources become final only in earlier
 // waves (the wavefront of Sec. I), block-ordered within each wave.  Two
 // schedules run them:
 //  - ACLZ_MODE_WAVES: one kernel per wave (k_wave_copy), kernel boundaries
-//    as the wave barrier;
+//    as the wave barrier.  Where ACLZ_MODE_AUTO takes this schedule it goes
+//    by levels instead of waves when the upload found them (every match of a
+//    level is independent of the others, so no chain is left inside a step),
+//    and consecutive small steps run in one launch of one thread-block
+//    cluster (k_wave_run), the cluster barrier between them;
 //  - ACLZ_MODE_PERSISTENT: one cooperative launch (k_ranges) over ranges of
 //    consecutive (block, wave) segments in wave-major order, with bounded
 //    waits on per-block completed-wave bits instead of wave barriers, so a
@@ -37,22 +41,21 @@ constexpr int kThreads = 256;
 // per-wave copy CTAs, and the CTAs of that size per SM the register cap
 // is set for (the same 85 registers a thread as 3 x 256)
 constexpr int kWaveThreads = 64, kWaveMinCtas = 768 / kWaveThreads;
-// chunks per lane per round in the wave-0 pass: before per-wave copies
-// (short matches; more resident warps without spills) and before the
-// persistent schedule (long in-order matches)
-constexpr int kUnrollWaveShort = 1, kUnrollWaveLong = 2;
+// literal copies: CTA size, CTAs of that size per SM the register cap is set
+// for, chunks per lane per round
+constexpr int kLitThreads = 128, kLitMinCtas = 6, kUnrollLits = 3;
+// small levels and waves: one cluster of kRunCtas CTAs runs consecutive
+// ones of at most kRunMost matches each, one window of 32 per warp
+constexpr int kRunThreads = 512, kRunCtas = 8;
+constexpr uint64_t kRunMost = (uint64_t)kRunThreads * kRunCtas;
 constexpr int kUnrollCopy = 3;   // chunks per lane per round in per-wave match copies
 constexpr int kUnrollRanges = 4; // the same in the persistent schedule's register copies
 // staged (TMA) copies: jobs of at least kTmaMin bytes, pieces of <= kPiece
-constexpr uint32_t kTmaMin = 192;
+constexpr uint32_t kTmaMin = (uint32_t)kPersistentMin;
 constexpr uint32_t kPiece = 2048;
 constexpr uint32_t kSmemPerSm = 220u * 1024u;  // stage memory shared by the CTAs of one SM
 // per-wave kernels are launched with programmatic stream serialization
 constexpr int kWavePdl = 1;
-// wave 0 reads literals through the non-coherent L1 path; before
-// per-wave copies (short tokens) it also prefetches the next window's
-// literal lines into L1 and the tokens two windows ahead into L2
-constexpr bool kWave0Ro = true;
 
 __device__ __forceinline__ uint64_t tri_dst(const uint4 t) { return (uint64_t)t.x | ((uint64_t)(t.y & 0xffu) << 32); }
 __device__ __forceinline__ uint64_t tri_src(const uint4 t) { return (uint64_t)t.z | ((uint64_t)(t.w & 0xffu) << 32); }
@@ -126,93 +129,54 @@ __device__ __forceinline__ unsigned same_wave_deps(const Group<G> &g, bool v, ui
 
 // ------------------------------------------------------------- wave 0
 
-// Wave 0 of one block: scan, literal runs, in-order (tag 0) matches, and
-// the deferred matches' triplets.  The next window's tokens are loaded
-// while the current window is copied.
-template <int G, int UW, bool PF>
-__device__ __forceinline__ void block_wave0(const Group<G> &g, uint32_t b, const uint4 *__restrict__ tok,
-                                            const uint8_t *__restrict__ lit,
-                                            const uint64_t *__restrict__ blk_tok,
-                                            const uint64_t *__restrict__ blk_lit,
-                                            const uint32_t *__restrict__ slot, uint4 *tri, uint8_t *out,
-                                            uint32_t log2bs) {
-    const uint64_t t0 = blk_tok[b], t1 = blk_tok[b + 1];
-    uint64_t lbase = blk_lit[b];
-    const uint64_t lend = blk_lit[b + 1];
-    uint64_t pos = (uint64_t)b << log2bs;
-    // the next window's tokens and worklist slots are loaded while the
-    // current window is copied
-    uint4 nt = t0 + g.lane < t1 ? __ldg(tok + t0 + g.lane) : make_uint4(0, 0, 0, 0);
-    uint32_t ns = (tri && t0 + g.lane < t1) ? __ldg(slot + t0 + g.lane) : 0u;
-    for (uint64_t w = t0; w < t1; w += G) {
-        const uint64_t i = w + g.lane;
-        const bool v = i < t1;
-        const uint4 t = v ? nt : make_uint4(0, 0, 0, 0);
-        const uint32_t sl = ns;
-        if (w + G + g.lane < t1) {
-            nt = __ldg(tok + w + G + g.lane);
-            if (tri) ns = __ldg(slot + w + G + g.lane);
-        }
-        const uint32_t ll = t.x, ml = t.y;
-        const uint32_t tag = t.w >> 8;
-        const uint64_t src = (uint64_t)t.z | ((uint64_t)(t.w & 0xffu) << 32);
-        const uint32_t incl = g.scan_incl(ll + ml);
-        const uint32_t lincl = g.scan_incl(ll);
-        const uint64_t dl = pos + incl - (ll + ml);
-        const uint64_t dm = dl + ll;
-        // deferred matches go to their wave's worklist
-        if (tri && v && ml && tag) {
-            __stcg(tri + sl, make_uint4((uint32_t)dm, (uint32_t)(dm >> 32), (uint32_t)src,
-                                        (uint32_t)(src >> 32) | (ml << 8)));
-        }
-        // literal runs: sources in the literal array, always independent
-        if (PF) {  // addresses inside this block's literals and tokens only
-            const uint64_t nl = lbase + g.shfl(lincl, G - 1) + 128 * g.lane;
-            if (g.lane < 2 && nl < lend) asm volatile("prefetch.global.L1 [%0];" ::"l"(lit + nl));
-            const uint64_t nt2 = w + 2 * G + 8 * (g.lane - 4);
-            if (g.lane >= 4 && g.lane < 8 && nt2 < t1) asm volatile("prefetch.global.L2 [%0];" ::"l"(tok + nt2));
-        }
-        group_copy<G, UW, kWave0Ro>(g, out, dl, lit + (lbase + lincl - ll), ll);
-        g.sync();
-        // in-order matches, batched so no batch reads what it writes: each
-        // batch takes the lanes whose sources overlap no output of a lane
-        // still to be copied (exact pairwise overlaps; the sources of
-        // in-order matches lie in their own block)
-        const bool m0 = v && ml && tag == 0;
-        unsigned rem = g.ballot(m0);
-        const unsigned deps0 = rem ? same_wave_deps<G>(g, m0, dm, src, ml, log2bs) & rem : 0u;
-        while (rem) {
-            const unsigned batch = g.ballot(((rem >> g.lane) & 1u) && (deps0 & rem) == 0u);
-            const bool mine = (batch >> g.lane) & 1u;
-            group_copy<G, UW>(g, out, dm, out + src, mine ? ml : 0u);
-            g.sync();
-            rem &= ~batch;
-        }
-        pos += g.shfl(incl, G - 1);
-        lbase += g.shfl(lincl, G - 1);
-    }
-}
-
-// Wave 0 of every block, one group per block.  With done non-null (the
+// Literal runs: one group per literal unit {block, first token, literal
+// range within the block}.  A window of G tokens needs no prefix sums, only
+// the tokens' output and literal offsets from the upload; a token's run ends
+// where the next token's literals start.  With done non-null (the
 // persistent schedule follows), each block's done bits start as its empty
 // waves plus wave 0.
-template <int G, int UW, bool PF>
-__global__ void __launch_bounds__(kThreads, 3) k_wave0(const uint4 *__restrict__ tok,
-                                                       const uint8_t *__restrict__ lit,
-                                                       const uint64_t *__restrict__ blk_tok,
-                                                       const uint64_t *__restrict__ blk_lit,
-                                                       const uint32_t *__restrict__ slot,
-                                                       uint4 *__restrict__ tri, uint8_t *out, uint32_t nb,
-                                                       uint32_t log2bs, const uint64_t *__restrict__ pending,
-                                                       uint64_t *done, uint32_t ww) {
+//
+// Bound by the latency of the unit's one or two rounds and by instruction
+// issue.  Units, and not blocks, are the work items because a stream has few
+// blocks (512 in 32 MiB at 64 KiB) and very unequal amounts of literals in
+// them: the literals and in-order matches of 32 MiB of word text at 6/8/10/12
+// took 786 us with one warp walking each block's tokens, the literals take
+// 56 us here (64 MiB of FASTQ-like text 108 -> 57 us, 256 KiB of Markov
+// bytes 97 -> 6 us).
+template <int G>
+__global__ void __launch_bounds__(kLitThreads, kLitMinCtas)
+    k_lits(const uint4 *__restrict__ units, uint64_t n_units, const uint8_t *__restrict__ lit,
+           const uint64_t *__restrict__ blk_tok, const uint64_t *__restrict__ blk_lit,
+           const uint32_t *__restrict__ tokdst, const uint32_t *__restrict__ toklit, uint8_t *out, uint32_t log2bs,
+           const uint64_t *__restrict__ pending, uint64_t *done, uint64_t n_done, uint32_t ww) {
     Group<G> g;
     griddep_launch_dependents();
-    const uint32_t b = (uint32_t)((blockIdx.x * (uint64_t)kThreads + threadIdx.x) / G);
-    if (b >= nb) return;
-    block_wave0<G, UW, PF>(g, b, tok, lit, blk_tok, blk_lit, slot, tri, out, log2bs);
-    if (done)
-        for (uint32_t k = g.lane; k < ww; k += G)
-            done[(uint64_t)b * ww + k] = ~__ldg(pending + (uint64_t)b * ww + k) | (k == 0 ? 1ULL : 0ULL);
+    const uint64_t tid = blockIdx.x * (uint64_t)kLitThreads + threadIdx.x;
+    for (uint64_t k = tid; k < n_done; k += (uint64_t)gridDim.x * kLitThreads)
+        done[k] = ~__ldg(pending + k) | (k % ww == 0 ? 1ULL : 0ULL);
+    if (tid / G >= n_units) return;
+    const uint4 u = __ldg(units + tid / G);
+    const uint32_t lo = u.z, hi = u.w;
+    if (lo == hi) return;
+    const uint64_t t1 = __ldg(blk_tok + u.x + 1);
+    const uint8_t *ls = lit + __ldg(blk_lit + u.x);
+    const uint64_t bpos = (uint64_t)u.x << log2bs;
+    uint64_t w = u.y;
+    // literal and output offset of this lane's token, the next window's
+    // loaded ahead (tokens past the block's end start at hi: no run)
+    uint32_t nl = w + g.lane < t1 ? __ldg(toklit + w + g.lane) : hi;
+    uint32_t nd = w + g.lane < t1 ? __ldg(tokdst + w + g.lane) : 0u;
+    for (;;) {
+        const uint32_t l0 = nl, d0 = nd;
+        w += G;
+        nl = w + g.lane < t1 ? __ldg(toklit + w + g.lane) : hi;
+        nd = w + g.lane < t1 ? __ldg(tokdst + w + g.lane) : 0u;
+        const uint32_t after = g.shfl(nl, 0), right = g.shfl(l0, (g.lane + 1) & (G - 1));
+        const uint32_t l1 = g.lane == G - 1 ? after : right;
+        const uint32_t x = max(l0, lo), y = min(l1, hi);
+        group_copy<G, kUnrollLits, true>(g, out, bpos + d0 + (x - l0), ls + x, y > x ? y - x : 0u);
+        if (after >= hi) break;
+    }
 }
 
 // ------------------------------------------------ persistent schedule
@@ -391,13 +355,10 @@ __global__ void __launch_bounds__(kThreads, STAGED ? 2 : 3)
 // internal chain, marked at upload) is copied as it stands: no dependency
 // test, no look at its neighbours.  Otherwise the group owns the segments
 // (runs of one block) that start in its window, and cuttable triplets in
-// it; a segment crossing the window's end is finished by the group that
-// started it.  PDL: sources are read after griddep_wait only.
 template <int G, bool PDL>
 __device__ __forceinline__ void wave_window(const Group<G> &g, const uint4 *__restrict__ tri, uint64_t n, uint64_t a,
-                                            uint8_t *out, uint32_t log2bs) {
+                                            const uint4 t0, uint8_t *out, uint32_t log2bs) {
     const uint4 z4 = make_uint4(0, 0, 0, 0);
-    const uint4 t0 = a + g.lane < n ? __ldg(tri + a + g.lane) : z4;
     if (!g.ballot(a + g.lane < n && !tri_cut(t0))) {
         if (PDL) griddep_wait();
         group_copy<G, kUnrollCopy>(g, out, tri_dst(t0), out + tri_src(t0), tri_len(t0));
@@ -458,48 +419,139 @@ __global__ void __launch_bounds__(kWaveThreads, kWaveMinCtas) k_wave_copy(const 
     Group<G> g;
     griddep_launch_dependents();
     const uint64_t a = (blockIdx.x * (uint64_t)kWaveThreads + threadIdx.x) / G * G;
-    if (a < n) wave_window<G, true>(g, tri, n, a, out, log2bs);
+    if (a >= n) return;
+    const uint4 t0 = a + g.lane < n ? __ldg(tri + a + g.lane) : make_uint4(0, 0, 0, 0);
+    wave_window<G, true>(g, tri, n, a, t0, out, log2bs);
+}
+
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Consecutive small steps (in-order levels, waves) by one thread-block
+// cluster: every group takes windows of G triplets of the step in turn, and
+// the cluster barrier separates the steps.
+//
+// Bound by the latency of a step: its sources from L2, its stores to L2
+// before the barrier, and the issue of one window of copies, about 3.7 us in
+// all where one kernel per step takes 5 to 10 us.  8 CTAs of 512 threads hold
+// 4096 lanes at 128 registers; 16 CTAs, or steps of up to 8192 matches, were
+// no faster, 768 threads at 80 registers 20% slower.  256 KiB of Markov
+// bytes (12 levels) 159 -> 52 us, the steps of 64 MiB of FASTQ-like text
+// 137 -> 95 us.
+template <int G>
+__global__ void __launch_bounds__(kRunThreads) k_wave_run(const Step *__restrict__ steps, uint32_t count, uint8_t *out,
+                                                          uint32_t log2bs) {
+    Group<G> g;
+    griddep_launch_dependents();
+    const uint64_t a0 = (blockIdx.x * (uint64_t)kRunThreads + threadIdx.x) / G * G;
+    const uint64_t stride = (uint64_t)gridDim.x * kRunThreads;
+    const ulonglong2 *list = reinterpret_cast<const ulonglong2 *>(steps);
+    const uint4 z4 = make_uint4(0, 0, 0, 0);
+    // this step's and the next step's descriptor and first window are loaded
+    // before the barrier that the sources wait for
+    ulonglong2 cur = __ldg(list), nx = count > 1 ? __ldg(list + 1) : make_ulonglong2(0, 0);
+    auto window = [&](const ulonglong2 &s, uint64_t a) {
+        return a + g.lane < s.y ? __ldg(reinterpret_cast<const uint4 *>(s.x) + a + g.lane) : z4;
+    };
+    uint4 t0 = window(cur, a0);
+    griddep_wait();
+    for (uint32_t k = 0; k < count; k++) {
+        const uint4 *tri = reinterpret_cast<const uint4 *>(cur.x);
+        for (uint64_t a = a0; a < cur.y; a += stride) {
+            const uint4 t = t0;
+            if (a + stride < cur.y) t0 = window(cur, a + stride);
+            wave_window<G, false>(g, tri, cur.y, a, t, out, log2bs);
+        }
+        if (k + 1 == count) break;
+        cur = nx;
+        t0 = window(cur, a0);
+        if (k + 2 < count) nx = __ldg(list + k + 2);
+        cluster_barrier();
+    }
+}
+
+// Length of the run of small steps from step i on that share one cluster
+// launch (0: step i has a kernel of its own).
+uint32_t run_length(const std::vector<Step> &s, uint32_t i, uint32_t i1, bool merge) {
+    uint32_t j = i;
+    while (merge && j < i1 && s[j].n <= kRunMost) j++;
+    return j - i;
+}
+
+// Kernel launches of the steps [i0, i1).
+uint32_t count_steps(const std::vector<Step> &s, uint32_t i0, uint32_t i1, bool merge) {
+    uint32_t n = 0;
+    for (uint32_t i = i0; i < i1; n++) i += std::max(1u, run_length(s, i, i1, merge));
+    return n;
 }
 
 template <int G>
-int launch_waves(aclz_handle *h, uint8_t *out, cudaStream_t st, cudaEvent_t phase) {
-    constexpr int gpc = kThreads / G;  // groups per CTA
-    const unsigned grid0 = (h->n_blocks + gpc - 1) / gpc;
-    k_wave0<G, kUnrollWaveShort, true><<<grid0, kThreads, 0, st>>>((const uint4 *)h->d_tok, h->d_lit, h->d_blk_tok,
-                                                              h->d_blk_lit, h->d_slot, nullptr, out,
-                                                              h->n_blocks, h->log2_bs, nullptr, nullptr, 0);
-    if (phase) cudaEventRecord(phase, st);
-    for (uint32_t w = 1; w < h->n_waves; w++) {
-        const uint64_t a = h->wave_start[w], n = h->wave_start[w + 1] - a;
-        if (!n) continue;
-        const uint64_t groups = (n + G - 1) / G;
-        constexpr int gpcw = kWaveThreads / G;
-        const unsigned grid = (unsigned)((groups + gpcw - 1) / gpcw);
-        const uint4 *t = (const uint4 *)h->d_tri + a;
-        auto k = k_wave_copy<G>;
-        // programmatic stream serialization: this wave's CTAs may start (and
-        // load their worklist) while the previous kernel's last CTAs finish
-        cudaLaunchConfig_t lc = {};
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[0].val.programmaticStreamSerializationAllowed = kWavePdl;
-        lc.gridDim = dim3(grid);
-        lc.blockDim = dim3(kWaveThreads);
-        lc.dynamicSmemBytes = 0;
-        lc.stream = st;
-        lc.attrs = at;
-        lc.numAttrs = 1;
-        uint32_t lb = h->log2_bs;
-        if (cudaError_t e = cudaLaunchKernelEx(&lc, k, t, n, out, lb); e != cudaSuccess) {
+int launch_steps(const aclz_handle *h, const std::vector<Step> &steps, const void *d_steps, uint8_t *out,
+                 cudaStream_t st, uint32_t i0, uint32_t i1, bool merge) {
+    // programmatic stream serialization: a step's CTAs may start (and load
+    // their worklist) while the previous kernel's last CTAs finish
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = kWavePdl;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = kRunCtas;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.dynamicSmemBytes = 0;
+    lc.stream = st;
+    lc.attrs = at;
+    const uint32_t lb = h->log2_bs;
+    for (uint32_t i = i0; i < i1;) {
+        const uint32_t run = run_length(steps, i, i1, merge);
+        cudaError_t e;
+        if (run) {
+            lc.gridDim = dim3(kRunCtas);
+            lc.blockDim = dim3(kRunThreads);
+            lc.numAttrs = 2;
+            e = cudaLaunchKernelEx(&lc, k_wave_run<G>, (const Step *)d_steps + i, run, out, lb);
+        } else {
+            const uint64_t n = steps[i].n, groups = (n + G - 1) / G;
+            constexpr int gpcw = kWaveThreads / G;
+            lc.gridDim = dim3((unsigned)((groups + gpcw - 1) / gpcw));
+            lc.blockDim = dim3(kWaveThreads);
+            lc.numAttrs = 1;
+            e = cudaLaunchKernelEx(&lc, k_wave_copy<G>, (const uint4 *)steps[i].tri, n, out, lb);
+        }
+        if (e != cudaSuccess) {
             note_cuda_error(e);
             return ACLZ_E_CUDA;
         }
+        i += std::max(1u, run);
     }
+    return ACLZ_OK;
+}
+
+template <int G>
+int launch_lits(aclz_handle *h, uint8_t *out, cudaStream_t st, bool persistent) {
+    constexpr int gpc = kLitThreads / G;
+    const uint64_t n_done = persistent ? (uint64_t)h->n_blocks * h->n_wave_words : 0;
+    const unsigned grid = (unsigned)((h->n_lunits + gpc - 1) / gpc);
+    k_lits<G><<<grid, kLitThreads, 0, st>>>((const uint4 *)h->d_lunits, h->n_lunits, h->d_lit, h->d_blk_tok,
+                                            h->d_blk_lit, h->d_tokdst, h->d_toklit, out, h->log2_bs, h->d_pending,
+                                            h->d_done, n_done, h->n_wave_words);
     if (cudaError_t e = cudaGetLastError(); e != cudaSuccess) {
         note_cuda_error(e);
         return ACLZ_E_CUDA;
     }
     return ACLZ_OK;
+}
+
+template <int G>
+int launch_waves(aclz_handle *h, uint8_t *out, cudaStream_t st, cudaEvent_t phase, bool merge) {
+    const uint32_t n = (uint32_t)h->steps.size(), no = h->n_ord_steps;
+    if (int rc = launch_lits<G>(h, out, st, false)) return rc;
+    if (merge && !phase && h->by_level)
+        return launch_steps<G>(h, h->lsteps, h->d_lsteps, out, st, 0, (uint32_t)h->lsteps.size(), true);
+    if (int rc = launch_steps<G>(h, h->steps, h->d_steps, out, st, 0, no, true)) return rc;
+    if (phase) cudaEventRecord(phase, st);
+    return launch_steps<G>(h, h->steps, h->d_steps, out, st, no, n, merge);
 }
 
 struct Occ {
@@ -515,22 +567,15 @@ size_t &smem_attr() {
     return v;
 }
 
-// Persistent mode: the wave-0 kernel (no dependencies) initialises the
-// per-block done bits, then one cooperative launch runs every range of
+// Persistent mode: the literal kernel initialises the per-block done bits;
+// after the in-order levels one cooperative launch runs every range of
 // waves >= 1.
 template <int G, bool STAGED>
 int launch_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaStream_t st, cudaEvent_t phase) {
     constexpr int gpc = kThreads / G;
-    const unsigned grid0 = (h->n_blocks + gpc - 1) / gpc;
-    k_wave0<G, kUnrollWaveLong, false><<<grid0, kThreads, 0, st>>>((const uint4 *)h->d_tok, h->d_lit, h->d_blk_tok,
-                                                             h->d_blk_lit, h->d_slot, nullptr, out,
-                                                             h->n_blocks, h->log2_bs, h->d_pending, h->d_done,
-                                                             h->n_wave_words);
+    if (int rc = launch_lits<G>(h, out, st, true)) return rc;
+    if (int rc = launch_steps<G>(h, h->steps, h->d_steps, out, st, 0, h->n_ord_steps, true)) return rc;
     if (phase) cudaEventRecord(phase, st);
-    if (cudaError_t e = cudaGetLastError(); e != cudaSuccess) {
-        note_cuda_error(e);
-        return ACLZ_E_CUDA;
-    }
     if (!h->n_ranges) return ACLZ_OK;
     auto fn = k_ranges<G, STAGED>;
     static int sms = 0;
@@ -621,6 +666,10 @@ int launch_persistent_auto(aclz_handle *h, uint8_t *out, const aclz_decode_cfg &
 
 namespace {
 
+// Small waves share a launch only when the caller left the mode open: an
+// explicit ACLZ_MODE_WAVES is one kernel per wave.
+bool is_auto(const aclz_decode_cfg *cfg) { return !cfg || cfg->mode == ACLZ_MODE_AUTO; }
+
 // Checks cfg and resolves ACLZ_MODE_AUTO for this handle.
 int resolve_cfg(const aclz_handle *h, const aclz_decode_cfg *cfg, aclz_decode_cfg &c) {
     c = {32, ACLZ_MODE_AUTO, 0, 0};
@@ -649,12 +698,13 @@ extern "C" int aclz_decode_plan(const aclz_handle *h, const aclz_decode_cfg *cfg
     if (int rc = resolve_cfg(h, cfg, c)) return rc;
     uint32_t n = 0;
     if (h->n_blocks) {
-        n = 1;
-        if (c.mode == ACLZ_MODE_PERSISTENT) {
-            n += h->n_ranges ? 1 : 0;
-        } else {
-            for (uint32_t w = 1; w < h->n_waves; w++) n += h->wave_start[w + 1] > h->wave_start[w];
-        }
+        const uint32_t no = h->n_ord_steps, ns = (uint32_t)h->steps.size();
+        if (c.mode == ACLZ_MODE_PERSISTENT)
+            n = 1 + count_steps(h->steps, 0, no, true) + (h->n_ranges ? 1 : 0);
+        else if (is_auto(cfg) && h->by_level)
+            n = 1 + count_steps(h->lsteps, 0, (uint32_t)h->lsteps.size(), true);
+        else
+            n = 1 + count_steps(h->steps, 0, no, true) + count_steps(h->steps, no, ns, is_auto(cfg));
     }
     if (resolved) *resolved = c;
     if (launches) *launches = n;
@@ -680,9 +730,9 @@ extern "C" int aclz_decode_all_ev(aclz_handle *h, void *d_out, uint64_t cap, con
         }
     }
     switch (c.G) {
-        case 8: return launch_waves<8>(h, out, st, ev);
-        case 16: return launch_waves<16>(h, out, st, ev);
-        default: return launch_waves<32>(h, out, st, ev);
+        case 8: return launch_waves<8>(h, out, st, ev, is_auto(cfg));
+        case 16: return launch_waves<16>(h, out, st, ev, is_auto(cfg));
+        default: return launch_waves<32>(h, out, st, ev, is_auto(cfg));
     }
 }
 

@@ -50,10 +50,13 @@ struct Group {
     __device__ __forceinline__ unsigned lanemask_lt() const { return (1u << lane) - 1u; }
     // bitwise or over the group's lanes
     __device__ __forceinline__ unsigned or_all(unsigned v) const {
-        if constexpr (G == 32) return __reduce_or_sync(0xffffffffu, v);
+        if constexpr (G == 32) {
+            return __reduce_or_sync(0xffffffffu, v);
+        } else {
 #pragma unroll
-        for (int o = 1; o < G; o <<= 1) v |= __shfl_xor_sync(mask, v, o, G);
-        return v;
+            for (int o = 1; o < G; o <<= 1) v |= __shfl_xor_sync(mask, v, o, G);
+            return v;
+        }
     }
 };
 

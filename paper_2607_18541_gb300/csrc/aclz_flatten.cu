@@ -361,7 +361,9 @@ extern "C" int aclz_flatten(aclz_handle *h, void *stream) {
     h->wave_start[2] = np;
     h->mean_deferred_len = (double)def_bytes / (double)np;
     h->flat = true;
-    return aclz_set_range_bytes(h, h->range_bytes, stream);
+    h->by_level = false;  // the pieces are one step after the in-order levels
+    if (int rc = aclz_set_range_bytes(h, h->range_bytes, stream)) return rc;
+    return build_steps(h, stream);
 }
 
 // ------------------------------------------------------------- reshape

@@ -4,11 +4,16 @@
 //                    validation (lengths fill the block, every source lies
 //                    strictly before its target, Sec. I), block-relative
 //                    token offsets for the seek path.
-//  2. k_tags_min     minimal wave tags (a match waits one wave for every
-//                    cross-block hop of its source chain; same-block sources
-//                    are ordered within the block), computed in one launch:
-//                    blocks are taken in increasing order and a block waits
-//                    (bounded) for the earlier blocks its sources lie in.
+//  2. k_cover, k_relax  the tokens each match reads, then by passes over
+//                    them its minimal wave tag (a match waits one wave for
+//                    every cross-block hop of its source chain; same-block
+//                    sources are ordered within the block) and its level
+//                    (the length of the longest chain of matches that ends
+//                    in it).
+//     k_tags_min     the tags of streams whose chains are too deep for the
+//                    passes, in one launch: blocks are taken in increasing
+//                    order and a block waits (bounded) for the earlier
+//                    blocks its sources lie in.
 //     k_tags_check   legality of tags supplied by the container.
 //  3. k_wave_hist, an exclusive scan and k_slots: the wave-major, block-
 //     ordered worklist slot of every deferred match.
@@ -307,51 +312,111 @@ __global__ void __launch_bounds__(256) k_tags_check(const uint4 *__restrict__ to
     if (g.ballot(bad) && g.lane == 0) atomicOr(err, kErrCorrupt);
 }
 
-// One pass of the parallel minimal-tag computation: every match's tag is
-// raised to its requirement under the current tags (read as other warps
-// leave them).  Requirements only grow with the tags, so from all-zero
-// tags the passes climb to the least fixed point, which is the minimal
-// tagging; a pass that raises nothing (changed stays 0) proves it reached.
-// Also folds the largest tag into *maxtag.
-__global__ void __launch_bounds__(256) k_tags_relax(const uint4 *__restrict__ tok,
-                                                    const uint64_t *__restrict__ blk_tok,
-                                                    const uint32_t *__restrict__ tokdst, uint32_t *tags,
-                                                    uint32_t nb, uint32_t log2bs, uint64_t n_tok,
-                                                    uint32_t *changed, uint32_t *maxtag) {
-    Group<32> g;
+// cover[i] of a match token i: the tokens whose match bytes its source
+// reads, as {first token, of them in other blocks, of them in its own block,
+// 1 when any source byte lies in another block}; zero for other tokens.
+// Covering tokens are consecutive, other blocks' first.
+__global__ void __launch_bounds__(256) k_cover(const uint4 *__restrict__ tok, const uint64_t *__restrict__ blk_tok,
+                                               const uint32_t *__restrict__ tokdst, uint32_t nb, uint32_t log2bs,
+                                               uint64_t n_tok, uint4 *__restrict__ cover) {
     const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (b >= nb) return;
     const uint64_t t0 = blk_tok[b], t1 = blk_tok[b + 1];
-    uint32_t mx = 0;
-    bool raised = false;
-    for (uint64_t w = t0; w < t1; w += 32) {
-        const uint64_t i = w + g.lane;
-        if (i < t1) {
-            const uint4 t = __ldg(tok + i);
-            if (t.y) {
-                const uint64_t src = ((uint64_t)t.z | ((uint64_t)t.w << 32)) & kSrcMask;
-                bool inwin = false;
-                const uint32_t req = match_requirement(tok, blk_tok, tokdst, tags, src, t.y, b, log2bs, n_tok,
-                                                       n_tok, &inwin);
-                const uint32_t cur = __ldcg(tags + i);
-                if (req > cur) {
-                    __stcg(tags + i, req);
-                    raised = true;
+    for (uint64_t i = t0 + lane; i < t1; i += 32) {
+        const uint4 tk = __ldg(tok + i);
+        uint4 c = make_uint4(0, 0, 0, 0);
+        if (tk.y) {
+            const uint64_t src = ((uint64_t)tk.z | ((uint64_t)tk.w << 32)) & kSrcMask, e = src + tk.y;
+            uint64_t bp = src >> log2bs;
+            uint64_t lo = __ldg(blk_tok + bp), hi = __ldg(blk_tok + bp + 1) - 1;
+            const uint32_t rel = (uint32_t)(src - (bp << log2bs));
+            // last token of block bp that starts at or before src
+            while (lo < hi) {
+                const uint64_t mid = (lo + hi + 1) >> 1;
+                if (__ldg(tokdst + mid) <= rel) lo = mid; else hi = mid - 1;
+            }
+            uint64_t t = lo, bend = __ldg(blk_tok + bp + 1), first = ~0ULL, last = 0;
+            for (;;) {
+                const uint64_t ts = (bp << log2bs) + __ldg(tokdst + t);
+                if (ts >= e) break;
+                const uint4 y = __ldg(tok + t);
+                const uint64_t le = ts + y.x;
+                if (y.y && le < e && le + y.y > src) {
+                    if (first == ~0ULL) first = t;
+                    last = t;
                 }
-                mx = max(mx, max(req, cur));
+                if (++t >= n_tok) break;
+                if (t >= bend) bend = __ldg(blk_tok + ++bp + 1);
+            }
+            c.w = (src >> log2bs) != b;
+            if (first != ~0ULL) {
+                const uint32_t total = (uint32_t)(last - first) + 1u;
+                const uint32_t other = first >= t0 ? 0u : (last < t0 ? total : (uint32_t)(t0 - first));
+                c.x = (uint32_t)first;
+                c.y = other;
+                c.z = total - other;
             }
         }
-        g.sync();
+        cover[i] = c;
     }
-    for (int o = 16; o; o >>= 1) mx = max(mx, g.shfl(mx, (g.lane + o) & 31));
-    if (g.ballot(raised) && g.lane == 0) *changed = 1u;
-    if (g.lane == 0 && mx) atomicMax(maxtag, mx);
+}
+
+// One pass over the matches: val[i] = {level, tag} of token i raised to what
+// its covering tokens ask for under their current values (read as other
+// warps leave them): level = 1 + their largest level, tag = the largest of
+// their tags, plus one in another block.  Both only grow, from zero to the
+// least fixed point, which is the longest chain and the minimal tagging.
+// After pass k every match of true level up to k has its final values, and
+// no value exceeds its true one, so a match whose level is below k is final:
+// pass k + 1 skips it after one 8-byte read.  A pass that raises nothing
+// (*changed stays 0) proves the fixed point reached.
+__global__ void __launch_bounds__(256) k_relax(const uint4 *__restrict__ cover, const uint4 *__restrict__ tok,
+                                               uint64_t n, uint32_t pass, unsigned long long *val,
+                                               uint32_t *changed, uint32_t *maxes) {
+    uint32_t mt = 0, ml = 0;
+    bool raised = false;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+        const unsigned long long cur = __ldcg(val + i);
+        if (pass > 1 && (uint32_t)(cur >> 32) + 1u < pass) continue;
+        const uint4 c = __ldg(cover + i);
+        if (pass == 1 && !__ldg(&tok[i].y)) continue;
+        uint32_t lv = 0, tg = c.w;
+        for (uint32_t k = 0; k < c.y + c.z; k++) {
+            const unsigned long long v = __ldcg(val + c.x + k);
+            lv = max(lv, (uint32_t)(v >> 32));
+            // a literal-only token among them has value 0 and asks for nothing
+            if (v) tg = max(tg, (uint32_t)v + (k < c.y ? 1u : 0u));
+        }
+        const unsigned long long nv = ((unsigned long long)(lv + 1u) << 32) | max(tg, (uint32_t)cur);
+        if (nv != cur) {
+            __stcg(val + i, nv);
+            raised = true;
+        }
+        ml = max(ml, lv + 1u);
+        mt = max(mt, (uint32_t)nv);
+    }
+    ml = __reduce_max_sync(0xffffffffu, ml);
+    mt = __reduce_max_sync(0xffffffffu, mt);
+    if (__any_sync(0xffffffffu, raised) && (threadIdx.x & 31) == 0) {
+        *changed = 1u;
+        atomicMax(maxes, mt);
+        atomicMax(maxes + 1, ml);
+    }
 }
 
 __global__ void k_extract_tags(const uint4 *__restrict__ tok, uint32_t *tags, uint64_t n) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
          i += (uint64_t)gridDim.x * blockDim.x)
         tags[i] = __ldg(tok + i).w >> 8;
+}
+
+__global__ void k_store_val_tags(uint4 *tok, const unsigned long long *val, uint64_t n) {
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
+         i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint4 t = tok[i];
+        tok[i].w = (t.w & 0xffu) | ((uint32_t)val[i] << 8);
+    }
 }
 
 __global__ void k_store_tags(uint4 *tok, const uint32_t *tags, uint64_t n) {
@@ -692,27 +757,32 @@ int aclz::device_excl_scan(uint32_t *d, uint64_t n, uint32_t *d_total, void *str
     return cuda_rc(cudaGetLastError());
 }
 
-// Minimal wave tags of h's tokens into d_tags (and the largest into
-// *d_maxtag) by parallel relaxation passes from all-zero tags, checked every
-// kRelaxBatch passes; true when a pass raised nothing within kRelaxMax
-// passes.  A stream whose copy chains are deeper than that is left to the
-// ordered pass (false; d_tags then holds partial tags).
+// Levels and minimal wave tags of h's tokens into d_val ({level, tag}, and
+// the largest tag and level into d_maxes[0..1]) by relaxation passes from
+// zero, checked every kRelaxBatch passes; true when a pass raised nothing
+// within kRelaxMax passes.  A stream whose copy chains are deeper than that
+// is left to the ordered pass (false; d_val is then part-way).
 namespace {
 constexpr uint32_t kRelaxBatch = 8, kRelaxMax = 512;
-bool relax_tags(aclz_handle *h, uint32_t *d_tags, uint32_t *d_maxtag, cudaStream_t st) {
+bool relax_levels(aclz_handle *h, unsigned long long *d_val, uint32_t *d_maxes, cudaStream_t st) {
     const uint32_t nb = h->n_blocks;
     const uint64_t nt = h->n_tokens;
-    if (!nb) return true;
-    Scratch flags;
+    Scratch flags, cover;
     if (flags.alloc(4 * kRelaxBatch, st) != cudaSuccess) return false;
+    if (cover.alloc(16 * (nt ? nt : 1), st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
     uint32_t *changed = (uint32_t *)flags.p;
-    if (cudaMemsetAsync(d_tags, 0, 4 * (nt ? nt : 1), st) != cudaSuccess) return false;
-    const unsigned wblocks = (nb + 7) / 8;
+    if (cudaMemsetAsync(d_val, 0, 8 * (nt ? nt : 1), st) != cudaSuccess) return false;
+    k_cover<<<(nb + 7) / 8, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, nb, h->log2_bs, nt,
+                                           (uint4 *)cover.p);
+    const unsigned grid = (unsigned)std::min<uint64_t>((nt + 255) / 256, 152 * 8 * 4);
     for (uint32_t done_passes = 0; done_passes < kRelaxMax; done_passes += kRelaxBatch) {
         if (cudaMemsetAsync(changed, 0, 4 * kRelaxBatch, st) != cudaSuccess) return false;
         for (uint32_t k = 0; k < kRelaxBatch; k++)
-            k_tags_relax<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, d_tags, nb,
-                                                   h->log2_bs, nt, changed + k, d_maxtag);
+            k_relax<<<grid, 256, 0, st>>>((const uint4 *)cover.p, (const uint4 *)h->d_tok, nt, done_passes + k + 1,
+                                          d_val, changed + k, d_maxes);
         uint32_t last = 1;
         if (cudaGetLastError() != cudaSuccess ||
             cudaMemcpyAsync(&last, changed + kRelaxBatch - 1, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -743,6 +813,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         dev_free(*pp, st);
         *pp = nullptr;
     }
+    free_wave0(h, st);
     h->n_seg = h->n_ranges = 0;
     h->n_deferred = 0;
     CK(dev_alloc((void **)&h->d_tokdst, 4 * (nt ? nt : 1), st));
@@ -753,8 +824,9 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     Scratch work;
     CK(work.alloc(64, st));
     uint32_t *d_maxtag = (uint32_t *)work.p, *d_ctr = d_maxtag + 1, *d_total = d_maxtag + 2;
-    // words: [0] max tag, [1] counter, [2] deferred total, [3] segment count,
-    // [4] range count; bytes 32..39: first bad token
+    // words: [0] max tag, [1] largest level, then the block counter, [2]
+    // deferred total, [3] segment count, [4] range count, [5] matches of the
+    // level list; bytes 32..39: first bad token
     unsigned long long *d_first_bad = (unsigned long long *)((char *)work.p + 32);
     CK(cudaMemsetAsync(work.p, 0, 32, st));
     CK(cudaMemsetAsync(d_first_bad, 0xff, 8, st));
@@ -768,9 +840,13 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     CK(cudaStreamSynchronize(st));
     if (herr) { cleanup(); return ACLZ_E_CORRUPT; }
     // tags
+    // {level, tag} of every token when the passes find them (8 bytes), or
+    // plain tags (4 bytes) in the same array
     Scratch tags, done;
-    CK(tags.alloc(4 * (nt ? nt : 1), st));
+    CK(tags.alloc(8 * (nt ? nt : 1), st));
     uint32_t *d_tags = (uint32_t *)tags.p;
+    unsigned long long *d_val = (unsigned long long *)tags.p;
+    bool levels = false;
     h->local_tags = false;
     if (has_tags) {
         k_extract_tags<<<1024, 256, 0, st>>>((const uint4 *)h->d_tok, d_tags, nt);
@@ -781,11 +857,12 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         k_tags_local<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, d_tags, nb,
                                                h->log2_bs, d_maxtag);
         k_store_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_tags, nt);
-    } else if (relax_tags(h, d_tags, d_maxtag, st)) {
-        // minimal tags by parallel passes (the chains were shallow enough)
-        k_store_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_tags, nt);
+    } else if (relax_levels(h, d_val, d_maxtag, st)) {
+        // by parallel passes (the chains were shallow enough)
+        levels = true;
+        k_store_val_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_val, nt);
     } else {
-        CK(cudaMemsetAsync(d_maxtag, 0, 4, st));
+        CK(cudaMemsetAsync(d_maxtag, 0, 8, st));
         CK(done.alloc(4 * nb, st));
         CK(cudaMemsetAsync(done.p, 0, 4 * nb, st));
         int dev_sms = 0;
@@ -800,9 +877,10 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         k_store_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_tags, nt);
     }
     CK(cudaGetLastError());
-    uint32_t hw[2] = {0, 0};
+    uint32_t hw[3] = {0, 0, 0};
     CK(cudaMemcpyAsync(&hw[0], d_maxtag, 4, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(&hw[1], h->d_err, 4, cudaMemcpyDeviceToHost, st));
+    if (levels) CK(cudaMemcpyAsync(&hw[2], d_maxtag + 1, 4, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (hw[1] & kErrTimeout) { cleanup(); return ACLZ_E_TIMEOUT; }
     if (hw[1]) { cleanup(); return ACLZ_E_CORRUPT; }
@@ -874,6 +952,16 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         rc = aclz_set_range_bytes(h, h->range_bytes, stream);
         if (rc) { cleanup(); return rc; }
     }
+    // the schedule by levels serves what ACLZ_MODE_AUTO decodes as waves: a
+    // container with tags of its own has its levels found here
+    const bool by_level = !flat_up && !h->needs_flatten && decodes_as_waves(h);
+    if (by_level && has_tags) {
+        CK(cudaMemsetAsync(d_maxtag, 0, 8, st));
+        levels = relax_levels(h, d_val, d_maxtag, st);
+        if (levels) CK(cudaMemcpyAsync(&hw[2], d_maxtag + 1, 4, cudaMemcpyDeviceToHost, st));
+    }
+    rc = build_wave0(h, levels ? d_val : nullptr, hw[2], by_level && levels, stream);
+    if (rc) { cleanup(); return rc; }
     if (!h->d_pending) {  // no deferred matches: wave 0 finishes every block
         h->n_wave_words = 1;
         std::vector<uint64_t> ones(nb, 1ULL);
@@ -882,7 +970,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     }
     CK(dev_alloc((void **)&h->d_done, 8 * (size_t)nb * h->n_wave_words, st));
     CK(cudaStreamSynchronize(st));
-    return ACLZ_OK;
+    return build_steps(h, stream);
 }
 
 extern "C" int aclz_upload(const void *host_buf, uint64_t n, void *stream, aclz_handle **out) {
@@ -983,6 +1071,7 @@ extern "C" int aclz_free(aclz_handle *h) {
     cudaGetDevice(&cur);
     if (cur != dev) cudaSetDevice(dev);
     cudaDeviceSynchronize();
+    free_wave0(h, nullptr);
     for (void *p : ps) dev_free(p, nullptr);
     if (cur != dev) cudaSetDevice(cur);
     delete h;

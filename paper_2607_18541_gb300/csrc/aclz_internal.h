@@ -59,11 +59,38 @@ void note_cuda_error(int cuda_error_code);
 // (device); stream-ordered, temporary storage allocated on the stream.
 int device_excl_scan(uint32_t *d, uint64_t n, uint32_t *d_total, void *stream);
 
+// Stable sort of n (key, value) pairs by the low 8 * passes bits of the key;
+// k1 and v1 are scratch of the same size, and on return k0 and v0 point to
+// the sorted pairs (the pointers are exchanged when passes is odd).
+int device_sort_pairs(uint32_t **k0, uint32_t **v0, uint32_t **k1, uint32_t **v1, uint64_t n, int passes,
+                      void *stream);
+
 }  // namespace aclz
 
 struct aclz_handle;
 
 namespace aclz {
+
+// Wave 0's index (aclz_wave0.cu): literal units, and the level list of the
+// in-order matches, or with all of every match.  d_val: {level, tag} of every
+// token and maxlvl the largest level, or null when the levels are not known
+// (the in-order ones are then found block by block).  The step tables follow
+// once the worklists are final.
+int build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlvl, bool all, void *stream);
+int build_steps(aclz_handle *h, void *stream);
+void free_wave0(aclz_handle *h, void *stream);
+
+// Deferred matches of at least this mean length are decoded by the
+// persistent schedule under ACLZ_MODE_AUTO (TMA staging pays), shorter ones
+// by waves.
+constexpr double kPersistentMin = 192.0;
+bool decodes_as_waves(const aclz_handle *h);
+
+// A list of matches that may be copied once everything before it is final:
+// device address of its triplets, and their number.
+struct Step {
+    uint64_t tri, n;
+};
 
 // Decode index of h from its device tokens (validation, offsets, wave tags,
 // worklists, schedule); see aclz_index.cu.
@@ -107,6 +134,22 @@ struct aclz_handle {
     void *d_tri = nullptr;        // n_deferred x 16 B triplets (dst, src, len), built at upload
     uint32_t *d_err = nullptr;    // latched device status bits
     std::vector<uint64_t> wave_start;  // n_waves + 1 entries into the triplet array
+    // wave 0: literal units {block, first token, literal range}
+    void *d_lunits = nullptr;
+    uint64_t n_lunits = 0;
+    // level list: triplets sorted by level, the in-order matches of a level
+    // before its deferred ones (which it holds only when by_level).  Level l
+    // (from 1) starts at lev_start[2l - 2], its deferred part at
+    // lev_start[2l - 1]; one entry more ends the list.
+    void *d_lev = nullptr;
+    std::vector<uint64_t> lev_start;
+    bool by_level = false;
+    // what follows the literals, in order: in steps the in-order levels
+    // (n_ord_steps of them), then the non-empty waves; in lsteps every
+    // level.  d_steps and d_lsteps are the same on the device.
+    std::vector<aclz::Step> steps, lsteps;
+    void *d_steps = nullptr, *d_lsteps = nullptr;
+    uint32_t n_ord_steps = 0;
     // persistent-mode schedule.  A segment is the run of one block's
     // matches in one wave's worklist: seg[s] = {block, wave, triplet offset,
     // count}, wave-major then block order.  A range is a run of consecutive
@@ -140,3 +183,5 @@ struct aclz_handle {
     bool local_tags = false;
     uint64_t n_matches_deferred = 0;  // deferred matches before flattening
 };
+
+inline bool aclz::decodes_as_waves(const aclz_handle *h) { return h->mean_deferred_len < kPersistentMin; }

@@ -481,6 +481,33 @@ __global__ void __launch_bounds__(256) k_emit(const uint8_t *__restrict__ x, uin
 
 }  // namespace
 
+int aclz::device_sort_pairs(uint32_t **k0, uint32_t **v0, uint32_t **k1, uint32_t **v1, uint64_t n, int passes,
+                            void *stream) {
+    if (!n) return ACLZ_OK;
+    cudaStream_t st = (cudaStream_t)stream;
+    const uint32_t ntiles = (uint32_t)((n + kSortTile - 1) / kSortTile);
+    const uint64_t hn = 256ULL * ntiles;
+    uint32_t *hist = nullptr;
+    cudaError_t e = dev_alloc((void **)&hist, 4 * (hn + 4), st);
+    int rc = ACLZ_OK;
+    for (int pass = 0; pass < passes && e == cudaSuccess && rc == ACLZ_OK; pass++) {
+        const int shift = 8 * pass;
+        k_rs_hist<<<ntiles, kSortThreads, 0, st>>>(*k0, n, shift, ntiles, hist);
+        rc = device_excl_scan(hist, hn, hist + hn, st);
+        if (rc) break;
+        k_rs_scatter<<<ntiles, kSortThreads, 0, st>>>(*k0, *v0, n, shift, ntiles, hist, *k1, *v1);
+        e = cudaGetLastError();
+        std::swap(*k0, *k1);
+        std::swap(*v0, *v1);
+    }
+    dev_free(hist, st);
+    if (e != cudaSuccess) {
+        note_cuda_error(e);
+        return e == cudaErrorMemoryAllocation ? ACLZ_E_NOMEM : ACLZ_E_CUDA;
+    }
+    return rc;
+}
+
 extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_encode_params *p,
                                const uint8_t *block_min_match, void *stream, void *host_out, uint64_t cap,
                                uint64_t *out_size) {
@@ -506,8 +533,7 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
         }
         return rc == ACLZ_OK;
     };
-    Scratch dx, dk0, dv0, dk1, dv1, dlen, dhist, dslots, dntok, dnlit, dtoff, dloff, dmm, dbmm, dcont;
-    const uint32_t ntiles = (uint32_t)((m + kSortTile - 1) / kSortTile);
+    Scratch dx, dk0, dv0, dk1, dv1, dlen, dslots, dntok, dnlit, dtoff, dloff, dmm, dbmm, dcont;
     // the input with 16 zero bytes after it (the 8-byte compares read
     // whole aligned words)
     if (!ck(dx.alloc(n + 64, st)) || !ck(cudaMemsetAsync((uint8_t *)dx.p + (n & ~(uint64_t)15), 0, 48, st)) ||
@@ -515,28 +541,14 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
         return rc;
     const uint64_t mm1 = m ? m : 1;
     if (!ck(dk0.alloc(4 * mm1, st)) || !ck(dv0.alloc(4 * mm1, st)) || !ck(dk1.alloc(4 * mm1, st)) ||
-        !ck(dv1.alloc(4 * mm1, st)) || !ck(dlen.alloc(n + 3 * kLenWindow, st)) ||
-        !ck(dhist.alloc(4 * (256ULL * (ntiles ? ntiles : 1) + 4), st)))
+        !ck(dv1.alloc(4 * mm1, st)) || !ck(dlen.alloc(n + 3 * kLenWindow, st)))
         return rc;
     uint32_t *k0 = (uint32_t *)dk0.p, *v0 = (uint32_t *)dv0.p, *k1 = (uint32_t *)dk1.p, *v1 = (uint32_t *)dv1.p;
     if (m) {
         const unsigned g = (unsigned)std::min<uint64_t>(8192, (m + 255) / 256);
         k_keys<<<g, 256, 0, st>>>((const uint8_t *)dx.p, m, k0, v0);
-        uint32_t *hist = (uint32_t *)dhist.p;
-        const uint64_t hn = 256ULL * ntiles;
-        for (int pass = 0; pass < 4 && rc == ACLZ_OK; pass++) {
-            const int shift = 8 * pass;
-            k_rs_hist<<<ntiles, kSortThreads, 0, st>>>(k0, m, shift, ntiles, hist);
-            ck(cudaGetLastError());
-            if (rc) break;
-            rc = device_excl_scan(hist, hn, hist + hn, st);
-            if (rc) break;
-            k_rs_scatter<<<ntiles, kSortThreads, 0, st>>>(k0, v0, m, shift, ntiles, hist, k1, v1);
-            ck(cudaGetLastError());
-            std::swap(k0, k1);
-            std::swap(v0, v1);
-        }
-        if (rc) return rc;
+        ck(cudaGetLastError());
+        if (rc || (rc = device_sort_pairs(&k0, &v0, &k1, &v1, m, 4, st))) return rc;
     }
     // thresholds
     if (!ck(dmm.alloc(16, st)) || !ck(cudaMemcpyAsync(dmm.p, p->min_match, 4, cudaMemcpyHostToDevice, st)))

@@ -1,0 +1,279 @@
+// Index of wave 0: what a decode can do before any deferred match.
+//
+//  - Literal units: the literal array cut at multiples of a unit size and at
+//    block boundaries, each unit with the token its first byte belongs to,
+//    so that literals are copied by as many groups as their bytes ask for,
+//    whatever the number of blocks.  Unit ids need no scan: the unit of
+//    block b holding the k-th stretch of the literal array is k + b (k never
+//    falls and b rises from block to block); ids nothing maps to stay empty.
+//  - Matches by level: level 1 reads literals only, level l + 1 matches of
+//    level l and below.  The matches of one level are independent of each
+//    other, in every block at once.  The list holds the in-order matches
+//    (tag 0: every source byte is a literal or an in-order match byte of the
+//    same block), for every schedule; for streams that are decoded as waves
+//    it holds the deferred ones too and is a schedule of its own: the fewest
+//    dependent steps there are (a wave hides its chains within a block:
+//    4 MiB of FASTQ-like text at 12/16/24/32 has 9 waves with chains adding
+//    up to 42 steps, and 14 levels).
+#include <algorithm>
+#include <cstring>
+#include <vector>
+
+#include "aclz_device.cuh"
+#include "aclz_internal.h"
+#include "aclz_mem.h"
+
+using namespace aclz;
+
+namespace {
+
+int rc_of(cudaError_t e) {
+    if (e == cudaSuccess) return ACLZ_OK;
+    note_cuda_error((int)e);
+    return e == cudaErrorMemoryAllocation ? ACLZ_E_NOMEM : ACLZ_E_CUDA;
+}
+
+#define W0CK(x)                  \
+    do {                         \
+        int _rc = rc_of(x);      \
+        if (_rc) return _rc;     \
+    } while (0)
+
+__device__ __forceinline__ uint64_t t_dst(const uint4 t) { return (uint64_t)t.x | ((uint64_t)(t.y & 0xffu) << 32); }
+__device__ __forceinline__ uint64_t t_src(const uint4 t) { return (uint64_t)t.z | ((uint64_t)(t.w & 0xffu) << 32); }
+__device__ __forceinline__ uint32_t t_len(const uint4 t) { return t.w >> 8; }
+
+// units[k + b] = {block b, first token, literal range within the block}, one
+// warp per block
+__global__ void __launch_bounds__(256) k_lit_units(const uint64_t *__restrict__ blk_tok,
+                                                   const uint64_t *__restrict__ blk_lit,
+                                                   const uint32_t *__restrict__ toklit, uint32_t nb, uint32_t log2u,
+                                                   uint4 *__restrict__ units) {
+    const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (b >= nb) return;
+    const uint64_t l0 = blk_lit[b], l1 = blk_lit[b + 1];
+    if (l1 == l0) return;
+    for (uint64_t k = (l0 >> log2u) + lane; k <= (l1 - 1) >> log2u; k += 32) {
+        const uint64_t x = max(l0, k << log2u), y = min(l1, (k + 1) << log2u);
+        const uint32_t lo = (uint32_t)(x - l0);
+        // last token whose literals start at or before lo: they hold lo
+        uint64_t a = blk_tok[b], e = blk_tok[b + 1] - 1;
+        while (a < e) {
+            const uint64_t mid = (a + e + 1) >> 1;
+            if (__ldg(toklit + mid) <= lo) a = mid; else e = mid - 1;
+        }
+        units[k + b] = make_uint4(b, (uint32_t)a, lo, (uint32_t)(y - l0));
+    }
+}
+
+// cnt[b] = matches of block b for the list (the in-order ones, or all)
+__global__ void __launch_bounds__(256) k_lev_count(const uint4 *__restrict__ tok, const uint64_t *__restrict__ blk_tok,
+                                                   uint32_t nb, bool all, uint32_t *cnt) {
+    const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (b >= nb) return;
+    uint32_t c = 0;
+    for (uint64_t i = blk_tok[b] + lane; i < blk_tok[b + 1]; i += 32) {
+        const uint4 t = __ldg(tok + i);
+        c += t.y && (all || !(t.w >> 8));
+    }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0) cnt[b] = c;
+}
+
+// triplets of those matches in token order (base: exclusive scan of the
+// counts), which may all be cut anywhere (bit 8 of .y), and with val their
+// sort keys 2 (level - 1) + deferred
+__global__ void __launch_bounds__(256) k_lev_build(const uint4 *__restrict__ tok, const uint64_t *__restrict__ blk_tok,
+                                                   const uint32_t *__restrict__ tokdst, uint32_t nb, uint32_t log2bs,
+                                                   const uint32_t *__restrict__ base, bool all,
+                                                   const unsigned long long *__restrict__ val, uint4 *__restrict__ tri,
+                                                   uint32_t *__restrict__ key, uint32_t *__restrict__ idx) {
+    const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (b >= nb) return;
+    uint32_t at = base[b];
+    if (base[b + 1] == at) return;
+    const uint64_t bstart = (uint64_t)b << log2bs, t1 = blk_tok[b + 1];
+    for (uint64_t w = blk_tok[b]; w < t1; w += 32) {
+        const uint64_t i = w + lane;
+        const uint4 t = i < t1 ? __ldg(tok + i) : make_uint4(0, 0, 0, 0);
+        const bool m = t.y && (all || !(t.w >> 8));
+        const unsigned bal = __ballot_sync(0xffffffffu, m);
+        if (m) {
+            const uint64_t d = bstart + __ldg(tokdst + i) + t.x;
+            const uint32_t k = at + __popc(bal & ((1u << lane) - 1u));
+            tri[k] = make_uint4((uint32_t)d, (uint32_t)(d >> 32) | 0x100u, t.z, (t.w & 0xffu) | (t.y << 8));
+            if (val) key[k] = 2u * ((uint32_t)(__ldg(val + i) >> 32) - 1u) + ((t.w >> 8) ? 1u : 0u);
+            idx[k] = k;
+        }
+        at += __popc(bal);
+    }
+}
+
+// Levels of the in-order matches, one CTA per block: windows of one match a
+// thread in token order, each iterated to its fixed point (a match reads
+// earlier ones only, so levels before the window are final and those in it
+// only grow).
+constexpr int kLevelThreads = 256;
+__global__ void __launch_bounds__(kLevelThreads) k_ord_levels(const uint4 *__restrict__ tri,
+                                                              const uint32_t *__restrict__ base, uint32_t *lvl,
+                                                              uint32_t *maxlvl, uint32_t *key) {
+    const uint32_t o0 = base[blockIdx.x], o1 = base[blockIdx.x + 1];
+    uint32_t mx = 0;
+    for (uint32_t w = o0; w < o1; w += kLevelThreads) {
+        const uint32_t i = w + threadIdx.x;
+        const bool v = i < o1;
+        uint64_t s = 0, e = 0;
+        uint32_t jl = i, cur = 1;
+        if (v) {
+            const uint4 t = __ldg(tri + i);
+            s = t_src(t);
+            e = s + t_len(t);
+            // first earlier match that ends past s
+            uint32_t lo = o0, hi = i;
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                const uint4 y = __ldg(tri + mid);
+                if (t_dst(y) + t_len(y) > s) hi = mid; else lo = mid + 1;
+            }
+            jl = lo;
+            __stcg(lvl + i, 1u);
+        }
+        bool pending = v;
+        __syncthreads();
+        for (;;) {
+            bool changed = false;
+            if (pending) {
+                uint32_t lv = 1;
+                bool inwin = false;
+                for (uint32_t j = jl; j < i && t_dst(__ldg(tri + j)) < e; j++) {
+                    lv = max(lv, __ldcg(lvl + j) + 1u);
+                    inwin = inwin || j >= w;
+                }
+                changed = lv != cur;
+                cur = lv;
+                if (changed) __stcg(lvl + i, cur);
+                pending = inwin;
+            }
+            if (!__syncthreads_or(changed)) break;
+        }
+        if (v) {
+            mx = max(mx, cur);
+            key[i] = 2u * (cur - 1u);
+        }
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0 && mx) atomicMax(maxlvl, mx);
+}
+
+// triplets in key order, and the first of each key present
+__global__ void k_lev_gather(const uint4 *__restrict__ tri, const uint32_t *__restrict__ key,
+                             const uint32_t *__restrict__ idx, uint64_t n, uint4 *__restrict__ out,
+                             uint32_t *__restrict__ start) {
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+        out[i] = __ldg(tri + idx[i]);
+        if (i == 0 || key[i] != key[i - 1]) start[key[i]] = (uint32_t)i;
+    }
+}
+
+}  // namespace
+
+void aclz::free_wave0(aclz_handle *h, void *stream) {
+    cudaStream_t st = (cudaStream_t)stream;
+    for (void **pp : {&h->d_lunits, &h->d_lev, &h->d_steps, &h->d_lsteps}) {
+        dev_free(*pp, st);
+        *pp = nullptr;
+    }
+    h->n_lunits = 0;
+    h->lev_start.clear();
+    h->by_level = false;
+    h->steps.clear();
+    h->lsteps.clear();
+}
+
+int aclz::build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlvl, bool all, void *stream) {
+    cudaStream_t st = (cudaStream_t)stream;
+    const uint32_t nb = h->n_blocks;
+    // units of 2 KiB, smaller in a short stream so that there are about 32
+    // of them per SM, down to 256 bytes
+    uint32_t lu = 11;
+    while (lu > 8 && (h->n_literals >> lu) < 152 * 32) lu--;
+    h->n_lunits = (h->n_literals >> lu) + nb + 1;
+    W0CK(dev_alloc(&h->d_lunits, 16 * h->n_lunits, st));
+    W0CK(cudaMemsetAsync(h->d_lunits, 0, 16 * h->n_lunits, st));
+    k_lit_units<<<(nb + 7) / 8, 256, 0, st>>>(h->d_blk_tok, h->d_blk_lit, h->d_toklit, nb, lu, (uint4 *)h->d_lunits);
+    W0CK(cudaGetLastError());
+    // level list
+    Scratch cnt, work, tri, key, idx, key2, idx2, start;
+    W0CK(cnt.alloc(4 * ((uint64_t)nb + 1), st));
+    k_lev_count<<<(nb + 7) / 8, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, nb, all, cnt.as<uint32_t>());
+    W0CK(cudaGetLastError());
+    if (int rc = device_excl_scan(cnt.as<uint32_t>(), nb, cnt.as<uint32_t>() + nb, st)) return rc;
+    uint32_t n = 0;
+    W0CK(cudaMemcpyAsync(&n, cnt.as<uint32_t>() + nb, 4, cudaMemcpyDeviceToHost, st));
+    W0CK(cudaStreamSynchronize(st));
+    if (!n) return ACLZ_OK;
+    h->by_level = all;
+    W0CK(tri.alloc(16 * (uint64_t)n, st));
+    W0CK(key.alloc(4 * (uint64_t)n, st));
+    W0CK(idx.alloc(4 * (uint64_t)n, st));
+    k_lev_build<<<(nb + 7) / 8, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, nb, h->log2_bs,
+                                              cnt.as<uint32_t>(), all, d_val, (uint4 *)tri.p, key.as<uint32_t>(), idx.as<uint32_t>());
+    W0CK(cudaGetLastError());
+    W0CK(key2.alloc(4 * (uint64_t)n, st));
+    if (!d_val) {
+        W0CK(work.alloc(16, st));
+        W0CK(cudaMemsetAsync(work.p, 0, 16, st));
+        k_ord_levels<<<nb, kLevelThreads, 0, st>>>((const uint4 *)tri.p, cnt.as<uint32_t>(), key2.as<uint32_t>(), work.as<uint32_t>(), key.as<uint32_t>());
+        W0CK(cudaGetLastError());
+        W0CK(cudaMemcpyAsync(&maxlvl, work.p, 4, cudaMemcpyDeviceToHost, st));
+        W0CK(cudaStreamSynchronize(st));
+    }
+    const uint64_t keys = 2 * (uint64_t)maxlvl;
+    W0CK(idx2.alloc(4 * (uint64_t)n, st));
+    W0CK(start.alloc(4 * keys, st));
+    W0CK(cudaMemsetAsync(start.p, 0xff, 4 * keys, st));
+    W0CK(dev_alloc(&h->d_lev, 16 * (uint64_t)n, st));
+    uint32_t *k0 = key.as<uint32_t>(), *v0 = idx.as<uint32_t>(), *k1 = key2.as<uint32_t>(), *v1 = idx2.as<uint32_t>();
+    const int passes = keys <= 256 ? 1 : keys <= 65536 ? 2 : keys <= (1u << 24) ? 3 : 4;
+    if (int rc = device_sort_pairs(&k0, &v0, &k1, &v1, n, passes, st)) return rc;
+    const unsigned grid = (unsigned)std::min<uint64_t>(4096, ((uint64_t)n + 255) / 256);
+    k_lev_gather<<<grid, 256, 0, st>>>((const uint4 *)tri.p, k0, v0, n, (uint4 *)h->d_lev, start.as<uint32_t>());
+    W0CK(cudaGetLastError());
+    std::vector<uint32_t> hs(keys);
+    W0CK(cudaMemcpyAsync(hs.data(), start.p, 4 * keys, cudaMemcpyDeviceToHost, st));
+    W0CK(cudaStreamSynchronize(st));
+    h->lev_start.assign(keys + 1, n);
+    for (uint64_t k = keys; k-- > 0;) h->lev_start[k] = hs[k] == 0xffffffffu ? h->lev_start[k + 1] : hs[k];
+    return ACLZ_OK;
+}
+
+int aclz::build_steps(aclz_handle *h, void *stream) {
+    cudaStream_t st = (cudaStream_t)stream;
+    for (void **pp : {&h->d_steps, &h->d_lsteps}) {
+        dev_free(*pp, st);
+        *pp = nullptr;
+    }
+    h->steps.clear();
+    h->lsteps.clear();
+    auto add = [](std::vector<Step> &v, const void *tri, uint64_t a, uint64_t b) {
+        if (b > a) v.push_back({(uint64_t)((const uint4 *)tri + a), b - a});
+    };
+    const std::vector<uint64_t> &ls = h->lev_start;
+    for (size_t k = 0; k + 2 < ls.size(); k += 2) {
+        add(h->steps, h->d_lev, ls[k], ls[k + 1]);
+        if (h->by_level) add(h->lsteps, h->d_lev, ls[k], ls[k + 2]);
+    }
+    h->n_ord_steps = (uint32_t)h->steps.size();
+    for (uint32_t w = 1; w < h->n_waves && h->d_tri; w++)
+        add(h->steps, h->d_tri, h->wave_start[w], h->wave_start[w + 1]);
+    for (auto &pr : {std::make_pair(&h->steps, &h->d_steps), std::make_pair(&h->lsteps, &h->d_lsteps)}) {
+        if (pr.first->empty()) continue;
+        W0CK(dev_alloc((void **)pr.second, sizeof(Step) * pr.first->size(), st));
+        W0CK(cudaMemcpyAsync(*pr.second, pr.first->data(), sizeof(Step) * pr.first->size(), cudaMemcpyHostToDevice, st));
+    }
+    W0CK(cudaStreamSynchronize(st));
+    return ACLZ_OK;
+}

@@ -1,0 +1,131 @@
+"""Wave 0 and the small steps where their tiling can go wrong: literal units
+around block and unit boundaries, in-order chains of more levels than one
+sort digit and of more matches than one window of the level pass, waves on
+both sides of the size that shares a cluster launch."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2607_18541_gb300 import aclz
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _decode_all_ways(c, flatten=True):
+    exp = oracle.decode(c)
+    s = torch.cuda.current_stream()
+    for flags in (0, aclz.ACLZ_UPLOAD_FLATTEN) if flatten else (0,):
+        h = aclz.aclz_upload(c, s, flags=flags)
+        try:
+            for G in (32, 16, 8):
+                for mode in (aclz.ACLZ_MODE_AUTO, aclz.ACLZ_MODE_WAVES, aclz.ACLZ_MODE_PERSISTENT):
+                    out = torch.full((exp.size + 32,), 0xA5, dtype=torch.uint8, device="cuda")
+                    aclz.aclz_decode_all(h, out, cap=exp.size, G=G, mode=mode, stream=s)
+                    assert aclz.aclz_device_status(h, s) == 0
+                    got = out.cpu().numpy()
+                    assert np.array_equal(got[:exp.size], exp), (flags, G, mode)
+                    assert (got[exp.size:] == 0xA5).all()
+        finally:
+            aclz.aclz_free(h)
+
+
+def _pack(total, bs, blocks, lits):
+    """blocks: per block a list of (lit_len, match_len, src)."""
+    ll = np.array([t[0] for b in blocks for t in b], dtype=np.uint32)
+    ml = np.array([t[1] for b in blocks for t in b], dtype=np.uint32)
+    sr = np.array([t[2] for b in blocks for t in b], dtype=np.uint64)
+    n = np.array([len(b) for b in blocks], dtype=np.uint32)
+    return aclz.aclz_pack(total, bs, (4, 4, 4, 4), n, ll, ml, sr, lits[:int(ll.sum())])
+
+
+LITS = np.random.RandomState(1).randint(0, 256, 1 << 22).astype(np.uint8)
+
+
+@pytest.mark.parametrize("bs", [64, 256, 1024, 4096])
+@pytest.mark.parametrize("total", [63, 64, 255, 256, 257, 2048, 4095, 4096, 4097, 70000])
+def test_all_literal_blocks(bs, total):
+    # units end where blocks end, blocks end where units end, short last block
+    blocks = [[(min(bs, total - p), 0, 0)] for p in range(0, total, bs)]
+    _decode_all_ways(_pack(total, bs, blocks, LITS))
+
+
+@pytest.mark.parametrize("seed", range(6))
+def test_blocks_with_and_without_literals(seed):
+    r = np.random.RandomState(seed)
+    bs, nb = int(r.choice([64, 128, 512, 2048])), 60
+    blocks = [[(bs, 0, 0)]]
+    for b in range(1, nb):
+        p, toks = b * bs, []
+        end = p + bs
+        while p < end:
+            lit = int(r.choice([0, 0, 0, 1, 3, 17, 300])) if b % 3 else 0
+            lit = min(lit, end - p)
+            p += lit
+            m = min(int(r.randint(1, 90)), end - p, p)
+            if m == 0:
+                toks.append((lit, 0, 0))
+                break
+            toks.append((lit, m, int(r.randint(0, p - m + 1))))
+            p += m
+        blocks.append(toks)
+    _decode_all_ways(_pack(nb * bs, bs, blocks, LITS))
+
+
+@pytest.mark.parametrize("chain", [1, 2, 255, 256, 257, 700])
+@pytest.mark.parametrize("width", [1, 5])
+def test_in_order_chains(chain, width):
+    # each match copies the match `width` tokens before it: `chain` levels
+    bs = 1 << 14
+    blocks = []
+    for b in range(3):
+        p = b * bs
+        toks, ends = [(40, 0, 0)], []
+        pos, lit = p + 40, 40
+        toks = []
+        starts = []
+        for k in range(chain * width):
+            ln = 7
+            src = starts[k - width] if k >= width else p + (k % 8)
+            toks.append((lit if k == 0 else k % 2, ln, src))
+            pos = pos + (0 if k == 0 else k % 2)
+            starts.append(pos)
+            pos += ln
+            if pos + 10 > p + bs:
+                break
+        toks.append((p + bs - pos, 0, 0))
+        blocks.append(toks)
+    c = _pack(3 * bs, bs, blocks, LITS)
+    assert oracle.validate(c) == 0
+    _decode_all_ways(c)
+
+
+@pytest.mark.parametrize("n", [4095, 4096, 4097])
+def test_steps_around_the_shared_launch(n):
+    # waves 1 and 3 of n matches, waves 2 and 4 of a few: AUTO shares launches
+    bs, ln = 1 << 17, 8
+    blocks, pos = [[(bs, 0, 0)]], bs
+    src, readable = 0, bs  # what the wave before wrote at the start of its first block
+    for cnt in (n, 40, n, 3):
+        start, left = pos, cnt
+        while left:
+            k = min(left, bs // ln)
+            toks = [(0, ln, src + (ln * i) % readable) for i in range(k)]
+            if k * ln < bs:
+                toks.append((bs - k * ln, 0, 0))
+            blocks.append(toks)
+            left -= k
+            pos += bs
+        src, readable = start, min(cnt, bs // ln) * ln
+    c = _pack(pos, bs, blocks, LITS)
+    assert oracle.validate(c) == 0
+    s = torch.cuda.current_stream()
+    h = aclz.aclz_upload(c, s)
+    try:
+        counts = aclz.aclz_wave_counts(h)
+        assert counts[1:].tolist() == [n, 40, n, 3]
+        assert aclz.aclz_decode_plan(h, mode=aclz.ACLZ_MODE_WAVES)[1] == 5
+        assert aclz.aclz_decode_plan(h)[1] == (2 if n <= 4096 else 5)
+    finally:
+        aclz.aclz_free(h)
+    _decode_all_ways(c)
