@@ -299,6 +299,19 @@ int make_pieces(aclz_handle *h, cudaStream_t st, int max_rounds, Pieces &pc) {
 
 }  // namespace
 
+namespace {
+
+// slot[t] = first piece of deferred match t (others keep ~0)
+__global__ void k_fl_slot(const uint4 *__restrict__ tok, const uint32_t *__restrict__ defscan,
+                          const uint64_t *__restrict__ off, uint64_t nt, uint32_t *slot) {
+    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < nt; t += (uint64_t)gridDim.x * blockDim.x) {
+        const uint4 tk = __ldg(tok + t);
+        if (tk.y && (tk.w >> 8)) slot[t] = (uint32_t)off[defscan[t]];
+    }
+}
+
+}  // namespace
+
 extern "C" int aclz_flatten(aclz_handle *h, void *stream) {
     if (!h) return ACLZ_E_INVAL;
     if (h->flat) return ACLZ_OK;
@@ -323,6 +336,8 @@ extern "C" int aclz_flatten(aclz_handle *h, void *stream) {
     FCK(tri.alloc(16 * np, st));
     k_fl_tri<<<grid_for(np), 256, 0, st>>>(P.as<uint4>(), owner.as<uint32_t>(), dmk.as<uint64_t>(), np,
                                             tri.as<uint4>());
+    k_fl_slot<<<grid_for(h->n_tokens), 256, 0, st>>>((const uint4 *)h->d_tok, defscan.as<uint32_t>(),
+                                                      off.as<uint64_t>(), h->n_tokens, h->d_slot);
     FCK(bflag.alloc(4 * ((uint64_t)nb + 1), st));
     FCK(pending.alloc(8 * (uint64_t)nb, st));
     FCK(done.alloc(8 * (uint64_t)nb, st));

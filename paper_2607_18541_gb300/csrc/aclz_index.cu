@@ -46,12 +46,14 @@ __global__ void __launch_bounds__(256) k_index_scan(const uint4 *__restrict__ to
                                                     const uint64_t *__restrict__ blk_tok,
                                                     const uint64_t *__restrict__ blk_lit,
                                                     uint32_t *__restrict__ tokdst,
-                                                    uint32_t *__restrict__ toklit, uint32_t nb,
+                                                    uint32_t *__restrict__ toklit, uint32_t *__restrict__ cell,
+                                                    uint64_t n_cells, uint32_t log2c, uint64_t nt, uint32_t nb,
                                                     uint32_t log2bs, uint64_t total, int has_tags,
                                                     uint32_t *err, unsigned long long *first_bad) {
     Group<32> g;
     const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (b >= nb) return;
+    if (b == 0 && g.lane == 0) cell[n_cells] = (uint32_t)nt;
     const uint64_t t0 = blk_tok[b], t1 = blk_tok[b + 1];
     const uint64_t bstart = (uint64_t)b << log2bs;
     const uint64_t blen = min((uint64_t)1 << log2bs, total - bstart);
@@ -83,6 +85,12 @@ __global__ void __launch_bounds__(256) k_index_scan(const uint4 *__restrict__ to
             }
             tokdst[i] = (uint32_t)rel;
             toklit[i] = (uint32_t)(lcarry + lsum - lit);
+            // the cells that start in this token's bytes
+            if (ok) {
+                const uint64_t ts = bstart + rel;
+                for (uint64_t c = (ts + (1ULL << log2c) - 1) >> log2c; c << log2c < ts + tot; c++)
+                    cell[c] = (uint32_t)i;
+            }
         }
         carry += g.shfl(incl, 31);
         lcarry += g.shfl(lsum, 31);
@@ -808,7 +816,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     const uint32_t nb = h->n_blocks;
     const uint64_t nt = h->n_tokens;
     int rc = ACLZ_OK;
-    for (void **pp : {(void **)&h->d_tokdst, (void **)&h->d_toklit, (void **)&h->d_slot, &h->d_tri, &h->d_seg,
+    for (void **pp : {(void **)&h->d_tokdst, (void **)&h->d_toklit, (void **)&h->d_slot, (void **)&h->d_cell, &h->d_tri, &h->d_seg,
                       &h->d_ranges, (void **)&h->d_pending, (void **)&h->d_done}) {
         dev_free(*pp, st);
         *pp = nullptr;
@@ -819,6 +827,11 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     CK(dev_alloc((void **)&h->d_tokdst, 4 * (nt ? nt : 1), st));
     CK(dev_alloc((void **)&h->d_toklit, 4 * (nt ? nt : 1), st));
     CK(dev_alloc((void **)&h->d_slot, 4 * (nt ? nt : 1), st));
+    // cells of at least the mean token length, 64 bytes to one block
+    h->log2_cell = 6;
+    while (h->log2_cell < h->log2_bs && (h->total_len >> h->log2_cell) > nt) h->log2_cell++;
+    h->n_cells = (h->total_len + (1ULL << h->log2_cell) - 1) >> h->log2_cell;
+    CK(dev_alloc((void **)&h->d_cell, 4 * (h->n_cells + 1), st));
     CK(cudaMemsetAsync(h->d_err, 0, 64, st));
     // scratch words: [0] err (handle), work: maxtag, counter, total, first_bad
     Scratch work;
@@ -832,7 +845,8 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     CK(cudaMemsetAsync(d_first_bad, 0xff, 8, st));
     const unsigned wblocks = (nb + 7) / 8;  // 8 warps per CTA
     k_index_scan<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_blk_lit, h->d_tokdst,
-                                           h->d_toklit, nb, h->log2_bs, h->total_len, has_tags, h->d_err,
+                                           h->d_toklit, h->d_cell, h->n_cells, h->log2_cell, nt, nb, h->log2_bs,
+                                           h->total_len, has_tags, h->d_err,
                                            d_first_bad);
     CK(cudaGetLastError());
     uint32_t herr = 0;
@@ -1065,7 +1079,7 @@ extern "C" int aclz_free(aclz_handle *h) {
     if (!h) return ACLZ_E_INVAL;
     void *ps[] = {h->d_tok, h->d_lit,    h->d_blk_tok, h->d_blk_lit,      h->d_slot,      h->d_tokdst,
                   h->d_toklit, h->d_tri, h->d_err,     h->d_seg,          h->d_ranges,    h->d_seg_pieces,
-                  h->d_seg_cnt, h->d_pending, h->d_done};
+                  h->d_seg_cnt, h->d_pending, h->d_done, h->d_cell};
     // work in flight on any stream may still read them
     int dev = h->device, cur = h->device;
     cudaGetDevice(&cur);

@@ -128,9 +128,15 @@ struct aclz_handle {
     uint8_t *d_lit = nullptr;     // n_literals + 32 zero bytes of padding
     uint64_t *d_blk_tok = nullptr;  // n_blocks + 1 token offsets
     uint64_t *d_blk_lit = nullptr;  // n_blocks + 1 literal offsets
-    uint32_t *d_slot = nullptr;   // per token: triplet slot of a deferred match, else ~0u
+    uint32_t *d_slot = nullptr;   // per token: triplet slot of a deferred match (flattened: of its first piece), else ~0u
     uint32_t *d_tokdst = nullptr; // per token: block-relative offset of its first byte
     uint32_t *d_toklit = nullptr; // per token: block-relative offset of its first literal
+    // cell c: the token covering output position c << log2_cell; one entry
+    // more holds n_tokens.  Cells are as many as tokens or fewer, and no
+    // larger than a block.
+    uint32_t *d_cell = nullptr;
+    uint64_t n_cells = 0;
+    uint32_t log2_cell = 0;
     void *d_tri = nullptr;        // n_deferred x 16 B triplets (dst, src, len), built at upload
     uint32_t *d_err = nullptr;    // latched device status bits
     std::vector<uint64_t> wave_start;  // n_waves + 1 entries into the triplet array
