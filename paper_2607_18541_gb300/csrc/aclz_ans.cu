@@ -7,8 +7,8 @@
 // states (byte i of the tile on state i mod 32) in [2^16, 2^32), and one
 // stream of 16-bit renormalisation words, taken in increasing lane order
 // within each step of 32 bytes.  One warp decodes one tile: lane k owns
-// state k, a slot-to-symbol table of 4096 entries sits in shared memory, and
-// every step writes 32 consecutive bytes.  The planes are then transposed
+// state k, a table of the 4096 slots and a ring of words sit in shared
+// memory, and every step writes 32 consecutive bytes.  The planes are then transposed
 // into 16-byte tokens and the upload continues as for a v1 container.
 #include <algorithm>
 #include <cstring>
@@ -27,8 +27,9 @@ constexpr uint32_t kStreams = 17;
 constexpr uint32_t kProbBits = 12, kProb = 1u << kProbBits;
 constexpr uint32_t kStateLow = 1u << 16;
 constexpr uint32_t kTileHeader = 512 + 4 * 32 + 4;  // freq[256], state[32], n_words
-constexpr int kWarps = 8;                             // tiles per CTA
-constexpr uint32_t kWarpSmem = 4096 + 512 + 512;      // slot table, freq[256], cum[256]
+constexpr int kWarps = 1;                             // tiles per CTA (12 of them per SM)
+constexpr uint32_t kGroup = 128, kRing = 4 * kGroup;  // words: a group, the ring of them
+constexpr uint32_t kWarpSmem = 4 * kProb + 2 * kRing; // slot table, ring
 
 struct TileDesc {
     uint64_t payload;  // offset in the payload area
@@ -43,6 +44,19 @@ uint32_t rd32le(const uint8_t *p) {
 }
 uint64_t rd64le(const uint8_t *p) { return (uint64_t)rd32le(p) | ((uint64_t)rd32le(p + 4) << 32); }
 
+// A tile is a chain of up to 2048 steps, each depending on the one before,
+// and there are few tiles per SM (1035 of them in 64 MiB of FASTQ-like text),
+// so the kernel is bound by the latency of a step: one shared-memory load
+// (symbol, frequency and offset of a slot packed in a word), a multiply-add,
+// a ballot and a load of the word.  The words come through a ring of four
+// groups in shared memory, filled by asynchronous copies three groups (some
+// 50 steps) ahead; four steps take at most one group, so the ring is looked
+// after once every four steps.  With separate symbol, frequency and offset
+// tables and words loaded from global memory one step took 360 ns, 85 ns
+// now: the tiles of 64 MiB of FASTQ-like text 740 -> 203 us, of 1 GiB 1.90 ->
+// 1.69 ms (12 tiles per SM at a time; 4 tiles per CTA 1.84 ms).  Words in
+// registers, shuffled, were no faster than 390 us: a register queue waits
+// for its newest load at every move.
 __global__ void __launch_bounds__(kWarps * 32) k_ans_tiles(const uint8_t *__restrict__ pay,
                                                           const TileDesc *__restrict__ td, uint64_t n_tiles,
                                                           uint8_t *planes, uint64_t plane_bytes, uint8_t *lits,
@@ -51,20 +65,15 @@ __global__ void __launch_bounds__(kWarps * 32) k_ans_tiles(const uint8_t *__rest
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint64_t t = (uint64_t)blockIdx.x * kWarps + warp;
     if (t >= n_tiles) return;
-    uint8_t *lut = sm + warp * kWarpSmem;
-    uint16_t *freq = reinterpret_cast<uint16_t *>(lut + 4096);
-    uint16_t *cum = freq + 256;
+    uint32_t *lut = reinterpret_cast<uint32_t *>(sm + warp * kWarpSmem);
     const TileDesc d = td[t];
     const uint8_t *p = pay + d.payload;
     // frequencies: 8 per lane, cumulative by a warp scan
     const uint4 fv = __ldg(reinterpret_cast<const uint4 *>(p) + lane);
     const uint32_t fw[4] = {fv.x, fv.y, fv.z, fv.w};
-    uint32_t f8[8], local = 0;
+    uint32_t local = 0;
 #pragma unroll
-    for (int k = 0; k < 8; k++) {
-        f8[k] = (fw[k >> 1] >> (16 * (k & 1))) & 0xffffu;
-        local += f8[k];
-    }
+    for (int k = 0; k < 8; k++) local += (fw[k >> 1] >> (16 * (k & 1))) & 0xffffu;
     uint32_t incl = local;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -72,56 +81,86 @@ __global__ void __launch_bounds__(kWarps * 32) k_ans_tiles(const uint8_t *__rest
         if (lane >= o) incl += v;
     }
     const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-    if (d.m && total != kProb) {  // checked on the host; never index the table with a bad one
+    if (total != kProb) {  // checked on the host; never fill the table from a bad one
         if (lane == 0) atomicOr(err, kErrCorrupt);
         return;
     }
+    uint32_t x = __ldg(reinterpret_cast<const uint32_t *>(p + 512) + lane);  // little-endian
+    // the ring holds the payload from its last aligned 16 bytes before the
+    // words on: word i is at place i + kLead of that stream
+    constexpr uint32_t kLead = (kTileHeader & 15u) / 2;
+    uint8_t *ring = sm + warp * kWarpSmem + 4 * kProb;
+    const uint8_t *stream = p + (kTileHeader & ~15u);
+    const uint32_t stream_bytes = 2 * (d.n_words + kLead);
+    // one group (8 bytes per lane), whole copies that start inside the
+    // payload: they end inside the padded buffer
+    auto fetch = [&](uint32_t group) {
+        const uint32_t at = group * 2 * kGroup + 8 * lane;
+        if (at < stream_bytes)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(ring + (at & (2 * kRing - 1)))),
+                         "l"(stream + at)
+                         : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (uint32_t k = 0; k < 4; k++) fetch(k);
+    // slot r of symbol s: (r - cum) | s << 12 | (freq - 1) << 20
     uint32_t c = incl - local;
 #pragma unroll
     for (int k = 0; k < 8; k++) {
-        freq[8 * lane + k] = (uint16_t)f8[k];
-        cum[8 * lane + k] = (uint16_t)c;
-        c += f8[k];
-    }
-    __syncwarp();
-    // slot r -> the last symbol s with cum[s] <= r (its frequency is then > 0)
-    if (d.m) {
-        for (uint32_t r = lane; r < kProb; r += 32) {
-            uint32_t lo = 0, hi = 255;
-            while (lo < hi) {
-                const uint32_t mid = (lo + hi + 1) >> 1;
-                if (cum[mid] <= r) lo = mid; else hi = mid - 1;
-            }
-            lut[r] = (uint8_t)lo;
+        const uint32_t f = (fw[k >> 1] >> (16 * (k & 1))) & 0xffffu;
+        for (int l = 0; l < 32; l++) {
+            const uint32_t fl = __shfl_sync(0xffffffffu, f, l), cl = __shfl_sync(0xffffffffu, c, l);
+            const uint32_t e = ((uint32_t)(8 * l + k) << 12) | ((fl - 1u) << 20);
+            for (uint32_t j = lane; j < fl; j += 32) lut[cl + j] = e | j;
         }
+        c += f;
     }
     __syncwarp();
-    uint32_t x = __ldg(reinterpret_cast<const uint32_t *>(p + 512) + lane);  // little-endian
-    const uint16_t *words = reinterpret_cast<const uint16_t *>(p + kTileHeader);
     uint8_t *out = d.dst < plane_bytes ? planes + d.dst : lits + (d.dst - plane_bytes);
-    uint32_t next = 0;
+    uint32_t pos = kLead, group = 0;  // next word's place, and the group it lies in
     bool bad = x < kStateLow;
-    for (uint32_t base = 0; base < d.m; base += 32) {
-        const uint32_t i = base + (uint32_t)lane;
-        const bool act = i < d.m && !bad;
-        uint32_t y = x;
-        if (act) {
-            const uint32_t r = x & (kProb - 1);
-            const uint32_t s = lut[r];
-            out[i] = (uint8_t)s;
-            y = (uint32_t)freq[s] * (x >> kProbBits) + r - cum[s];
-        }
+    const unsigned below = (1u << lane) - 1u;
+    const uint32_t ring_at = smem_u32(ring);
+    // one step: the state's symbol, and a word for every lane whose state
+    // fell below kStateLow, in lane order (past the end it takes whatever the
+    // ring holds; the count at the end then differs)
+    auto step = [&](uint8_t *to, bool act) {
+        const uint32_t e = lut[x & (kProb - 1)], xh = x >> kProbBits;
+        const uint32_t y = (e >> 20) * xh + (xh + (e & (kProb - 1)));
         const bool need = act && y < kStateLow;
         const unsigned bm = __ballot_sync(0xffffffffu, need);
-        const uint32_t idx = next + (uint32_t)__popc(bm & ((1u << lane) - 1u));
-        if (need) {
-            if (idx < d.n_words) y = (y << 16) | (uint32_t)__ldg(words + idx);
-            else bad = true;
+        const uint32_t o = pos + (uint32_t)__popc(bm & below);
+        uint16_t w;
+        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(w) : "r"(ring_at + ((2 * o) & (2 * kRing - 1))));
+        if (act) *to = (uint8_t)(e >> 12);
+        x = act ? (need ? (y << 16) | w : y) : x;
+        pos += (uint32_t)__popc(bm);
+    };
+    // the groups of the next four steps have landed: all but the newest two
+    auto look = [&]() {
+        if (pos / kGroup != group) {
+            __syncwarp();  // every lane is past the group that is overwritten
+            fetch(group + 4);
+            group++;
+            asm volatile("cp.async.wait_group 2;" ::: "memory");
+            __syncwarp();
         }
-        next += (uint32_t)__popc(bm);
-        x = y;
+    };
+    asm volatile("cp.async.wait_group 2;" ::: "memory");
+    __syncwarp();
+    uint8_t *to = out + lane;
+    const uint32_t whole = d.m >> 5;
+    uint32_t i = 0;
+    for (; i + 4 <= whole; i += 4, to += 128) {
+        step(to, true);
+        step(to + 32, true);
+        step(to + 64, true);
+        step(to + 96, true);
+        look();
     }
-    if (next != d.n_words || x != kStateLow) bad = true;  // every state back where encoding began
+    for (; i < whole; i++, to += 32) step(to, true);
+    if (d.m & 31u) step(to, (uint32_t)lane < (d.m & 31u));
+    if (pos != d.n_words + kLead || x != kStateLow) bad = true;  // every state back where encoding began
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(err, kErrCorrupt);
 }
 
@@ -158,14 +197,15 @@ int fill_from_acle(aclz_handle *h, const View &v, const void *ctx, void *stream)
         return rc == ACLZ_OK;
     };
     const uint64_t nt = a.tiles.size();
-    if (ck(dev_alloc((void **)&d_pay, a.pay_bytes ? a.pay_bytes : 16, st)) &&
+    if (ck(dev_alloc((void **)&d_pay, a.pay_bytes + 16, st)) &&
         ck(dev_alloc((void **)&d_td, sizeof(TileDesc) * (nt ? nt : 1), st)) &&
         ck(dev_alloc((void **)&d_planes, a.plane_bytes ? a.plane_bytes : 16, st)) && ck(dev_alloc((void **)&d_err, 4, st)) &&
         ck(cudaMemsetAsync(d_err, 0, 4, st)) &&
         (!a.pay_bytes || ck(cudaMemcpyAsync(d_pay, a.pay, a.pay_bytes, cudaMemcpyHostToDevice, st))) &&
         (!nt || ck(cudaMemcpyAsync(d_td, a.tiles.data(), sizeof(TileDesc) * nt, cudaMemcpyHostToDevice, st)))) {
         if (a.ev_begin) ck(cudaEventRecord(a.ev_begin, st));
-        if (nt) {
+        if (nt && ck(cudaFuncSetAttribute(k_ans_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          kWarps * kWarpSmem))) {
             const unsigned grid = (unsigned)((nt + kWarps - 1) / kWarps);
             k_ans_tiles<<<grid, kWarps * 32, kWarps * kWarpSmem, st>>>(d_pay, d_td, nt, d_planes, a.plane_bytes,
                                                                          h->d_lit, d_err);
@@ -234,8 +274,14 @@ extern "C" int aclz_upload_acle_ev(const void *host_buf, uint64_t n, uint32_t fl
             if (m != want || po % 16 || sz < kTileHeader || po > a.pay_bytes || sz > a.pay_bytes - po)
                 return ACLZ_E_CORRUPT;
             const uint8_t *tp = a.pay + po;
-            uint32_t fsum = 0;
-            for (int s = 0; s < 256; s++) fsum += (uint32_t)tp[2 * s] | ((uint32_t)tp[2 * s + 1] << 8);
+            // sum of the 256 little-endian 16-bit frequencies, four at a time
+            uint64_t lo = 0, hi = 0;
+            for (int q = 0; q < 64; q++) {
+                const uint64_t w = rd64le(tp + 8 * q);
+                lo += w & 0x0000ffff0000ffffULL;
+                hi += (w >> 16) & 0x0000ffff0000ffffULL;
+            }
+            const uint64_t fsum = (lo & 0xffffffffULL) + (lo >> 32) + (hi & 0xffffffffULL) + (hi >> 32);
             const uint32_t nw = rd32le(tp + 512 + 128);
             if (fsum != kProb || (uint64_t)kTileHeader + 2ull * nw != sz) return ACLZ_E_CORRUPT;
             TileDesc d{};
