@@ -11,10 +11,9 @@
 // schedules run them:
 //  - ACLZ_MODE_WAVES: one kernel per wave (k_wave_copy), kernel boundaries
 //    as the wave barrier.  Where ACLZ_MODE_AUTO takes this schedule it goes
-//    by levels instead of waves when the upload found them (every match of a
-//    level is independent of the others, so no chain is left inside a step),
-//    and consecutive small steps run in one launch of one thread-block
-//    cluster (k_wave_run), the cluster barrier between them;
+//    by levels instead of waves when the upload found them, one kernel per
+//    level (k_level): every match of a level is independent of the others,
+//    so no chain is left inside a step;
 //  - ACLZ_MODE_PERSISTENT: one cooperative launch (k_ranges) over ranges of
 //    consecutive (block, wave) segments in wave-major order, with bounded
 //    waits on per-block completed-wave bits instead of wave barriers, so a
@@ -38,20 +37,22 @@ using namespace aclz;
 namespace {
 
 constexpr int kThreads = 256;
-// per-wave copy CTAs, and the CTAs of that size per SM the register cap
-// is set for (the same 85 registers a thread as 3 x 256)
-constexpr int kWaveThreads = 64, kWaveMinCtas = 768 / kWaveThreads;
+// per-wave copy CTAs, and the CTAs of that size per SM the register cap is
+// set for
+constexpr int kWaveThreads = 64, kWaveMinCtas = 1024 / kWaveThreads;
+// per-level copies: CTA size, CTAs per SM, stage bytes per warp (16 matches
+// of up to 192 bytes), and the level sizes up to which a group of G lanes
+// takes G / 4 and G / 8 matches instead of G / 2
+constexpr int kLevelThreads = 128, kLevelMinCtas = 9;
+constexpr uint32_t kStageWarp = 3584;
+constexpr uint64_t kLevelQuarter = 40000, kLevelEighth = 20000;
 // literal copies: CTA size, CTAs of that size per SM the register cap is set
 // for, chunks per lane per round
-constexpr int kLitThreads = 128, kLitMinCtas = 6, kUnrollLits = 3;
-// small levels and waves: one cluster of kRunCtas CTAs runs consecutive
-// ones of at most kRunMost matches each, one window of 32 per warp
-constexpr int kRunThreads = 512, kRunCtas = 8;
-constexpr uint64_t kRunMost = (uint64_t)kRunThreads * kRunCtas;
-constexpr int kUnrollCopy = 3;   // chunks per lane per round in per-wave match copies
+constexpr int kLitThreads = 128, kLitMinCtas = 8, kUnrollLits = 2;
+constexpr int kUnrollCopy = 2;   // chunks per lane per round in per-wave match copies
 constexpr int kUnrollRanges = 4; // the same in the persistent schedule's register copies
 // staged (TMA) copies: jobs of at least kTmaMin bytes, pieces of <= kPiece
-constexpr uint32_t kTmaMin = (uint32_t)kPersistentMin;
+constexpr uint32_t kTmaMin = 192;
 constexpr uint32_t kPiece = 2048;
 constexpr uint32_t kSmemPerSm = 220u * 1024u;  // stage memory shared by the CTAs of one SM
 // per-wave kernels are launched with programmatic stream serialization
@@ -174,7 +175,7 @@ __global__ void __launch_bounds__(kLitThreads, kLitMinCtas)
         const uint32_t after = g.shfl(nl, 0), right = g.shfl(l0, (g.lane + 1) & (G - 1));
         const uint32_t l1 = g.lane == G - 1 ? after : right;
         const uint32_t x = max(l0, lo), y = min(l1, hi);
-        group_copy<G, kUnrollLits, true>(g, out, bpos + d0 + (x - l0), ls + x, y > x ? y - x : 0u);
+        group_copy<G, kUnrollLits, kFromConst>(g, out, bpos + d0 + (x - l0), ls + x, y > x ? y - x : 0u);
         if (after >= hi) break;
     }
 }
@@ -355,12 +356,12 @@ __global__ void __launch_bounds__(kThreads, STAGED ? 2 : 3)
 // internal chain, marked at upload) is copied as it stands: no dependency
 // test, no look at its neighbours.  Otherwise the group owns the segments
 // (runs of one block) that start in its window, and cuttable triplets in
-template <int G, bool PDL>
+template <int G>
 __device__ __forceinline__ void wave_window(const Group<G> &g, const uint4 *__restrict__ tri, uint64_t n, uint64_t a,
                                             const uint4 t0, uint8_t *out, uint32_t log2bs) {
     const uint4 z4 = make_uint4(0, 0, 0, 0);
     if (!g.ballot(a + g.lane < n && !tri_cut(t0))) {
-        if (PDL) griddep_wait();
+        griddep_wait();
         group_copy<G, kUnrollCopy>(g, out, tri_dst(t0), out + tri_src(t0), tri_len(t0));
         return;
     }
@@ -379,7 +380,7 @@ __device__ __forceinline__ void wave_window(const Group<G> &g, const uint4 *__re
     uint4 nt = s + g.lane < n ? __ldg(tri + s + g.lane) : z4;
     uint64_t prev_blk = ~0ULL;
     // the worklist was written at upload; the sources, by earlier waves
-    if (PDL) griddep_wait();
+    griddep_wait();
     for (uint64_t cur = s; cur < n; cur += G) {
         const uint64_t i = cur + g.lane;
         const bool v = i < n;
@@ -421,110 +422,87 @@ __global__ void __launch_bounds__(kWaveThreads, kWaveMinCtas) k_wave_copy(const 
     const uint64_t a = (blockIdx.x * (uint64_t)kWaveThreads + threadIdx.x) / G * G;
     if (a >= n) return;
     const uint4 t0 = a + g.lane < n ? __ldg(tri + a + g.lane) : make_uint4(0, 0, 0, 0);
-    wave_window<G, true>(g, tri, n, a, t0, out, log2bs);
+    wave_window<G>(g, tri, n, a, t0, out, log2bs);
 }
 
-__device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-}
-
-// Consecutive small steps (in-order levels, waves) by one thread-block
-// cluster: every group takes windows of G triplets of the step in turn, and
-// the cluster barrier separates the steps.
+// One level's matches (all independent) through the groups' stages.
 //
-// Bound by the latency of a step: its sources from L2, its stores to L2
-// before the barrier, and the issue of one window of copies, about 3.7 us in
-// all where one kernel per step takes 5 to 10 us.  8 CTAs of 512 threads hold
-// 4096 lanes at 128 registers; 16 CTAs, or steps of up to 8192 matches, were
-// no faster, 768 threads at 80 registers 20% slower.  256 KiB of Markov
-// bytes (12 levels) 159 -> 52 us, the steps of 64 MiB of FASTQ-like text
-// 137 -> 95 us.
-template <int G>
-__global__ void __launch_bounds__(kRunThreads) k_wave_run(const Step *__restrict__ steps, uint32_t count, uint8_t *out,
-                                                          uint32_t log2bs) {
+// Bound by the latency of a window and its instruction count (about 1200
+// instructions for 32 matches of 128 bytes): most levels have fewer windows
+// than the GPU has resident groups, so a level takes as long as one window.
+// Hence few matches per group (G / 2, in small levels less), with heads and
+// tails in one step, and the sources of the whole window in flight at once.
+// Launches overlap (programmatic dependent launch): a small level costs 2.5
+// us.  512 MiB copy sweep at L = 128 899 -> 721 us against one window of G
+// matches per group through registers with small levels run one after another
+// by one thread-block cluster (3.7 us a level); 256 MiB at L = 32 / 64 / 185
+// 910 / 662 / 492 -> 792 / 563 / 337 us, 64 MiB of FASTQ-like text 154 -> 112
+// us, 64 batched streams 70 -> 48 us, 256 KiB of Markov bytes 52 -> 36 us.
+template <int G, int J>
+__global__ void __launch_bounds__(kLevelThreads, kLevelMinCtas)
+    k_level(const uint4 *__restrict__ tri, uint64_t n, uint8_t *out, uint32_t *err) {
+    constexpr int kGroups = kLevelThreads / G;
+    constexpr uint32_t kBytes = kStageWarp / 32 * G;
+    __shared__ __align__(128) uint8_t buf[kGroups][kBytes];
+    __shared__ __align__(8) uint64_t bar[kGroups];
     Group<G> g;
     griddep_launch_dependents();
-    const uint64_t a0 = (blockIdx.x * (uint64_t)kRunThreads + threadIdx.x) / G * G;
-    const uint64_t stride = (uint64_t)gridDim.x * kRunThreads;
-    const ulonglong2 *list = reinterpret_cast<const ulonglong2 *>(steps);
-    const uint4 z4 = make_uint4(0, 0, 0, 0);
-    // this step's and the next step's descriptor and first window are loaded
-    // before the barrier that the sources wait for
-    ulonglong2 cur = __ldg(list), nx = count > 1 ? __ldg(list + 1) : make_ulonglong2(0, 0);
-    auto window = [&](const ulonglong2 &s, uint64_t a) {
-        return a + g.lane < s.y ? __ldg(reinterpret_cast<const uint4 *>(s.x) + a + g.lane) : z4;
-    };
-    uint4 t0 = window(cur, a0);
+    const int gi = threadIdx.x / G;
+    Stage st = {buf[gi], bar + gi, kBytes, 0};
+    const uint64_t i = (blockIdx.x * (uint64_t)kLevelThreads + threadIdx.x) / G * J + g.lane;
+    const uint4 t = g.lane < J && i < n ? __ldg(tri + i) : make_uint4(0, 0, 0, 0);
+    if (g.lane == 0) mbar_init(st.bar, 1);
+    fence_mbar_init();
+    g.sync();
     griddep_wait();
-    for (uint32_t k = 0; k < count; k++) {
-        const uint4 *tri = reinterpret_cast<const uint4 *>(cur.x);
-        for (uint64_t a = a0; a < cur.y; a += stride) {
-            const uint4 t = t0;
-            if (a + stride < cur.y) t0 = window(cur, a + stride);
-            wave_window<G, false>(g, tri, cur.y, a, t, out, log2bs);
-        }
-        if (k + 1 == count) break;
-        cur = nx;
-        t0 = window(cur, a0);
-        if (k + 2 < count) nx = __ldg(list + k + 2);
-        cluster_barrier();
-    }
+    fence_proxy_async_global();
+    group_copy_staged<G, J>(g, st, out, tri_dst(t), out + tri_src(t), tri_len(t), err);
 }
 
-// Length of the run of small steps from step i on that share one cluster
-// launch (0: step i has a kernel of its own).
-uint32_t run_length(const std::vector<Step> &s, uint32_t i, uint32_t i1, bool merge) {
-    uint32_t j = i;
-    while (merge && j < i1 && s[j].n <= kRunMost) j++;
-    return j - i;
-}
-
-// Kernel launches of the steps [i0, i1).
-uint32_t count_steps(const std::vector<Step> &s, uint32_t i0, uint32_t i1, bool merge) {
-    uint32_t n = 0;
-    for (uint32_t i = i0; i < i1; n++) i += std::max(1u, run_length(s, i, i1, merge));
-    return n;
-}
-
-template <int G>
-int launch_steps(const aclz_handle *h, const std::vector<Step> &steps, const void *d_steps, uint8_t *out,
-                 cudaStream_t st, uint32_t i0, uint32_t i1, bool merge) {
-    // programmatic stream serialization: a step's CTAs may start (and load
-    // their worklist) while the previous kernel's last CTAs finish
-    cudaLaunchAttribute at[2];
+// Launch of one step kernel with programmatic stream serialization: its CTAs
+// may start (and load their worklist) while the previous kernel's last ones
+// finish.
+template <class... P, class... A>
+int launch_step(void (*k)(P...), uint64_t n, unsigned per_cta, unsigned threads, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = kWavePdl;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = kRunCtas;
-    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t lc = {};
-    lc.dynamicSmemBytes = 0;
+    lc.gridDim = dim3((unsigned)((n + per_cta - 1) / per_cta));
+    lc.blockDim = dim3(threads);
     lc.stream = st;
     lc.attrs = at;
-    const uint32_t lb = h->log2_bs;
-    for (uint32_t i = i0; i < i1;) {
-        const uint32_t run = run_length(steps, i, i1, merge);
-        cudaError_t e;
-        if (run) {
-            lc.gridDim = dim3(kRunCtas);
-            lc.blockDim = dim3(kRunThreads);
-            lc.numAttrs = 2;
-            e = cudaLaunchKernelEx(&lc, k_wave_run<G>, (const Step *)d_steps + i, run, out, lb);
-        } else {
-            const uint64_t n = steps[i].n, groups = (n + G - 1) / G;
-            constexpr int gpcw = kWaveThreads / G;
-            lc.gridDim = dim3((unsigned)((groups + gpcw - 1) / gpcw));
-            lc.blockDim = dim3(kWaveThreads);
-            lc.numAttrs = 1;
-            e = cudaLaunchKernelEx(&lc, k_wave_copy<G>, (const uint4 *)steps[i].tri, n, out, lb);
-        }
-        if (e != cudaSuccess) {
-            note_cuda_error(e);
-            return ACLZ_E_CUDA;
-        }
-        i += std::max(1u, run);
+    lc.numAttrs = 1;
+    if (cudaError_t e = cudaLaunchKernelEx(&lc, k, static_cast<P>(args)...); e != cudaSuccess) {
+        note_cuda_error(e);
+        return ACLZ_E_CUDA;
     }
+    return ACLZ_OK;
+}
+
+// Levels: one kernel each, fewer matches per group in the small ones, whose
+// groups are all resident at once and take as long as their own window.
+template <int G>
+int launch_levels(const aclz_handle *h, const std::vector<Step> &levels, uint32_t count, uint8_t *out,
+                  cudaStream_t st) {
+    for (uint32_t i = 0; i < count; i++) {
+        const uint64_t n = levels[i].n;
+        const int part = n <= kLevelEighth ? 8 : n <= kLevelQuarter ? 4 : 2;
+        auto k = part == 8 ? k_level<G, G / 8> : part == 4 ? k_level<G, G / 4> : k_level<G, G / 2>;
+        if (int rc = launch_step(k, n, kLevelThreads / part, kLevelThreads, st, (const uint4 *)levels[i].tri, n, out,
+                                 h->d_err))
+            return rc;
+    }
+    return ACLZ_OK;
+}
+
+// Waves >= 1: one kernel each.
+template <int G>
+int launch_wave_steps(const aclz_handle *h, uint8_t *out, cudaStream_t st) {
+    for (size_t i = h->n_ord_steps; i < h->steps.size(); i++)
+        if (int rc = launch_step(k_wave_copy<G>, h->steps[i].n, kWaveThreads, kWaveThreads, st,
+                                 (const uint4 *)h->steps[i].tri, h->steps[i].n, out, h->log2_bs))
+            return rc;
     return ACLZ_OK;
 }
 
@@ -543,15 +521,15 @@ int launch_lits(aclz_handle *h, uint8_t *out, cudaStream_t st, bool persistent) 
     return ACLZ_OK;
 }
 
+// By levels where the caller left the mode open and the upload found them;
+// else the in-order levels, then one kernel per wave.
 template <int G>
-int launch_waves(aclz_handle *h, uint8_t *out, cudaStream_t st, cudaEvent_t phase, bool merge) {
-    const uint32_t n = (uint32_t)h->steps.size(), no = h->n_ord_steps;
+int launch_waves(aclz_handle *h, uint8_t *out, cudaStream_t st, cudaEvent_t phase, bool by_level) {
     if (int rc = launch_lits<G>(h, out, st, false)) return rc;
-    if (merge && !phase && h->by_level)
-        return launch_steps<G>(h, h->lsteps, h->d_lsteps, out, st, 0, (uint32_t)h->lsteps.size(), true);
-    if (int rc = launch_steps<G>(h, h->steps, h->d_steps, out, st, 0, no, true)) return rc;
+    if (by_level && !phase) return launch_levels<G>(h, h->lsteps, (uint32_t)h->lsteps.size(), out, st);
+    if (int rc = launch_levels<G>(h, h->steps, h->n_ord_steps, out, st)) return rc;
     if (phase) cudaEventRecord(phase, st);
-    return launch_steps<G>(h, h->steps, h->d_steps, out, st, no, n, merge);
+    return launch_wave_steps<G>(h, out, st);
 }
 
 struct Occ {
@@ -574,7 +552,7 @@ template <int G, bool STAGED>
 int launch_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaStream_t st, cudaEvent_t phase) {
     constexpr int gpc = kThreads / G;
     if (int rc = launch_lits<G>(h, out, st, true)) return rc;
-    if (int rc = launch_steps<G>(h, h->steps, h->d_steps, out, st, 0, h->n_ord_steps, true)) return rc;
+    if (int rc = launch_levels<G>(h, h->steps, h->n_ord_steps, out, st)) return rc;
     if (phase) cudaEventRecord(phase, st);
     if (!h->n_ranges) return ACLZ_OK;
     auto fn = k_ranges<G, STAGED>;
@@ -666,9 +644,11 @@ int launch_persistent_auto(aclz_handle *h, uint8_t *out, const aclz_decode_cfg &
 
 namespace {
 
-// Small waves share a launch only when the caller left the mode open: an
+// Levels take the place of waves only when the caller left the mode open: an
 // explicit ACLZ_MODE_WAVES is one kernel per wave.
-bool is_auto(const aclz_decode_cfg *cfg) { return !cfg || cfg->mode == ACLZ_MODE_AUTO; }
+bool goes_by_level(const aclz_handle *h, const aclz_decode_cfg *cfg) {
+    return h->by_level && (!cfg || cfg->mode == ACLZ_MODE_AUTO);
+}
 
 // Checks cfg and resolves ACLZ_MODE_AUTO for this handle.
 int resolve_cfg(const aclz_handle *h, const aclz_decode_cfg *cfg, aclz_decode_cfg &c) {
@@ -679,8 +659,8 @@ int resolve_cfg(const aclz_handle *h, const aclz_decode_cfg *cfg, aclz_decode_cf
         return ACLZ_E_INVAL;
     if (c.mode == ACLZ_MODE_AUTO) {
         // long deferred matches: one persistent launch with TMA staging;
-        // short ones: the per-wave kernels
-        c.mode = h->mean_deferred_len >= (double)kTmaMin ? ACLZ_MODE_PERSISTENT : ACLZ_MODE_WAVES;
+        // short ones: by levels (or waves)
+        c.mode = decodes_as_waves(h) ? ACLZ_MODE_WAVES : ACLZ_MODE_PERSISTENT;
         if (c.mode == ACLZ_MODE_PERSISTENT && !(c.flags & ACLZ_FLAG_REGISTERS)) c.flags |= ACLZ_FLAG_STAGED;
     }
     if ((c.flags & ACLZ_FLAG_STAGED) && (c.flags & ACLZ_FLAG_REGISTERS)) return ACLZ_E_INVAL;
@@ -698,13 +678,10 @@ extern "C" int aclz_decode_plan(const aclz_handle *h, const aclz_decode_cfg *cfg
     if (int rc = resolve_cfg(h, cfg, c)) return rc;
     uint32_t n = 0;
     if (h->n_blocks) {
-        const uint32_t no = h->n_ord_steps, ns = (uint32_t)h->steps.size();
         if (c.mode == ACLZ_MODE_PERSISTENT)
-            n = 1 + count_steps(h->steps, 0, no, true) + (h->n_ranges ? 1 : 0);
-        else if (is_auto(cfg) && h->by_level)
-            n = 1 + count_steps(h->lsteps, 0, (uint32_t)h->lsteps.size(), true);
+            n = 1 + h->n_ord_steps + (h->n_ranges ? 1 : 0);
         else
-            n = 1 + count_steps(h->steps, 0, no, true) + count_steps(h->steps, no, ns, is_auto(cfg));
+            n = 1 + (uint32_t)(goes_by_level(h, cfg) ? h->lsteps.size() : h->steps.size());
     }
     if (resolved) *resolved = c;
     if (launches) *launches = n;
@@ -730,9 +707,9 @@ extern "C" int aclz_decode_all_ev(aclz_handle *h, void *d_out, uint64_t cap, con
         }
     }
     switch (c.G) {
-        case 8: return launch_waves<8>(h, out, st, ev, is_auto(cfg));
-        case 16: return launch_waves<16>(h, out, st, ev, is_auto(cfg));
-        default: return launch_waves<32>(h, out, st, ev, is_auto(cfg));
+        case 8: return launch_waves<8>(h, out, st, ev, goes_by_level(h, cfg));
+        case 16: return launch_waves<16>(h, out, st, ev, goes_by_level(h, cfg));
+        default: return launch_waves<32>(h, out, st, ev, goes_by_level(h, cfg));
     }
 }
 

@@ -86,21 +86,26 @@ __device__ __forceinline__ uint4 window16(uint4 a, uint4 b, uint32_t r) {
     return o;
 }
 
-// One aligned source word: L2 (bytes other kernels wrote), or the
-// non-coherent L1 path (RO: bytes nobody writes during the kernel).
-template <bool RO>
+// Where a copy reads: L2 (bytes other kernels wrote), the non-coherent L1
+// path (bytes nobody writes during the kernel), or shared memory (addresses
+// in the shared window).
+enum Source { kFromL2, kFromConst, kFromShared };
+
+// One aligned source word.
+template <Source SRC>
 __device__ __forceinline__ uint4 ld_word(uintptr_t a) {
-    return RO ? __ldg(reinterpret_cast<const uint4 *>(a)) : __ldcg(reinterpret_cast<const uint4 *>(a));
+    if (SRC == kFromShared) return lds16_u32((uint32_t)a);
+    return SRC == kFromConst ? __ldg(reinterpret_cast<const uint4 *>(a)) : __ldcg(reinterpret_cast<const uint4 *>(a));
 }
 
 // The 16 bytes from s on, of which the first n (1 <= n <= 16) are wanted:
 // only the aligned words holding wanted bytes are read.
-template <bool RO>
+template <Source SRC>
 __device__ __forceinline__ uint4 load_bytes(uintptr_t s, uint32_t n) {
     const uint32_t r = (uint32_t)s & 15u;
     const uintptr_t base = s & ~(uintptr_t)15;
-    uint4 a = ld_word<RO>(base), b = a;
-    if (r + n > 16) b = ld_word<RO>(base + 16);
+    uint4 a = ld_word<SRC>(base), b = a;
+    if (r + n > 16) b = ld_word<SRC>(base + 16);
     return window16(a, b, r);
 }
 
@@ -174,7 +179,7 @@ __device__ __forceinline__ int select_bit(unsigned m, uint32_t o) {
 // before stores.  The job of a chunk is found from the starts of the jobs
 // within the slot of G chunks: one bit per start, or-reduced over the group,
 // counted up to the own lane.
-template <int G, int U, bool RO>
+template <int G, int U, Source SRC>
 __device__ __forceinline__ void copy_full_chunks(const Group<G> &g, uintptr_t P, uintptr_t S, uint32_t c,
                                                  unsigned have) {
     if (have & (have + 1u)) {  // bring the jobs to the lowest lanes
@@ -212,8 +217,8 @@ __device__ __forceinline__ void copy_full_chunks(const Group<G> &g, uintptr_t P,
                 dst[u] = dj;
                 r[u] = (uint32_t)sj & 15u;
                 const uintptr_t w = sj & ~(uintptr_t)15;
-                a[u] = ld_word<RO>(w);
-                if (r[u]) b[u] = ld_word<RO>(w + 16);
+                a[u] = ld_word<SRC>(w);
+                if (r[u]) b[u] = ld_word<SRC>(w + 16);
             }
         }
 #pragma unroll
@@ -222,14 +227,13 @@ __device__ __forceinline__ void copy_full_chunks(const Group<G> &g, uintptr_t P,
     }
 }
 
-// Packed group copy.  Each lane holds one job (d: output offset, s: source
-// pointer, n: length; n == 0 for none).  A job of at most 16 bytes is copied
+// Packed group copy.  Each lane holds one job (p: output address, q:
+// source address, n: length; n == 0 for none).  A job of at most 16 bytes is copied
 // by its own lane; of a longer one the lane copies the bytes before the
 // first and after the last 16-byte boundary of the output, and the full
 // chunks between are dealt to the whole group (copy_full_chunks).  Jobs must
 // be independent: no job's source may overlap another job's output in the
-// same call.  RO: the source is global memory that no thread writes during
-// the kernel.
+// same call.
 //
 // The copy is issue-bound, so it is built to take few instructions.  Against
 // a form that searched every chunk's job by shuffles and cut its partial
@@ -237,20 +241,24 @@ __device__ __forceinline__ void copy_full_chunks(const Group<G> &g, uintptr_t P,
 // decodes on GB300: 32 MiB of word text at 6/8/10/12, flattened (pieces of
 // 3 bytes), 1217 -> 911 us; the 512 MiB copy sweep at L = 128 1096 -> 1038 us;
 // 64 MiB of FASTQ-like text at 12/16/24/32 244 -> 230 us.
-template <int G, int U, bool RO = false>
-__device__ __forceinline__ void group_copy(const Group<G> &g, uint8_t *out, uint64_t d, const uint8_t *s,
-                                           uint32_t n) {
-    const uintptr_t p = reinterpret_cast<uintptr_t>(out) + d, q = reinterpret_cast<uintptr_t>(s);
+template <int G, int U, Source SRC>
+__device__ __forceinline__ void group_copy_from(const Group<G> &g, uintptr_t p, uintptr_t q, uint32_t n) {
     const uint32_t head = n <= 16 ? n : (0u - (uint32_t)p) & 15u;
     const uint32_t rest = n - head;           // of a job longer than 16 bytes
     const uint32_t tail = rest & 15u, c = rest >> 4;
     uint4 hv = make_uint4(0, 0, 0, 0), tv = hv;
-    if (head) hv = load_bytes<RO>(q, head);
-    if (tail) tv = load_bytes<RO>(q + n - tail, tail);
+    if (head) hv = load_bytes<SRC>(q, head);
+    if (tail) tv = load_bytes<SRC>(q + n - tail, tail);
     const unsigned have = g.ballot(c > 0);
-    if (have) copy_full_chunks<G, U, RO>(g, p + head, q + head, c, have);
+    if (have) copy_full_chunks<G, U, SRC>(g, p + head, q + head, c, have);
     if (g.ballot(head > 0)) store_bytes(p, hv, head);
     if (g.ballot(tail > 0)) store_bytes(p + n - tail, tv, tail);
+}
+
+template <int G, int U, Source SRC = kFromL2>
+__device__ __forceinline__ void group_copy(const Group<G> &g, uint8_t *out, uint64_t d, const uint8_t *s,
+                                           uint32_t n) {
+    group_copy_from<G, U, SRC>(g, reinterpret_cast<uintptr_t>(out) + d, reinterpret_cast<uintptr_t>(s), n);
 }
 
 // Bytes [r, r + 16) of a || b for a shift r that is the same on every lane
@@ -449,6 +457,64 @@ __device__ __forceinline__ bool staged_copy_fills(const Group<G> &g, Stage &st, 
         if (!fill_consume<G>(g, st, out, d, f, err)) return false;
         if (!fill_issue<G>(g, st, s, n, piece, f)) return true;
     }
+}
+
+// Packed group copy of at most J <= G / 2 jobs, in the lowest lanes (n == 0
+// in the others), from shared memory: the next J lanes copy what the first
+// ones have after their jobs' last 16-byte boundary, so that heads and tails
+// take one step together.
+template <int G, int J>
+__device__ __forceinline__ void group_copy_few(const Group<G> &g, uintptr_t p, uintptr_t q, uint32_t n) {
+    const uint32_t head = n <= 16 ? n : (0u - (uint32_t)p) & 15u;
+    const uint32_t rest = n - head, c = rest >> 4;
+    const int from = g.lane & (J - 1);
+    const uintptr_t pe = (uintptr_t)g.shfl((unsigned long long)(p + n), from);
+    const uint32_t qe = g.shfl((uint32_t)q + n, from), tail = g.shfl(rest & 15u, from);
+    const bool second = g.lane >= J;
+    const uintptr_t ep = second ? pe - tail : p, eq = second ? qe - tail : (uint32_t)q;
+    const uint32_t en = !second ? head : g.lane < 2 * J ? tail : 0u;
+    uint4 ev = make_uint4(0, 0, 0, 0);
+    if (en) ev = load_bytes<kFromShared>(eq, en);
+    const unsigned have = g.ballot(c > 0);
+    if (have) copy_full_chunks<G, 1, kFromShared>(g, p + head, q + head, c, have);
+    store_bytes(ep, ev, en);
+}
+
+// Copy of at most J <= G / 2 jobs (in the lowest lanes) through the group's
+// stage: every job's aligned source span by one bulk copy, as many
+// jobs at a time as the stage holds, then the packed copy from shared
+// memory.  All of a window's source bytes are in flight at once and each is
+// fetched once, where the copy through registers has U rounds of chunks in
+// flight and reads every word of an unaligned source twice.  Jobs larger
+// than the stage are copied through registers.  The sources are final and
+// visible to bulk copies.  False when a wait timed out (see stage_wait).
+template <int G, int J>
+__device__ __forceinline__ bool group_copy_staged(const Group<G> &g, Stage &st, uint8_t *out, uint64_t d,
+                                                  const uint8_t *s, uint32_t n, uint32_t *err) {
+    const uintptr_t q = reinterpret_cast<uintptr_t>(s), qa = q & ~(uintptr_t)15;
+    uint32_t span = n ? (uint32_t)(((q + n + 15) & ~(uintptr_t)15) - qa) : 0u;
+    while (g.ballot(span > 0)) {
+        const uint32_t incl = g.scan_incl(span);
+        const bool take = span > 0 && incl <= st.bytes;
+        const unsigned tm = g.ballot(take);
+        if (!tm) {
+            group_copy<G, 1>(g, out, d, s, span ? n : 0u);
+            return true;
+        }
+        const uint32_t tx = g.shfl(incl, 31 - __clz(tm)), off = incl - span;
+        if (g.lane == 0) mbar_expect_tx(st.bar, tx);
+        g.sync();
+        if (take) tma_load_1d(st.buf + off, reinterpret_cast<const void *>(qa), span, st.bar);
+        if (g.ballot(!stage_wait(st, err))) return false;
+        group_copy_few<G, J>(g, reinterpret_cast<uintptr_t>(out) + d, smem_u32(st.buf) + off + (uint32_t)(q - qa),
+                           take ? n : 0u);
+        if (take) span = 0;
+        if (g.ballot(span > 0)) {  // the stage is filled again
+            g.sync();
+            fence_proxy_async_shared();
+        }
+    }
+    return true;
 }
 
 }  // namespace aclz

@@ -984,7 +984,8 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     }
     CK(dev_alloc((void **)&h->d_done, 8 * (size_t)nb * h->n_wave_words, st));
     CK(cudaStreamSynchronize(st));
-    return build_steps(h, stream);
+    build_steps(h);
+    return ACLZ_OK;
 }
 
 extern "C" int aclz_upload(const void *host_buf, uint64_t n, void *stream, aclz_handle **out) {

@@ -74,10 +74,10 @@ namespace aclz {
 // Wave 0's index (aclz_wave0.cu): literal units, and the level list of the
 // in-order matches, or with all of every match.  d_val: {level, tag} of every
 // token and maxlvl the largest level, or null when the levels are not known
-// (the in-order ones are then found block by block).  The step tables follow
+// (the in-order ones are then found block by block).  The step lists follow
 // once the worklists are final.
 int build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlvl, bool all, void *stream);
-int build_steps(aclz_handle *h, void *stream);
+void build_steps(aclz_handle *h);
 void free_wave0(aclz_handle *h, void *stream);
 
 // Deferred matches of at least this mean length are decoded by the
@@ -152,9 +152,8 @@ struct aclz_handle {
     bool by_level = false;
     // what follows the literals, in order: in steps the in-order levels
     // (n_ord_steps of them), then the non-empty waves; in lsteps every
-    // level.  d_steps and d_lsteps are the same on the device.
+    // level
     std::vector<aclz::Step> steps, lsteps;
-    void *d_steps = nullptr, *d_lsteps = nullptr;
     uint32_t n_ord_steps = 0;
     // persistent-mode schedule.  A segment is the run of one block's
     // matches in one wave's worklist: seg[s] = {block, wave, triplet offset,

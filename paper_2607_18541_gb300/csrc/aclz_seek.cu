@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kSeekThreads, 6) k_seek(const SeekReq *__restr
                     ls = ix.lit + __ldg(ix.blk_lit + bb) + __ldg(ix.toklit + ti) + (lx - ts);
                 }
             }
-            group_copy<32, 1, true>(g, out, ld, ls, ln);
+            group_copy<32, 1, kFromConst>(g, out, ld, ls, ln);
             // what a match covers of the window, its first stretch from one
             // source, is the lane's own piece; the rest waits on the stack
             uint64_t a = 0;
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kSeekThreads, 6) k_seek(const SeekReq *__restr
                 rm = g.ballot(rest > 0);
                 if (rest) stk[sp + __popc(rm & g.lanemask_lt())] = pack_piece(from, rest, co + (cl ? cl : n));
                 sp += __popc(rm);
-                if (g.ballot(cl > 0)) group_copy<32, 1, true>(g, out, co, cs, cl);
+                if (g.ballot(cl > 0)) group_copy<32, 1, kFromConst>(g, out, co, cs, cl);
                 __syncwarp();
             }
             at = wend;

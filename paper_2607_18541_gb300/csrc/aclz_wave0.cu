@@ -182,7 +182,7 @@ __global__ void k_lev_gather(const uint4 *__restrict__ tri, const uint32_t *__re
 
 void aclz::free_wave0(aclz_handle *h, void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
-    for (void **pp : {&h->d_lunits, &h->d_lev, &h->d_steps, &h->d_lsteps}) {
+    for (void **pp : {&h->d_lunits, &h->d_lev}) {
         dev_free(*pp, st);
         *pp = nullptr;
     }
@@ -250,12 +250,7 @@ int aclz::build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t 
     return ACLZ_OK;
 }
 
-int aclz::build_steps(aclz_handle *h, void *stream) {
-    cudaStream_t st = (cudaStream_t)stream;
-    for (void **pp : {&h->d_steps, &h->d_lsteps}) {
-        dev_free(*pp, st);
-        *pp = nullptr;
-    }
+void aclz::build_steps(aclz_handle *h) {
     h->steps.clear();
     h->lsteps.clear();
     auto add = [](std::vector<Step> &v, const void *tri, uint64_t a, uint64_t b) {
@@ -269,11 +264,4 @@ int aclz::build_steps(aclz_handle *h, void *stream) {
     h->n_ord_steps = (uint32_t)h->steps.size();
     for (uint32_t w = 1; w < h->n_waves && h->d_tri; w++)
         add(h->steps, h->d_tri, h->wave_start[w], h->wave_start[w + 1]);
-    for (auto &pr : {std::make_pair(&h->steps, &h->d_steps), std::make_pair(&h->lsteps, &h->d_lsteps)}) {
-        if (pr.first->empty()) continue;
-        W0CK(dev_alloc((void **)pr.second, sizeof(Step) * pr.first->size(), st));
-        W0CK(cudaMemcpyAsync(*pr.second, pr.first->data(), sizeof(Step) * pr.first->size(), cudaMemcpyHostToDevice, st));
-    }
-    W0CK(cudaStreamSynchronize(st));
-    return ACLZ_OK;
 }

@@ -1,7 +1,8 @@
 """Wave 0 and the small steps where their tiling can go wrong: literal units
 around block and unit boundaries, in-order chains of more levels than one
-sort digit and of more matches than one window of the level pass, waves on
-both sides of the size that shares a cluster launch."""
+sort digit and of more matches than one window of the level pass, levels on
+both sides of the sizes that change the matches per group, matches around
+and past the size of a group's stage."""
 import numpy as np
 import pytest
 
@@ -100,9 +101,9 @@ def test_in_order_chains(chain, width):
     _decode_all_ways(c)
 
 
-@pytest.mark.parametrize("n", [4095, 4096, 4097])
-def test_steps_around_the_shared_launch(n):
-    # waves 1 and 3 of n matches, waves 2 and 4 of a few: AUTO shares launches
+@pytest.mark.parametrize("n", [20000, 20001, 40000, 40001])
+def test_levels_around_the_sizes_per_group(n):
+    # levels 1 and 3 of n matches, levels 2 and 4 of a few
     bs, ln = 1 << 17, 8
     blocks, pos = [[(bs, 0, 0)]], bs
     src, readable = 0, bs  # what the wave before wrote at the start of its first block
@@ -125,7 +126,27 @@ def test_steps_around_the_shared_launch(n):
         counts = aclz.aclz_wave_counts(h)
         assert counts[1:].tolist() == [n, 40, n, 3]
         assert aclz.aclz_decode_plan(h, mode=aclz.ACLZ_MODE_WAVES)[1] == 5
-        assert aclz.aclz_decode_plan(h)[1] == (2 if n <= 4096 else 5)
+        assert aclz.aclz_decode_plan(h)[1] == 5
     finally:
         aclz.aclz_free(h)
+    _decode_all_ways(c)
+
+
+@pytest.mark.parametrize("ln", [1, 15, 16, 17, 31, 33, 176, 177, 192, 200, 208, 224, 900, 3568, 3569, 3584, 5000])
+def test_match_lengths_around_the_stage(ln):
+    # every source alignment, matches that leave the stage room for 16, for
+    # fewer, for one and for none
+    bs = 1 << 15
+    blocks = [[(bs, 0, 0)]]
+    for b in range(1, 5):
+        toks, p = [], b * bs
+        k = 0
+        while p + ln + 3 <= (b + 1) * bs:
+            toks.append((k % 3, ln, (b - 1) * bs + (k * 37 + b) % (bs - ln)))
+            p += k % 3 + ln
+            k += 1
+        toks.append(((b + 1) * bs - p, 0, 0))
+        blocks.append(toks)
+    c = _pack(5 * bs, bs, blocks, LITS)
+    assert oracle.validate(c) == 0
     _decode_all_ways(c)
