@@ -266,7 +266,8 @@ int aclz_flatten(aclz_handle *h, void *stream);
  * After any other error the handle is left part-way and must be freed. */
 int aclz_reshape(aclz_handle *h, uint32_t rounds, void *stream);
 
-/* Regroup the persistent schedule into work ranges: runs of consecutive
+/* Regroup the persistent schedule's work ranges (used with register copies,
+ * and staged where the upload found no dependency levels): runs of consecutive
  * deferred matches of one wave (wave-major, block order), of about
  * range_bytes of matches (at least 8 matches, at most 4096) in large waves;
  * a wave with fewer matches than about 16 ranges per SM of that size is cut
@@ -285,24 +286,27 @@ typedef struct aclz_decode_cfg {
 } aclz_decode_cfg;
 
 #define ACLZ_MODE_WAVES 0      /* wave 0, then one kernel per wave */
-#define ACLZ_MODE_PERSISTENT 1 /* wave 0, then one launch with bounded per-block waits */
-#define ACLZ_MODE_AUTO 2       /* persistent + staged when deferred matches average >= 192 B, else waves */
+#define ACLZ_MODE_PERSISTENT 1 /* wave 0, then one launch with bounded waits */
+#define ACLZ_MODE_AUTO 2       /* persistent + staged when deferred matches average >= 1024 B, else waves, one
+                                  kernel per dependency level where the upload found the levels */
 #define ACLZ_FLAG_STAGED 1u    /* persistent: stage long matches through shared memory (TMA) */
 #define ACLZ_FLAG_REGISTERS 2u /* persistent: copy through registers only */
 
 /* Decode the whole stream into d_out (cap >= total_len bytes, 16-byte
  * aligned).  Enqueues on stream; capturable in a CUDA graph (no allocation,
  * no synchronization).  cfg NULL = {32, ACLZ_MODE_AUTO, 0, 0}.  The
- * persistent mode stages long matches through shared memory when the
- * deferred matches average at least 192 bytes, unless a flag forces one
- * copy path. */
+ * persistent mode stages matches through shared memory when the deferred
+ * matches average at least 192 bytes, unless a flag forces one copy path;
+ * staged, it runs the dependency levels found at upload, where there are
+ * any, else the work ranges of aclz_set_range_bytes. */
 int aclz_decode_all(aclz_handle *h, void *d_out, uint64_t cap, const aclz_decode_cfg *cfg,
                     void *stream);
 
 /* aclz_decode_all that also records phase_event (a cudaEvent_t owned by the
- * caller) on stream between its two phases: after the wave-0 kernel
+ * caller) on stream between its two phases: after wave 0
  * (literals and in-order matches; the wavefront decode of Sec. I) and before the deferred
- * matches of waves >= 1.  With its own events before and after the call a
+ * matches of waves >= 1 (so the decode goes by waves, not by levels that hold
+ * both kinds of match).  With its own events before and after the call a
  * caller times each phase on the launching stream.  phase_event NULL is
  * aclz_decode_all; a failed record is reported by the next CUDA call. */
 int aclz_decode_all_ev(aclz_handle *h, void *d_out, uint64_t cap, const aclz_decode_cfg *cfg,
@@ -310,8 +314,11 @@ int aclz_decode_all_ev(aclz_handle *h, void *d_out, uint64_t cap, const aclz_dec
 
 /* What aclz_decode_all would launch for this handle and cfg (no GPU work):
  * *resolved = cfg with ACLZ_MODE_AUTO resolved and the copy-path flag set;
- * *launches = kernel launches of one call (wave 0, then one persistent
- * launch or one per non-empty wave >= 1; 0 for an empty stream).  Either
+ * *launches = kernel launches of one call: the literal kernel, then for
+ * ACLZ_MODE_AUTO by levels one per level; else one per level of in-order
+ * matches (none in most streams without short distances; in the staged
+ * persistent launch where it runs levels) and one persistent launch or one
+ * per non-empty wave >= 1; 0 for an empty stream.  Either
  * output may be NULL.  ACLZ_E_INVAL for a bad cfg, as aclz_decode_all. */
 int aclz_decode_plan(const aclz_handle *h, const aclz_decode_cfg *cfg, aclz_decode_cfg *resolved,
                      uint32_t *launches);

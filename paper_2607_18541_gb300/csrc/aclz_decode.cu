@@ -14,11 +14,13 @@
 //    by levels instead of waves when the upload found them, one kernel per
 //    level (k_level): every match of a level is independent of the others,
 //    so no chain is left inside a step;
-//  - ACLZ_MODE_PERSISTENT: one cooperative launch (k_ranges) over ranges of
-//    consecutive (block, wave) segments in wave-major order, with bounded
-//    waits on per-block completed-wave bits instead of wave barriers, so a
-//    match is copied as soon as the blocks it reads have finished the waves
-//    below its own.
+//  - ACLZ_MODE_PERSISTENT: one cooperative launch.  With staged copies it
+//    runs the levels, with a bounded grid barrier between them
+//    (k_levels_persistent); with register copies, or when the upload found no
+//    levels (chains too deep), ranges of consecutive (block, wave) segments
+//    in wave-major order (k_ranges), with bounded waits on per-block
+//    completed-wave bits instead of barriers, so a match is copied as soon as
+//    the blocks it reads have finished the waves below its own.
 //
 // All copies are 16-byte vectorised with every lane owning aligned output
 // chunks, so short matches from several tokens share one pass instead of
@@ -40,11 +42,13 @@ constexpr int kThreads = 256;
 // per-wave copy CTAs, and the CTAs of that size per SM the register cap is
 // set for
 constexpr int kWaveThreads = 64, kWaveMinCtas = 1024 / kWaveThreads;
-// per-level copies: CTA size, CTAs per SM, stage bytes per warp (16 matches
-// of up to 192 bytes), and the level sizes up to which a group of G lanes
-// takes G / 4 and G / 8 matches instead of G / 2
+// per-level copies: CTA size, the CTAs per SM the register cap is set for,
+// stage bytes per warp (16 matches of up to 192 bytes; more when the deferred
+// matches average kStageLongMin bytes or more), and the level sizes up to
+// which a group of G lanes takes G / 4 and G / 8 matches instead of G / 2
 constexpr int kLevelThreads = 128, kLevelMinCtas = 9;
-constexpr uint32_t kStageWarp = 3584;
+constexpr uint32_t kStageWarp = 3584, kStageWarpLong = 6144;
+constexpr double kStageLongMin = 224.0;
 constexpr uint64_t kLevelQuarter = 40000, kLevelEighth = 20000;
 // literal copies: CTA size, CTAs of that size per SM the register cap is set
 // for, chunks per lane per round
@@ -54,6 +58,8 @@ constexpr int kUnrollRanges = 4; // the same in the persistent schedule's regist
 // staged (TMA) copies: jobs of at least kTmaMin bytes, pieces of <= kPiece
 constexpr uint32_t kTmaMin = 192;
 constexpr uint32_t kPiece = 2048;
+// persistent level copies: CTA size, CTAs per SM
+constexpr int kPersThreads = 512, kPersCtas = 2;
 constexpr uint32_t kSmemPerSm = 220u * 1024u;  // stage memory shared by the CTAs of one SM
 // per-wave kernels are launched with programmatic stream serialization
 constexpr int kWavePdl = 1;
@@ -149,9 +155,10 @@ __global__ void __launch_bounds__(kLitThreads, kLitMinCtas)
     k_lits(const uint4 *__restrict__ units, uint64_t n_units, const uint8_t *__restrict__ lit,
            const uint64_t *__restrict__ blk_tok, const uint64_t *__restrict__ blk_lit,
            const uint32_t *__restrict__ tokdst, const uint32_t *__restrict__ toklit, uint8_t *out, uint32_t log2bs,
-           const uint64_t *__restrict__ pending, uint64_t *done, uint64_t n_done, uint32_t ww) {
+           const uint64_t *__restrict__ pending, uint64_t *done, uint64_t n_done, uint32_t ww, uint32_t *barrier) {
     Group<G> g;
     griddep_launch_dependents();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *barrier = 0;
     const uint64_t tid = blockIdx.x * (uint64_t)kLitThreads + threadIdx.x;
     for (uint64_t k = tid; k < n_done; k += (uint64_t)gridDim.x * kLitThreads)
         done[k] = ~__ldg(pending + k) | (k % ww == 0 ? 1ULL : 0ULL);
@@ -440,15 +447,13 @@ __global__ void __launch_bounds__(kWaveThreads, kWaveMinCtas) k_wave_copy(const 
 // us, 64 batched streams 70 -> 48 us, 256 KiB of Markov bytes 52 -> 36 us.
 template <int G, int J>
 __global__ void __launch_bounds__(kLevelThreads, kLevelMinCtas)
-    k_level(const uint4 *__restrict__ tri, uint64_t n, uint8_t *out, uint32_t *err) {
-    constexpr int kGroups = kLevelThreads / G;
-    constexpr uint32_t kBytes = kStageWarp / 32 * G;
-    __shared__ __align__(128) uint8_t buf[kGroups][kBytes];
-    __shared__ __align__(8) uint64_t bar[kGroups];
+    k_level(const uint4 *__restrict__ tri, uint64_t n, uint8_t *out, uint32_t stage_bytes, uint32_t *err) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ __align__(8) uint64_t bar[kLevelThreads / G];
     Group<G> g;
     griddep_launch_dependents();
     const int gi = threadIdx.x / G;
-    Stage st = {buf[gi], bar + gi, kBytes, 0};
+    Stage st = {smem + (size_t)gi * stage_bytes, bar + gi, stage_bytes, 0};
     const uint64_t i = (blockIdx.x * (uint64_t)kLevelThreads + threadIdx.x) / G * J + g.lane;
     const uint4 t = g.lane < J && i < n ? __ldg(tri + i) : make_uint4(0, 0, 0, 0);
     if (g.lane == 0) mbar_init(st.bar, 1);
@@ -459,17 +464,110 @@ __global__ void __launch_bounds__(kLevelThreads, kLevelMinCtas)
     group_copy_staged<G, J>(g, st, out, tri_dst(t), out + tri_src(t), tri_len(t), err);
 }
 
+// Word of a handle's status array that counts the CTAs at the grid barrier.
+constexpr uint32_t kBarrierWord = 8;
+
+// Bounded grid barrier of a cooperative launch: the CTA's writes are visible
+// to every CTA that leaves it.  target: CTAs times barriers so far.  False,
+// on every thread, when a thread of the CTA comes with ok false, when the
+// wait ran out, or when another CTA already gave up.
+__device__ __forceinline__ bool grid_barrier(uint32_t *count, uint32_t target, bool ok, uint32_t *err) {
+    if (__syncthreads_or(!ok)) return false;
+    bool out = false;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(count, 1u);
+        uint32_t spins = 0, v;
+        for (;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+            if (v >= target) break;
+            if (++spins > kSpinLimitMax) {
+                atomicOr(err, kErrTimeout);
+                out = true;
+                break;
+            }
+            if ((spins & 255) == 0 && (*(volatile uint32_t *)err & kErrTimeout)) {
+                out = true;
+                break;
+            }
+            if (spins > 64) __nanosleep(64);
+        }
+        __threadfence();
+    }
+    return !__syncthreads_or(out);
+}
+
+// Every level in one cooperative launch.  A level's matches are dealt out
+// evenly, at most G / 2 per group at a time, through the groups' stages; the
+// next level's first window is loaded before the barrier.
+//
+// 32 warps per SM at 64 registers; with the level's barrier (2 to 3 us) it
+// takes 593 us for the 1 GiB copy sweep at L = 1024 where k_ranges takes 627
+// (1 GiB at L = 512 / 192: 750 / 1152 against 845 / 1710; one kernel per
+// level 657 / 1044).
+template <int G>
+__global__ void __launch_bounds__(kPersThreads, kPersCtas)
+    k_levels_persistent(const Step *__restrict__ steps, uint32_t count, uint8_t *out, uint32_t stage_bytes,
+                        uint32_t *err) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    constexpr int kGroups = kPersThreads / G;
+    Group<G> g;
+    const int gi = threadIdx.x / G;
+    Stage st;
+    st.bar = reinterpret_cast<uint64_t *>(smem) + gi;
+    st.buf = smem + 128 * ((8 * kGroups + 127) / 128) + (size_t)gi * stage_bytes;
+    st.bytes = stage_bytes;
+    st.phase = 0;
+    if (g.lane == 0) mbar_init(st.bar, 1);
+    fence_mbar_init();
+    __syncthreads();
+    const uint32_t gid = (blockIdx.x * kPersThreads + threadIdx.x) / G;
+    const uint32_t ng = gridDim.x * kGroups;
+    const ulonglong2 *list = reinterpret_cast<const ulonglong2 *>(steps);
+    const uint4 z4 = make_uint4(0, 0, 0, 0);
+    auto share = [&](uint64_t n) {  // matches per group at a time
+        const uint32_t e = ((uint32_t)n + ng - 1) / ng;
+        return e < G / 2 ? e : (uint32_t)G / 2;
+    };
+    auto window = [&](const ulonglong2 &s, uint32_t per, uint32_t a) {
+        return (uint32_t)g.lane < per && a + g.lane < (uint32_t)s.y
+                   ? __ldg(reinterpret_cast<const uint4 *>(s.x) + a + g.lane) : z4;
+    };
+    ulonglong2 cur = __ldg(list), nx = count > 1 ? __ldg(list + 1) : make_ulonglong2(0, 0);
+    uint32_t per = share(cur.y);
+    uint4 t0 = window(cur, per, gid * per);
+    bool ok = true;
+    for (uint32_t k = 0; k < count; k++) {
+        fence_proxy_async_global();
+        for (uint32_t a = gid * per; ok && a < (uint32_t)cur.y; a += ng * per) {
+            const uint4 t = t0;
+            t0 = window(cur, per, a + ng * per);
+            ok = group_copy_staged<G, G / 2>(g, st, out, tri_dst(t), out + tri_src(t), tri_len(t), err);
+            g.sync();
+            fence_proxy_async_shared();  // before the stage is filled again
+        }
+        if (k + 1 == count) break;
+        cur = nx;
+        per = share(cur.y);
+        t0 = window(cur, per, gid * per);
+        if (k + 2 < count) nx = __ldg(list + k + 2);
+        if (!grid_barrier(err + kBarrierWord, (k + 1) * gridDim.x, ok, err)) return;
+    }
+}
+
 // Launch of one step kernel with programmatic stream serialization: its CTAs
 // may start (and load their worklist) while the previous kernel's last ones
 // finish.
 template <class... P, class... A>
-int launch_step(void (*k)(P...), uint64_t n, unsigned per_cta, unsigned threads, cudaStream_t st, A... args) {
+int launch_step(void (*k)(P...), uint64_t n, unsigned per_cta, unsigned threads, size_t smem, cudaStream_t st,
+                A... args) {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = kWavePdl;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3((unsigned)((n + per_cta - 1) / per_cta));
     lc.blockDim = dim3(threads);
+    lc.dynamicSmemBytes = smem;
     lc.stream = st;
     lc.attrs = at;
     lc.numAttrs = 1;
@@ -485,12 +583,14 @@ int launch_step(void (*k)(P...), uint64_t n, unsigned per_cta, unsigned threads,
 template <int G>
 int launch_levels(const aclz_handle *h, const std::vector<Step> &levels, uint32_t count, uint8_t *out,
                   cudaStream_t st) {
+    const uint32_t stage = (h->mean_deferred_len >= kStageLongMin ? kStageWarpLong : kStageWarp) / 32 * G;
+    constexpr int gpc = kLevelThreads / G;
     for (uint32_t i = 0; i < count; i++) {
         const uint64_t n = levels[i].n;
         const int part = n <= kLevelEighth ? 8 : n <= kLevelQuarter ? 4 : 2;
         auto k = part == 8 ? k_level<G, G / 8> : part == 4 ? k_level<G, G / 4> : k_level<G, G / 2>;
-        if (int rc = launch_step(k, n, kLevelThreads / part, kLevelThreads, st, (const uint4 *)levels[i].tri, n, out,
-                                 h->d_err))
+        if (int rc = launch_step(k, n, kLevelThreads / part, kLevelThreads, (size_t)gpc * stage, st,
+                                 (const uint4 *)levels[i].tri, n, out, stage, h->d_err))
             return rc;
     }
     return ACLZ_OK;
@@ -500,20 +600,20 @@ int launch_levels(const aclz_handle *h, const std::vector<Step> &levels, uint32_
 template <int G>
 int launch_wave_steps(const aclz_handle *h, uint8_t *out, cudaStream_t st) {
     for (size_t i = h->n_ord_steps; i < h->steps.size(); i++)
-        if (int rc = launch_step(k_wave_copy<G>, h->steps[i].n, kWaveThreads, kWaveThreads, st,
+        if (int rc = launch_step(k_wave_copy<G>, h->steps[i].n, kWaveThreads, kWaveThreads, 0, st,
                                  (const uint4 *)h->steps[i].tri, h->steps[i].n, out, h->log2_bs))
             return rc;
     return ACLZ_OK;
 }
 
 template <int G>
-int launch_lits(aclz_handle *h, uint8_t *out, cudaStream_t st, bool persistent) {
+int launch_lits(aclz_handle *h, uint8_t *out, cudaStream_t st, bool ranges) {
     constexpr int gpc = kLitThreads / G;
-    const uint64_t n_done = persistent ? (uint64_t)h->n_blocks * h->n_wave_words : 0;
+    const uint64_t n_done = ranges ? (uint64_t)h->n_blocks * h->n_wave_words : 0;
     const unsigned grid = (unsigned)((h->n_lunits + gpc - 1) / gpc);
     k_lits<G><<<grid, kLitThreads, 0, st>>>((const uint4 *)h->d_lunits, h->n_lunits, h->d_lit, h->d_blk_tok,
                                             h->d_blk_lit, h->d_tokdst, h->d_toklit, out, h->log2_bs, h->d_pending,
-                                            h->d_done, n_done, h->n_wave_words);
+                                            h->d_done, n_done, h->n_wave_words, h->d_err + kBarrierWord);
     if (cudaError_t e = cudaGetLastError(); e != cudaSuccess) {
         note_cuda_error(e);
         return ACLZ_E_CUDA;
@@ -630,12 +730,49 @@ int launch_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaSt
     return ACLZ_OK;
 }
 
+// Staged persistent mode by levels: the literal kernel, then every level in
+// one cooperative launch.
+template <int G>
+int launch_levels_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaStream_t st, cudaEvent_t phase) {
+    if (int rc = launch_lits<G>(h, out, st, false)) return rc;
+    if (phase) cudaEventRecord(phase, st);
+    constexpr int gpc = kPersThreads / G;
+    const uint32_t ctas = ctas_per_sm ? std::min<uint32_t>(ctas_per_sm, kPersCtas) : kPersCtas;
+    constexpr uint32_t bar = 128 * ((8 * gpc + 127) / 128);
+    uint32_t stage = ((kSmemPerSm / ctas - bar) / gpc) & ~127u;
+    const size_t smem = bar + (size_t)gpc * stage;
+    int sms = 0;
+    auto fn = k_levels_persistent<G>;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    // the attribute is the largest any call needs, the same on every call
+    constexpr uint32_t most = ((kSmemPerSm - bar) / gpc) & ~127u;
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(bar + (size_t)gpc * most));
+    const Step *steps = (const Step *)h->d_levels;
+    uint32_t count = h->n_levels, *err = h->d_err;
+    void *args[] = {&steps, &count, &out, &stage, &err};
+    if (e == cudaSuccess)
+        e = cudaLaunchCooperativeKernel((const void *)fn, dim3((unsigned)sms * ctas), dim3(kPersThreads), args, smem, st);
+    if (e == cudaErrorCooperativeLaunchTooLarge && ctas > 1) {
+        cudaGetLastError();
+        e = cudaLaunchCooperativeKernel((const void *)fn, dim3((unsigned)sms), dim3(kPersThreads), args, smem, st);
+    }
+    if (e != cudaSuccess) {
+        note_cuda_error(e);
+        return ACLZ_E_CUDA;
+    }
+    return ACLZ_OK;
+}
+
 template <int G>
 int launch_persistent_auto(aclz_handle *h, uint8_t *out, const aclz_decode_cfg &c, cudaStream_t st,
                            cudaEvent_t phase) {
     bool staged = h->mean_deferred_len >= (double)kTmaMin;
     if (c.flags & ACLZ_FLAG_STAGED) staged = true;
     if (c.flags & ACLZ_FLAG_REGISTERS) staged = false;
+    // levels hold in-order and deferred matches: no place for the event then
+    if (staged && h->n_levels && !(phase && h->n_ord_steps))
+        return launch_levels_persistent<G>(h, out, c.ctas_per_sm, st, phase);
     return staged ? launch_persistent<G, true>(h, out, c.ctas_per_sm, st, phase)
                   : launch_persistent<G, false>(h, out, c.ctas_per_sm, st, phase);
 }
@@ -647,7 +784,7 @@ namespace {
 // Levels take the place of waves only when the caller left the mode open: an
 // explicit ACLZ_MODE_WAVES is one kernel per wave.
 bool goes_by_level(const aclz_handle *h, const aclz_decode_cfg *cfg) {
-    return h->by_level && (!cfg || cfg->mode == ACLZ_MODE_AUTO);
+    return h->by_level && decodes_as_waves(h) && (!cfg || cfg->mode == ACLZ_MODE_AUTO);
 }
 
 // Checks cfg and resolves ACLZ_MODE_AUTO for this handle.
@@ -679,7 +816,7 @@ extern "C" int aclz_decode_plan(const aclz_handle *h, const aclz_decode_cfg *cfg
     uint32_t n = 0;
     if (h->n_blocks) {
         if (c.mode == ACLZ_MODE_PERSISTENT)
-            n = 1 + h->n_ord_steps + (h->n_ranges ? 1 : 0);
+            n = (c.flags & ACLZ_FLAG_STAGED) && h->n_levels ? 2 : 1 + h->n_ord_steps + (h->n_ranges ? 1 : 0);
         else
             n = 1 + (uint32_t)(goes_by_level(h, cfg) ? h->lsteps.size() : h->steps.size());
     }

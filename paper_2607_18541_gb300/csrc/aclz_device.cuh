@@ -473,43 +473,41 @@ __device__ __forceinline__ void group_copy_few(const Group<G> &g, uintptr_t p, u
     const bool second = g.lane >= J;
     const uintptr_t ep = second ? pe - tail : p, eq = second ? qe - tail : (uint32_t)q;
     const uint32_t en = !second ? head : g.lane < 2 * J ? tail : 0u;
-    uint4 ev = make_uint4(0, 0, 0, 0);
-    if (en) ev = load_bytes<kFromShared>(eq, en);
     const unsigned have = g.ballot(c > 0);
     if (have) copy_full_chunks<G, 1, kFromShared>(g, p + head, q + head, c, have);
-    store_bytes(ep, ev, en);
+    if (en) store_bytes(ep, load_bytes<kFromShared>(eq, en), en);
 }
 
 // Copy of at most J <= G / 2 jobs (in the lowest lanes) through the group's
-// stage: every job's aligned source span by one bulk copy, as many
-// jobs at a time as the stage holds, then the packed copy from shared
-// memory.  All of a window's source bytes are in flight at once and each is
-// fetched once, where the copy through registers has U rounds of chunks in
-// flight and reads every word of an unaligned source twice.  Jobs larger
-// than the stage are copied through registers.  The sources are final and
-// visible to bulk copies.  False when a wait timed out (see stage_wait).
+// stage: every job's aligned source span by one bulk copy, as many jobs at a
+// time as the stage holds (a job larger than the stage in pieces), then the
+// packed copy from shared memory.  All of a window's source bytes are in
+// flight at once and each is fetched once, where the copy through registers
+// has U rounds of chunks in flight and reads every word of an unaligned
+// source twice.  The sources are final and visible to bulk copies, and the
+// stage is free for them.  False when a wait timed out (see stage_wait).
 template <int G, int J>
 __device__ __forceinline__ bool group_copy_staged(const Group<G> &g, Stage &st, uint8_t *out, uint64_t d,
                                                   const uint8_t *s, uint32_t n, uint32_t *err) {
-    const uintptr_t q = reinterpret_cast<uintptr_t>(s), qa = q & ~(uintptr_t)15;
-    uint32_t span = n ? (uint32_t)(((q + n + 15) & ~(uintptr_t)15) - qa) : 0u;
-    while (g.ballot(span > 0)) {
-        const uint32_t incl = g.scan_incl(span);
-        const bool take = span > 0 && incl <= st.bytes;
-        const unsigned tm = g.ballot(take);
-        if (!tm) {
-            group_copy<G, 1>(g, out, d, s, span ? n : 0u);
-            return true;
-        }
-        const uint32_t tx = g.shfl(incl, 31 - __clz(tm)), off = incl - span;
+    uintptr_t p = reinterpret_cast<uintptr_t>(out) + d, q = reinterpret_cast<uintptr_t>(s);
+    while (g.ballot(n > 0)) {
+        uint32_t m = n < st.bytes - 32 ? n : st.bytes - 32;  // this fill's piece of the job
+        const uint32_t lead = (uint32_t)q & 15u, span = m ? (lead + m + 15u) & ~15u : 0u;
+        const uint32_t incl = g.scan_incl(span), off = incl - span;
+        const bool take = m > 0 && incl <= st.bytes;
+        const uint32_t tx = g.shfl(incl, 31 - __clz(g.ballot(take)));
         if (g.lane == 0) mbar_expect_tx(st.bar, tx);
         g.sync();
-        if (take) tma_load_1d(st.buf + off, reinterpret_cast<const void *>(qa), span, st.bar);
+        if (take)
+            tma_load_1d(st.buf + off, reinterpret_cast<const void *>(q - lead), span, st.bar);
+        else
+            m = 0;
         if (g.ballot(!stage_wait(st, err))) return false;
-        group_copy_few<G, J>(g, reinterpret_cast<uintptr_t>(out) + d, smem_u32(st.buf) + off + (uint32_t)(q - qa),
-                           take ? n : 0u);
-        if (take) span = 0;
-        if (g.ballot(span > 0)) {  // the stage is filled again
+        group_copy_few<G, J>(g, p, smem_u32(st.buf) + off + lead, m);
+        p += m;
+        q += m;
+        n -= m;
+        if (g.ballot(n > 0)) {  // the stage is filled again
             g.sync();
             fence_proxy_async_shared();
         }

@@ -378,8 +378,7 @@ extern "C" int aclz_flatten(aclz_handle *h, void *stream) {
     h->flat = true;
     h->by_level = false;  // the pieces are one step after the in-order levels
     if (int rc = aclz_set_range_bytes(h, h->range_bytes, stream)) return rc;
-    build_steps(h);
-    return ACLZ_OK;
+    return build_steps(h, stream);
 }
 
 // ------------------------------------------------------------- reshape

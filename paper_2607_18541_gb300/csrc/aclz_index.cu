@@ -966,9 +966,9 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         rc = aclz_set_range_bytes(h, h->range_bytes, stream);
         if (rc) { cleanup(); return rc; }
     }
-    // the schedule by levels serves what ACLZ_MODE_AUTO decodes as waves: a
-    // container with tags of its own has its levels found here
-    const bool by_level = !flat_up && !h->needs_flatten && decodes_as_waves(h);
+    // the schedule by levels; a container with tags of its own has its levels
+    // found here
+    const bool by_level = !flat_up && !h->needs_flatten;
     if (by_level && has_tags) {
         CK(cudaMemsetAsync(d_maxtag, 0, 8, st));
         levels = relax_levels(h, d_val, d_maxtag, st);
@@ -984,8 +984,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     }
     CK(dev_alloc((void **)&h->d_done, 8 * (size_t)nb * h->n_wave_words, st));
     CK(cudaStreamSynchronize(st));
-    build_steps(h);
-    return ACLZ_OK;
+    return build_steps(h, stream);
 }
 
 extern "C" int aclz_upload(const void *host_buf, uint64_t n, void *stream, aclz_handle **out) {

@@ -77,13 +77,14 @@ namespace aclz {
 // (the in-order ones are then found block by block).  The step lists follow
 // once the worklists are final.
 int build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlvl, bool all, void *stream);
-void build_steps(aclz_handle *h);
+int build_steps(aclz_handle *h, void *stream);
 void free_wave0(aclz_handle *h, void *stream);
 
 // Deferred matches of at least this mean length are decoded by the
-// persistent schedule under ACLZ_MODE_AUTO (TMA staging pays), shorter ones
-// by waves.
-constexpr double kPersistentMin = 192.0;
+// persistent schedule under ACLZ_MODE_AUTO, shorter ones by levels (or waves),
+// one kernel each: 1 GiB copy sweep at L = 192 / 512 1152 / 750 us persistent
+// and 1044 / 657 us by level kernels; at L = 1024 they are level (593 us).
+constexpr double kPersistentMin = 1024.0;
 bool decodes_as_waves(const aclz_handle *h);
 
 // A list of matches that may be copied once everything before it is final:
@@ -138,7 +139,7 @@ struct aclz_handle {
     uint64_t n_cells = 0;
     uint32_t log2_cell = 0;
     void *d_tri = nullptr;        // n_deferred x 16 B triplets (dst, src, len), built at upload
-    uint32_t *d_err = nullptr;    // latched device status bits
+    uint32_t *d_err = nullptr;    // latched device status bits; word 8: grid barrier count of a persistent decode
     std::vector<uint64_t> wave_start;  // n_waves + 1 entries into the triplet array
     // wave 0: literal units {block, first token, literal range}
     void *d_lunits = nullptr;
@@ -152,8 +153,12 @@ struct aclz_handle {
     bool by_level = false;
     // what follows the literals, in order: in steps the in-order levels
     // (n_ord_steps of them), then the non-empty waves; in lsteps every
-    // level
+    // level.  d_levels is, on the device, the list whose steps hold
+    // independent matches only: lsteps, or the steps of a flattened handle
+    // (n_levels 0: there is none).
     std::vector<aclz::Step> steps, lsteps;
+    void *d_levels = nullptr;
+    uint32_t n_levels = 0;
     uint32_t n_ord_steps = 0;
     // persistent-mode schedule.  A segment is the run of one block's
     // matches in one wave's worklist: seg[s] = {block, wave, triplet offset,

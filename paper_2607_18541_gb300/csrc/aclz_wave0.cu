@@ -67,7 +67,12 @@ __global__ void __launch_bounds__(256) k_lit_units(const uint64_t *__restrict__ 
     }
 }
 
-// cnt[b] = matches of block b for the list (the in-order ones, or all)
+// A match longer than this goes into the list as several, which groups copy
+// side by side (at L = 16000 a level has few matches: the 1 GiB copy sweep takes
+// 496 us instead of 826; pieces of 512 bytes cost 10% at L = 1024).
+constexpr uint32_t kSplit = 1024;
+
+// cnt[b] = triplets of block b for the list (of its in-order matches, or all)
 __global__ void __launch_bounds__(256) k_lev_count(const uint4 *__restrict__ tok, const uint64_t *__restrict__ blk_tok,
                                                    uint32_t nb, bool all, uint32_t *cnt) {
     const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -76,13 +81,13 @@ __global__ void __launch_bounds__(256) k_lev_count(const uint4 *__restrict__ tok
     uint32_t c = 0;
     for (uint64_t i = blk_tok[b] + lane; i < blk_tok[b + 1]; i += 32) {
         const uint4 t = __ldg(tok + i);
-        c += t.y && (all || !(t.w >> 8));
+        if (all || !(t.w >> 8)) c += (t.y + kSplit - 1) / kSplit;
     }
     c = __reduce_add_sync(0xffffffffu, c);
     if (lane == 0) cnt[b] = c;
 }
 
-// triplets of those matches in token order (base: exclusive scan of the
+// those triplets in token order (base: exclusive scan of the
 // counts), which may all be cut anywhere (bit 8 of .y), and with val their
 // sort keys 2 (level - 1) + deferred
 __global__ void __launch_bounds__(256) k_lev_build(const uint4 *__restrict__ tok, const uint64_t *__restrict__ blk_tok,
@@ -99,16 +104,27 @@ __global__ void __launch_bounds__(256) k_lev_build(const uint4 *__restrict__ tok
     for (uint64_t w = blk_tok[b]; w < t1; w += 32) {
         const uint64_t i = w + lane;
         const uint4 t = i < t1 ? __ldg(tok + i) : make_uint4(0, 0, 0, 0);
-        const bool m = t.y && (all || !(t.w >> 8));
-        const unsigned bal = __ballot_sync(0xffffffffu, m);
-        if (m) {
-            const uint64_t d = bstart + __ldg(tokdst + i) + t.x;
-            const uint32_t k = at + __popc(bal & ((1u << lane) - 1u));
-            tri[k] = make_uint4((uint32_t)d, (uint32_t)(d >> 32) | 0x100u, t.z, (t.w & 0xffu) | (t.y << 8));
-            if (val) key[k] = 2u * ((uint32_t)(__ldg(val + i) >> 32) - 1u) + ((t.w >> 8) ? 1u : 0u);
-            idx[k] = k;
+        const uint32_t c = all || !(t.w >> 8) ? (t.y + kSplit - 1) / kSplit : 0u;
+        uint32_t incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
         }
-        at += __popc(bal);
+        if (c) {
+            const uint64_t d = bstart + __ldg(tokdst + i) + t.x;
+            const uint64_t src = (uint64_t)t.z | ((uint64_t)(t.w & 0xffu) << 32);
+            const uint32_t kk = val ? 2u * ((uint32_t)(__ldg(val + i) >> 32) - 1u) + ((t.w >> 8) ? 1u : 0u) : 0u;
+            for (uint32_t q = 0; q < c; q++) {
+                const uint32_t k = at + incl - c + q, n = min(t.y - q * kSplit, kSplit);
+                const uint64_t pd = d + (uint64_t)q * kSplit, ps = src + (uint64_t)q * kSplit;
+                tri[k] = make_uint4((uint32_t)pd, (uint32_t)(pd >> 32) | 0x100u, (uint32_t)ps,
+                                    (uint32_t)(ps >> 32) | (n << 8));
+                if (val) key[k] = kk;
+                idx[k] = k;
+            }
+        }
+        at += __shfl_sync(0xffffffffu, incl, 31);
     }
 }
 
@@ -182,7 +198,7 @@ __global__ void k_lev_gather(const uint4 *__restrict__ tri, const uint32_t *__re
 
 void aclz::free_wave0(aclz_handle *h, void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
-    for (void **pp : {&h->d_lunits, &h->d_lev}) {
+    for (void **pp : {&h->d_lunits, &h->d_lev, &h->d_levels}) {
         dev_free(*pp, st);
         *pp = nullptr;
     }
@@ -191,6 +207,7 @@ void aclz::free_wave0(aclz_handle *h, void *stream) {
     h->by_level = false;
     h->steps.clear();
     h->lsteps.clear();
+    h->n_levels = 0;
 }
 
 int aclz::build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlvl, bool all, void *stream) {
@@ -250,7 +267,8 @@ int aclz::build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t 
     return ACLZ_OK;
 }
 
-void aclz::build_steps(aclz_handle *h) {
+int aclz::build_steps(aclz_handle *h, void *stream) {
+    cudaStream_t st = (cudaStream_t)stream;
     h->steps.clear();
     h->lsteps.clear();
     auto add = [](std::vector<Step> &v, const void *tri, uint64_t a, uint64_t b) {
@@ -264,4 +282,15 @@ void aclz::build_steps(aclz_handle *h) {
     h->n_ord_steps = (uint32_t)h->steps.size();
     for (uint32_t w = 1; w < h->n_waves && h->d_tri; w++)
         add(h->steps, h->d_tri, h->wave_start[w], h->wave_start[w + 1]);
+    dev_free(h->d_levels, st);
+    h->d_levels = nullptr;
+    const std::vector<Step> &list = h->by_level ? h->lsteps : h->steps;
+    h->n_levels = h->by_level || h->flat ? (uint32_t)list.size() : 0;
+    for (const Step &x : list)
+        if (x.n >= 1ULL << 31) h->n_levels = 0;  // the kernel over them counts in 32 bits
+    if (!h->n_levels) return ACLZ_OK;
+    W0CK(dev_alloc(&h->d_levels, sizeof(Step) * list.size(), st));
+    W0CK(cudaMemcpyAsync(h->d_levels, list.data(), sizeof(Step) * list.size(), cudaMemcpyHostToDevice, st));
+    W0CK(cudaStreamSynchronize(st));
+    return ACLZ_OK;
 }

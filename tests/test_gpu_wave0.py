@@ -2,7 +2,7 @@
 around block and unit boundaries, in-order chains of more levels than one
 sort digit and of more matches than one window of the level pass, levels on
 both sides of the sizes that change the matches per group, matches around
-and past the size of a group's stage."""
+the size of a group's stage and of a piece."""
 import numpy as np
 import pytest
 
@@ -132,10 +132,10 @@ def test_levels_around_the_sizes_per_group(n):
     _decode_all_ways(c)
 
 
-@pytest.mark.parametrize("ln", [1, 15, 16, 17, 31, 33, 176, 177, 192, 200, 208, 224, 900, 3568, 3569, 3584, 5000])
+@pytest.mark.parametrize("ln", [1, 15, 16, 17, 31, 33, 176, 177, 192, 200, 208, 224, 900, 1023, 1024, 1025, 2049, 5000])
 def test_match_lengths_around_the_stage(ln):
-    # every source alignment, matches that leave the stage room for 16, for
-    # fewer, for one and for none
+    # every source alignment, matches that leave the stage room for 16 and
+    # for fewer, and matches that go into the list in pieces
     bs = 1 << 15
     blocks = [[(bs, 0, 0)]]
     for b in range(1, 5):
