@@ -211,9 +211,9 @@ def aclz_encode_gpu(src, params: aclz_encode_params, block_min_match=None, strea
         bmm = np.ascontiguousarray(block_min_match, dtype=np.uint8)
     size = ctypes.c_uint64(0)
     bp = _hptr(bmm) if bmm is not None else None
-    _ck(lib().aclz_encode_gpu(_hptr(x), x.size, ctypes.byref(params), bp, _stream(stream), None, 0,
-                              ctypes.byref(size)), "aclz_encode_gpu")
-    out = np.empty(max(1, size.value), dtype=np.uint8)
+    # room for any container, so that the parse runs once (untouched pages of
+    # it are never backed)
+    out = np.empty(max(1, aclz_encode_bound(x.size, params.block_size)), dtype=np.uint8)
     _ck(lib().aclz_encode_gpu(_hptr(x), x.size, ctypes.byref(params), bp, _stream(stream), _hptr(out), out.size,
                               ctypes.byref(size)), "aclz_encode_gpu")
     return out[:size.value]

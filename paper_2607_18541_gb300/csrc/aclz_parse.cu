@@ -158,12 +158,14 @@ __device__ __forceinline__ uint32_t class_min(uint32_t d, uint32_t T) {
 // kCap bytes.
 //
 // Neighbouring ranks share their candidates, so a CTA stages the entries of
-// its ranks and of the kHalo before them (prefix, position and the 16 bytes
-// after the prefix) in shared memory: a candidate costs a 64-bit compare
-// against the bytes it must match to win, and only those that match all 20
-// staged bytes go back to the input.  Issue-bound; the whole of 16 MiB of
-// word text at depth 64 is scored in 1.6 ms, where one warp per block
-// scoring one position at a time took 135 ms.
+// its ranks and of the kHalo before them (prefix, position and the 32 bytes
+// after the prefix) in shared memory.  A round first tests its candidates
+// against the bytes any match must have (a 64-bit compare each, no branch),
+// then scores those that passed, each lane its own; only candidates that
+// match all 36 staged bytes go back to the input.  Issue-bound; 16 MiB of
+// word text at depth 64 is scored in 0.93 ms (1.6 ms when each candidate was
+// tested and scored in turn with 16 bytes staged; 135 ms with one warp per
+// block scoring one position at a time).
 __global__ void __launch_bounds__(kBestThreads) k_best(const uint8_t *__restrict__ x, uint64_t n, uint64_t m,
                                                        uint32_t log2bs, const uint32_t *__restrict__ key_s,
                                                        const uint32_t *__restrict__ val_s, const uint8_t *mm,
@@ -171,12 +173,12 @@ __global__ void __launch_bounds__(kBestThreads) k_best(const uint8_t *__restrict
                                                        uint64_t window, uint8_t *__restrict__ best_len,
                                                        uint32_t *__restrict__ best_src) {
     __shared__ uint32_t skey[kBestThreads + kHalo], spos[kBestThreads + kHalo];
-    __shared__ ulonglong2 swin[kBestThreads + kHalo];
+    __shared__ unsigned long long swin[4][kBestThreads + kHalo];  // the 32 bytes after the prefix
     const uint64_t r0 = (uint64_t)blockIdx.x * kBestThreads;
     const uint64_t r = r0 + threadIdx.x;
     bool live = r < m;
     uint32_t kp = 0, p = 0, T = 0, rem = 0, need = 0, blen = 0, bsrc = 0;
-    unsigned long long w0 = 0, w1 = 0, mask = 0;
+    unsigned long long own[4] = {0, 0, 0, 0}, mask = 0;
     const uint32_t no_key = ~__ldg(key_s);  // differs from any chain that reaches rank 0
     // bytes 4 .. need - 1 of a candidate must match (up to 12 of them)
     auto set_need = [&](uint32_t v) {
@@ -187,22 +189,31 @@ __global__ void __launch_bounds__(kBestThreads) k_best(const uint8_t *__restrict
         for (uint32_t i = threadIdx.x; i < kBestThreads + kHalo; i += kBestThreads) {
             const long long rr = (long long)r0 - (long long)kb - (long long)kHalo + (long long)i;
             uint32_t k = no_key, q = 0;
-            ulonglong2 w = make_ulonglong2(0, 0);
             if (rr >= 0 && (uint64_t)rr < m) {
                 k = __ldg(key_s + rr);
                 q = __ldg(val_s + rr);
-                w = make_ulonglong2(ld8u(x + q + 4), ld8u(x + q + 12));
             }
             skey[i] = k;
             spos[i] = q;
-            swin[i] = w;
+            // 32 bytes from five aligned words (the input is readable, zero,
+            // for 64 bytes past its end)
+            const uintptr_t at = reinterpret_cast<uintptr_t>(x + q + 4);
+            const uint64_t *w = reinterpret_cast<const uint64_t *>(at & ~(uintptr_t)7);
+            const uint32_t sh = (uint32_t)(at & 7) * 8;
+            uint64_t a = __ldg(w);
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const uint64_t b = __ldg(w + j + 1);
+                swin[j][i] = sh ? (a >> sh) | (b << (64 - sh)) : a;
+                a = b;
+            }
         }
         __syncthreads();
         if (kb == 0 && live) {
             kp = skey[threadIdx.x + kHalo];
             p = spos[threadIdx.x + kHalo];
-            w0 = swin[threadIdx.x + kHalo].x;
-            w1 = swin[threadIdx.x + kHalo].y;
+#pragma unroll
+            for (int j = 0; j < 4; j++) own[j] = swin[j][threadIdx.x + kHalo];
             const uint32_t b = p >> log2bs;
             const uint64_t bend = min((uint64_t)(b + 1) << log2bs, n);
             rem = (uint32_t)(bend - p);
@@ -211,35 +222,53 @@ __global__ void __launch_bounds__(kBestThreads) k_best(const uint8_t *__restrict
             set_need(min(min((uint32_t)Tp[0], (uint32_t)Tp[1]), min((uint32_t)Tp[2], (uint32_t)Tp[3])));
             if (rem < need) live = false;
         }
-        const uint32_t kn = min(kHalo, depth - kb);
-        for (uint32_t k = 0; live && k < kn; k++) {
-            const uint32_t e = threadIdx.x + kHalo - 1 - k;  // rank r - 1 - (kb + k)
-            const uint32_t q = spos[e];
-            if (skey[e] != kp || (uint64_t)(p - q) > window) {
+        // candidates of this round: the entries with this prefix (the keys are
+        // in order, so they are a run that ends just before the own entry)
+        uint32_t kn = 0;
+        if (live) {
+            const uint32_t top = threadIdx.x + kHalo;  // entry of rank r - kb
+            uint32_t lo = top - kHalo, hi = top;
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (skey[mid] == kp) hi = mid; else lo = mid + 1;
+            }
+            kn = top - lo;
+            live = kn == kHalo;  // the chain may go on past this round
+            if (kn > depth - kb) kn = depth - kb;
+        }
+        // bit k: candidate k (rank r - 1 - (kb + k)) has the bytes it needs
+        unsigned long long hits = 0;
+#pragma unroll 16
+        for (int k = 0; k < (int)kHalo; k++)
+            if (!((swin[0][threadIdx.x + kHalo - 1 - k] ^ own[0]) & mask)) hits |= 1ULL << k;
+        if (kn < kHalo) hits &= (1ULL << kn) - 1ULL;
+        for (; hits; hits &= hits - 1) {
+            const uint32_t e = threadIdx.x + kHalo - (uint32_t)__ffsll((long long)hits);
+            const uint32_t q = spos[e], d = p - q;
+            if ((uint64_t)d > window) {
                 live = false;
                 break;
             }
-            const unsigned long long x0 = swin[e].x ^ w0;
-            if (x0 & mask) continue;
-            const uint32_t d = p - q;
             const uint32_t lim = d < rem ? d : rem;
-            if (lim < need) continue;
-            uint32_t len;
-            if (x0) {
-                len = 4 + (uint32_t)(__ffsll((long long)x0) - 1) / 8;
-            } else {
-                const unsigned long long x1 = swin[e].y ^ w1;
-                if (x1) {
-                    len = 12 + (uint32_t)(__ffsll((long long)x1) - 1) / 8;
-                } else {
-                    const uint32_t cap = lim < kCap ? lim : kCap;
-                    len = cap <= 20 ? cap : 20 + common_len(x, (uint64_t)q + 20, (uint64_t)p + 20, cap - 20);
-                    if (len >= kCap) {
-                        blen = kLong;
-                        bsrc = (uint32_t)r;
-                        live = false;
-                        break;
-                    }
+            if (((swin[0][e] ^ own[0]) & mask) || lim < need) continue;
+            uint32_t len = 4;
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+                const unsigned long long xj = swin[j][e] ^ own[j];
+                if (xj) {
+                    len += (uint32_t)(__ffsll((long long)xj) - 1) / 8;
+                    break;
+                }
+                len += 8;
+            }
+            if (len == 36) {
+                const uint32_t cap = lim < kCap ? lim : kCap;
+                if (cap > 36) len = 36 + common_len(x, (uint64_t)q + 36, (uint64_t)p + 36, cap - 36);
+                if (len >= kCap) {
+                    blen = kLong;
+                    bsrc = (uint32_t)r;
+                    live = false;
+                    break;
                 }
             }
             len = len < lim ? len : lim;
@@ -247,7 +276,10 @@ __global__ void __launch_bounds__(kBestThreads) k_best(const uint8_t *__restrict
                 blen = len;
                 bsrc = q;
                 set_need(len + 1 > need ? len + 1 : need);
-                if (need > rem) live = false;  // no longer match fits the block
+                if (need > rem) {  // no longer match fits the block
+                    live = false;
+                    break;
+                }
             }
         }
         if (!__syncthreads_or(live && kb + kHalo < depth)) break;
@@ -317,8 +349,8 @@ __device__ __forceinline__ void best_long(const uint8_t *__restrict__ x, const u
 // next window loaded ahead; a step finds the first position with a match
 // at or after p, emits its token and moves past it.  Lane i keeps token i of
 // the current 32 and looks its source up when they are written.  Tokens go
-// to slots[b * cap_tok ...]; ntok[b] and nlit[b] receive the counts.
-// best_len is readable, zero, for two windows past the input.
+// to slots[b * cap_tok ...], the place of every 32nd one to starts; ntok[b]
+// and nlit[b] receive the counts.  best_len is readable, zero, for two windows past the input.
 __global__ void __launch_bounds__(256) k_parse_blocks(const uint8_t *__restrict__ x, uint64_t n, uint32_t bs,
                                                       uint32_t nb, const uint32_t *__restrict__ key_s,
                                                       const uint32_t *__restrict__ val_s,
@@ -326,7 +358,8 @@ __global__ void __launch_bounds__(256) k_parse_blocks(const uint8_t *__restrict_
                                                       const uint32_t *__restrict__ best_src, const uint8_t *mm,
                                                       const uint8_t *__restrict__ block_mm, uint32_t depth,
                                                       uint64_t window, uint32_t cap_tok, TokOut *__restrict__ slots,
-                                                      uint32_t *__restrict__ ntok, uint32_t *__restrict__ nlit) {
+                                                      uint2 *__restrict__ starts, uint32_t *__restrict__ ntok,
+                                                      uint32_t *__restrict__ nlit) {
     const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (b >= nb) return;
@@ -335,8 +368,10 @@ __global__ void __launch_bounds__(256) k_parse_blocks(const uint8_t *__restrict_
     const uint64_t bstart = (uint64_t)b * bs;
     const uint64_t bend = bstart + bs < n ? bstart + bs : n;
     TokOut *out = slots + (uint64_t)b * cap_tok;
+    uint2 *win = starts + (uint64_t)b * (cap_tok / 32 + 1);
     uint64_t p = bstart, lit_start = bstart;
     uint32_t cnt = 0, lits = 0;
+    if (lane == 0) win[0] = make_uint2(0u, 0u);
     // this lane's token of the current 32: literals, length, source (or the
     // position whose source is still to be looked up)
     uint32_t t_lit = 0, t_len = 0, t_src = 0;
@@ -354,7 +389,11 @@ __global__ void __launch_bounds__(256) k_parse_blocks(const uint8_t *__restrict_
         }
         lits += lit;
         cnt++;
-        if (!(cnt & 31u)) flush(32);
+        if (!(cnt & 31u)) {
+            flush(32);
+            // where the next 32 tokens start, in the block and in its literals
+            if (lane == 0) win[cnt / 32] = make_uint2((uint32_t)(lit_start + lit + len - bstart), lits);
+        }
     };
     auto load = [&](uint64_t at) { return __ldg(reinterpret_cast<const uint4 *>(best_len + at) + lane); };
     // bit i: position 16 * lane + i of the window has a match
@@ -411,25 +450,26 @@ __global__ void __launch_bounds__(256) k_parse_blocks(const uint8_t *__restrict_
     }
 }
 
-// One warp per block: directory entry, tokens and literal bytes of the
-// container (tok_off / lit_off: exclusive scans of the counts).
-__global__ void __launch_bounds__(256) k_emit(const uint8_t *__restrict__ x, uint64_t n, uint32_t bs, uint32_t nb,
-                                              const TokOut *__restrict__ slots, uint32_t cap_tok,
-                                              const uint32_t *__restrict__ ntok, const uint32_t *__restrict__ tok_off,
+// One CTA per block: directory entry, tokens and literal bytes of the
+// container (tok_off / lit_off: exclusive scans of the counts; starts: place
+// of every 32nd token), 32 tokens a warp at a time.
+__global__ void __launch_bounds__(256) k_emit(const uint8_t *__restrict__ x, uint32_t bs,
+                                              const TokOut *__restrict__ slots, const uint2 *__restrict__ starts,
+                                              uint32_t cap_tok, const uint32_t *__restrict__ ntok,
+                                              const uint32_t *__restrict__ tok_off,
                                               const uint32_t *__restrict__ lit_off, const uint8_t *mm,
                                               const uint8_t *__restrict__ block_mm, uint8_t *__restrict__ dir,
                                               uint8_t *__restrict__ tok, uint8_t *__restrict__ lit) {
-    const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (b >= nb) return;
+    Group<32> g;
+    const uint32_t b = blockIdx.x;
     const uint32_t nt = ntok[b];
     const uint64_t t0 = tok_off[b], l0 = lit_off[b];
-    if (lane < 8) {
+    if (threadIdx.x < 8) {
         // tok_off u64, lit_off u64, n_tok u32, max_wave u16 0, flags u16 0,
         // min_match[4], pad u32 0: 32 bytes as eight words
         const uint8_t *T = block_mm ? block_mm + 4 * (uint64_t)b : mm;
         uint32_t v = 0;
-        switch (lane) {
+        switch (threadIdx.x) {
             case 0: v = (uint32_t)t0; break;
             case 1: v = (uint32_t)(t0 >> 32); break;
             case 2: v = (uint32_t)l0; break;
@@ -438,27 +478,18 @@ __global__ void __launch_bounds__(256) k_emit(const uint8_t *__restrict__ x, uin
             case 6: v = (uint32_t)T[0] | ((uint32_t)T[1] << 8) | ((uint32_t)T[2] << 16) | ((uint32_t)T[3] << 24); break;
             default: v = 0; break;
         }
-        reinterpret_cast<uint32_t *>(dir + 32 * (uint64_t)b)[lane] = v;
+        reinterpret_cast<uint32_t *>(dir + 32 * (uint64_t)b)[threadIdx.x] = v;
     }
     const TokOut *in = slots + (uint64_t)b * cap_tok;
-    uint64_t pos = (uint64_t)b * bs, lbase = l0;
-    for (uint32_t w = 0; w < nt; w += 32) {
-        const uint32_t i = w + lane;
+    const uint2 *win = starts + (uint64_t)b * (cap_tok / 32 + 1);
+    for (uint32_t w = 32 * (threadIdx.x / 32); w < nt; w += 256) {
+        const uint32_t i = w + g.lane;
         const bool v = i < nt;
+        const uint2 at = win[w / 32];
         const TokOut t = v ? in[i] : TokOut{0u, 0u, 0ULL};
-        // output position of this token's literals: block start + the
-        // lengths of the tokens before it
-        uint64_t tot = (uint64_t)t.lit + t.len, incl = tot;
-        uint64_t lincl = t.lit;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint64_t a = __shfl_up_sync(0xffffffffu, incl, o);
-            const uint64_t c = __shfl_up_sync(0xffffffffu, lincl, o);
-            if (lane >= o) {
-                incl += a;
-                lincl += c;
-            }
-        }
+        // place of this token's literals in the block and in its literals:
+        // those of the window plus the lengths of the tokens before it
+        const uint32_t incl = g.scan_incl(t.lit + t.len), lincl = g.scan_incl(t.lit);
         if (v) {
             uint32_t *tw = reinterpret_cast<uint32_t *>(tok + 16 * (t0 + i));
             tw[0] = t.lit;
@@ -466,16 +497,8 @@ __global__ void __launch_bounds__(256) k_emit(const uint8_t *__restrict__ x, uin
             tw[2] = t.len ? (uint32_t)t.src : 0u;
             tw[3] = t.len ? (uint32_t)(t.src >> 32) & 0xffu : 0u;
         }
-        // literal runs, one after another, each copied by the whole warp
-        const uint64_t ps = pos + incl - tot;        // first literal byte in the input
-        const uint64_t ls = lbase + lincl - t.lit;   // its place in the literal array
-        for (int j = 0; j < 32; j++) {
-            const uint32_t lj = __shfl_sync(0xffffffffu, v ? t.lit : 0u, j);
-            const uint64_t pj = __shfl_sync(0xffffffffu, ps, j), qj = __shfl_sync(0xffffffffu, ls, j);
-            for (uint32_t k = lane; k < lj; k += 32) lit[qj + k] = x[pj + k];
-        }
-        pos += __shfl_sync(0xffffffffu, incl, 31);
-        lbase += __shfl_sync(0xffffffffu, lincl, 31);
+        const uint64_t from = (uint64_t)b * bs + at.x + incl - (t.lit + t.len);
+        group_copy<32, 2, kFromConst>(g, lit, l0 + at.y + lincl - t.lit, x + from, t.lit);
     }
 }
 
@@ -533,7 +556,7 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
         }
         return rc == ACLZ_OK;
     };
-    Scratch dx, dk0, dv0, dk1, dv1, dlen, dslots, dntok, dnlit, dtoff, dloff, dmm, dbmm, dcont;
+    Scratch dx, dk0, dv0, dk1, dv1, dlen, dslots, dstarts, dntok, dnlit, dtoff, dloff, dmm, dbmm, dcont;
     // the input with 16 zero bytes after it (the 8-byte compares read
     // whole aligned words)
     if (!ck(dx.alloc(n + 64, st)) || !ck(cudaMemsetAsync((uint8_t *)dx.p + (n & ~(uint64_t)15), 0, 48, st)) ||
@@ -557,6 +580,7 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
                             !ck(cudaMemcpyAsync(dbmm.p, block_min_match, 4ULL * nb, cudaMemcpyHostToDevice, st))))
         return rc;
     if (!ck(dslots.alloc(sizeof(TokOut) * (uint64_t)cap_tok * (nb ? nb : 1), st)) ||
+        !ck(dstarts.alloc(sizeof(uint2) * (uint64_t)(cap_tok / 32 + 1) * (nb ? nb : 1), st)) ||
         !ck(dntok.alloc(4ULL * nb + 16, st)) || !ck(dnlit.alloc(4ULL * nb + 16, st)) ||
         !ck(dtoff.alloc(4ULL * nb + 16, st)) || !ck(dloff.alloc(4ULL * nb + 16, st)))
         return rc;
@@ -571,7 +595,8 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
         k_parse_blocks<<<(nb + 7) / 8, 256, 0, st>>>((const uint8_t *)dx.p, n, bs, nb, k0, v0,
                                                      (const uint8_t *)dlen.p, v1, (const uint8_t *)dmm.p,
                                                      (const uint8_t *)dbmm.p, p->chain_depth, window, cap_tok,
-                                                     (TokOut *)dslots.p, (uint32_t *)dntok.p, (uint32_t *)dnlit.p);
+                                                     (TokOut *)dslots.p, (uint2 *)dstarts.p, (uint32_t *)dntok.p,
+                                                     (uint32_t *)dnlit.p);
         if (!ck(cudaGetLastError())) return rc;
         ck(cudaMemcpyAsync(dtoff.p, dntok.p, 4ULL * nb, cudaMemcpyDeviceToDevice, st));
         ck(cudaMemcpyAsync(dloff.p, dnlit.p, 4ULL * nb, cudaMemcpyDeviceToDevice, st));
@@ -594,11 +619,11 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
     if (!ck(dcont.alloc(need ? need : 16, st))) return rc;
     uint8_t *c = (uint8_t *)dcont.p;
     if (nb) {
-        k_emit<<<(nb + 7) / 8, 256, 0, st>>>((const uint8_t *)dx.p, n, bs, nb, (const TokOut *)dslots.p, cap_tok,
-                                             (const uint32_t *)dntok.p, (const uint32_t *)dtoff.p,
-                                             (const uint32_t *)dloff.p, (const uint8_t *)dmm.p,
-                                             (const uint8_t *)dbmm.p, c + kHdr, c + kHdr + (uint64_t)kDirent * nb,
-                                             c + kHdr + (uint64_t)kDirent * nb + (uint64_t)kTok * nt);
+        k_emit<<<nb, 256, 0, st>>>((const uint8_t *)dx.p, bs, (const TokOut *)dslots.p, (const uint2 *)dstarts.p,
+                                   cap_tok, (const uint32_t *)dntok.p, (const uint32_t *)dtoff.p,
+                                   (const uint32_t *)dloff.p, (const uint8_t *)dmm.p, (const uint8_t *)dbmm.p, c + kHdr,
+                                   c + kHdr + (uint64_t)kDirent * nb,
+                                   c + kHdr + (uint64_t)kDirent * nb + (uint64_t)kTok * nt);
         if (!ck(cudaGetLastError())) return rc;
     }
     // header: "ACLZ", v1, no tags, sizes, thresholds, distance bounds

@@ -64,3 +64,17 @@ def test_block_thresholds():
     nb = (x.size + 1023) // 1024
     bmm = np.random.RandomState(4).randint(4, 80, (nb, 4)).astype(np.uint8)
     _same(x, _params((6, 8, 10, 12), 1024, 64), bmm)
+
+
+@pytest.mark.parametrize("depth", [64, 65, 200])
+def test_staged_bytes(depth):
+    # many candidates that agree for 35, 36, 37 and more bytes, the longest
+    # among the first round's or a later round's
+    r = np.random.RandomState(depth)
+    stem = r.randint(0, 256, 80).astype(np.uint8)
+    parts = []
+    for k in range(180):
+        n = int(r.choice([34, 35, 36, 37, 38, 60, 63, 64, 65, 80]))
+        parts += [stem[:n], r.randint(0, 256, int(r.randint(1, 9))).astype(np.uint8)]
+    _same(np.concatenate(parts), _params((6, 8, 10, 12), 4096, depth))
+    _same(np.concatenate(parts), _params((30, 36, 37, 40), 65536, depth))
