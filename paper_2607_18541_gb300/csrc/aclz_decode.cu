@@ -91,7 +91,7 @@ __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wa
 // second) to 2^26: a range deep in a long chain legitimately waits for most
 // of the launch.  A wait also gives up when another group already gave up
 // (err has kErrTimeout), so one stuck wait ends the whole launch.
-constexpr uint32_t kSpinLimitMin = 1u << 22, kSpinLimitMax = 1u << 26;
+constexpr uint32_t kSpinLimitMin = 1u << 22;
 
 // Spin (bounded) until every wave below w of one block is done: its done
 // bits (ww 64-bit words, empty waves preset) are all set below bit w.
@@ -462,39 +462,6 @@ __global__ void __launch_bounds__(kLevelThreads, kLevelMinCtas)
     griddep_wait();
     fence_proxy_async_global();
     group_copy_staged<G, J>(g, st, out, tri_dst(t), out + tri_src(t), tri_len(t), err);
-}
-
-// Word of a handle's status array that counts the CTAs at the grid barrier.
-constexpr uint32_t kBarrierWord = 8;
-
-// Bounded grid barrier of a cooperative launch: the CTA's writes are visible
-// to every CTA that leaves it.  target: CTAs times barriers so far.  False,
-// on every thread, when a thread of the CTA comes with ok false, when the
-// wait ran out, or when another CTA already gave up.
-__device__ __forceinline__ bool grid_barrier(uint32_t *count, uint32_t target, bool ok, uint32_t *err) {
-    if (__syncthreads_or(!ok)) return false;
-    bool out = false;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(count, 1u);
-        uint32_t spins = 0, v;
-        for (;;) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
-            if (v >= target) break;
-            if (++spins > kSpinLimitMax) {
-                atomicOr(err, kErrTimeout);
-                out = true;
-                break;
-            }
-            if ((spins & 255) == 0 && (*(volatile uint32_t *)err & kErrTimeout)) {
-                out = true;
-                break;
-            }
-            if (spins > 64) __nanosleep(64);
-        }
-        __threadfence();
-    }
-    return !__syncthreads_or(out);
 }
 
 // Every level in one cooperative launch.  A level's matches are dealt out

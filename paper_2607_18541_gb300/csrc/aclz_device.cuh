@@ -16,6 +16,39 @@ constexpr uint32_t kErrTimeout = 1u;
 constexpr uint32_t kErrCorrupt = 2u;
 constexpr uint32_t kErrBounds = 4u;
 
+// most polls of any bounded wait
+constexpr uint32_t kSpinLimitMax = 1u << 26;
+
+// Bounded grid barrier of a cooperative launch: the CTA's writes are visible
+// to every CTA that leaves it.  target: CTAs times barriers so far (*count
+// starts at 0).  One release and one acquire on one word: every further hop
+// (a flag set by the last arrival, a tree of counters) cost 0.8 us more than
+// it saved.  False, on every thread, when a thread of the CTA comes with ok
+// false, when the wait ran out, or when another CTA already gave up.
+__device__ __forceinline__ bool grid_barrier(uint32_t *count, uint32_t target, bool ok, uint32_t *err) {
+    if (__syncthreads_or(!ok)) return false;
+    bool out = false;
+    if (threadIdx.x == 0) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+        uint32_t spins = 0, v;
+        for (;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+            if (v >= target) break;
+            if (++spins > kSpinLimitMax) {
+                atomicOr(err, kErrTimeout);
+                out = true;
+                break;
+            }
+            if ((spins & 255) == 0 && (*(volatile uint32_t *)err & kErrTimeout)) {
+                out = true;
+                break;
+            }
+            if (spins > 64) __nanosleep(64);
+        }
+    }
+    return !__syncthreads_or(out);
+}
+
 template <int G>
 struct Group {
     static_assert(G == 8 || G == 16 || G == 32, "G must be 8, 16 or 32");

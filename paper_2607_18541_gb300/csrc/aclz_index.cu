@@ -5,7 +5,7 @@
 //                    strictly before its target, Sec. I), block-relative
 //                    token offsets for the seek path.
 //  2. k_cover, k_relax  the tokens each match reads, then by passes over
-//                    them its minimal wave tag (a match waits one wave for
+//                    them (one launch) its minimal wave tag (a match waits one wave for
 //                    every cross-block hop of its source chain; same-block
 //                    sources are ordered within the block) and its level
 //                    (the length of the longest chain of matches that ends
@@ -370,47 +370,67 @@ __global__ void __launch_bounds__(256) k_cover(const uint4 *__restrict__ tok, co
     }
 }
 
-// One pass over the matches: val[i] = {level, tag} of token i raised to what
-// its covering tokens ask for under their current values (read as other
-// warps leave them): level = 1 + their largest level, tag = the largest of
-// their tags, plus one in another block.  Both only grow, from zero to the
-// least fixed point, which is the longest chain and the minimal tagging.
-// After pass k every match of true level up to k has its final values, and
-// no value exceeds its true one, so a match whose level is below k is final:
-// pass k + 1 skips it after one 8-byte read.  A pass that raises nothing
-// (*changed stays 0) proves the fixed point reached.
-__global__ void __launch_bounds__(256) k_relax(const uint4 *__restrict__ cover, const uint4 *__restrict__ tok,
-                                               uint64_t n, uint32_t pass, unsigned long long *val,
-                                               uint32_t *changed, uint32_t *maxes) {
-    uint32_t mt = 0, ml = 0;
-    bool raised = false;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        const unsigned long long cur = __ldcg(val + i);
-        if (pass > 1 && (uint32_t)(cur >> 32) + 1u < pass) continue;
-        const uint4 c = __ldg(cover + i);
-        if (pass == 1 && !__ldg(&tok[i].y)) continue;
-        uint32_t lv = 0, tg = c.w;
-        for (uint32_t k = 0; k < c.y + c.z; k++) {
-            const unsigned long long v = __ldcg(val + c.x + k);
-            lv = max(lv, (uint32_t)(v >> 32));
-            // a literal-only token among them has value 0 and asks for nothing
-            if (v) tg = max(tg, (uint32_t)v + (k < c.y ? 1u : 0u));
+// Passes over the matches, in one cooperative launch: val[i] = {level, tag}
+// of token i raised to what its covering tokens ask for under their current
+// values (read as other warps leave them): level = 1 + their largest level,
+// tag = the largest of their tags, plus one in another block.  Both only
+// grow, from zero to the least fixed point, which is the longest chain and
+// the minimal tagging.  After pass k every match of true level up to k has
+// its final values, and no value exceeds its true one, so a match whose level
+// is below k is final: pass k + 1 skips it after one 8-byte read.  A pass that
+// raises nothing proves the fixed point reached.  out: [0] largest tag, [1]
+// largest level, [2] 1 when the fixed point was reached within most passes;
+// state (kRelaxState words, zeroed): the barrier's count, from kRaised on the
+// raised flags of three passes in turn, then the bounded barrier's error word.
+//
+// A pass is bound by its barrier and the latency of three dependent loads,
+// about 5 us.  With one launch per pass and a look from the host every eighth
+// the 14 to 25 levels of 32 and 64 MiB streams took 16 to 32 launches of 4.6
+// us and two to four stops; with the host's other stops for counts read
+// together, uploads of 32 / 64 MiB took 819 / 1225 us before and 656 / 1122 us
+// now.
+constexpr int kRelaxThreads = 512, kRelaxCtas = 2;
+constexpr uint32_t kRaised = 32, kRelaxState = 64;  // the flags on a line of their own
+__global__ void __launch_bounds__(kRelaxThreads, kRelaxCtas)
+    k_relax(const uint4 *__restrict__ cover, const uint4 *__restrict__ tok, uint64_t n, uint32_t most,
+            unsigned long long *val, uint32_t *state, uint32_t *out) {
+    uint32_t mt = 0, ml = 0, pass = 1;
+    for (; pass <= most; pass++) {
+        bool raised = false;
+        for (uint64_t i = blockIdx.x * (uint64_t)kRelaxThreads + threadIdx.x; i < n;
+             i += (uint64_t)gridDim.x * kRelaxThreads) {
+            const unsigned long long cur = __ldcg(val + i);
+            if (pass > 1 && (uint32_t)(cur >> 32) + 1u < pass) continue;
+            if (pass == 1 && !__ldg(&tok[i].y)) continue;
+            const uint4 c = __ldg(cover + i);
+            uint32_t lv = 0, tg = c.w;
+            for (uint32_t k = 0; k < c.y + c.z; k++) {
+                const unsigned long long v = __ldcg(val + c.x + k);
+                lv = max(lv, (uint32_t)(v >> 32));
+                // a literal-only token among them has value 0 and asks for nothing
+                if (v) tg = max(tg, (uint32_t)v + (k < c.y ? 1u : 0u));
+            }
+            const unsigned long long nv = ((unsigned long long)(lv + 1u) << 32) | max(tg, (uint32_t)cur);
+            if (nv != cur) {
+                __stcg(val + i, nv);
+                raised = true;
+            }
+            ml = max(ml, lv + 1u);
+            mt = max(mt, (uint32_t)nv);
         }
-        const unsigned long long nv = ((unsigned long long)(lv + 1u) << 32) | max(tg, (uint32_t)cur);
-        if (nv != cur) {
-            __stcg(val + i, nv);
-            raised = true;
-        }
-        ml = max(ml, lv + 1u);
-        mt = max(mt, (uint32_t)nv);
+        // the flag of the next pass: every CTA is past its last reading
+        if (blockIdx.x == 0 && threadIdx.x == 0) state[kRaised + (pass + 1) % 3] = 0;
+        if (__any_sync(0xffffffffu, raised) && (threadIdx.x & 31) == 0) state[kRaised + pass % 3] = 1u;
+        if (!grid_barrier(state, pass * gridDim.x, true, state + kRaised + 3)) return;
+        if (!__ldcg(state + kRaised + pass % 3)) break;
     }
     ml = __reduce_max_sync(0xffffffffu, ml);
     mt = __reduce_max_sync(0xffffffffu, mt);
-    if (__any_sync(0xffffffffu, raised) && (threadIdx.x & 31) == 0) {
-        *changed = 1u;
-        atomicMax(maxes, mt);
-        atomicMax(maxes + 1, ml);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(out, mt);
+        atomicMax(out + 1, ml);
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) out[2] = pass <= most;
 }
 
 __global__ void k_extract_tags(const uint4 *__restrict__ tok, uint32_t *tags, uint64_t n) {
@@ -419,7 +439,9 @@ __global__ void k_extract_tags(const uint4 *__restrict__ tok, uint32_t *tags, ui
         tags[i] = __ldg(tok + i).w >> 8;
 }
 
-__global__ void k_store_val_tags(uint4 *tok, const unsigned long long *val, uint64_t n) {
+// tags of the values into the tokens, when *reached
+__global__ void k_store_val_tags(uint4 *tok, const unsigned long long *val, uint64_t n, const uint32_t *reached) {
+    if (!*reached) return;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
          i += (uint64_t)gridDim.x * blockDim.x) {
         const uint4 t = tok[i];
@@ -698,7 +720,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t *in
     if (threadIdx.x == 0) part[blockIdx.x] = tot;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_parts(uint32_t *part, uint64_t np) {
+__global__ void __launch_bounds__(kScanThreads) k_scan_parts(uint32_t *part, uint64_t np, uint32_t *total) {
     __shared__ uint32_t sh[32];
     uint32_t carry = 0;
     for (uint64_t b = 0; b < np; b += kScanThreads) {
@@ -709,7 +731,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_parts(uint32_t *part, uin
         if (i < np) part[i] = carry + ex;
         carry += tot;
     }
-    if (threadIdx.x == 0) part[np] = carry;
+    if (threadIdx.x == 0) *total = carry;
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_apply(uint32_t *io, uint64_t n,
@@ -727,6 +749,31 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(uint32_t *io, uint6
         if (base + k < n) io[base + k] = ex;
         ex += v[k];
     }
+}
+
+// Exclusive scan in place by one CTA (short arrays: one launch in the place
+// of three).
+__global__ void __launch_bounds__(kScanThreads) k_scan_one(uint32_t *io, uint32_t n, uint32_t *total) {
+    __shared__ uint32_t sh[32];
+    uint32_t carry = 0;
+    for (uint32_t b = 0; b < n; b += kScanTile) {
+        const uint32_t at = b + threadIdx.x * kScanItems;
+        uint32_t v[kScanItems], s = 0;
+#pragma unroll
+        for (int k = 0; k < kScanItems; k++) {
+            v[k] = at + k < n ? io[at + k] : 0;
+            s += v[k];
+        }
+        uint32_t tot;
+        uint32_t ex = carry + block_excl_scan(s, sh, &tot);
+#pragma unroll
+        for (int k = 0; k < kScanItems; k++) {
+            if (at + k < n) io[at + k] = ex;
+            ex += v[k];
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0) *total = carry;
 }
 
 __global__ void k_gather_starts(const uint32_t *base, uint64_t nb, uint32_t nw1, const uint32_t *total,
@@ -753,52 +800,51 @@ int cuda_rc(cudaError_t e) {
 // Temporary partials are allocated stream-ordered.
 int aclz::device_excl_scan(uint32_t *d, uint64_t n, uint32_t *d_total, void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
+    // one CTA takes 4 us for 4096 words and 1 us more for every 4096 after;
+    // three launches take 10 us
+    if (n <= 8 * kScanTile) {
+        k_scan_one<<<1, kScanThreads, 0, st>>>(d, (uint32_t)n, d_total);
+        return cuda_rc(cudaGetLastError());
+    }
     const uint64_t ntile = (n + kScanTile - 1) / kScanTile;
     uint32_t *part = nullptr;
-    cudaError_t e = dev_alloc((void **)&part, sizeof(uint32_t) * (ntile + 1), st);
+    cudaError_t e = dev_alloc((void **)&part, sizeof(uint32_t) * ntile, st);
     if (e != cudaSuccess) return cuda_rc(e);
-    if (ntile) k_scan_reduce<<<(unsigned)ntile, kScanThreads, 0, st>>>(d, n, part);
-    k_scan_parts<<<1, kScanThreads, 0, st>>>(part, ntile);
-    if (ntile) k_scan_apply<<<(unsigned)ntile, kScanThreads, 0, st>>>(d, n, part);
-    cudaMemcpyAsync(d_total, part + ntile, sizeof(uint32_t), cudaMemcpyDeviceToDevice, st);
+    k_scan_reduce<<<(unsigned)ntile, kScanThreads, 0, st>>>(d, n, part);
+    k_scan_parts<<<1, kScanThreads, 0, st>>>(part, ntile, d_total);
+    k_scan_apply<<<(unsigned)ntile, kScanThreads, 0, st>>>(d, n, part);
     dev_free(part, st);
     return cuda_rc(cudaGetLastError());
 }
 
-// Levels and minimal wave tags of h's tokens into d_val ({level, tag}, and
-// the largest tag and level into d_maxes[0..1]) by relaxation passes from
-// zero, checked every kRelaxBatch passes; true when a pass raised nothing
-// within kRelaxMax passes.  A stream whose copy chains are deeper than that
-// is left to the ordered pass (false; d_val is then part-way).
+// Levels and minimal wave tags of h's tokens into d_val ({level, tag}) by
+// relaxation passes from zero; d_out[0..2] as k_relax leaves them.  A stream
+// whose copy chains are deeper than kRelaxMax (d_out[2] = 0) is left to the
+// ordered pass; so is one whose cover list does not fit.
 namespace {
-constexpr uint32_t kRelaxBatch = 8, kRelaxMax = 512;
-bool relax_levels(aclz_handle *h, unsigned long long *d_val, uint32_t *d_maxes, cudaStream_t st) {
+constexpr uint32_t kRelaxMax = 512;
+int relax_levels(aclz_handle *h, unsigned long long *d_val, uint32_t *d_out, cudaStream_t st) {
     const uint32_t nb = h->n_blocks;
     const uint64_t nt = h->n_tokens;
-    Scratch flags, cover;
-    if (flags.alloc(4 * kRelaxBatch, st) != cudaSuccess) return false;
-    if (cover.alloc(16 * (nt ? nt : 1), st) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    uint32_t *changed = (uint32_t *)flags.p;
-    if (cudaMemsetAsync(d_val, 0, 8 * (nt ? nt : 1), st) != cudaSuccess) return false;
+    Scratch state, cover;
+    if (cudaMemsetAsync(d_out, 0, 12, st) != cudaSuccess) return ACLZ_E_CUDA;
+    if (state.alloc(4 * kRelaxState, st) != cudaSuccess || cover.alloc(16 * (nt ? nt : 1), st) != cudaSuccess) return ACLZ_OK;
+    if (cudaMemsetAsync(state.p, 0, 4 * kRelaxState, st) != cudaSuccess ||
+        cudaMemsetAsync(d_val, 0, 8 * (nt ? nt : 1), st) != cudaSuccess)
+        return ACLZ_E_CUDA;
     k_cover<<<(nb + 7) / 8, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, nb, h->log2_bs, nt,
                                            (uint4 *)cover.p);
-    const unsigned grid = (unsigned)std::min<uint64_t>((nt + 255) / 256, 152 * 8 * 4);
-    for (uint32_t done_passes = 0; done_passes < kRelaxMax; done_passes += kRelaxBatch) {
-        if (cudaMemsetAsync(changed, 0, 4 * kRelaxBatch, st) != cudaSuccess) return false;
-        for (uint32_t k = 0; k < kRelaxBatch; k++)
-            k_relax<<<grid, 256, 0, st>>>((const uint4 *)cover.p, (const uint4 *)h->d_tok, nt, done_passes + k + 1,
-                                          d_val, changed + k, d_maxes);
-        uint32_t last = 1;
-        if (cudaGetLastError() != cudaSuccess ||
-            cudaMemcpyAsync(&last, changed + kRelaxBatch - 1, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            return false;
-        if (!last) return true;
-    }
-    return false;
+    int sms = 0, per_sm = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_relax, kRelaxThreads, 0);
+    const uint64_t need = (nt + kRelaxThreads - 1) / kRelaxThreads;
+    const unsigned grid =
+        (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(need, (uint64_t)sms * std::min(per_sm, kRelaxCtas)));
+    const uint4 *c = (const uint4 *)cover.p, *tok = (const uint4 *)h->d_tok;
+    uint64_t n = nt;
+    uint32_t most = kRelaxMax, *s = (uint32_t *)state.p;
+    void *args[] = {&c, &tok, &n, &most, &d_val, &s, &d_out};
+    return cuda_rc(cudaLaunchCooperativeKernel((const void *)k_relax, dim3(grid), dim3(kRelaxThreads), args, 0, st));
 }
 }  // namespace
 
@@ -832,17 +878,28 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     while (h->log2_cell < h->log2_bs && (h->total_len >> h->log2_cell) > nt) h->log2_cell++;
     h->n_cells = (h->total_len + (1ULL << h->log2_cell) - 1) >> h->log2_cell;
     CK(dev_alloc((void **)&h->d_cell, 4 * (h->n_cells + 1), st));
-    CK(cudaMemsetAsync(h->d_err, 0, 64, st));
-    // scratch words: [0] err (handle), work: maxtag, counter, total, first_bad
+    CK(cudaMemsetAsync(h->d_err, 0, kErrBytes, st));
+    // scratch words, read by the host together: [0] max tag, [1] largest level
+    // (then the block counter of k_tags_min), [2] fixed point reached, [3]
+    // deferred matches, [4] segments, [5] triplets of the level list, [6]
+    // status; bytes 32..39: first bad token, 40..47: deferred bytes
+    struct Words {
+        uint32_t maxtag, maxlvl, reached, deferred, segs, lev, err, pad;
+        unsigned long long first_bad, def_bytes, pad2[2];
+    } hw;
+    static_assert(sizeof(Words) == 64, "scratch words");
     Scratch work;
     CK(work.alloc(64, st));
-    uint32_t *d_maxtag = (uint32_t *)work.p, *d_ctr = d_maxtag + 1, *d_total = d_maxtag + 2;
-    // words: [0] max tag, [1] largest level, then the block counter, [2]
-    // deferred total, [3] segment count, [4] range count, [5] matches of the
-    // level list; bytes 32..39: first bad token
-    unsigned long long *d_first_bad = (unsigned long long *)((char *)work.p + 32);
-    CK(cudaMemsetAsync(work.p, 0, 32, st));
+    uint32_t *d_maxtag = (uint32_t *)work.p, *d_ctr = d_maxtag + 1, *d_total = d_maxtag + 3;
+    unsigned long long *d_first_bad = (unsigned long long *)((char *)work.p + 32), *d_def_bytes = d_first_bad + 1;
+    CK(cudaMemsetAsync(work.p, 0, 64, st));
     CK(cudaMemsetAsync(d_first_bad, 0xff, 8, st));
+    // the words as they stand after the work enqueued so far (and the status)
+    auto read_words = [&]() {
+        cudaError_t e = cudaMemcpyAsync(d_maxtag + 6, h->d_err, 4, cudaMemcpyDeviceToDevice, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&hw, work.p, 64, cudaMemcpyDeviceToHost, st);
+        return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+    };
     const unsigned wblocks = (nb + 7) / 8;  // 8 warps per CTA
     k_index_scan<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_blk_lit, h->d_tokdst,
                                            h->d_toklit, h->d_cell, h->n_cells, h->log2_cell, nt, nb, h->log2_bs,
@@ -871,11 +928,16 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         k_tags_local<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, d_tags, nb,
                                                h->log2_bs, d_maxtag);
         k_store_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_tags, nt);
-    } else if (relax_levels(h, d_val, d_maxtag, st)) {
-        // by parallel passes (the chains were shallow enough)
-        levels = true;
-        k_store_val_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_val, nt);
     } else {
+        rc = relax_levels(h, d_val, d_maxtag, st);
+        if (rc) { cleanup(); return rc; }
+        k_store_val_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_val, nt, d_maxtag + 2);
+    }
+    CK(cudaGetLastError());
+    CK(read_words());
+    if (hw.reached) {
+        levels = true;
+    } else if (!has_tags && !flat_up) {  // chains too deep for the passes
         CK(cudaMemsetAsync(d_maxtag, 0, 8, st));
         CK(done.alloc(4 * nb, st));
         CK(cudaMemsetAsync(done.p, 0, 4 * nb, st));
@@ -889,34 +951,37 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
                                           (uint32_t *)done.p, d_ctr, nb, h->log2_bs, nt, d_maxtag,
                                           h->d_err);
         k_store_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_tags, nt);
+        CK(cudaGetLastError());
+        CK(read_words());
     }
-    CK(cudaGetLastError());
-    uint32_t hw[3] = {0, 0, 0};
-    CK(cudaMemcpyAsync(&hw[0], d_maxtag, 4, cudaMemcpyDeviceToHost, st));
-    CK(cudaMemcpyAsync(&hw[1], h->d_err, 4, cudaMemcpyDeviceToHost, st));
-    if (levels) CK(cudaMemcpyAsync(&hw[2], d_maxtag + 1, 4, cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    if (hw[1] & kErrTimeout) { cleanup(); return ACLZ_E_TIMEOUT; }
-    if (hw[1]) { cleanup(); return ACLZ_E_CORRUPT; }
-    const uint32_t maxtag = hw[0];
+    if (hw.err & kErrTimeout) { cleanup(); return ACLZ_E_TIMEOUT; }
+    if (hw.err) { cleanup(); return ACLZ_E_CORRUPT; }
+    const uint32_t maxtag = hw.maxtag;
+    uint32_t maxlvl = hw.maxlvl;
     if (maxtag > kMaxWave) { cleanup(); return ACLZ_E_UNSUPPORTED; }
     if (has_tags && given_waves != maxtag + 1) { cleanup(); return ACLZ_E_CORRUPT; }
     h->n_waves = maxtag + 1;
     h->wave_start.assign(h->n_waves + 1, 0);
     CK(cudaMemsetAsync(h->d_slot, 0xff, 4 * nt, st));
-    unsigned long long defb_total = 0;
     // The plain schedule keeps a dense (wave, block) count table and
     // per-block wave bitmasks, quadratic in the chain depth; beyond 2^28
     // cells the upload builds the flattened two-wave schedule instead.
     h->needs_flatten = maxtag > 0 && (uint64_t)maxtag * nb > (1ULL << 28);
-    if (maxtag > 0 && !h->needs_flatten) {
-        const uint64_t M = (uint64_t)maxtag * nb;
-        Scratch cnt, starts;
+    // the schedule by levels; a container with tags of its own has its levels
+    // found here
+    const bool by_level = !flat_up && !h->needs_flatten;
+    if (by_level && has_tags) {
+        rc = relax_levels(h, d_val, d_maxtag, st);
+        if (rc) { cleanup(); return rc; }
+    }
+    const bool waves = maxtag > 0 && !h->needs_flatten;
+    const uint64_t M = waves ? (uint64_t)maxtag * nb : 0;
+    Scratch cnt, starts, flag, levcnt;
+    if (waves) {
         CK(cnt.alloc(4 * M, st));
+        CK(flag.alloc(4 * M, st));
         CK(starts.alloc(8 * (maxtag + 1), st));
         CK(cudaMemsetAsync(cnt.p, 0, 4 * M, st));
-        unsigned long long *d_def_bytes = (unsigned long long *)((char *)work.p + 40);
-        CK(cudaMemsetAsync(d_def_bytes, 0, 8, st));
         k_wave_hist<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, (uint32_t *)cnt.p, nb,
                                               d_def_bytes);
         CK(cudaGetLastError());
@@ -924,37 +989,39 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         if (rc) { cleanup(); return rc; }
         k_gather_starts<<<(maxtag + 256) / 256, 256, 0, st>>>((const uint32_t *)cnt.p, nb, maxtag, d_total,
                                                             (uint64_t *)starts.p);
-        // persistent-mode segments and ranges, from the segment bases
-        // (before k_slots turns the bases into cursors)
-        {
-            Scratch flag;
-            CK(flag.alloc(4 * M, st));
-            k_seg_flags<<<1024, 256, 0, st>>>((const uint32_t *)cnt.p, M, d_total, (uint32_t *)flag.p);
-            uint32_t *d_nseg = d_total + 1;
-            rc = device_excl_scan((uint32_t *)flag.p, M, d_nseg, st);
-            if (rc) { cleanup(); return rc; }
-            uint32_t nseg = 0;
-            CK(cudaMemcpyAsync(&nseg, d_nseg, 4, cudaMemcpyDeviceToHost, st));
-            CK(cudaStreamSynchronize(st));
-            h->n_seg = nseg;
-            h->n_wave_words = (maxtag + 1 + 63) / 64;
-            CK(dev_alloc(&h->d_seg, 16 * (size_t)(nseg ? nseg : 1), st));
-            CK(dev_alloc((void **)&h->d_pending, 8 * (size_t)nb * h->n_wave_words, st));
-            k_segs_build<<<(nb + 255) / 256, 256, 0, st>>>((const uint32_t *)cnt.p, (const uint32_t *)flag.p,
-                                                          d_total, nb, maxtag, h->n_wave_words,
-                                                          (uint4 *)h->d_seg,
-                                                          (unsigned long long *)h->d_pending);
-            CK(cudaGetLastError());
-            CK(cudaMemcpyAsync(&defb_total, d_def_bytes, 8, cudaMemcpyDeviceToHost, st));
-            CK(cudaStreamSynchronize(st));
-            CK(cudaStreamSynchronize(st));
-        }
-        k_slots<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, (uint32_t *)cnt.p,
-                                          h->d_slot, nb);
-        CK(cudaGetLastError());
+        // persistent-mode segments, from the segment bases (before k_slots
+        // turns the bases into cursors)
+        k_seg_flags<<<1024, 256, 0, st>>>((const uint32_t *)cnt.p, M, d_total, (uint32_t *)flag.p);
+        rc = device_excl_scan((uint32_t *)flag.p, M, d_total + 1, st);
+        if (rc) { cleanup(); return rc; }
         // wave_start[0] = wave_start[1] = 0: wave 0 has no triplets
         CK(cudaMemcpyAsync(h->wave_start.data() + 1, starts.p, 8 * (maxtag + 1), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
+    }
+    CK(levcnt.alloc(4 * ((uint64_t)nb + 1), st));
+    // whether the level list holds every match is known to the device only in
+    // a container with tags; it is counted for both there
+    rc = count_levels(h, by_level && !has_tags ? levels : by_level, (uint32_t *)levcnt.p, d_total + 2, st);
+    if (rc) { cleanup(); return rc; }
+    CK(read_words());
+    if (by_level && has_tags) {
+        levels = hw.reached;
+        maxlvl = hw.maxlvl;
+        if (!levels) {  // the in-order matches only
+            rc = count_levels(h, false, (uint32_t *)levcnt.p, d_total + 2, st);
+            if (rc) { cleanup(); return rc; }
+            CK(read_words());
+        }
+    }
+    if (waves) {
+        h->n_seg = hw.segs;
+        h->n_wave_words = (maxtag + 1 + 63) / 64;
+        CK(dev_alloc(&h->d_seg, 16 * (size_t)(h->n_seg ? h->n_seg : 1), st));
+        CK(dev_alloc((void **)&h->d_pending, 8 * (size_t)nb * h->n_wave_words, st));
+        k_segs_build<<<(nb + 255) / 256, 256, 0, st>>>((const uint32_t *)cnt.p, (const uint32_t *)flag.p, d_total, nb,
+                                                      maxtag, h->n_wave_words, (uint4 *)h->d_seg,
+                                                      (unsigned long long *)h->d_pending);
+        k_slots<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, (uint32_t *)cnt.p, h->d_slot, nb);
+        CK(cudaGetLastError());
         h->n_deferred = h->wave_start[h->n_waves];
         if (h->n_deferred) {
             CK(dev_alloc(&h->d_tri, 16 * h->n_deferred, st));
@@ -962,19 +1029,11 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
                                                   nb, h->log2_bs, (uint4 *)h->d_tri);
             CK(cudaGetLastError());
         }
-        h->mean_deferred_len = h->n_deferred ? (double)defb_total / (double)h->n_deferred : 0.0;
+        h->mean_deferred_len = h->n_deferred ? (double)hw.def_bytes / (double)h->n_deferred : 0.0;
         rc = aclz_set_range_bytes(h, h->range_bytes, stream);
         if (rc) { cleanup(); return rc; }
     }
-    // the schedule by levels; a container with tags of its own has its levels
-    // found here
-    const bool by_level = !flat_up && !h->needs_flatten;
-    if (by_level && has_tags) {
-        CK(cudaMemsetAsync(d_maxtag, 0, 8, st));
-        levels = relax_levels(h, d_val, d_maxtag, st);
-        if (levels) CK(cudaMemcpyAsync(&hw[2], d_maxtag + 1, 4, cudaMemcpyDeviceToHost, st));
-    }
-    rc = build_wave0(h, levels ? d_val : nullptr, hw[2], by_level && levels, stream);
+    rc = build_wave0(h, levels ? d_val : nullptr, maxlvl, by_level && levels, (uint32_t *)levcnt.p, hw.lev, stream);
     if (rc) { cleanup(); return rc; }
     if (!h->d_pending) {  // no deferred matches: wave 0 finishes every block
         h->n_wave_words = 1;
@@ -983,8 +1042,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         CK(cudaMemcpyAsync(h->d_pending, ones.data(), 8 * (size_t)nb, cudaMemcpyHostToDevice, st));
     }
     CK(dev_alloc((void **)&h->d_done, 8 * (size_t)nb * h->n_wave_words, st));
-    CK(cudaStreamSynchronize(st));
-    return build_steps(h, stream);
+    return build_steps(h, stream);  // synchronizes
 }
 
 extern "C" int aclz_upload(const void *host_buf, uint64_t n, void *stream, aclz_handle **out) {
@@ -1037,8 +1095,8 @@ int upload_view(const View &v, uint32_t flags, void *stream, FillFn fill, const 
     CK(dev_alloc((void **)&h->d_lit, v.n_literals + 32, st));
     CK(dev_alloc((void **)&h->d_blk_tok, 8 * (nb + 1), st));
     CK(dev_alloc((void **)&h->d_blk_lit, 8 * (nb + 1), st));
-    CK(dev_alloc((void **)&h->d_err, 64, st));
-    CK(cudaMemsetAsync(h->d_err, 0, 64, st));
+    CK(dev_alloc((void **)&h->d_err, kErrBytes, st));
+    CK(cudaMemsetAsync(h->d_err, 0, kErrBytes, st));
     CK(cudaMemsetAsync(h->d_lit + v.n_literals, 0, 32, st));
     if (int rc = fill(h, v, ctx, stream); rc != ACLZ_OK) {
         cleanup();

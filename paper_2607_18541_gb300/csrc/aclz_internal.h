@@ -71,12 +71,17 @@ struct aclz_handle;
 
 namespace aclz {
 
-// Wave 0's index (aclz_wave0.cu): literal units, and the level list of the
-// in-order matches, or with all of every match.  d_val: {level, tag} of every
-// token and maxlvl the largest level, or null when the levels are not known
-// (the in-order ones are then found block by block).  The step lists follow
-// once the worklists are final.
-int build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlvl, bool all, void *stream);
+// Wave 0's index (aclz_wave0.cu).  count_levels: the triplets of the level
+// list of every block (of its in-order matches, or with all of every match),
+// scanned into d_cnt (n_blocks + 1 words), their total to *d_total.
+// build_wave0: literal units, and the list from that scan (n triplets).
+// d_val: {level, tag} of every token and maxlvl the largest level, or null
+// when the levels are not known (the in-order ones are then found block by
+// block).  build_steps: the step lists, once the worklists are final;
+// synchronizes the stream.
+int count_levels(aclz_handle *h, bool all, uint32_t *d_cnt, uint32_t *d_total, void *stream);
+int build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlvl, bool all, const uint32_t *d_cnt,
+                uint32_t n, void *stream);
 int build_steps(aclz_handle *h, void *stream);
 void free_wave0(aclz_handle *h, void *stream);
 
@@ -86,6 +91,10 @@ void free_wave0(aclz_handle *h, void *stream);
 // and 1044 / 657 us by level kernels; at L = 1024 they are level (593 us).
 constexpr double kPersistentMin = 1024.0;
 bool decodes_as_waves(const aclz_handle *h);
+
+// A handle's status array: the status word and, on a line of its own, the
+// count of the grid barrier.
+constexpr uint32_t kBarrierWord = 32, kErrBytes = 256;
 
 // A list of matches that may be copied once everything before it is final:
 // device address of its triplets, and their number.
@@ -139,7 +148,7 @@ struct aclz_handle {
     uint64_t n_cells = 0;
     uint32_t log2_cell = 0;
     void *d_tri = nullptr;        // n_deferred x 16 B triplets (dst, src, len), built at upload
-    uint32_t *d_err = nullptr;    // latched device status bits; word 8: grid barrier count of a persistent decode
+    uint32_t *d_err = nullptr;    // latched device status bits; word kBarrierWord: a persistent decode's grid barrier
     std::vector<uint64_t> wave_start;  // n_waves + 1 entries into the triplet array
     // wave 0: literal units {block, first token, literal range}
     void *d_lunits = nullptr;

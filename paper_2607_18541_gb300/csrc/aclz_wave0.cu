@@ -210,7 +210,16 @@ void aclz::free_wave0(aclz_handle *h, void *stream) {
     h->n_levels = 0;
 }
 
-int aclz::build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlvl, bool all, void *stream) {
+int aclz::count_levels(aclz_handle *h, bool all, uint32_t *d_cnt, uint32_t *d_total, void *stream) {
+    const uint32_t nb = h->n_blocks;
+    k_lev_count<<<(nb + 7) / 8, 256, 0, (cudaStream_t)stream>>>((const uint4 *)h->d_tok, h->d_blk_tok, nb, all, d_cnt);
+    W0CK(cudaGetLastError());
+    if (int rc = device_excl_scan(d_cnt, nb, d_cnt + nb, stream)) return rc;
+    return rc_of(cudaMemcpyAsync(d_total, d_cnt + nb, 4, cudaMemcpyDeviceToDevice, (cudaStream_t)stream));
+}
+
+int aclz::build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlvl, bool all,
+                      const uint32_t *d_cnt, uint32_t n, void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
     const uint32_t nb = h->n_blocks;
     // units of 2 KiB, smaller in a short stream so that there are about 32
@@ -223,27 +232,20 @@ int aclz::build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t 
     k_lit_units<<<(nb + 7) / 8, 256, 0, st>>>(h->d_blk_tok, h->d_blk_lit, h->d_toklit, nb, lu, (uint4 *)h->d_lunits);
     W0CK(cudaGetLastError());
     // level list
-    Scratch cnt, work, tri, key, idx, key2, idx2, start;
-    W0CK(cnt.alloc(4 * ((uint64_t)nb + 1), st));
-    k_lev_count<<<(nb + 7) / 8, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, nb, all, cnt.as<uint32_t>());
-    W0CK(cudaGetLastError());
-    if (int rc = device_excl_scan(cnt.as<uint32_t>(), nb, cnt.as<uint32_t>() + nb, st)) return rc;
-    uint32_t n = 0;
-    W0CK(cudaMemcpyAsync(&n, cnt.as<uint32_t>() + nb, 4, cudaMemcpyDeviceToHost, st));
-    W0CK(cudaStreamSynchronize(st));
+    Scratch work, tri, key, idx, key2, idx2, start;
     if (!n) return ACLZ_OK;
     h->by_level = all;
     W0CK(tri.alloc(16 * (uint64_t)n, st));
     W0CK(key.alloc(4 * (uint64_t)n, st));
     W0CK(idx.alloc(4 * (uint64_t)n, st));
     k_lev_build<<<(nb + 7) / 8, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, nb, h->log2_bs,
-                                              cnt.as<uint32_t>(), all, d_val, (uint4 *)tri.p, key.as<uint32_t>(), idx.as<uint32_t>());
+                                              d_cnt, all, d_val, (uint4 *)tri.p, key.as<uint32_t>(), idx.as<uint32_t>());
     W0CK(cudaGetLastError());
     W0CK(key2.alloc(4 * (uint64_t)n, st));
     if (!d_val) {
         W0CK(work.alloc(16, st));
         W0CK(cudaMemsetAsync(work.p, 0, 16, st));
-        k_ord_levels<<<nb, kLevelThreads, 0, st>>>((const uint4 *)tri.p, cnt.as<uint32_t>(), key2.as<uint32_t>(), work.as<uint32_t>(), key.as<uint32_t>());
+        k_ord_levels<<<nb, kLevelThreads, 0, st>>>((const uint4 *)tri.p, d_cnt, key2.as<uint32_t>(), work.as<uint32_t>(), key.as<uint32_t>());
         W0CK(cudaGetLastError());
         W0CK(cudaMemcpyAsync(&maxlvl, work.p, 4, cudaMemcpyDeviceToHost, st));
         W0CK(cudaStreamSynchronize(st));
@@ -288,7 +290,7 @@ int aclz::build_steps(aclz_handle *h, void *stream) {
     h->n_levels = h->by_level || h->flat ? (uint32_t)list.size() : 0;
     for (const Step &x : list)
         if (x.n >= 1ULL << 31) h->n_levels = 0;  // the kernel over them counts in 32 bits
-    if (!h->n_levels) return ACLZ_OK;
+    if (!h->n_levels) return rc_of(cudaStreamSynchronize(st));
     W0CK(dev_alloc(&h->d_levels, sizeof(Step) * list.size(), st));
     W0CK(cudaMemcpyAsync(h->d_levels, list.data(), sizeof(Step) * list.size(), cudaMemcpyHostToDevice, st));
     W0CK(cudaStreamSynchronize(st));
