@@ -59,7 +59,7 @@ constexpr int kUnrollRanges = 4; // the same in the persistent schedule's regist
 constexpr uint32_t kTmaMin = 192;
 constexpr uint32_t kPiece = 2048;
 // persistent level copies: CTA size, CTAs per SM
-constexpr int kPersThreads = 512, kPersCtas = 2;
+constexpr int kPersThreads = 256, kPersCtas = 2;
 constexpr uint32_t kSmemPerSm = 220u * 1024u;  // stage memory shared by the CTAs of one SM
 // per-wave kernels are launched with programmatic stream serialization
 constexpr int kWavePdl = 1;
@@ -141,7 +141,9 @@ __device__ __forceinline__ unsigned same_wave_deps(const Group<G> &g, bool v, ui
 // the tokens' output and literal offsets from the upload; a token's run ends
 // where the next token's literals start.  With done non-null (the
 // persistent schedule follows), each block's done bits start as its empty
-// waves plus wave 0.
+// waves plus wave 0; with barrier non-null (the persistent level schedule
+// follows) its count starts at 0.  The other schedules leave both alone: they
+// may run on one handle in several streams.
 //
 // Bound by the latency of the unit's one or two rounds and by instruction
 // issue.  Units, and not blocks, are the work items because a stream has few
@@ -158,7 +160,7 @@ __global__ void __launch_bounds__(kLitThreads, kLitMinCtas)
            const uint64_t *__restrict__ pending, uint64_t *done, uint64_t n_done, uint32_t ww, uint32_t *barrier) {
     Group<G> g;
     griddep_launch_dependents();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *barrier = 0;
+    if (barrier && blockIdx.x == 0 && threadIdx.x == 0) *barrier = 0;
     const uint64_t tid = blockIdx.x * (uint64_t)kLitThreads + threadIdx.x;
     for (uint64_t k = tid; k < n_done; k += (uint64_t)gridDim.x * kLitThreads)
         done[k] = ~__ldg(pending + k) | (k % ww == 0 ? 1ULL : 0ULL);
@@ -465,13 +467,16 @@ __global__ void __launch_bounds__(kLevelThreads, kLevelMinCtas)
 }
 
 // Every level in one cooperative launch.  A level's matches are dealt out
-// evenly, at most G / 2 per group at a time, through the groups' stages; the
-// next level's first window is loaded before the barrier.
+// evenly, at most G / 2 per group at a time, through the group's two stages
+// in turn; the next level's first window is loaded before the barrier.
 //
-// 32 warps per SM at 64 registers; with the level's barrier (2 to 3 us) it
-// takes 593 us for the 1 GiB copy sweep at L = 1024 where k_ranges takes 627
-// (1 GiB at L = 512 / 192: 750 / 1152 against 845 / 1710; one kernel per
-// level 657 / 1044).
+// Bound by a window's chain of fill, copy out, fill: a kilobyte match leaves
+// three to a stage, so a window takes five fills or more.  With one stage per
+// group and 32 warps per SM the 1 GiB copy sweep at L = 1024 / 4096 took
+// 600 / 521 us; with two stages in turn, 16 warps per SM of up to 128
+// registers and matches copied out one by one (their chunks need no search),
+// 556 / 490 us, and 64 MiB at L = 1024 158 -> 125 us (k_ranges took 627 us at
+// L = 1024).
 template <int G>
 __global__ void __launch_bounds__(kPersThreads, kPersCtas)
     k_levels_persistent(const Step *__restrict__ steps, uint32_t count, uint8_t *out, uint32_t stage_bytes,
@@ -480,12 +485,14 @@ __global__ void __launch_bounds__(kPersThreads, kPersCtas)
     constexpr int kGroups = kPersThreads / G;
     Group<G> g;
     const int gi = threadIdx.x / G;
-    Stage st;
-    st.bar = reinterpret_cast<uint64_t *>(smem) + gi;
-    st.buf = smem + 128 * ((8 * kGroups + 127) / 128) + (size_t)gi * stage_bytes;
-    st.bytes = stage_bytes;
-    st.phase = 0;
-    if (g.lane == 0) mbar_init(st.bar, 1);
+    Stage st[2];
+    for (int k = 0; k < 2; k++) {
+        st[k].bar = reinterpret_cast<uint64_t *>(smem) + 2 * gi + k;
+        st[k].buf = smem + 128 * ((16 * kGroups + 127) / 128) + (size_t)(2 * gi + k) * stage_bytes;
+        st[k].bytes = stage_bytes;
+        st[k].phase = 0;
+        if (g.lane == 0) mbar_init(st[k].bar, 1);
+    }
     fence_mbar_init();
     __syncthreads();
     const uint32_t gid = (blockIdx.x * kPersThreads + threadIdx.x) / G;
@@ -509,16 +516,18 @@ __global__ void __launch_bounds__(kPersThreads, kPersCtas)
         for (uint32_t a = gid * per; ok && a < (uint32_t)cur.y; a += ng * per) {
             const uint4 t = t0;
             t0 = window(cur, per, a + ng * per);
-            ok = group_copy_staged<G, G / 2>(g, st, out, tri_dst(t), out + tri_src(t), tri_len(t), err);
-            g.sync();
-            fence_proxy_async_shared();  // before the stage is filled again
+            ok = group_copy_piped<G, G / 2>(g, st, out, tri_dst(t), out + tri_src(t), tri_len(t), err);
         }
         if (k + 1 == count) break;
         cur = nx;
         per = share(cur.y);
         t0 = window(cur, per, gid * per);
         if (k + 2 < count) nx = __ldg(list + k + 2);
-        if (!grid_barrier(err + kBarrierWord, (k + 1) * gridDim.x, ok, err)) return;
+        if (!grid_barrier(err + kBarrierWord, (k + 1) * gridDim.x, ok, err)) break;
+    }
+    if (!ok) {  // a wait timed out: leave no fill in flight
+        stage_wait(st[0], err);
+        stage_wait(st[1], err);
     }
 }
 
@@ -574,13 +583,13 @@ int launch_wave_steps(const aclz_handle *h, uint8_t *out, cudaStream_t st) {
 }
 
 template <int G>
-int launch_lits(aclz_handle *h, uint8_t *out, cudaStream_t st, bool ranges) {
+int launch_lits(aclz_handle *h, uint8_t *out, cudaStream_t st, bool ranges, bool levels) {
     constexpr int gpc = kLitThreads / G;
     const uint64_t n_done = ranges ? (uint64_t)h->n_blocks * h->n_wave_words : 0;
     const unsigned grid = (unsigned)((h->n_lunits + gpc - 1) / gpc);
     k_lits<G><<<grid, kLitThreads, 0, st>>>((const uint4 *)h->d_lunits, h->n_lunits, h->d_lit, h->d_blk_tok,
                                             h->d_blk_lit, h->d_tokdst, h->d_toklit, out, h->log2_bs, h->d_pending,
-                                            h->d_done, n_done, h->n_wave_words, h->d_err + kBarrierWord);
+                                            h->d_done, n_done, h->n_wave_words, levels ? h->d_err + kBarrierWord : nullptr);
     if (cudaError_t e = cudaGetLastError(); e != cudaSuccess) {
         note_cuda_error(e);
         return ACLZ_E_CUDA;
@@ -592,7 +601,7 @@ int launch_lits(aclz_handle *h, uint8_t *out, cudaStream_t st, bool ranges) {
 // else the in-order levels, then one kernel per wave.
 template <int G>
 int launch_waves(aclz_handle *h, uint8_t *out, cudaStream_t st, cudaEvent_t phase, bool by_level) {
-    if (int rc = launch_lits<G>(h, out, st, false)) return rc;
+    if (int rc = launch_lits<G>(h, out, st, false, false)) return rc;
     if (by_level && !phase) return launch_levels<G>(h, h->lsteps, (uint32_t)h->lsteps.size(), out, st);
     if (int rc = launch_levels<G>(h, h->steps, h->n_ord_steps, out, st)) return rc;
     if (phase) cudaEventRecord(phase, st);
@@ -618,7 +627,7 @@ size_t &smem_attr() {
 template <int G, bool STAGED>
 int launch_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaStream_t st, cudaEvent_t phase) {
     constexpr int gpc = kThreads / G;
-    if (int rc = launch_lits<G>(h, out, st, true)) return rc;
+    if (int rc = launch_lits<G>(h, out, st, true, false)) return rc;
     if (int rc = launch_levels<G>(h, h->steps, h->n_ord_steps, out, st)) return rc;
     if (phase) cudaEventRecord(phase, st);
     if (!h->n_ranges) return ACLZ_OK;
@@ -701,20 +710,20 @@ int launch_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaSt
 // one cooperative launch.
 template <int G>
 int launch_levels_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaStream_t st, cudaEvent_t phase) {
-    if (int rc = launch_lits<G>(h, out, st, false)) return rc;
+    if (int rc = launch_lits<G>(h, out, st, false, true)) return rc;
     if (phase) cudaEventRecord(phase, st);
     constexpr int gpc = kPersThreads / G;
     const uint32_t ctas = ctas_per_sm ? std::min<uint32_t>(ctas_per_sm, kPersCtas) : kPersCtas;
-    constexpr uint32_t bar = 128 * ((8 * gpc + 127) / 128);
-    uint32_t stage = ((kSmemPerSm / ctas - bar) / gpc) & ~127u;
-    const size_t smem = bar + (size_t)gpc * stage;
+    constexpr uint32_t bar = 128 * ((16 * gpc + 127) / 128);
+    uint32_t stage = ((kSmemPerSm / ctas - bar) / (2 * gpc)) & ~127u;
+    const size_t smem = bar + (size_t)2 * gpc * stage;
     int sms = 0;
     auto fn = k_levels_persistent<G>;
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     // the attribute is the largest any call needs, the same on every call
-    constexpr uint32_t most = ((kSmemPerSm - bar) / gpc) & ~127u;
+    constexpr uint32_t most = ((kSmemPerSm - bar) / (2 * gpc)) & ~127u;
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(bar + (size_t)gpc * most));
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(bar + (size_t)2 * gpc * most));
     const Step *steps = (const Step *)h->d_levels;
     uint32_t count = h->n_levels, *err = h->d_err;
     void *args[] = {&steps, &count, &out, &stage, &err};

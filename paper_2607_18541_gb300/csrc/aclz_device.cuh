@@ -492,6 +492,40 @@ __device__ __forceinline__ bool staged_copy_fills(const Group<G> &g, Stage &st, 
     }
 }
 
+// The full chunks of the group's jobs from shared memory (S: shared address),
+// one job after another: for jobs of about G chunks or more, whose chunks
+// need no search for their job and share one shift.
+template <int G>
+__device__ __forceinline__ void copy_full_by_job(const Group<G> &g, uintptr_t P, uint32_t S, uint32_t c,
+                                                 unsigned have) {
+    for (; have; have &= have - 1) {
+        const int j = __ffs(have) - 1;
+        uint8_t *pj = reinterpret_cast<uint8_t *>((uintptr_t)g.shfl((unsigned long long)P, j));
+        const uint32_t sj = g.shfl(S, j), cj = g.shfl(c, j);
+        const uint32_t r = sj & 15u, base = sj & ~15u, q = r >> 2, sh = (r & 3u) * 8u;
+        auto word = [&](uint32_t k) {
+            const uint4 x = lds16_u32(base + 16 * k);
+            return r ? window16_uniform(x, lds16_u32(base + 16 * k + 16), q, sh) : x;
+        };
+        uint32_t k = g.lane, left = cj;
+        for (; left > G; k += 2 * G, left = left > 2 * G ? left - 2 * G : 0) {  // two a lane
+            const uint4 v = word(k);
+            const bool two = k + G < cj;
+            const uint4 v2 = word(two ? k + G : k);
+            *reinterpret_cast<uint4 *>(pj + 16 * (uint64_t)k) = v;
+            if (two) *reinterpret_cast<uint4 *>(pj + 16 * (uint64_t)(k + G)) = v2;
+        }
+        if (g.lane < left) *reinterpret_cast<uint4 *>(pj + 16 * (uint64_t)k) = word(k);
+    }
+}
+
+// Jobs of at least this many full chunks (of 32 lanes; in proportion for
+// narrower groups) are copied out one by one: below it more than a third of
+// the lanes would idle.  1 GiB copy sweep at L = 384 / 512 / 1000 (23, 31 and
+// 61 chunks) by level kernels 802 / 685 / 617 us packed and 790 / 663 / 577 us
+// one by one; at L = 256 (15 chunks) 944 and 960 us.
+constexpr uint32_t kByJobMin = 20;
+
 // Packed group copy of at most J <= G / 2 jobs, in the lowest lanes (n == 0
 // in the others), from shared memory: the next J lanes copy what the first
 // ones have after their jobs' last 16-byte boundary, so that heads and tails
@@ -506,8 +540,12 @@ __device__ __forceinline__ void group_copy_few(const Group<G> &g, uintptr_t p, u
     const bool second = g.lane >= J;
     const uintptr_t ep = second ? pe - tail : p, eq = second ? qe - tail : (uint32_t)q;
     const uint32_t en = !second ? head : g.lane < 2 * J ? tail : 0u;
+    // job by job when every job fills most of the lanes by itself
     const unsigned have = g.ballot(c > 0);
-    if (have) copy_full_chunks<G, 1, kFromShared>(g, p + head, q + head, c, have);
+    if (have && !g.ballot(c > 0 && c < kByJobMin * G / 32))
+        copy_full_by_job<G>(g, p + head, (uint32_t)q + head, c, have);
+    else if (have)
+        copy_full_chunks<G, 1, kFromShared>(g, p + head, q + head, c, have);
     if (en) store_bytes(ep, load_bytes<kFromShared>(eq, en), en);
 }
 
@@ -546,6 +584,61 @@ __device__ __forceinline__ bool group_copy_staged(const Group<G> &g, Stage &st, 
         }
     }
     return true;
+}
+
+// The same with two stages in turn: the next fill is in flight while the
+// current one is copied out (jobs of a kilobyte take several fills a window).
+// After a wait that timed out the next fill may be in flight: the caller
+// drains both stages before it returns.
+template <int G, int J>
+__device__ __forceinline__ bool group_copy_piped(const Group<G> &g, Stage (&st)[2], uint8_t *out, uint64_t d,
+                                                 const uint8_t *s, uint32_t n, uint32_t *err) {
+    uintptr_t p = reinterpret_cast<uintptr_t>(out) + d, q = reinterpret_cast<uintptr_t>(s);
+    // a fill of stage t: its piece of this lane's job (at, from, m)
+    uintptr_t at = 0, at2 = 0;
+    uint32_t from = 0, m = 0, from2 = 0, m2 = 0;
+    auto issue = [&](Stage &t, uintptr_t &a, uint32_t &f, uint32_t &k) {
+        k = n < t.bytes - 32 ? n : t.bytes - 32;
+        const uint32_t lead = (uint32_t)q & 15u, span = k ? (lead + k + 15u) & ~15u : 0u;
+        const uint32_t incl = g.scan_incl(span);
+        const bool take = k > 0 && incl <= t.bytes;
+        const uint32_t tx = g.shfl(incl, 31 - __clz(g.ballot(take)));
+        if (g.lane == 0) mbar_expect_tx(t.bar, tx);
+        g.sync();
+        a = p;
+        f = smem_u32(t.buf) + incl - span + lead;
+        if (take)
+            tma_load_1d(t.buf + (incl - span), reinterpret_cast<const void *>(q - lead), span, t.bar);
+        else
+            k = 0;
+        p += k;
+        q += k;
+        n -= k;
+    };
+    if (!g.ballot(n > 0)) return true;
+    issue(st[0], at, from, m);
+    for (;;) {
+#pragma unroll
+        for (int b = 0; b < 2; b++) {
+            const bool next = g.ballot(n > 0) != 0;
+            if (next) issue(st[b ^ 1], at2, from2, m2);
+            if (g.ballot(!stage_wait(st[b], err))) return false;
+            group_copy_few<G, J>(g, at, from, m);
+            g.sync();
+            fence_proxy_async_shared();  // the stage may be filled again
+            if (!next) {
+                if (b == 0) {  // the stages keep their order
+                    const Stage t = st[0];
+                    st[0] = st[1];
+                    st[1] = t;
+                }
+                return true;
+            }
+            at = at2;
+            from = from2;
+            m = m2;
+        }
+    }
 }
 
 }  // namespace aclz

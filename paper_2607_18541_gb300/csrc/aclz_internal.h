@@ -87,8 +87,9 @@ void free_wave0(aclz_handle *h, void *stream);
 
 // Deferred matches of at least this mean length are decoded by the
 // persistent schedule under ACLZ_MODE_AUTO, shorter ones by levels (or waves),
-// one kernel each: 1 GiB copy sweep at L = 192 / 512 1152 / 750 us persistent
-// and 1044 / 657 us by level kernels; at L = 1024 they are level (593 us).
+// one kernel each: 1 GiB copy sweep at L = 384 / 512 / 768 / 1000 873 / 717 /
+// 639 / 570 us persistent and 794 / 665 / 617 / 580 us by level kernels (64 MiB
+// at L = 768 137 and 140 us): they meet at a kilobyte.
 constexpr double kPersistentMin = 1024.0;
 bool decodes_as_waves(const aclz_handle *h);
 
