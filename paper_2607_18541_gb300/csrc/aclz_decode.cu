@@ -4,7 +4,8 @@
 // (k_lits, over literal units of about equal bytes), then the in-order
 // matches, whose source bytes are literals or in-order match bytes of the
 // same block, level by level (a level's matches are independent; the levels
-// are found at upload).
+// are found at upload): one kernel per level, or, where the deferred matches
+// go by waves or origin pieces, one over the blocks (k_ord_blocks).
 //
 // Waves w >= 1 hold the matches whose sources become final only in earlier
 // waves (the wavefront of Sec. I), block-ordered within each wave.  Two
@@ -50,6 +51,13 @@ constexpr int kLevelThreads = 128, kLevelMinCtas = 9;
 constexpr uint32_t kStageWarp = 3584, kStageWarpLong = 6144;
 constexpr double kStageLongMin = 224.0;
 constexpr uint64_t kLevelQuarter = 40000, kLevelEighth = 20000;
+// in-order levels by block: CTA size, and the same for blocks below kOrdSmall
+// bytes (16 MiB of text flattened, 4 KiB blocks: 118 us with 128 threads,
+// 131 us with 512; 32 MiB, 64 KiB blocks: 225 and 213 us); the length above
+// which a match is copied by a warp
+constexpr int kOrdThreads = 512, kOrdThreadsSmall = 128;
+constexpr uint32_t kOrdSmall = 1u << 14;
+constexpr uint32_t kOrdLong = 64;
 // literal copies: CTA size, CTAs of that size per SM the register cap is set
 // for, chunks per lane per round
 constexpr int kLitThreads = 128, kLitMinCtas = 8, kUnrollLits = 2;
@@ -531,6 +539,79 @@ __global__ void __launch_bounds__(kPersThreads, kPersCtas)
     }
 }
 
+// Every in-order level of one block per CTA, in shared memory: the block comes
+// in as the literal copies left it, a level's matches are copied by one thread
+// each (longer ones by their warp), and the block goes out again, bytes of
+// deferred matches as they were.  Bytes of another block that a match reads
+// are literals.
+//
+// Bound by the latency of a level's barrier, shared loads and narrow shared
+// stores, not by bytes.  With one kernel per level (about 3 us each)
+// 32 MiB of word text at 6/8/10/12, flattened, took 250 us and takes 213 us,
+// 256 KiB of it 69 and 32 us, 16 MiB of FASTQ-like text 55 and 37 us.
+__global__ void __launch_bounds__(kOrdThreads)
+    k_ord_blocks(const uint4 *__restrict__ ord, const uint32_t *__restrict__ base, uint8_t *out, uint32_t log2bs,
+                 uint64_t total) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    griddep_launch_dependents();
+    const uint32_t o0 = __ldg(base + blockIdx.x), o1 = __ldg(base + blockIdx.x + 1);
+    if (o0 == o1) {
+        griddep_wait();  // the grid ends after the one before it
+        return;
+    }
+    const uint32_t tid = threadIdx.x, nt = blockDim.x;
+    auto at = [&](uint32_t i) { return i < o1 ? __ldg(ord + i) : make_uint4(0, 0, 0, 0); };
+    uint4 next = at(o0 + tid);
+    const uint64_t bpos = (uint64_t)blockIdx.x << log2bs;
+    const uint32_t len = (uint32_t)min((uint64_t)1 << log2bs, total - bpos), words = len >> 4;
+    uint8_t *blk = out + bpos;
+    griddep_wait();
+    uint4 *sw = reinterpret_cast<uint4 *>(smem), *gw = reinterpret_cast<uint4 *>(blk);
+#pragma unroll 8
+    for (uint32_t i = tid; i < words; i += nt) sw[i] = __ldcg(gw + i);
+    if (16 * words + tid < len && tid < 16) smem[16 * words + tid] = __ldcg(blk + 16 * words + tid);
+    __syncthreads();
+    const uintptr_t sbase = smem_u32(smem), gbase = reinterpret_cast<uintptr_t>(smem);
+    auto piece = [&](uint32_t d, uint32_t s, uint32_t n) {
+        store_bytes(gbase + d, load_bytes<kFromShared>(sbase + s, n), n);
+    };
+    for (uint32_t w = o0; w < o1; w += nt) {
+        const uint4 t = next;
+        next = at(w + nt + tid);
+        const uint32_t mine = w + tid < o1 ? t.y >> 9 : 0xffffffffu;
+        const uint32_t l1 = __ldg(&ord[min(w + nt, o1) - 1].y) >> 9;
+        uint32_t d = (uint32_t)(tri_dst(t) - bpos), n = tri_len(t);
+        const uint64_t src = tri_src(t);
+        for (uint32_t l = __ldg(&ord[w].y) >> 9; l <= l1; l++) {
+            const bool go = mine == l;
+            uint32_t s = (uint32_t)(src - bpos);
+            if (go && src < bpos) {  // from the blocks before
+                uint64_t a = src;
+                while (n && a < bpos) {
+                    const uint32_t m = (uint32_t)min((uint64_t)min(n, 16u), bpos - a);
+                    store_bytes(gbase + d, load_bytes<kFromL2>(reinterpret_cast<uintptr_t>(out) + a, m), m);
+                    a += m;
+                    d += m;
+                    n -= m;
+                }
+                s = (uint32_t)(a - bpos);
+            }
+            if (go && n <= kOrdLong)
+                for (uint32_t k = 0; k < n; k += 16) piece(d + k, s + k, min(n - k, 16u));
+            for (unsigned m = __ballot_sync(0xffffffffu, go && n > kOrdLong); m; m &= m - 1) {
+                const int j = __ffs(m) - 1;
+                const uint32_t dj = __shfl_sync(0xffffffffu, d, j), sj = __shfl_sync(0xffffffffu, s, j),
+                               nj = __shfl_sync(0xffffffffu, n, j);
+                for (uint32_t k = 16 * (tid & 31); k < nj; k += 512) piece(dj + k, sj + k, min(nj - k, 16u));
+            }
+            __syncthreads();
+        }
+    }
+#pragma unroll 8
+    for (uint32_t i = tid; i < words; i += nt) gw[i] = sw[i];
+    if (16 * words + tid < len && tid < 16) blk[16 * words + tid] = smem[16 * words + tid];
+}
+
 // Launch of one step kernel with programmatic stream serialization: its CTAs
 // may start (and load their worklist) while the previous kernel's last ones
 // finish.
@@ -572,6 +653,22 @@ int launch_levels(const aclz_handle *h, const std::vector<Step> &levels, uint32_
     return ACLZ_OK;
 }
 
+// The in-order levels: by block where the handle lists them so.
+template <int G>
+int launch_order(const aclz_handle *h, uint8_t *out, cudaStream_t st) {
+    if (!h->d_ord) return launch_levels<G>(h, h->steps, h->n_ord_steps, out, st);
+    const size_t smem = std::max<size_t>(h->block_size, 16);
+    // the attribute is the largest any call needs, the same on every call
+    if (cudaError_t e = cudaFuncSetAttribute(k_ord_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize, 1 << 17);
+        e != cudaSuccess) {
+        note_cuda_error(e);
+        return ACLZ_E_CUDA;
+    }
+    const int threads = h->block_size < kOrdSmall ? kOrdThreadsSmall : kOrdThreads;
+    return launch_step(k_ord_blocks, h->n_blocks, 1, threads, smem, st, (const uint4 *)h->d_ord,
+                       (const uint32_t *)h->d_ord_base, out, h->log2_bs, h->total_len);
+}
+
 // Waves >= 1: one kernel each.
 template <int G>
 int launch_wave_steps(const aclz_handle *h, uint8_t *out, cudaStream_t st) {
@@ -603,7 +700,7 @@ template <int G>
 int launch_waves(aclz_handle *h, uint8_t *out, cudaStream_t st, cudaEvent_t phase, bool by_level) {
     if (int rc = launch_lits<G>(h, out, st, false, false)) return rc;
     if (by_level && !phase) return launch_levels<G>(h, h->lsteps, (uint32_t)h->lsteps.size(), out, st);
-    if (int rc = launch_levels<G>(h, h->steps, h->n_ord_steps, out, st)) return rc;
+    if (int rc = launch_order<G>(h, out, st)) return rc;
     if (phase) cudaEventRecord(phase, st);
     return launch_wave_steps<G>(h, out, st);
 }
@@ -628,7 +725,7 @@ template <int G, bool STAGED>
 int launch_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaStream_t st, cudaEvent_t phase) {
     constexpr int gpc = kThreads / G;
     if (int rc = launch_lits<G>(h, out, st, true, false)) return rc;
-    if (int rc = launch_levels<G>(h, h->steps, h->n_ord_steps, out, st)) return rc;
+    if (int rc = launch_order<G>(h, out, st)) return rc;
     if (phase) cudaEventRecord(phase, st);
     if (!h->n_ranges) return ACLZ_OK;
     auto fn = k_ranges<G, STAGED>;
@@ -711,6 +808,8 @@ int launch_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaSt
 template <int G>
 int launch_levels_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaStream_t st, cudaEvent_t phase) {
     if (int rc = launch_lits<G>(h, out, st, false, true)) return rc;
+    if (h->d_ord)
+        if (int rc = launch_order<G>(h, out, st)) return rc;
     if (phase) cudaEventRecord(phase, st);
     constexpr int gpc = kPersThreads / G;
     const uint32_t ctas = ctas_per_sm ? std::min<uint32_t>(ctas_per_sm, kPersCtas) : kPersCtas;
@@ -795,6 +894,7 @@ extern "C" int aclz_decode_plan(const aclz_handle *h, const aclz_decode_cfg *cfg
             n = (c.flags & ACLZ_FLAG_STAGED) && h->n_levels ? 2 : 1 + h->n_ord_steps + (h->n_ranges ? 1 : 0);
         else
             n = 1 + (uint32_t)(goes_by_level(h, cfg) ? h->lsteps.size() : h->steps.size());
+        if (h->d_ord) n++;
     }
     if (resolved) *resolved = c;
     if (launches) *launches = n;

@@ -161,6 +161,11 @@ struct aclz_handle {
     void *d_lev = nullptr;
     std::vector<uint64_t> lev_start;
     bool by_level = false;
+    // the same list's in-order matches by block and level (level from bit 9 of
+    // .y on), and each block's first: they take the place of the in-order
+    // levels' steps where they are built
+    void *d_ord = nullptr;
+    uint32_t *d_ord_base = nullptr;
     // what follows the literals, in order: in steps the in-order levels
     // (n_ord_steps of them), then the non-empty waves; in lsteps every
     // level.  d_levels is, on the device, the list whose steps hold

@@ -194,11 +194,95 @@ __global__ void k_lev_gather(const uint4 *__restrict__ tri, const uint32_t *__re
     }
 }
 
+// The in-order matches of the level list in one order (level after level): a
+// level is the last one whose first place is at most i.
+__device__ __forceinline__ uint32_t level_of(const uint2 *__restrict__ lev, uint32_t n_lev, uint32_t i) {
+    uint32_t lo = 0, hi = n_lev - 1;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi + 1) >> 1;
+        if (__ldg(&lev[mid].x) <= i) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+// key[i] = block of the i-th of them
+__global__ void k_ord_keys(const uint4 *__restrict__ list, const uint2 *__restrict__ lev, uint32_t n_lev, uint32_t n,
+                           uint32_t log2bs, uint32_t *__restrict__ key, uint32_t *__restrict__ idx) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const uint2 l = __ldg(lev + level_of(lev, n_lev, i));
+        key[i] = (uint32_t)(t_dst(__ldg(list + l.y + (i - l.x))) >> log2bs);
+        idx[i] = i;
+    }
+}
+
+// their triplets in block order, the level from bit 9 of .y on, and every
+// block's first place (base: nb + 1 entries)
+__global__ void k_ord_gather(const uint4 *__restrict__ list, const uint2 *__restrict__ lev, uint32_t n_lev, uint32_t n,
+                             const uint32_t *__restrict__ key, const uint32_t *__restrict__ idx, uint32_t nb,
+                             uint4 *__restrict__ out, uint32_t *__restrict__ base) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const uint32_t at = idx[i], k = level_of(lev, n_lev, at);
+        const uint2 l = __ldg(lev + k);
+        uint4 t = __ldg(list + l.y + (at - l.x));
+        t.y = (t.y & 0x1ffu) | (k << 9);
+        out[i] = t;
+        for (uint32_t b = i ? key[i - 1] + 1 : 0; b <= key[i]; b++) base[b] = i;
+        if (i + 1 == n)
+            for (uint32_t b = key[i] + 1; b <= nb; b++) base[b] = n;
+    }
+}
+
+// In-order levels from which their matches are listed by block: one kernel
+// over the blocks then takes their place (k_ord_blocks).  It moves every block
+// in and out of shared memory, about what three level kernels take.  Blocks up
+// to kOrdBlockMax bytes are held there.
+constexpr uint32_t kOrdLevelsMin = 4;
+constexpr uint32_t kOrdBlockMax = 1u << 17;
+
+// The list by block.  Without memory for it the levels stay as they are.
+int build_ord_blocks(aclz_handle *h, cudaStream_t st) {
+    const std::vector<uint64_t> &ls = h->lev_start;
+    std::vector<uint2> lev;  // {first place, first triplet} of every level with in-order matches
+    uint64_t n = 0;
+    for (size_t k = 0; k + 2 < ls.size(); k += 2)
+        if (ls[k + 1] > ls[k]) {
+            lev.push_back(make_uint2((uint32_t)n, (uint32_t)ls[k]));
+            n += ls[k + 1] - ls[k];
+        }
+    if (lev.size() < kOrdLevelsMin || lev.size() >= 1u << 23 || h->block_size > kOrdBlockMax || n >= 1ULL << 31)
+        return ACLZ_OK;
+    Scratch dl, key, idx, key2, idx2, out, base;
+    const uint32_t nb = h->n_blocks, n_lev = (uint32_t)lev.size();
+    for (cudaError_t e : {dl.alloc(8 * lev.size(), st), key.alloc(4 * n, st), idx.alloc(4 * n, st),
+                          key2.alloc(4 * n, st), idx2.alloc(4 * n, st), out.alloc(16 * n, st),
+                          base.alloc(4 * ((uint64_t)nb + 1), st)})
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return e == cudaErrorMemoryAllocation ? ACLZ_OK : rc_of(e);
+        }
+    W0CK(cudaMemcpyAsync(dl.p, lev.data(), 8 * lev.size(), cudaMemcpyHostToDevice, st));
+    W0CK(cudaStreamSynchronize(st));  // lev is this call's
+    uint32_t *k0 = key.as<uint32_t>(), *v0 = idx.as<uint32_t>(), *k1 = key2.as<uint32_t>(), *v1 = idx2.as<uint32_t>();
+    const unsigned grid = (unsigned)std::min<uint64_t>(4096, (n + 255) / 256);
+    k_ord_keys<<<grid, 256, 0, st>>>((const uint4 *)h->d_lev, dl.as<uint2>(), n_lev, (uint32_t)n, h->log2_bs, k0, v0);
+    W0CK(cudaGetLastError());
+    const int passes = nb <= 256 ? 1 : nb <= 65536 ? 2 : nb <= (1u << 24) ? 3 : 4;
+    if (int rc = device_sort_pairs(&k0, &v0, &k1, &v1, n, passes, st)) return rc;
+    k_ord_gather<<<grid, 256, 0, st>>>((const uint4 *)h->d_lev, dl.as<uint2>(), n_lev, (uint32_t)n, k0, v0, nb,
+                                       out.as<uint4>(), base.as<uint32_t>());
+    W0CK(cudaGetLastError());
+    h->d_ord = out.p;
+    out.p = nullptr;
+    h->d_ord_base = base.as<uint32_t>();
+    base.p = nullptr;
+    return ACLZ_OK;
+}
+
 }  // namespace
 
 void aclz::free_wave0(aclz_handle *h, void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
-    for (void **pp : {&h->d_lunits, &h->d_lev, &h->d_levels}) {
+    for (void **pp : {&h->d_lunits, &h->d_lev, &h->d_levels, &h->d_ord, (void **)&h->d_ord_base}) {
         dev_free(*pp, st);
         *pp = nullptr;
     }
@@ -277,8 +361,14 @@ int aclz::build_steps(aclz_handle *h, void *stream) {
         if (b > a) v.push_back({(uint64_t)((const uint4 *)tri + a), b - a});
     };
     const std::vector<uint64_t> &ls = h->lev_start;
+    dev_free(h->d_ord, st);
+    dev_free(h->d_ord_base, st);
+    h->d_ord = nullptr;
+    h->d_ord_base = nullptr;
+    if (!h->by_level && h->d_lev)
+        if (int rc = build_ord_blocks(h, st)) return rc;
     for (size_t k = 0; k + 2 < ls.size(); k += 2) {
-        add(h->steps, h->d_lev, ls[k], ls[k + 1]);
+        if (!h->d_ord) add(h->steps, h->d_lev, ls[k], ls[k + 1]);
         if (h->by_level) add(h->lsteps, h->d_lev, ls[k], ls[k + 2]);
     }
     h->n_ord_steps = (uint32_t)h->steps.size();

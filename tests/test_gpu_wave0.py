@@ -150,3 +150,55 @@ def test_match_lengths_around_the_stage(ln):
     c = _pack(5 * bs, bs, blocks, LITS)
     assert oracle.validate(c) == 0
     _decode_all_ways(c)
+
+
+@pytest.mark.parametrize("bs,width,levels,ln,lit", [
+    (256, 1, 4, 16, 40), (256, 2, 3, 17, 40), (1024, 3, 5, 15, 40), (4096, 40, 6, 7, 40), (1 << 14, 255, 4, 9, 40),
+    (1 << 14, 256, 4, 9, 40), (1 << 14, 257, 5, 9, 40), (1 << 14, 6, 8, 63, 40), (1 << 14, 6, 8, 64, 40),
+    (1 << 14, 6, 8, 65, 40), (1 << 16, 3, 7, 1025, 40), (1 << 17, 600, 12, 13, 40), (1 << 18, 300, 6, 33, 40),
+    (1 << 14, 6, 8, 63, 80), (1 << 14, 6, 8, 64, 80), (1 << 14, 6, 8, 65, 80), (1 << 14, 6, 8, 81, 90),
+    (1 << 16, 3, 7, 1025, 1100), (1 << 17, 40, 5, 513, 600), (256, 2, 4, 17, 40)])
+def test_in_order_levels_by_block(bs, width, levels, ln, lit):
+    # levels of `width` matches of ln bytes in every other block, every source
+    # alignment, matches that read the block before among them and after them
+    # (they are deferred, and what reads them); a short last block
+    r = np.random.RandomState(bs + width + ln)
+    nb = 7
+    total = nb * bs - 5
+    blocks = [[(bs, 0, 0)]]
+    for b in range(1, nb):
+        toks, at, p, end = [], b * bs, b * bs + lit, min((b + 1) * bs, total)
+        before = None
+        for _ in range(levels if b % 2 else 0):
+            starts = []
+            for k in range(width):
+                if before is not None:
+                    src = before[int(r.randint(width))]
+                elif ln <= lit:
+                    src = at - 7 if k == 0 else at + k % (lit - ln + 1)
+                else:
+                    src = k % 8
+                toks.append((0 if toks else lit, ln, src))
+                starts.append(p)
+                p += ln
+            before = starts
+        if b % 2 and b > 2:
+            toks.append((3, 11, (b - 2) * bs + lit + 2))
+            p += 14
+        if not toks:
+            p = at
+        assert p <= end
+        toks.append((end - p, 0, 0))
+        blocks.append(toks)
+    c = _pack(total, bs, blocks, LITS)
+    assert oracle.validate(c) == 0
+    _decode_all_ways(c)
+    s = torch.cuda.current_stream()
+    h = aclz.aclz_upload(c, s, flags=aclz.ACLZ_UPLOAD_FLATTEN)
+    try:
+        n = levels if levels < 4 or bs > 1 << 17 else 1
+        if ln > lit or width == 1:
+            n = 0  # all of them start from another block's bytes
+        assert aclz.aclz_decode_plan(h, mode=aclz.ACLZ_MODE_WAVES)[1] == 1 + n + 1
+    finally:
+        aclz.aclz_free(h)
