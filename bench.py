@@ -140,8 +140,8 @@ def peaks():
 
 
 def kernel_sources_sha() -> str:
-    """Hash of the sources of the decode kernels (k_wave0, k_ranges and the
-    copy helpers they inline): recorded traffic is valid only for these."""
+    """Hash of the sources of the decode kernels (k_lits, the level,
+    wave and range kernels and the copy helpers they inline): recorded traffic is valid only for these."""
     d = os.path.join(ROOT, "paper_2607_18541_gb300", "csrc")
     h = hashlib.sha256()
     for f in ("aclz_decode.cu", "aclz_device.cuh"):
@@ -152,9 +152,9 @@ def kernel_sources_sha() -> str:
 
 def recorded_traffic(workload: str):
     """DRAM bytes per launch of the dominant kernel from the committed ncu
-    summary (profiles/traffic_k_ranges_<workload>.txt, lines "key: value"),
+    summary (profiles/traffic_k_levels_persistent_<workload>.txt, lines "key: value"),
     if it was taken on the current kernel sources; else None."""
-    p = os.path.join(ROOT, "profiles", f"traffic_k_ranges_{workload}.txt")
+    p = os.path.join(ROOT, "profiles", f"traffic_k_levels_persistent_{workload}.txt")
     if not os.path.exists(p):
         return None
     d = {}
@@ -305,7 +305,7 @@ def workload_config(args, extra):
 
 MODE = {"auto": 2, "waves": 0, "persistent": 1}
 LIB_RANGE_BYTES = 20480  # the work-range size an upload picks
-KERNEL = {0: "k_wave_copy (one launch per wave >= 1)", 1: "k_ranges (persistent, deferred matches)"}
+KERNEL = {0: "k_wave_copy (one launch per wave >= 1)", 1: "k_levels_persistent (every level in one launch)"}
 
 
 def sweep_leg(args, dev, st, peak):
@@ -479,7 +479,7 @@ def run_ours(args):
         kern, kbytes, kms = KERNEL[plan["mode"]], def_bytes, d_ms
         klaunch = launches_per_step - 1
     else:
-        kern, kbytes, kms = "k_wave0 (tokens, literals, in-order matches)", w0_bytes, w0_ms
+        kern, kbytes, kms = "k_lits (literals)", w0_bytes, w0_ms
         klaunch = 1
     achieved = kbytes / (kms * 1e-3) / 1e9
     workload = workload_config(args, None)["workload"]

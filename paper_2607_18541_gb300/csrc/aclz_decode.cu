@@ -26,8 +26,8 @@
 // All copies are 16-byte vectorised with every lane owning aligned output
 // chunks, so short matches from several tokens share one pass instead of
 // leaving most of the group idle (the work-granularity mechanism of
-// Sec. III-C); long matches in the persistent schedule are staged through
-// shared memory by TMA bulk copies (cp.async.bulk + mbarrier).
+// Sec. III-C).  Matches copied by levels, and long ones in work ranges, are
+// staged through shared memory by TMA bulk copies (cp.async.bulk + mbarrier).
 #include <algorithm>
 #include <cstring>
 #include <mutex>
