@@ -46,11 +46,11 @@ constexpr int kWaveThreads = 64, kWaveMinCtas = 1024 / kWaveThreads;
 // per-level copies: CTA size, the CTAs per SM the register cap is set for,
 // stage bytes per warp (16 matches of up to 192 bytes; more when the deferred
 // matches average kStageLongMin bytes or more), and the level sizes up to
-// which a group of G lanes takes G / 4 and G / 8 matches instead of G / 2
+// which a group of G lanes takes G / 4, G / 8 and one match instead of G / 2
 constexpr int kLevelThreads = 128, kLevelMinCtas = 9;
 constexpr uint32_t kStageWarp = 3584, kStageWarpLong = 6144;
 constexpr double kStageLongMin = 224.0;
-constexpr uint64_t kLevelQuarter = 40000, kLevelEighth = 20000;
+constexpr uint64_t kLevelQuarter = 40000, kLevelEighth = 20000, kLevelOne = 5000;
 // in-order levels by block: CTA size, and the same for blocks below kOrdSmall
 // bytes (16 MiB of text flattened, 4 KiB blocks: 118 us with 128 threads,
 // 131 us with 512; 32 MiB, 64 KiB blocks: 225 and 213 us); the length above
@@ -636,7 +636,11 @@ int launch_step(void (*k)(P...), uint64_t n, unsigned per_cta, unsigned threads,
 }
 
 // Levels: one kernel each, fewer matches per group in the small ones, whose
-// groups are all resident at once and take as long as their own window.
+// groups are all resident at once and take as long as their own window.  Up
+// to kLevelOne (about the warps resident at a time) a group takes one match:
+// 64 MiB copy sweep at L = 900 137 -> 115 us, 256 KiB of Markov bytes 38.5 ->
+// 36 us, 64 MiB of FASTQ-like text 120 -> 116 us; up to 20000 instead the
+// 512 MiB sweep at L = 128 goes from 756 to 780 us.
 template <int G>
 int launch_levels(const aclz_handle *h, const std::vector<Step> &levels, uint32_t count, uint8_t *out,
                   cudaStream_t st) {
@@ -644,8 +648,8 @@ int launch_levels(const aclz_handle *h, const std::vector<Step> &levels, uint32_
     constexpr int gpc = kLevelThreads / G;
     for (uint32_t i = 0; i < count; i++) {
         const uint64_t n = levels[i].n;
-        const int part = n <= kLevelEighth ? 8 : n <= kLevelQuarter ? 4 : 2;
-        auto k = part == 8 ? k_level<G, G / 8> : part == 4 ? k_level<G, G / 4> : k_level<G, G / 2>;
+        const int part = n <= kLevelOne ? G : n <= kLevelEighth ? 8 : n <= kLevelQuarter ? 4 : 2;
+        auto k = part == G ? k_level<G, 1> : part == 8 ? k_level<G, G / 8> : part == 4 ? k_level<G, G / 4> : k_level<G, G / 2>;
         if (int rc = launch_step(k, n, kLevelThreads / part, kLevelThreads, (size_t)gpc * stage, st,
                                  (const uint4 *)levels[i].tri, n, out, stage, h->d_err))
             return rc;

@@ -89,7 +89,7 @@ void free_wave0(aclz_handle *h, void *stream);
 // persistent schedule under ACLZ_MODE_AUTO, shorter ones by levels (or waves),
 // one kernel each: 1 GiB copy sweep at L = 384 / 512 / 768 / 1000 873 / 717 /
 // 639 / 570 us persistent and 794 / 665 / 617 / 580 us by level kernels (64 MiB
-// at L = 768 137 and 140 us): they meet at a kilobyte.
+// at L = 900 136 and 115 us): they meet at a kilobyte.
 constexpr double kPersistentMin = 1024.0;
 bool decodes_as_waves(const aclz_handle *h);
 

@@ -101,7 +101,7 @@ def test_in_order_chains(chain, width):
     _decode_all_ways(c)
 
 
-@pytest.mark.parametrize("n", [20000, 20001, 40000, 40001])
+@pytest.mark.parametrize("n", [5000, 5001, 20000, 20001, 40000, 40001])
 def test_levels_around_the_sizes_per_group(n):
     # levels 1 and 3 of n matches, levels 2 and 4 of a few
     bs, ln = 1 << 17, 8
