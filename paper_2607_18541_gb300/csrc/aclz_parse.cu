@@ -179,7 +179,6 @@ __global__ void __launch_bounds__(kBestThreads) k_best(const uint8_t *__restrict
     bool live = r < m;
     uint32_t kp = 0, p = 0, T = 0, rem = 0, need = 0, blen = 0, bsrc = 0;
     unsigned long long own[4] = {0, 0, 0, 0}, mask = 0;
-    const uint32_t no_key = ~__ldg(key_s);  // differs from any chain that reaches rank 0
     // bytes 4 .. need - 1 of a candidate must match (up to 12 of them)
     auto set_need = [&](uint32_t v) {
         need = v;
@@ -188,7 +187,7 @@ __global__ void __launch_bounds__(kBestThreads) k_best(const uint8_t *__restrict
     for (uint32_t kb = 0; kb < depth; kb += kHalo) {
         for (uint32_t i = threadIdx.x; i < kBestThreads + kHalo; i += kBestThreads) {
             const long long rr = (long long)r0 - (long long)kb - (long long)kHalo + (long long)i;
-            uint32_t k = no_key, q = 0;
+            uint32_t k = 0, q = 0;  // places before rank 0 are never looked at
             if (rr >= 0 && (uint64_t)rr < m) {
                 k = __ldg(key_s + rr);
                 q = __ldg(val_s + rr);
@@ -223,11 +222,13 @@ __global__ void __launch_bounds__(kBestThreads) k_best(const uint8_t *__restrict
             if (rem < need) live = false;
         }
         // candidates of this round: the entries with this prefix (the keys are
-        // in order, so they are a run that ends just before the own entry)
+        // in order from rank 0 on, so they are a run that ends just before the
+        // own entry; a live position has rank kb or more)
         uint32_t kn = 0;
         if (live) {
             const uint32_t top = threadIdx.x + kHalo;  // entry of rank r - kb
-            uint32_t lo = top - kHalo, hi = top;
+            const uint32_t rank0 = kb + kHalo > r0 ? (uint32_t)(kb + kHalo - r0) : 0u;  // entry of rank 0
+            uint32_t lo = max(top - kHalo, rank0), hi = top;
             while (lo < hi) {
                 const uint32_t mid = (lo + hi) >> 1;
                 if (skey[mid] == kp) hi = mid; else lo = mid + 1;
