@@ -558,9 +558,10 @@ extern "C" int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_enco
         return rc == ACLZ_OK;
     };
     Scratch dx, dk0, dv0, dk1, dv1, dlen, dslots, dstarts, dntok, dnlit, dtoff, dloff, dmm, dbmm, dcont;
-    // the input with 16 zero bytes after it (the 8-byte compares read
-    // whole aligned words)
-    if (!ck(dx.alloc(n + 64, st)) || !ck(cudaMemsetAsync((uint8_t *)dx.p + (n & ~(uint64_t)15), 0, 48, st)) ||
+    // the input with 64 zero bytes after it (the 8-byte compares read whole
+    // aligned words, the staging of k_best 40 bytes from a prefix on)
+    const uint64_t tail = n & ~(uint64_t)15;
+    if (!ck(dx.alloc(n + 64, st)) || !ck(cudaMemsetAsync((uint8_t *)dx.p + tail, 0, n + 64 - tail, st)) ||
         (n && !ck(cudaMemcpyAsync(dx.p, host_src, n, cudaMemcpyHostToDevice, st))))
         return rc;
     const uint64_t mm1 = m ? m : 1;
