@@ -5,7 +5,9 @@
 // matches, whose source bytes are literals or in-order match bytes of the
 // same block, level by level (a level's matches are independent; the levels
 // are found at upload): one kernel per level, or, where the deferred matches
-// go by waves or origin pieces, one over the blocks (k_ord_blocks).
+// go by waves or origin pieces, one over the blocks (k_ord_blocks).  Where
+// most matches read the ones just before them they are walked in token order,
+// block by block (k_ord_walk).
 //
 // Waves w >= 1 hold the matches whose sources become final only in earlier
 // waves (the wavefront of Sec. I), block-ordered within each wave.  Two
@@ -612,6 +614,46 @@ __global__ void __launch_bounds__(kOrdThreads)
     if (16 * words + tid < len && tid < 16) blk[16 * words + tid] = smem[16 * words + tid];
 }
 
+// The in-order matches of one block per group, in token order: windows of G
+// tokens, each copied in batches that read nothing a match still to be copied
+// writes.  For blocks whose matches mostly read the ones just before them, or
+// whose levels are too many to list: a step of a chain takes 0.4 us here (a
+// store, a load of it from L2), 1.7 us as a level of its own.  12 CTAs per SM
+// (80 registers): with 16 it spills.
+template <int G>
+__global__ void __launch_bounds__(kWaveThreads, 12)
+    k_ord_walk(const uint4 *__restrict__ tok, const uint64_t *__restrict__ blk_tok, const uint32_t *__restrict__ tokdst,
+               uint8_t *out, uint32_t nb, uint32_t log2bs) {
+    Group<G> g;
+    griddep_launch_dependents();
+    const uint64_t b = (blockIdx.x * (uint64_t)kWaveThreads + threadIdx.x) / G;
+    if (b >= nb) return;
+    const uint64_t t0 = __ldg(blk_tok + b), t1 = __ldg(blk_tok + b + 1), bpos = b << log2bs;
+    const uint4 z4 = make_uint4(0, 0, 0, 0);
+    uint4 nt = t0 + g.lane < t1 ? __ldg(tok + t0 + g.lane) : z4;
+    uint32_t nd = t0 + g.lane < t1 ? __ldg(tokdst + t0 + g.lane) : 0u;
+    griddep_wait();
+    for (uint64_t w = t0; w < t1; w += G) {
+        const uint4 t = nt;
+        const uint64_t d = bpos + nd + t.x;
+        const bool more = w + G + g.lane < t1;
+        nt = more ? __ldg(tok + w + G + g.lane) : z4;
+        nd = more ? __ldg(tokdst + w + G + g.lane) : 0u;
+        const uint64_t src = (uint64_t)t.z | ((uint64_t)(t.w & 0xffu) << 32);
+        const bool mine = t.y && !(t.w >> 8);
+        unsigned rem = g.ballot(mine);
+        if (!rem) continue;
+        const unsigned deps = same_wave_deps<G>(g, mine, d, src, t.y, log2bs) & rem;
+        while (rem) {
+            const bool now = ((rem >> g.lane) & 1u) && (deps & rem) == 0u;
+            const unsigned batch = g.ballot(now);
+            group_copy<G, kUnrollCopy>(g, out, d, out + src, now ? t.y : 0u);
+            g.sync();
+            rem &= ~batch;
+        }
+    }
+}
+
 // Launch of one step kernel with programmatic stream serialization: its CTAs
 // may start (and load their worklist) while the previous kernel's last ones
 // finish.
@@ -657,9 +699,13 @@ int launch_levels(const aclz_handle *h, const std::vector<Step> &levels, uint32_
     return ACLZ_OK;
 }
 
-// The in-order levels: by block where the handle lists them so.
+// The in-order matches: walked, or by levels, by block where the handle lists
+// them so.
 template <int G>
 int launch_order(const aclz_handle *h, uint8_t *out, cudaStream_t st) {
+    if (h->walk)
+        return launch_step(k_ord_walk<G>, h->n_blocks, kWaveThreads / G, kWaveThreads, 0, st, (const uint4 *)h->d_tok,
+                           h->d_blk_tok, h->d_tokdst, out, h->n_blocks, h->log2_bs);
     if (!h->d_ord) return launch_levels<G>(h, h->steps, h->n_ord_steps, out, st);
     const size_t smem = std::max<size_t>(h->block_size, 16);
     // the attribute is the largest any call needs, the same on every call
@@ -812,7 +858,7 @@ int launch_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaSt
 template <int G>
 int launch_levels_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaStream_t st, cudaEvent_t phase) {
     if (int rc = launch_lits<G>(h, out, st, false, true)) return rc;
-    if (h->d_ord)
+    if (h->d_ord || h->walk)
         if (int rc = launch_order<G>(h, out, st)) return rc;
     if (phase) cudaEventRecord(phase, st);
     constexpr int gpc = kPersThreads / G;
@@ -898,7 +944,7 @@ extern "C" int aclz_decode_plan(const aclz_handle *h, const aclz_decode_cfg *cfg
             n = (c.flags & ACLZ_FLAG_STAGED) && h->n_levels ? 2 : 1 + h->n_ord_steps + (h->n_ranges ? 1 : 0);
         else
             n = 1 + (uint32_t)(goes_by_level(h, cfg) ? h->lsteps.size() : h->steps.size());
-        if (h->d_ord) n++;
+        if (h->d_ord || h->walk) n++;
     }
     if (resolved) *resolved = c;
     if (launches) *launches = n;

@@ -71,17 +71,19 @@ struct aclz_handle;
 
 namespace aclz {
 
-// Wave 0's index (aclz_wave0.cu).  count_levels: the triplets of the level
-// list of every block (of its in-order matches, or with all of every match),
-// scanned into d_cnt (n_blocks + 1 words), their total to *d_total.
-// build_wave0: literal units, and the list from that scan (n triplets).
+// Wave 0's index (aclz_wave0.cu).  build_units: literal units.  count_levels:
+// the triplets of the level list of every block (of its in-order matches, or
+// with all of every match), scanned into d_cnt (n_blocks + 1 words), their
+// total to *d_total.  build_levels: the list from that scan (n triplets).
 // d_val: {level, tag} of every token and maxlvl the largest level, or null
 // when the levels are not known (the in-order ones are then found block by
-// block).  build_steps: the step lists, once the worklists are final;
-// synchronizes the stream.
+// block).  Where there are more than kOrdLevelsMost of those, it leaves the
+// in-order matches to the walk, without a list.  build_steps: the step lists,
+// once the worklists are final; synchronizes the stream.
+int build_units(aclz_handle *h, void *stream);
 int count_levels(aclz_handle *h, bool all, uint32_t *d_cnt, uint32_t *d_total, void *stream);
-int build_wave0(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlvl, bool all, const uint32_t *d_cnt,
-                uint32_t n, void *stream);
+int build_levels(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlvl, bool all, const uint32_t *d_cnt,
+                 uint32_t n, void *stream);
 int build_steps(aclz_handle *h, void *stream);
 void free_wave0(aclz_handle *h, void *stream);
 
@@ -161,6 +163,10 @@ struct aclz_handle {
     void *d_lev = nullptr;
     std::vector<uint64_t> lev_start;
     bool by_level = false;
+    // the in-order matches have no list: each block's are walked in token
+    // order (most matches read the ones just before them, or the levels are
+    // too many, or the list does not fit)
+    bool walk = false;
     // the same list's in-order matches by block and level (level from bit 9 of
     // .y on), and each block's first: they take the place of the in-order
     // levels' steps where they are built
