@@ -306,14 +306,14 @@ __global__ void __launch_bounds__(kThreads, STAGED ? 2 : 3)
                 if (STAGED) {
                     if (!issued) fence_proxy_async_global();
                     const bool longj = mine && len >= kTmaMin;
-                    group_copy<G, 2>(g, out, d, out + sr, (mine && !longj) ? len : 0u);
+                    group_copy_batch<G, 2>(g, out, d, out + sr, (mine && !longj) ? len : 0u);
                     if (issued || g.ballot(longj)) {
                         if (!staged_copy_fills<G>(g, st, out, d, out + sr, longj ? len : 0u, piece, pre, issued,
                                                   err))
                             return;  // a bulk copy did not complete: no further copies into the stage
                     }
                 } else {
-                    group_copy<G, kUnrollRanges>(g, out, d, out + sr, mine ? len : 0u);
+                    group_copy_batch<G, kUnrollRanges>(g, out, d, out + sr, mine ? len : 0u);
                 }
                 g.sync();
                 rem &= ~batch;
@@ -423,7 +423,7 @@ __device__ __forceinline__ void wave_window(const Group<G> &g, const uint4 *__re
         while (rem) {
             const unsigned batch = g.ballot(((rem >> g.lane) & 1u) && (deps & rem) == 0u);
             const bool mine = (batch >> g.lane) & 1u;
-            group_copy<G, kUnrollCopy>(g, out, d, out + sr, mine ? len : 0u);
+            group_copy_batch<G, kUnrollCopy>(g, out, d, out + sr, mine ? len : 0u);
             g.sync();
             rem &= ~batch;
         }
@@ -647,7 +647,7 @@ __global__ void __launch_bounds__(kWaveThreads, 12)
         while (rem) {
             const bool now = ((rem >> g.lane) & 1u) && (deps & rem) == 0u;
             const unsigned batch = g.ballot(now);
-            group_copy<G, kUnrollCopy>(g, out, d, out + src, now ? t.y : 0u);
+            group_copy_batch<G, kUnrollCopy>(g, out, d, out + src, now ? t.y : 0u);
             g.sync();
             rem &= ~batch;
         }

@@ -297,6 +297,37 @@ __device__ __forceinline__ void group_copy(const Group<G> &g, uint8_t *out, uint
     group_copy_from<G, U, SRC>(g, reinterpret_cast<uintptr_t>(out) + d, reinterpret_cast<uintptr_t>(s), n);
 }
 
+// The same for one batch of a chain, where the next batch waits for this one:
+// a single job (lane j's) is dealt to the lanes by its chunks at once, without
+// the search for every chunk's job.  A step of a chain of 64-byte matches
+// takes 0.38 us instead of 0.80 us (0.59 us with a packed copy that found every
+// chunk's job by shuffles): 1 MiB of zeros in one block 13.2 -> 6.3 ms, 256 KiB in 16
+// KiB blocks by waves 3.11 -> 1.57 ms, by ranges 3.55 -> 1.88 ms.
+template <int G, int U, Source SRC = kFromL2>
+__device__ __forceinline__ void group_copy_batch(const Group<G> &g, uint8_t *out, uint64_t d, const uint8_t *s,
+                                                 uint32_t n) {
+    const unsigned jobs = g.ballot(n > 0);
+    if (jobs & (jobs - 1u)) {
+        group_copy<G, U, SRC>(g, out, d, s, n);
+        return;
+    }
+    const int j = __ffs(jobs) - 1;
+    if (j < 0) return;
+    const uintptr_t p = (uintptr_t)g.shfl((unsigned long long)(reinterpret_cast<uintptr_t>(out) + d), j);
+    const uintptr_t q = (uintptr_t)g.shfl((unsigned long long)reinterpret_cast<uintptr_t>(s), j);
+    const uint32_t m = g.shfl(n, j);
+    // stretches of the output between 16-byte boundaries, one a lane
+    const uint32_t lead = (uint32_t)p & 15u;
+    for (uint32_t k = g.lane; 16 * k < lead + m; k += G) {
+        const uint32_t a = k ? 16 * k - lead : 0u, e = min(16 * k + 16 - lead, m);
+        const uint4 v = load_bytes<SRC>(q + a, e - a);
+        if (e - a == 16)
+            *reinterpret_cast<uint4 *>(p + a) = v;
+        else
+            store_bytes(p + a, v, e - a);
+    }
+}
+
 // Bytes [r, r + 16) of a || b for a shift r that is the same on every lane
 // (a uniform branch picks the word offset).
 __device__ __forceinline__ uint4 window16_uniform(const uint4 &a, const uint4 &b, uint32_t q, uint32_t sh) {

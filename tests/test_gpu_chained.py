@@ -96,3 +96,32 @@ def test_chains_of_neighbours(nb, bs, ln, width, short):
 def test_more_levels_than_are_listed(nb, bs, ln, width):
     # 1137 to 2047 levels, no match near the one it reads
     _decode_all_ways(_chains(nb, bs, ln, width), (1, 1))
+
+
+@pytest.mark.parametrize("top", [17, 40, 300, 1100])
+@pytest.mark.parametrize("cross", [False, True])
+def test_chain_of_all_lengths(top, cross):
+    # one match after another, each reading bytes of the one before it (or,
+    # across, of the block before and then of the one before it): every length
+    # up to `top`, at every alignment of source and output
+    r = np.random.RandomState(top)
+    bs, nb, lit0 = 1 << 15, 3, top + 64
+    ll, ml, sr, nt = [], [], [], []
+    for b in range(nb):
+        at, end = b * bs, (b + 1) * bs
+        p, toks = at + lit0, 0
+        if cross and b:
+            ll.append(0), ml.append(lit0), sr.append(at - lit0 - 3)
+            toks = 1
+        while p + 2 * top <= end:
+            n = int(r.randint(1, top + 1)) if toks % 3 else top
+            ll.append(lit0 if toks == 0 else 0), ml.append(n), sr.append(p - n - int(r.randint(0, 20)))
+            p += n
+            toks += 1
+        ll.append(end - p), ml.append(0), sr.append(0)
+        nt.append(toks + 1)
+    ll = np.array(ll, dtype=np.uint32)
+    c = aclz.aclz_pack(nb * bs, bs, (4, 4, 4, 4), np.array(nt, dtype=np.uint32), ll, np.array(ml, dtype=np.uint32),
+                       np.array(sr, dtype=np.uint64), r.randint(0, 256, int(ll.sum())).astype(np.uint8))
+    assert oracle.validate(c) == 0
+    _decode_all_ways(c, (None, None))
