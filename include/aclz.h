@@ -287,8 +287,9 @@ typedef struct aclz_decode_cfg {
 
 #define ACLZ_MODE_WAVES 0      /* wave 0, then one kernel per wave */
 #define ACLZ_MODE_PERSISTENT 1 /* wave 0, then one launch with bounded waits */
-#define ACLZ_MODE_AUTO 2       /* persistent + staged when deferred matches average >= 1024 B, else waves, one
-                                  kernel per dependency level where the upload found the levels */
+#define ACLZ_MODE_AUTO 2       /* persistent + staged when deferred matches average >= 1024 B, else one kernel per
+                                  dependency level; where the upload found no levels, or with a phase event, persistent
+                                  + staged from 192 B on, else waves (a flattened handle's one wave: up to 1024 B) */
 #define ACLZ_FLAG_STAGED 1u    /* persistent: stage long matches through shared memory (TMA) */
 #define ACLZ_FLAG_REGISTERS 2u /* persistent: copy through registers only */
 

@@ -749,7 +749,7 @@ int launch_lits(aclz_handle *h, uint8_t *out, cudaStream_t st, bool ranges, bool
 template <int G>
 int launch_waves(aclz_handle *h, uint8_t *out, cudaStream_t st, cudaEvent_t phase, bool by_level) {
     if (int rc = launch_lits<G>(h, out, st, false, false)) return rc;
-    if (by_level && !phase) return launch_levels<G>(h, h->lsteps, (uint32_t)h->lsteps.size(), out, st);
+    if (by_level) return launch_levels<G>(h, h->lsteps, (uint32_t)h->lsteps.size(), out, st);
     if (int rc = launch_order<G>(h, out, st)) return rc;
     if (phase) cudaEventRecord(phase, st);
     return launch_wave_steps<G>(h, out, st);
@@ -906,14 +906,16 @@ int launch_persistent_auto(aclz_handle *h, uint8_t *out, const aclz_decode_cfg &
 
 namespace {
 
-// Levels take the place of waves only when the caller left the mode open: an
-// explicit ACLZ_MODE_WAVES is one kernel per wave.
-bool goes_by_level(const aclz_handle *h, const aclz_decode_cfg *cfg) {
-    return h->by_level && decodes_as_waves(h) && (!cfg || cfg->mode == ACLZ_MODE_AUTO);
+// Levels take the place of waves only when the caller left the mode open (an
+// explicit ACLZ_MODE_WAVES is one kernel per wave) and no event goes between
+// the phases.
+bool goes_by_level(const aclz_handle *h, const aclz_decode_cfg *cfg, bool phase) {
+    return h->by_level && !phase && (!cfg || cfg->mode == ACLZ_MODE_AUTO) && h->mean_deferred_len < kPersistentMin;
 }
 
-// Checks cfg and resolves ACLZ_MODE_AUTO for this handle.
-int resolve_cfg(const aclz_handle *h, const aclz_decode_cfg *cfg, aclz_decode_cfg &c) {
+// Checks cfg and resolves ACLZ_MODE_AUTO for this handle; phase: an event is
+// recorded between the phases.
+int resolve_cfg(const aclz_handle *h, const aclz_decode_cfg *cfg, bool phase, aclz_decode_cfg &c) {
     c = {32, ACLZ_MODE_AUTO, 0, 0};
     if (cfg) c = *cfg;
     if (c.G != 8 && c.G != 16 && c.G != 32) return ACLZ_E_INVAL;
@@ -922,7 +924,8 @@ int resolve_cfg(const aclz_handle *h, const aclz_decode_cfg *cfg, aclz_decode_cf
     if (c.mode == ACLZ_MODE_AUTO) {
         // long deferred matches: one persistent launch with TMA staging;
         // short ones: by levels (or waves)
-        c.mode = decodes_as_waves(h) ? ACLZ_MODE_WAVES : ACLZ_MODE_PERSISTENT;
+        const double least = (h->by_level && !phase) || h->flat ? kPersistentMin : kPersistentMinWaves;
+        c.mode = h->mean_deferred_len < least ? ACLZ_MODE_WAVES : ACLZ_MODE_PERSISTENT;
         if (c.mode == ACLZ_MODE_PERSISTENT && !(c.flags & ACLZ_FLAG_REGISTERS)) c.flags |= ACLZ_FLAG_STAGED;
     }
     if ((c.flags & ACLZ_FLAG_STAGED) && (c.flags & ACLZ_FLAG_REGISTERS)) return ACLZ_E_INVAL;
@@ -937,13 +940,13 @@ extern "C" int aclz_decode_plan(const aclz_handle *h, const aclz_decode_cfg *cfg
                                 uint32_t *launches) {
     if (!h) return ACLZ_E_INVAL;
     aclz_decode_cfg c;
-    if (int rc = resolve_cfg(h, cfg, c)) return rc;
+    if (int rc = resolve_cfg(h, cfg, false, c)) return rc;
     uint32_t n = 0;
     if (h->n_blocks) {
         if (c.mode == ACLZ_MODE_PERSISTENT)
             n = (c.flags & ACLZ_FLAG_STAGED) && h->n_levels ? 2 : 1 + h->n_ord_steps + (h->n_ranges ? 1 : 0);
         else
-            n = 1 + (uint32_t)(goes_by_level(h, cfg) ? h->lsteps.size() : h->steps.size());
+            n = 1 + (uint32_t)(goes_by_level(h, cfg, false) ? h->lsteps.size() : h->steps.size());
         if (h->d_ord || h->walk) n++;
     }
     if (resolved) *resolved = c;
@@ -957,7 +960,7 @@ extern "C" int aclz_decode_all_ev(aclz_handle *h, void *d_out, uint64_t cap, con
     if (cap < h->total_len) return ACLZ_E_CAPACITY;
     if (reinterpret_cast<uintptr_t>(d_out) & 15) return ACLZ_E_INVAL;
     aclz_decode_cfg c;
-    if (int rc = resolve_cfg(h, cfg, c)) return rc;
+    if (int rc = resolve_cfg(h, cfg, phase_event != nullptr, c)) return rc;
     if (h->n_blocks == 0) return ACLZ_OK;
     cudaStream_t st = (cudaStream_t)stream;
     cudaEvent_t ev = (cudaEvent_t)phase_event;
@@ -969,10 +972,11 @@ extern "C" int aclz_decode_all_ev(aclz_handle *h, void *d_out, uint64_t cap, con
             default: return launch_persistent_auto<32>(h, out, c, st, ev);
         }
     }
+    const bool by_level = goes_by_level(h, cfg, ev != nullptr);
     switch (c.G) {
-        case 8: return launch_waves<8>(h, out, st, ev, goes_by_level(h, cfg));
-        case 16: return launch_waves<16>(h, out, st, ev, goes_by_level(h, cfg));
-        default: return launch_waves<32>(h, out, st, ev, goes_by_level(h, cfg));
+        case 8: return launch_waves<8>(h, out, st, ev, by_level);
+        case 16: return launch_waves<16>(h, out, st, ev, by_level);
+        default: return launch_waves<32>(h, out, st, ev, by_level);
     }
 }
 

@@ -87,13 +87,19 @@ int build_levels(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlv
 int build_steps(aclz_handle *h, void *stream);
 void free_wave0(aclz_handle *h, void *stream);
 
-// Deferred matches of at least this mean length are decoded by the
-// persistent schedule under ACLZ_MODE_AUTO, shorter ones by levels (or waves),
-// one kernel each: 1 GiB copy sweep at L = 384 / 512 / 768 / 1000 873 / 717 /
-// 639 / 570 us persistent and 794 / 665 / 617 / 580 us by level kernels (64 MiB
-// at L = 900 136 and 115 us): they meet at a kilobyte.
+// Deferred matches of at least this mean length are decoded by the persistent
+// schedule under ACLZ_MODE_AUTO, shorter ones by levels (or, of a flattened
+// handle, as one wave), one kernel each: 1 GiB copy sweep at L = 384 / 512 /
+// 768 / 1000 873 / 717 / 639 / 570 us persistent and 794 / 665 / 617 / 580 us
+// by level kernels, which meet at a kilobyte; at 64 MiB the level kernels are
+// ahead at L = 900 too (115 us, 136 us persistent).
 constexpr double kPersistentMin = 1024.0;
-bool decodes_as_waves(const aclz_handle *h);
+// The same where the deferred matches go by waves: no levels (chains too deep
+// or too narrow for them), or an event between the phases.  600 blocks of
+// 16 KiB, each copied from the one before at L = 256: 3.2 ms by waves, 1.9 ms
+// by ranges; 16 MiB copy sweep at L = 512 with the event: 411 us by waves, 108
+// us by levels in the persistent launch (it has no in-order matches).
+constexpr double kPersistentMinWaves = 192.0;
 
 // A handle's status array: the status word and, on a line of its own, the
 // count of the grid barrier.
@@ -215,4 +221,3 @@ struct aclz_handle {
     uint64_t n_matches_deferred = 0;  // deferred matches before flattening
 };
 
-inline bool aclz::decodes_as_waves(const aclz_handle *h) { return h->mean_deferred_len < kPersistentMin; }
