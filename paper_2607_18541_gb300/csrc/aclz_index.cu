@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256) k_index_scan(const uint4 *__restrict__ to
                                                     uint64_t n_cells, uint32_t log2c, uint64_t nt, uint32_t nb,
                                                     uint32_t log2bs, uint64_t total, int has_tags,
                                                     uint32_t *err, unsigned long long *first_bad,
-                                                    long long *near_matches) {
+                                                    long long *near_matches, uint32_t *crosses) {
     Group<32> g;
     const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (b >= nb) return;
@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(256) k_index_scan(const uint4 *__restrict__ to
     const uint64_t blen = min((uint64_t)1 << log2bs, total - bstart);
     uint64_t carry = 0, lcarry = 0;
     int near = 0;  // matches that read the match before them, less the others (of 31 in 32)
-    bool bad = false;
+    bool bad = false, cross = false;  // cross: a source starts in another block
     for (uint64_t w = t0; w < t1; w += 32) {
         const uint64_t i = w + g.lane;
         const bool v = i < t1;
@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(256) k_index_scan(const uint4 *__restrict__ to
         const uint64_t rel = carry + incl - tot;
         const uint64_t lsum = g.scan_incl(lit);
         const uint64_t m1 = g.shfl_up(rel + lit, 1);  // where the match before starts
+        cross = cross || (v && ml && (sw & kSrcMask) < bstart);
         if (v && ml && g.lane)
             near += (sw & kSrcMask) + ml > bstart + m1 && (sw & kSrcMask) < bstart + rel ? 1 : -1;
         if (v) {
@@ -102,6 +103,7 @@ __global__ void __launch_bounds__(256) k_index_scan(const uint4 *__restrict__ to
     }
     if (g.lane == 0 && (carry != blen || blk_lit[b] + lcarry != blk_lit[b + 1])) bad = true;
     if (g.ballot(bad) && g.lane == 0) atomicOr(err, kErrCorrupt);
+    if (g.ballot(cross) && g.lane == 0) *crosses = 1u;
     near = __reduce_add_sync(0xffffffffu, near);
     if (g.lane == 0 && near) atomicAdd((unsigned long long *)near_matches, (unsigned long long)(long long)near);
 }
@@ -828,8 +830,12 @@ int aclz::device_excl_scan(uint32_t *d, uint64_t n, uint32_t *d_total, void *str
 // relaxation passes from zero; d_out[0..2] as k_relax leaves them.  A stream
 // whose copy chains are deeper than kRelaxMax (d_out[2] = 0) is left to the
 // ordered pass; so is one whose cover list does not fit.
+// Without a match that reads another block every tag is 0, and with
+// kRelaxBlocks blocks or more the in-order levels are found faster block by
+// block (256 blocks of 16 KiB with 102 levels: upload 1509 -> 401 us; a single
+// block of 16 MiB and 505 levels takes 158 ms by passes, 202 ms by one CTA).
 namespace {
-constexpr uint32_t kRelaxMax = 512;
+constexpr uint32_t kRelaxMax = 512, kRelaxBlocks = 64;
 int relax_levels(aclz_handle *h, unsigned long long *d_val, uint32_t *d_out, cudaStream_t st) {
     const uint32_t nb = h->n_blocks;
     const uint64_t nt = h->n_tokens;
@@ -889,10 +895,10 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     // scratch words, read by the host together: [0] max tag, [1] largest level
     // (then the block counter of k_tags_min), [2] fixed point reached, [3]
     // deferred matches, [4] segments, [5] triplets of the level list, [6]
-    // status; bytes 32..39: first bad token, 40..47: deferred bytes, 48..55:
-    // matches near what they read less the others
+    // status, [7] a match reads another block; bytes 32..39: first bad token,
+    // 40..47: deferred bytes, 48..55: matches near what they read less the others
     struct Words {
-        uint32_t maxtag, maxlvl, reached, deferred, segs, lev, err, pad;
+        uint32_t maxtag, maxlvl, reached, deferred, segs, lev, err, crosses;
         unsigned long long first_bad, def_bytes;
         long long near, pad2;
     } hw;
@@ -913,7 +919,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     k_index_scan<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_blk_lit, h->d_tokdst,
                                            h->d_toklit, h->d_cell, h->n_cells, h->log2_cell, nt, nb, h->log2_bs,
                                            h->total_len, has_tags, h->d_err,
-                                           d_first_bad, (long long *)(d_first_bad + 2));
+                                           d_first_bad, (long long *)(d_first_bad + 2), d_maxtag + 7);
     CK(cudaGetLastError());
     CK(read_words());
     if (hw.err) { cleanup(); return ACLZ_E_CORRUPT; }
@@ -943,7 +949,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         k_tags_local<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, d_tags, nb,
                                                h->log2_bs, d_maxtag);
         k_store_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_tags, nt);
-    } else if (!chained) {
+    } else if (!chained && (hw.crosses || nb < kRelaxBlocks)) {
         rc = relax_levels(h, d_val, d_maxtag, st);
         if (rc) { cleanup(); return rc; }
         k_store_val_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_val, nt, d_maxtag + 2);
@@ -952,7 +958,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     CK(read_words());
     if (hw.reached) {
         levels = true;
-    } else if (!has_tags && !flat_up) {  // chains too deep for the passes (or too narrow)
+    } else if (!has_tags && !flat_up && hw.crosses) {  // chains too deep for the passes (or too narrow)
         CK(cudaMemsetAsync(d_maxtag, 0, 8, st));
         CK(done.alloc(4 * nb, st));
         CK(cudaMemsetAsync(done.p, 0, 4 * nb, st));
@@ -982,9 +988,12 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     // per-block wave bitmasks, quadratic in the chain depth; beyond 2^28
     // cells the upload builds the flattened two-wave schedule instead.
     h->needs_flatten = maxtag > 0 && (uint64_t)maxtag * nb > (1ULL << 28);
-    // the schedule by levels; a container with tags of its own has its levels
-    // found here
-    const bool by_level = !flat_up && !h->needs_flatten && !chained;
+    // The schedule by levels; a container with tags of its own has its levels
+    // found here.  Without deferred matches there is nothing for it to join:
+    // the in-order levels by block take less (1024 blocks of 64 KiB with 64
+    // levels each 351 -> 190 us, 256 blocks of 16 KiB with 102 levels 299 -> 75
+    // us, one launch a level and one over the blocks).
+    const bool by_level = !flat_up && !h->needs_flatten && !chained && maxtag > 0;
     if (by_level && has_tags) {
         rc = relax_levels(h, d_val, d_maxtag, st);
         if (rc) { cleanup(); return rc; }

@@ -125,3 +125,9 @@ def test_chain_of_all_lengths(top, cross):
                        np.array(sr, dtype=np.uint64), r.randint(0, 256, int(ll.sum())).astype(np.uint8))
     assert oracle.validate(c) == 0
     _decode_all_ways(c, (None, None))
+
+
+@pytest.mark.parametrize("nb,bs,ln,width", [(9, 4096, 20, 8), (300, 16384, 20, 8), (4, 1 << 16, 16, 64), (5, 1024, 16, 12)])
+def test_in_order_levels_without_deferred_matches(nb, bs, ln, width):
+    # 4 to 102 levels: by block in one launch, in the plain handle too
+    _decode_all_ways(_chains(nb, bs, ln, width, 5), (1, 1))
