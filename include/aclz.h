@@ -316,8 +316,9 @@ int aclz_decode_all_ev(aclz_handle *h, void *d_out, uint64_t cap, const aclz_dec
 /* What aclz_decode_all would launch for this handle and cfg (no GPU work):
  * *resolved = cfg with ACLZ_MODE_AUTO resolved and the copy-path flag set;
  * *launches = kernel launches of one call: the literal kernel, then for
- * ACLZ_MODE_AUTO by levels one per level; else one per level of in-order
- * matches, or one for all of them by block where the handle lists them so
+ * ACLZ_MODE_AUTO by levels one per level (one for a run of eight or more
+ * levels of at most 64 matches); else one per level of in-order
+ * matches, or one for all of them by block where the handle lists or walks them so
  * (none in most streams without short distances; in the staged persistent
  * launch where it runs levels of both kinds) and one persistent launch or one
  * per non-empty wave >= 1; 0 for an empty stream.  Either output may be NULL.  ACLZ_E_INVAL for a bad cfg, as aclz_decode_all. */

@@ -53,6 +53,8 @@ constexpr int kLevelThreads = 128, kLevelMinCtas = 9;
 constexpr uint32_t kStageWarp = 3584, kStageWarpLong = 6144;
 constexpr double kStageLongMin = 224.0;
 constexpr uint64_t kLevelQuarter = 40000, kLevelEighth = 20000, kLevelOne = 5000;
+// runs of narrow levels: CTA size
+constexpr int kRunThreads = 512;
 // in-order levels by block: CTA size, and the same for blocks below kOrdSmall
 // bytes (16 MiB of text flattened, 4 KiB blocks: 118 us with 128 threads,
 // 131 us with 512; 32 MiB, 64 KiB blocks: 225 and 213 us); the length above
@@ -476,6 +478,37 @@ __global__ void __launch_bounds__(kLevelThreads, kLevelMinCtas)
     group_copy_staged<G, J>(g, st, out, tri_dst(t), out + tri_src(t), tri_len(t), err);
 }
 
+// A run of narrow levels by one CTA: a group takes a match or a few, loads the
+// next level's while it copies, and a barrier of the CTA ends the level.
+//
+// Bound by a level's chain of L2 load, store and barrier (0.5 us for a match of
+// 64 bytes), which a launch of its own makes 1.7 us: 16 MiB of FASTQ-like text
+// with 24 KiB of zeros in it (386 levels, 360 of them of one or two matches)
+// 630 -> 228 us, 1024 levels of 64 matches 1654 -> 806 us.
+template <int G>
+__global__ void __launch_bounds__(kRunThreads, 1) k_level_run(const Step *__restrict__ steps, uint32_t count,
+                                                              uint8_t *out) {
+    Group<G> g;
+    griddep_launch_dependents();
+    constexpr uint32_t kGroups = kRunThreads / G;
+    const uint32_t gi = threadIdx.x / G;
+    const ulonglong2 *list = reinterpret_cast<const ulonglong2 *>(steps);
+    auto window = [&](const ulonglong2 &s) {
+        const uint32_t n = (uint32_t)s.y, per = (n + kGroups - 1) / kGroups, i = gi * per + (uint32_t)g.lane;
+        return (uint32_t)g.lane < per && i < n ? __ldg(reinterpret_cast<const uint4 *>(s.x) + i) : make_uint4(0, 0, 0, 0);
+    };
+    uint4 next = window(__ldg(list));
+    ulonglong2 after = count > 1 ? __ldg(list + 1) : make_ulonglong2(0, 0);
+    griddep_wait();
+    for (uint32_t k = 0; k < count; k++) {
+        const uint4 t = next;
+        next = window(after);
+        after = k + 2 < count ? __ldg(list + k + 2) : make_ulonglong2(0, 0);
+        group_copy_batch<G, kUnrollCopy>(g, out, tri_dst(t), out + tri_src(t), tri_len(t));
+        __syncthreads();
+    }
+}
+
 // Every level in one cooperative launch.  A level's matches are dealt out
 // evenly, at most G / 2 per group at a time, through the group's two stages
 // in turn; the next level's first window is loaded before the barrier.
@@ -677,18 +710,39 @@ int launch_step(void (*k)(P...), uint64_t n, unsigned per_cta, unsigned threads,
     return ACLZ_OK;
 }
 
-// Levels: one kernel each, fewer matches per group in the small ones, whose
+// Levels from `first` on that go in one launch as a run of narrow ones (0: the
+// level goes by itself).
+uint32_t narrow_run(const std::vector<Step> &levels, uint32_t first, uint32_t count, const void *d_steps) {
+    uint32_t e = first;
+    while (d_steps && e < count && levels[e].n <= kRunMost) e++;
+    return e - first >= kRunMin ? e - first : 0;
+}
+
+// Launches of launch_levels.
+uint32_t level_launches(const std::vector<Step> &levels, uint32_t count, const void *d_steps) {
+    uint32_t n = 0;
+    for (uint32_t i = 0; i < count; i += std::max(1u, narrow_run(levels, i, count, d_steps))) n++;
+    return n;
+}
+
+// Levels: one kernel each (runs of narrow ones one kernel together), fewer matches per group in the small ones, whose
 // groups are all resident at once and take as long as their own window.  Up
 // to kLevelOne (about the warps resident at a time) a group takes one match:
 // 64 MiB copy sweep at L = 900 137 -> 115 us, 256 KiB of Markov bytes 38.5 ->
 // 36 us, 64 MiB of FASTQ-like text 120 -> 116 us; up to 20000 instead the
 // 512 MiB sweep at L = 128 goes from 756 to 780 us.
 template <int G>
-int launch_levels(const aclz_handle *h, const std::vector<Step> &levels, uint32_t count, uint8_t *out,
-                  cudaStream_t st) {
+int launch_levels(const aclz_handle *h, const std::vector<Step> &levels, uint32_t count, const void *d_steps,
+                  uint8_t *out, cudaStream_t st) {
     const uint32_t stage = (h->mean_deferred_len >= kStageLongMin ? kStageWarpLong : kStageWarp) / 32 * G;
     constexpr int gpc = kLevelThreads / G;
     for (uint32_t i = 0; i < count; i++) {
+        if (const uint32_t run = narrow_run(levels, i, count, d_steps)) {
+            if (int rc = launch_step(k_level_run<G>, 1, 1, kRunThreads, 0, st, (const Step *)d_steps + i, run, out))
+                return rc;
+            i += run - 1;
+            continue;
+        }
         const uint64_t n = levels[i].n;
         const int part = n <= kLevelOne ? G : n <= kLevelEighth ? 8 : n <= kLevelQuarter ? 4 : 2;
         auto k = part == G ? k_level<G, 1> : part == 8 ? k_level<G, G / 8> : part == 4 ? k_level<G, G / 4> : k_level<G, G / 2>;
@@ -706,7 +760,7 @@ int launch_order(const aclz_handle *h, uint8_t *out, cudaStream_t st) {
     if (h->walk)
         return launch_step(k_ord_walk<G>, h->n_blocks, kWaveThreads / G, kWaveThreads, 0, st, (const uint4 *)h->d_tok,
                            h->d_blk_tok, h->d_tokdst, out, h->n_blocks, h->log2_bs);
-    if (!h->d_ord) return launch_levels<G>(h, h->steps, h->n_ord_steps, out, st);
+    if (!h->d_ord) return launch_levels<G>(h, h->steps, h->n_ord_steps, h->d_steps, out, st);
     const size_t smem = std::max<size_t>(h->block_size, 16);
     // the attribute is the largest any call needs, the same on every call
     if (cudaError_t e = cudaFuncSetAttribute(k_ord_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize, 1 << 17);
@@ -749,7 +803,7 @@ int launch_lits(aclz_handle *h, uint8_t *out, cudaStream_t st, bool ranges, bool
 template <int G>
 int launch_waves(aclz_handle *h, uint8_t *out, cudaStream_t st, cudaEvent_t phase, bool by_level) {
     if (int rc = launch_lits<G>(h, out, st, false, false)) return rc;
-    if (by_level) return launch_levels<G>(h, h->lsteps, (uint32_t)h->lsteps.size(), out, st);
+    if (by_level) return launch_levels<G>(h, h->lsteps, (uint32_t)h->lsteps.size(), h->d_lsteps, out, st);
     if (int rc = launch_order<G>(h, out, st)) return rc;
     if (phase) cudaEventRecord(phase, st);
     return launch_wave_steps<G>(h, out, st);
@@ -943,10 +997,13 @@ extern "C" int aclz_decode_plan(const aclz_handle *h, const aclz_decode_cfg *cfg
     if (int rc = resolve_cfg(h, cfg, false, c)) return rc;
     uint32_t n = 0;
     if (h->n_blocks) {
+        const uint32_t order = level_launches(h->steps, h->n_ord_steps, h->d_steps);
         if (c.mode == ACLZ_MODE_PERSISTENT)
-            n = (c.flags & ACLZ_FLAG_STAGED) && h->n_levels ? 2 : 1 + h->n_ord_steps + (h->n_ranges ? 1 : 0);
+            n = (c.flags & ACLZ_FLAG_STAGED) && h->n_levels ? 2 : 1 + order + (h->n_ranges ? 1 : 0);
+        else if (goes_by_level(h, cfg, false))
+            n = 1 + level_launches(h->lsteps, (uint32_t)h->lsteps.size(), h->d_lsteps);
         else
-            n = 1 + (uint32_t)(goes_by_level(h, cfg, false) ? h->lsteps.size() : h->steps.size());
+            n = 1 + order + (uint32_t)h->steps.size() - h->n_ord_steps;
         if (h->d_ord || h->walk) n++;
     }
     if (resolved) *resolved = c;

@@ -111,6 +111,11 @@ struct Step {
     uint64_t tri, n;
 };
 
+// Levels of at most kRunMost matches are narrow; kRunMin or more of them in a
+// row go in one launch, by one CTA.
+constexpr uint64_t kRunMost = 64;
+constexpr uint32_t kRunMin = 8;
+
 // Decode index of h from its device tokens (validation, offsets, wave tags,
 // worklists, schedule); see aclz_index.cu.
 int build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool flat_local, void *stream);
@@ -187,6 +192,8 @@ struct aclz_handle {
     void *d_levels = nullptr;
     uint32_t n_levels = 0;
     uint32_t n_ord_steps = 0;
+    // the two lists on the device, where they hold runs of narrow levels
+    void *d_steps = nullptr, *d_lsteps = nullptr;
     // persistent-mode schedule.  A segment is the run of one block's
     // matches in one wave's worklist: seg[s] = {block, wave, triplet offset,
     // count}, wave-major then block order.  A range is a run of consecutive

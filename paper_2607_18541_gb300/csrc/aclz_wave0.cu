@@ -289,7 +289,8 @@ int build_ord_blocks(aclz_handle *h, cudaStream_t st) {
 
 void aclz::free_wave0(aclz_handle *h, void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
-    for (void **pp : {&h->d_lunits, &h->d_lev, &h->d_levels, &h->d_ord, (void **)&h->d_ord_base}) {
+    for (void **pp : {&h->d_lunits, &h->d_lev, &h->d_levels, &h->d_ord, (void **)&h->d_ord_base, &h->d_steps,
+                      &h->d_lsteps}) {
         dev_free(*pp, st);
         *pp = nullptr;
     }
@@ -368,6 +369,26 @@ int aclz::build_levels(aclz_handle *h, const unsigned long long *d_val, uint32_t
     return ACLZ_OK;
 }
 
+namespace {
+
+// The first count steps on the device, when they hold a run of narrow levels.
+// Without memory for them every level is a launch.
+int copy_runs(const std::vector<Step> &v, uint32_t count, void **d, cudaStream_t st) {
+    dev_free(*d, st);
+    *d = nullptr;
+    uint32_t run = 0, most = 0;
+    for (uint32_t i = 0; i < count; i++) {
+        run = v[i].n <= kRunMost ? run + 1 : 0;
+        most = std::max(most, run);
+    }
+    if (most < kRunMin) return ACLZ_OK;
+    if (cudaError_t e = dev_alloc(d, sizeof(Step) * count, st); e != cudaSuccess)
+        return e == cudaErrorMemoryAllocation ? ACLZ_OK : rc_of(e);
+    return rc_of(cudaMemcpyAsync(*d, v.data(), sizeof(Step) * count, cudaMemcpyHostToDevice, st));
+}
+
+}  // namespace
+
 int aclz::build_steps(aclz_handle *h, void *stream) {
     cudaStream_t st = (cudaStream_t)stream;
     h->steps.clear();
@@ -389,6 +410,8 @@ int aclz::build_steps(aclz_handle *h, void *stream) {
     h->n_ord_steps = (uint32_t)h->steps.size();
     for (uint32_t w = 1; w < h->n_waves && h->d_tri; w++)
         add(h->steps, h->d_tri, h->wave_start[w], h->wave_start[w + 1]);
+    if (int rc = copy_runs(h->steps, h->n_ord_steps, &h->d_steps, st)) return rc;
+    if (int rc = copy_runs(h->lsteps, (uint32_t)h->lsteps.size(), &h->d_lsteps, st)) return rc;
     dev_free(h->d_levels, st);
     h->d_levels = nullptr;
     const std::vector<Step> &list = h->by_level ? h->lsteps : h->steps;

@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 import oracle
-from paper_2607_18541_gb300 import aclz
+from paper_2607_18541_gb300 import aclz, synth
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -131,3 +131,57 @@ def test_chain_of_all_lengths(top, cross):
 def test_in_order_levels_without_deferred_matches(nb, bs, ln, width):
     # 4 to 102 levels: by block in one launch, in the plain handle too
     _decode_all_ways(_chains(nb, bs, ln, width, 5), (1, 1))
+
+
+def _narrow(runs, seed):
+    """Levels of the given numbers of matches, each match reading one of the
+    level before: in-order chains in blocks of their own and, from block to
+    block, deferred ones.  Many literal blocks with far matches go first, so
+    that most matches are not near what they read."""
+    r = np.random.RandomState(seed)
+    bs, blocks, lits = 1 << 12, [[(1 << 12, 0, 0)]], 0
+    for _ in range(12):
+        at = len(blocks) * bs
+        blocks.append([(8, 8, int(r.randint(0, bs - 8))) for _ in range(bs // 16)])
+    prev = [(0, bs)]  # (place, bytes) of what the next level may read
+    for w in runs:
+        place, toks, here = len(blocks) * bs, [], []
+        for k in range(w):
+            n = int(r.choice([1 if k else 9, 7, 16, 33, 64, 130]))
+            a, m = prev[int(r.randint(len(prev)))]
+            n = min(n, m)
+            p = place + sum(t[0] + t[1] for t in toks)
+            if p + n + 8 > place + bs:
+                break
+            toks.append((int(r.randint(0, 3)), n, a + int(r.randint(0, m - n + 1))))
+            here.append((p + toks[-1][0], n))
+        toks.append((place + bs - place - sum(t[0] + t[1] for t in toks), 0, 0))
+        blocks.append(toks)
+        prev = [x for x in here if x[1] > 6]
+    ll = np.array([t[0] for b in blocks for t in b], dtype=np.uint32)
+    ml = np.array([t[1] for b in blocks for t in b], dtype=np.uint32)
+    sr = np.array([t[2] for b in blocks for t in b], dtype=np.uint64)
+    return aclz.aclz_pack(len(blocks) * bs, bs, (4, 4, 4, 4), np.array([len(b) for b in blocks], dtype=np.uint32), ll, ml,
+                          sr, r.randint(0, 256, int(ll.sum())).astype(np.uint8))
+
+
+@pytest.mark.parametrize("seed,runs", [(1, [1] * 7), (2, [1] * 8), (3, [1, 2, 3, 64, 64, 1, 63, 5, 40, 17]),
+                                       (4, [65] * 3 + [1] * 40 + [70] * 2 + [33] * 9 + [66] + [16] * 7)])
+def test_runs_of_narrow_levels(seed, runs):
+    c = _narrow(runs, seed)
+    assert oracle.validate(c) == 0
+    _decode_all_ways(c, (None, None))
+
+
+def test_launches_of_a_narrow_run():
+    # a run of zeros in text: hundreds of levels of a match or two
+    x = synth.wordtext(1 << 20, seed=3)
+    x[300000:300000 + (20 << 10)] = 0
+    c = _encode(x, 16 << 10, (6, 8, 10, 12))
+    h = aclz.aclz_upload(c, torch.cuda.current_stream())
+    try:
+        assert 2 < aclz.aclz_decode_plan(h)[1] < 130
+        assert aclz.aclz_decode_plan(h, mode=WAVES)[1] < 200
+    finally:
+        aclz.aclz_free(h)
+    _decode_all_ways(c, (None, None))
