@@ -371,6 +371,17 @@ int aclz::build_levels(aclz_handle *h, const unsigned long long *d_val, uint32_t
 
 namespace {
 
+// Whether the staged persistent launch is left to the work ranges: many narrow
+// levels, three quarters of all or more.  Its grid barrier makes each of them
+// take 2 us (16 MiB of FASTQ-like text with 24 KiB of zeros in it, 380 narrow
+// levels of 386: 792 us by levels, 228 us by ranges; 4 MiB of word text with
+// the zeros, 240 of 387: 965 and 1404 us).
+constexpr uint32_t kNarrowMost = 64;
+bool mostly_narrow(const std::vector<Step> &v) {
+    const size_t n = std::count_if(v.begin(), v.end(), [](const Step &s) { return s.n <= kRunMost; });
+    return n > kNarrowMost && 4 * n >= 3 * v.size();
+}
+
 // The first count steps on the device, when they hold a run of narrow levels.
 // Without memory for them every level is a launch.
 int copy_runs(const std::vector<Step> &v, uint32_t count, void **d, cudaStream_t st) {
@@ -418,6 +429,7 @@ int aclz::build_steps(aclz_handle *h, void *stream) {
     h->n_levels = h->by_level || h->flat ? (uint32_t)list.size() : 0;
     for (const Step &x : list)
         if (x.n >= 1ULL << 31) h->n_levels = 0;  // the kernel over them counts in 32 bits
+    if (mostly_narrow(list)) h->n_levels = 0;
     if (!h->n_levels) return rc_of(cudaStreamSynchronize(st));
     W0CK(dev_alloc(&h->d_levels, sizeof(Step) * list.size(), st));
     W0CK(cudaMemcpyAsync(h->d_levels, list.data(), sizeof(Step) * list.size(), cudaMemcpyHostToDevice, st));

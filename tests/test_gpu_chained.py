@@ -185,3 +185,16 @@ def test_launches_of_a_narrow_run():
     finally:
         aclz.aclz_free(h)
     _decode_all_ways(c, (None, None))
+
+
+def test_staged_launch_with_mostly_narrow_levels():
+    # it goes by ranges, after the in-order levels in launches of their own
+    x = synth.fastq(4 << 20, seed=3)
+    x[300000:300000 + (20 << 10)] = 0
+    c = _encode(x, 16 << 10, (12, 16, 24, 32))
+    h = aclz.aclz_upload(c, torch.cuda.current_stream())
+    try:
+        assert aclz.aclz_decode_plan(h, mode=PERSISTENT, flags=aclz.ACLZ_FLAG_STAGED)[1] > 2
+    finally:
+        aclz.aclz_free(h)
+    _decode_all_ways(c, (None, None))
