@@ -577,8 +577,7 @@ __global__ void __launch_bounds__(kPersThreads, kPersCtas)
 // Every in-order level of one block per CTA, in shared memory: the block comes
 // in as the literal copies left it, a level's matches are copied by one thread
 // each (longer ones by their warp), and the block goes out again, bytes of
-// deferred matches as they were.  Bytes of another block that a match reads
-// are literals.
+// deferred matches as they were.  An in-order match reads its own block only.
 //
 // Bound by the latency of a level's barrier, shared loads and narrow shared
 // stores, not by bytes.  With one kernel per level (about 3 us each)
@@ -615,22 +614,9 @@ __global__ void __launch_bounds__(kOrdThreads)
         next = at(w + nt + tid);
         const uint32_t mine = w + tid < o1 ? t.y >> 9 : 0xffffffffu;
         const uint32_t l1 = __ldg(&ord[min(w + nt, o1) - 1].y) >> 9;
-        uint32_t d = (uint32_t)(tri_dst(t) - bpos), n = tri_len(t);
-        const uint64_t src = tri_src(t);
+        const uint32_t d = (uint32_t)(tri_dst(t) - bpos), s = (uint32_t)(tri_src(t) - bpos), n = tri_len(t);
         for (uint32_t l = __ldg(&ord[w].y) >> 9; l <= l1; l++) {
             const bool go = mine == l;
-            uint32_t s = (uint32_t)(src - bpos);
-            if (go && src < bpos) {  // from the blocks before
-                uint64_t a = src;
-                while (n && a < bpos) {
-                    const uint32_t m = (uint32_t)min((uint64_t)min(n, 16u), bpos - a);
-                    store_bytes(gbase + d, load_bytes<kFromL2>(reinterpret_cast<uintptr_t>(out) + a, m), m);
-                    a += m;
-                    d += m;
-                    n -= m;
-                }
-                s = (uint32_t)(a - bpos);
-            }
             if (go && n <= kOrdLong)
                 for (uint32_t k = 0; k < n; k += 16) piece(d + k, s + k, min(n - k, 16u));
             for (unsigned m = __ballot_sync(0xffffffffu, go && n > kOrdLong); m; m &= m - 1) {
