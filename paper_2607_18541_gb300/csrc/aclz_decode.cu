@@ -582,7 +582,9 @@ __global__ void __launch_bounds__(kPersThreads, kPersCtas)
 // Bound by the latency of a level's barrier, shared loads and narrow shared
 // stores, not by bytes.  With one kernel per level (about 3 us each)
 // 32 MiB of word text at 6/8/10/12, flattened, took 250 us and takes 213 us,
-// 256 KiB of it 69 and 32 us, 16 MiB of FASTQ-like text 55 and 37 us.
+// 256 KiB of it 69 and 32 us, 16 MiB of FASTQ-like text 55 and 37 us (with 24
+// KiB of zeros in it, a chain of 256 matches of 64 bytes, 216 us when one
+// thread copied each whole, 113 us now).
 __global__ void __launch_bounds__(kOrdThreads)
     k_ord_blocks(const uint4 *__restrict__ ord, const uint32_t *__restrict__ base, uint8_t *out, uint32_t log2bs,
                  uint64_t total) {
@@ -617,9 +619,17 @@ __global__ void __launch_bounds__(kOrdThreads)
         const uint32_t d = (uint32_t)(tri_dst(t) - bpos), s = (uint32_t)(tri_src(t) - bpos), n = tri_len(t);
         for (uint32_t l = __ldg(&ord[w].y) >> 9; l <= l1; l++) {
             const bool go = mine == l;
-            if (go && n <= kOrdLong)
+            // the warp shares its matches longer than kOrdLong, or its only one
+            // longer than half of that; a thread copies the others piece by piece
+            unsigned big = __ballot_sync(0xffffffffu, go && n > kOrdLong / 2);
+            uint32_t alone = kOrdLong / 2;
+            if (big & (big - 1u)) {
+                big = __ballot_sync(0xffffffffu, go && n > kOrdLong);
+                alone = kOrdLong;
+            }
+            if (go && n <= alone)
                 for (uint32_t k = 0; k < n; k += 16) piece(d + k, s + k, min(n - k, 16u));
-            for (unsigned m = __ballot_sync(0xffffffffu, go && n > kOrdLong); m; m &= m - 1) {
+            for (unsigned m = big; m; m &= m - 1) {
                 const int j = __ffs(m) - 1;
                 const uint32_t dj = __shfl_sync(0xffffffffu, d, j), sj = __shfl_sync(0xffffffffu, s, j),
                                nj = __shfl_sync(0xffffffffu, n, j);

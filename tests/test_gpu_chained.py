@@ -198,3 +198,31 @@ def test_staged_launch_with_mostly_narrow_levels():
     finally:
         aclz.aclz_free(h)
     _decode_all_ways(c, (None, None))
+
+
+@pytest.mark.parametrize("width", [1, 2, 3, 4, 33])
+@pytest.mark.parametrize("ln", [15, 16, 17, 47, 64, 65])
+def test_few_matches_of_a_level_by_block(width, ln):
+    # levels of `width` matches in a block held in shared memory, one warp's
+    # matches or several warps', short and longer ones among them; a match
+    # reads two levels back, so that most are not near what they read
+    r = np.random.RandomState(width + ln)
+    bs, nb = 1 << 14, 4
+    lit0 = 3 * ln * width + 40
+    ll, ml, sr, nt = [], [], [], []
+    for b in range(nb):
+        at = b * bs
+        p, k = at + lit0, 0
+        while p + 200 < at + bs:
+            n = ln if k % 3 else int(r.randint(1, ln + 1))
+            back = ln * (width + 1) + int(r.randint(0, ln))
+            ll.append(lit0 if k == 0 else 0), ml.append(n), sr.append(p - back - n)
+            p += n
+            k += 1
+        ll.append(at + bs - p), ml.append(0), sr.append(0)
+        nt.append(k + 1)
+    ll = np.array(ll, dtype=np.uint32)
+    c = aclz.aclz_pack(nb * bs, bs, (4, 4, 4, 4), np.array(nt, dtype=np.uint32), ll, np.array(ml, dtype=np.uint32),
+                       np.array(sr, dtype=np.uint64), r.randint(0, 256, int(ll.sum())).astype(np.uint8))
+    assert oracle.validate(c) == 0
+    _decode_all_ways(c, (1, 1))
