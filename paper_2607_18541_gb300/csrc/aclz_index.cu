@@ -442,10 +442,57 @@ __global__ void __launch_bounds__(kRelaxThreads, kRelaxCtas)
     if (blockIdx.x == 0 && threadIdx.x == 0) out[2] = pass <= most;
 }
 
+// One pass of the same over blocks: every match's tag is raised to its
+// requirement under the current tags (read as other warps leave them), one
+// warp per block in token order, so that a chain inside a block settles in few
+// passes however long it is.  The tags start anywhere between zero and the
+// least fixed point; a pass that raises nothing (*changed stays 0) proves it
+// reached.  *maxtag: the largest tag.
+__global__ void __launch_bounds__(256) k_tags_relax(const uint4 *__restrict__ tok,
+                                                    const uint64_t *__restrict__ blk_tok,
+                                                    const uint32_t *__restrict__ tokdst, uint32_t *tags, uint32_t nb,
+                                                    uint32_t log2bs, uint64_t n_tok, uint32_t *changed,
+                                                    uint32_t *maxtag) {
+    Group<32> g;
+    const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (b >= nb) return;
+    const uint64_t t1 = blk_tok[b + 1];
+    uint32_t mx = 0;
+    bool raised = false;
+    for (uint64_t w = blk_tok[b]; w < t1; w += 32) {
+        const uint64_t i = w + g.lane;
+        if (i < t1) {
+            const uint4 t = __ldg(tok + i);
+            if (t.y) {
+                const uint64_t src = ((uint64_t)t.z | ((uint64_t)t.w << 32)) & kSrcMask;
+                bool inwin = false;
+                const uint32_t req = match_requirement(tok, blk_tok, tokdst, tags, src, t.y, b, log2bs, n_tok, n_tok,
+                                                       &inwin);
+                const uint32_t cur = __ldcg(tags + i);
+                if (req > cur) {
+                    __stcg(tags + i, req);
+                    raised = true;
+                }
+                mx = max(mx, max(req, cur));
+            }
+        }
+        g.sync();
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (g.ballot(raised) && g.lane == 0) *changed = 1u;
+    if (g.lane == 0 && mx) atomicMax(maxtag, mx);
+}
+
 __global__ void k_extract_tags(const uint4 *__restrict__ tok, uint32_t *tags, uint64_t n) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
          i += (uint64_t)gridDim.x * blockDim.x)
         tags[i] = __ldg(tok + i).w >> 8;
+}
+
+__global__ void k_val_tags(const unsigned long long *__restrict__ val, uint32_t *__restrict__ tags, uint64_t n) {
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
+         i += (uint64_t)gridDim.x * blockDim.x)
+        tags[i] = (uint32_t)val[i];
 }
 
 // tags of the values into the tokens, when *reached
@@ -859,6 +906,39 @@ int relax_levels(aclz_handle *h, unsigned long long *d_val, uint32_t *d_out, cud
     void *args[] = {&c, &tok, &n, &most, &d_val, &s, &d_out};
     return cuda_rc(cudaLaunchCooperativeKernel((const void *)k_relax, dim3(grid), dim3(kRelaxThreads), args, 0, st));
 }
+// Minimal tags from a lower bound of them in d_tags by passes over blocks,
+// looked at every kBlockBatch passes; *reached when one raised nothing within
+// kBlockPasses.
+//
+// Where k_relax stops short.  It takes a pass for every level of the longest
+// chain, this about one for every wave; the ordered pass (k_tags_min) takes
+// the blocks one after another.  128 MiB of word text at 6/8/10/12 in blocks of
+// 1 MiB (128 waves, over 512 levels) uploads in 1.03 s by these passes alone,
+// in 4.26 s by k_relax and the ordered pass and in 0.20 s by k_relax and these.  A stream of few tokens takes
+// the ordered pass at once (4096 matches in one chain, 16 blocks: 19 ms by
+// these passes and then it, 9 ms by it), and so does one whose chains mostly
+// go from block to block, for which these passes are as many as k_relax's.
+constexpr uint32_t kBlockBatch = 8, kBlockPasses = 512;
+constexpr uint64_t kOrderedTokens = 1u << 17;
+int relax_blocks(aclz_handle *h, uint32_t *d_tags, uint32_t *d_maxtag, bool *reached, cudaStream_t st) {
+    *reached = false;
+    Scratch flags;
+    if (flags.alloc(4 * kBlockBatch, st) != cudaSuccess) return ACLZ_OK;
+    uint32_t *changed = flags.as<uint32_t>(), last = 1;
+    const unsigned wblocks = (h->n_blocks + 7) / 8;
+    for (uint32_t pass = 0; pass < kBlockPasses && last; pass += kBlockBatch) {
+        if (cudaError_t e = cudaMemsetAsync(changed, 0, 4 * kBlockBatch, st); e != cudaSuccess) return cuda_rc(e);
+        for (uint32_t k = 0; k < kBlockBatch; k++)
+            k_tags_relax<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, d_tags,
+                                                   h->n_blocks, h->log2_bs, h->n_tokens, changed + k, d_maxtag);
+        cudaError_t e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&last, changed + kBlockBatch - 1, 4, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return cuda_rc(e);
+    }
+    *reached = !last;
+    return ACLZ_OK;
+}
 }  // namespace
 
 // Decode index of h from its device tokens (d_tok with n_tokens entries,
@@ -934,7 +1014,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     // tags
     // {level, tag} of every token when the passes find them (8 bytes), or
     // plain tags (4 bytes) in the same array
-    Scratch tags, done;
+    Scratch tags, tags2, done;
     CK(tags.alloc(8 * (nt ? nt : 1), st));
     uint32_t *d_tags = (uint32_t *)tags.p;
     unsigned long long *d_val = (unsigned long long *)tags.p;
@@ -960,18 +1040,29 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         levels = true;
     } else if (!has_tags && !flat_up && hw.crosses) {  // chains too deep for the passes (or too narrow)
         CK(cudaMemsetAsync(d_maxtag, 0, 8, st));
-        CK(done.alloc(4 * nb, st));
-        CK(cudaMemsetAsync(done.p, 0, 4 * nb, st));
-        int dev_sms = 0;
-        cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, h->device);
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tags_min, 256, 0);
-        unsigned grid = (unsigned)std::max(1, dev_sms * std::max(1, per_sm));
-        grid = std::min<unsigned>(grid, wblocks);
-        k_tags_min<<<grid, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, d_tags,
-                                          (uint32_t *)done.p, d_ctr, nb, h->log2_bs, nt, d_maxtag,
-                                          h->d_err);
-        k_store_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_tags, nt);
+        bool reached = false;
+        const bool local = 4 * hw.maxtag <= kRelaxMax;  // few waves in those many levels
+        if (!chained && local && nt > kOrderedTokens && tags2.alloc(4 * nt, st) == cudaSuccess) {
+            k_val_tags<<<1024, 256, 0, st>>>(d_val, tags2.as<uint32_t>(), nt);
+            rc = relax_blocks(h, tags2.as<uint32_t>(), d_maxtag, &reached, st);
+            if (rc) { cleanup(); return rc; }
+            if (reached) k_store_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, tags2.as<uint32_t>(), nt);
+            else CK(cudaMemsetAsync(d_maxtag, 0, 8, st));
+        }
+        if (!reached) {
+            CK(done.alloc(4 * nb, st));
+            CK(cudaMemsetAsync(done.p, 0, 4 * nb, st));
+            int dev_sms = 0;
+            cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, h->device);
+            int per_sm = 0;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tags_min, 256, 0);
+            unsigned grid = (unsigned)std::max(1, dev_sms * std::max(1, per_sm));
+            grid = std::min<unsigned>(grid, wblocks);
+            k_tags_min<<<grid, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, d_tags,
+                                              (uint32_t *)done.p, d_ctr, nb, h->log2_bs, nt, d_maxtag,
+                                              h->d_err);
+            k_store_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_tags, nt);
+        }
         CK(cudaGetLastError());
         CK(read_words());
     }
