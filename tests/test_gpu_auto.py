@@ -39,6 +39,11 @@ def test_chains_deeper_than_the_levels(L, persistent):
             assert plan["mode"] == aclz.ACLZ_MODE_PERSISTENT and plan["flags"] == aclz.ACLZ_FLAG_STAGED and n == 2
         else:
             assert plan["mode"] == aclz.ACLZ_MODE_WAVES and n == 600
+        # the container with its tags: the same, without passes for levels
+        t = aclz.aclz_upload(aclz.aclz_export(h), s)
+        assert aclz.aclz_decode_plan(t) == (plan, n)
+        assert np.array_equal(aclz.aclz_tags(t), aclz.aclz_tags(h))
+        aclz.aclz_free(t)
         for G in (32, 16, 8):
             out = torch.zeros(exp.size, dtype=torch.uint8, device="cuda")
             aclz.aclz_decode_all(h, out, G=G, stream=s)
