@@ -876,7 +876,8 @@ int aclz::device_excl_scan(uint32_t *d, uint64_t n, uint32_t *d_total, void *str
 // Levels and minimal wave tags of h's tokens into d_val ({level, tag}) by
 // relaxation passes from zero; d_out[0..2] as k_relax leaves them.  A stream
 // whose copy chains are deeper than kRelaxMax (d_out[2] = 0) is left to the
-// ordered pass; so is one whose cover list does not fit.
+// ordered pass; so is one whose cover list does not fit, and every one
+// when the cooperative launch does not fit the device.
 // Without a match that reads another block every tag is 0, and with
 // kRelaxBlocks blocks or more the in-order levels are found faster block by
 // block (256 blocks of 16 KiB with 102 levels: upload 1509 -> 401 us; a single
@@ -887,11 +888,11 @@ int relax_levels(aclz_handle *h, unsigned long long *d_val, uint32_t *d_out, cud
     const uint32_t nb = h->n_blocks;
     const uint64_t nt = h->n_tokens;
     Scratch state, cover;
-    if (cudaMemsetAsync(d_out, 0, 12, st) != cudaSuccess) return ACLZ_E_CUDA;
-    if (state.alloc(4 * kRelaxState, st) != cudaSuccess || cover.alloc(16 * (nt ? nt : 1), st) != cudaSuccess) return ACLZ_OK;
-    if (cudaMemsetAsync(state.p, 0, 4 * kRelaxState, st) != cudaSuccess ||
+    if (cudaMemsetAsync(d_out, 0, 12, st) != cudaSuccess ||
         cudaMemsetAsync(d_val, 0, 8 * (nt ? nt : 1), st) != cudaSuccess)
         return ACLZ_E_CUDA;
+    if (state.alloc(4 * kRelaxState, st) != cudaSuccess || cover.alloc(16 * (nt ? nt : 1), st) != cudaSuccess) return ACLZ_OK;
+    if (cudaMemsetAsync(state.p, 0, 4 * kRelaxState, st) != cudaSuccess) return ACLZ_E_CUDA;
     k_cover<<<(nb + 7) / 8, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, nb, h->log2_bs, nt,
                                            (uint4 *)cover.p);
     int sms = 0, per_sm = 0;
@@ -904,7 +905,20 @@ int relax_levels(aclz_handle *h, unsigned long long *d_val, uint32_t *d_out, cud
     uint64_t n = nt;
     uint32_t most = kRelaxMax, *s = (uint32_t *)state.p;
     void *args[] = {&c, &tok, &n, &most, &d_val, &s, &d_out};
-    return cuda_rc(cudaLaunchCooperativeKernel((const void *)k_relax, dim3(grid), dim3(kRelaxThreads), args, 0, st));
+    auto launch = [&](unsigned ctas) {
+        return cudaLaunchCooperativeKernel((const void *)k_relax, dim3(ctas), dim3(kRelaxThreads), args, 0, st);
+    };
+    cudaError_t e = launch(grid);
+    if (e == cudaErrorCooperativeLaunchTooLarge && grid > (unsigned)sms) {
+        // fewer co-resident CTAs than the occupancy estimate: one per SM
+        cudaGetLastError();
+        e = launch((unsigned)sms);
+    }
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        return ACLZ_OK;
+    }
+    return cuda_rc(e);
 }
 // Minimal tags from a lower bound of them in d_tags by passes over blocks,
 // looked at every kBlockBatch passes; *reached when one raised nothing within
