@@ -143,7 +143,12 @@ typedef struct aclz_handle aclz_handle;
  * src + match_len <= dst), wave tags (the minimal legal tags when the
  * container has none; a legality check when it has them), and the
  * wave-ordered worklist slots of deferred matches.  Synchronizes the
- * stream.  ACLZ_E_CORRUPT for an invalid container. */
+ * stream.  ACLZ_E_CORRUPT for an invalid container.
+ * Device memory of a handle: the literals, up to 32 bytes per token, 16 per
+ * deferred match and 16 per match for the list of dependency levels; while
+ * it is built up to 56 bytes per match more.  ACLZ_E_NOMEM when what a decode
+ * cannot do without does not fit; without room for the list alone the handle
+ * has none and decodes by waves. */
 int aclz_upload(const void *host_buf, uint64_t n, void *stream, aclz_handle **out);
 
 /* aclz_upload with options.  ACLZ_UPLOAD_FLATTEN: build the two-wave

@@ -1029,7 +1029,11 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     // {level, tag} of every token when the passes find them (8 bytes), or
     // plain tags (4 bytes) in the same array
     Scratch tags, tags2, done;
-    CK(tags.alloc(8 * (nt ? nt : 1), st));
+    const cudaError_t room = tags.alloc(8 * (nt ? nt : 1), st);
+    if (room != cudaSuccess) {
+        if (room != cudaErrorMemoryAllocation) CK(room);
+        CK(tags.alloc(4 * (nt ? nt : 1), st));  // room for plain tags: no levels
+    }
     uint32_t *d_tags = (uint32_t *)tags.p;
     unsigned long long *d_val = (unsigned long long *)tags.p;
     bool levels = false;
@@ -1043,7 +1047,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         k_tags_local<<<wblocks, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, d_tags, nb,
                                                h->log2_bs, d_maxtag);
         k_store_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_tags, nt);
-    } else if (!chained && (hw.crosses || nb < kRelaxBlocks)) {
+    } else if (!chained && room == cudaSuccess && (hw.crosses || nb < kRelaxBlocks)) {
         rc = relax_levels(h, d_val, d_maxtag, st);
         if (rc) { cleanup(); return rc; }
         k_store_val_tags<<<1024, 256, 0, st>>>((uint4 *)h->d_tok, d_val, nt, d_maxtag + 2);
@@ -1056,7 +1060,7 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
         CK(cudaMemsetAsync(d_maxtag, 0, 8, st));
         bool reached = false;
         const bool local = 4 * hw.maxtag <= kRelaxMax;  // few waves in those many levels
-        if (!chained && local && nt > kOrderedTokens && tags2.alloc(4 * nt, st) == cudaSuccess) {
+        if (!chained && room == cudaSuccess && local && nt > kOrderedTokens && tags2.alloc(4 * nt, st) == cudaSuccess) {
             k_val_tags<<<1024, 256, 0, st>>>(d_val, tags2.as<uint32_t>(), nt);
             rc = relax_blocks(h, tags2.as<uint32_t>(), d_maxtag, &reached, st);
             if (rc) { cleanup(); return rc; }
@@ -1100,7 +1104,8 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     // the in-order levels by block take less (1024 blocks of 64 KiB with 64
     // levels each 351 -> 190 us, 256 blocks of 16 KiB with 102 levels 299 -> 75
     // us, one launch a level and one over the blocks).
-    const bool by_level = !flat_up && !h->needs_flatten && !chained && maxtag > 0 && (!has_tags || maxtag < kRelaxMax);
+    const bool by_level = !flat_up && !h->needs_flatten && !chained && maxtag > 0 && room == cudaSuccess &&
+                          (!has_tags || maxtag < kRelaxMax);
     if (by_level && has_tags) {
         rc = relax_levels(h, d_val, d_maxtag, st);
         if (rc) { cleanup(); return rc; }
@@ -1131,13 +1136,14 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     CK(levcnt.alloc(4 * ((uint64_t)nb + 1), st));
     // whether the level list holds every match is known to the device only in
     // a container with tags; it is counted for both there
-    rc = count_levels(h, by_level && !has_tags ? levels : by_level, (uint32_t *)levcnt.p, d_total + 2, st);
+    const bool listed = list_counts_fit(nt, h->total_len);
+    if (listed) rc = count_levels(h, by_level && !has_tags ? levels : by_level, (uint32_t *)levcnt.p, d_total + 2, st);
     if (rc) { cleanup(); return rc; }
     CK(read_words());
     if (by_level && has_tags) {
         levels = hw.reached;
         maxlvl = hw.maxlvl;
-        if (!levels) {  // the in-order matches only
+        if (!levels && listed) {  // the in-order matches only
             rc = count_levels(h, false, (uint32_t *)levcnt.p, d_total + 2, st);
             if (rc) { cleanup(); return rc; }
             CK(read_words());
@@ -1166,19 +1172,32 @@ int aclz::build_index(aclz_handle *h, bool has_tags, uint32_t given_waves, bool 
     }
     rc = build_units(h, stream);
     if (rc) { cleanup(); return rc; }
-    if (chained) {
-        h->walk = hw.lev > 0;
-    } else {
-        rc = build_levels(h, levels ? d_val : nullptr, maxlvl, by_level && levels, (uint32_t *)levcnt.p, hw.lev, stream);
-        if (rc) { cleanup(); return rc; }
-    }
+    std::vector<uint64_t> ones;
     if (!h->d_pending) {  // no deferred matches: wave 0 finishes every block
         h->n_wave_words = 1;
-        std::vector<uint64_t> ones(nb, 1ULL);
+        ones.assign(nb, 1ULL);
         CK(dev_alloc((void **)&h->d_pending, 8 * (size_t)nb, st));
         CK(cudaMemcpyAsync(h->d_pending, ones.data(), 8 * (size_t)nb, cudaMemcpyHostToDevice, st));
     }
     CK(dev_alloc((void **)&h->d_done, 8 * (size_t)nb * h->n_wave_words, st));
+    // The level list comes last: without memory for it (48 bytes a match while
+    // it is built, 16 after) the stream goes by waves and the walk, which need
+    // none.
+    if (!listed) {
+        h->walk = true;
+    } else if (chained) {
+        h->walk = hw.lev > 0;
+    } else {
+        rc = build_levels(h, levels ? d_val : nullptr, maxlvl, by_level && levels, (uint32_t *)levcnt.p, hw.lev, stream);
+        if (rc == ACLZ_E_NOMEM) {
+            dev_free(h->d_lev, st);
+            h->d_lev = nullptr;
+            h->walk = true;
+        } else if (rc) {
+            cleanup();
+            return rc;
+        }
+    }
     return build_steps(h, stream);  // synchronizes
 }
 

@@ -80,6 +80,13 @@ namespace aclz {
 // block).  Where there are more than kOrdLevelsMost of those, it leaves the
 // in-order matches to the walk, without a list.  build_steps: the step lists,
 // once the worklists are final; synchronizes the stream.
+// list_counts_fit: the list of nt tokens with total bytes, however they are
+// cut, has fewer than 2^32 triplets (its counts and places are 32-bit).
+constexpr uint32_t kLevelPiece = 1024;  // a longer match goes into the list as several
+constexpr bool list_counts_fit(uint64_t nt, uint64_t total) { return nt + total / kLevelPiece < 0xffffffffULL; }
+static_assert(list_counts_fit(1ULL << 31, 1ULL << 40) && !list_counts_fit(3500000000ULL, 1ULL << 40) &&
+                  list_counts_fit(0xfffffffeULL, 1023) && !list_counts_fit(0xfffffffeULL, 1024),
+              "a terabyte of kilobyte pieces takes 2^30 of the triplets");
 int build_units(aclz_handle *h, void *stream);
 int count_levels(aclz_handle *h, bool all, uint32_t *d_cnt, uint32_t *d_total, void *stream);
 int build_levels(aclz_handle *h, const unsigned long long *d_val, uint32_t maxlvl, bool all, const uint32_t *d_cnt,

@@ -67,10 +67,9 @@ __global__ void __launch_bounds__(256) k_lit_units(const uint64_t *__restrict__ 
     }
 }
 
-// A match longer than this goes into the list as several, which groups copy
+// A match longer than kLevelPiece goes into the list as several, which groups copy
 // side by side (at L = 16000 a level has few matches: the 1 GiB copy sweep takes
 // 496 us instead of 826; pieces of 512 bytes cost 10% at L = 1024).
-constexpr uint32_t kSplit = 1024;
 
 // cnt[b] = triplets of block b for the list (of its in-order matches, or all)
 __global__ void __launch_bounds__(256) k_lev_count(const uint4 *__restrict__ tok, const uint64_t *__restrict__ blk_tok,
@@ -81,7 +80,7 @@ __global__ void __launch_bounds__(256) k_lev_count(const uint4 *__restrict__ tok
     uint32_t c = 0;
     for (uint64_t i = blk_tok[b] + lane; i < blk_tok[b + 1]; i += 32) {
         const uint4 t = __ldg(tok + i);
-        if (all || !(t.w >> 8)) c += (t.y + kSplit - 1) / kSplit;
+        if (all || !(t.w >> 8)) c += (t.y + kLevelPiece - 1) / kLevelPiece;
     }
     c = __reduce_add_sync(0xffffffffu, c);
     if (lane == 0) cnt[b] = c;
@@ -104,7 +103,7 @@ __global__ void __launch_bounds__(256) k_lev_build(const uint4 *__restrict__ tok
     for (uint64_t w = blk_tok[b]; w < t1; w += 32) {
         const uint64_t i = w + lane;
         const uint4 t = i < t1 ? __ldg(tok + i) : make_uint4(0, 0, 0, 0);
-        const uint32_t c = all || !(t.w >> 8) ? (t.y + kSplit - 1) / kSplit : 0u;
+        const uint32_t c = all || !(t.w >> 8) ? (t.y + kLevelPiece - 1) / kLevelPiece : 0u;
         uint32_t incl = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -116,8 +115,8 @@ __global__ void __launch_bounds__(256) k_lev_build(const uint4 *__restrict__ tok
             const uint64_t src = (uint64_t)t.z | ((uint64_t)(t.w & 0xffu) << 32);
             const uint32_t kk = val ? 2u * ((uint32_t)(__ldg(val + i) >> 32) - 1u) + ((t.w >> 8) ? 1u : 0u) : 0u;
             for (uint32_t q = 0; q < c; q++) {
-                const uint32_t k = at + incl - c + q, n = min(t.y - q * kSplit, kSplit);
-                const uint64_t pd = d + (uint64_t)q * kSplit, ps = src + (uint64_t)q * kSplit;
+                const uint32_t k = at + incl - c + q, n = min(t.y - q * kLevelPiece, kLevelPiece);
+                const uint64_t pd = d + (uint64_t)q * kLevelPiece, ps = src + (uint64_t)q * kLevelPiece;
                 tri[k] = make_uint4((uint32_t)pd, (uint32_t)(pd >> 32) | 0x100u, (uint32_t)ps,
                                     (uint32_t)(ps >> 32) | (n << 8));
                 if (val) key[k] = kk;
@@ -413,7 +412,7 @@ int aclz::build_steps(aclz_handle *h, void *stream) {
     h->d_ord = nullptr;
     h->d_ord_base = nullptr;
     if (!h->by_level && h->d_lev)
-        if (int rc = build_ord_blocks(h, st)) return rc;
+        if (int rc = build_ord_blocks(h, st); rc && rc != ACLZ_E_NOMEM) return rc;
     for (size_t k = 0; k + 2 < ls.size(); k += 2) {
         if (!h->d_ord) add(h->steps, h->d_lev, ls[k], ls[k + 1]);
         if (h->by_level) add(h->lsteps, h->d_lev, ls[k], ls[k + 2]);
@@ -426,13 +425,18 @@ int aclz::build_steps(aclz_handle *h, void *stream) {
     dev_free(h->d_levels, st);
     h->d_levels = nullptr;
     const std::vector<Step> &list = h->by_level ? h->lsteps : h->steps;
-    h->n_levels = h->by_level || h->flat ? (uint32_t)list.size() : 0;
+    h->n_levels = 0;
+    uint32_t n = h->by_level || h->flat ? (uint32_t)list.size() : 0;
     for (const Step &x : list)
-        if (x.n >= 1ULL << 31) h->n_levels = 0;  // the kernel over them counts in 32 bits
-    if (mostly_narrow(list)) h->n_levels = 0;
-    if (!h->n_levels) return rc_of(cudaStreamSynchronize(st));
-    W0CK(dev_alloc(&h->d_levels, sizeof(Step) * list.size(), st));
-    W0CK(cudaMemcpyAsync(h->d_levels, list.data(), sizeof(Step) * list.size(), cudaMemcpyHostToDevice, st));
+        if (x.n >= 1ULL << 31) n = 0;  // the kernel over them counts in 32 bits
+    if (mostly_narrow(list)) n = 0;
+    if (n) {  // without memory for it the persistent launch goes by ranges
+        cudaError_t e = dev_alloc(&h->d_levels, sizeof(Step) * list.size(), st);
+        if (e == cudaErrorMemoryAllocation) n = 0;
+        else W0CK(e);
+    }
+    if (n) W0CK(cudaMemcpyAsync(h->d_levels, list.data(), sizeof(Step) * list.size(), cudaMemcpyHostToDevice, st));
     W0CK(cudaStreamSynchronize(st));
+    h->n_levels = n;
     return ACLZ_OK;
 }
