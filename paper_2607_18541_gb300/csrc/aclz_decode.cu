@@ -827,7 +827,7 @@ int launch_persistent(aclz_handle *h, uint8_t *out, uint32_t ctas_per_sm, cudaSt
     if (int rc = launch_lits<G>(h, out, st, true, false)) return rc;
     if (int rc = launch_order<G>(h, out, st)) return rc;
     if (phase) cudaEventRecord(phase, st);
-    if (!h->n_ranges) return ACLZ_OK;
+    if (!h->n_ranges) return launch_wave_steps<G>(h, out, st);  // none, or no memory for the ranges
     auto fn = k_ranges<G, STAGED>;
     static int sms = 0;
     static Occ occ[5][33];  // [ctas_per_sm request 0..4][G]
@@ -995,7 +995,8 @@ extern "C" int aclz_decode_plan(const aclz_handle *h, const aclz_decode_cfg *cfg
     if (h->n_blocks) {
         const uint32_t order = level_launches(h->steps, h->n_ord_steps, h->d_steps);
         if (c.mode == ACLZ_MODE_PERSISTENT)
-            n = (c.flags & ACLZ_FLAG_STAGED) && h->n_levels ? 2 : 1 + order + (h->n_ranges ? 1 : 0);
+            n = (c.flags & ACLZ_FLAG_STAGED) && h->n_levels ? 2
+                : 1 + order + (h->n_ranges ? 1 : (uint32_t)h->steps.size() - h->n_ord_steps);
         else if (goes_by_level(h, cfg, false))
             n = 1 + level_launches(h->lsteps, (uint32_t)h->lsteps.size(), h->d_lsteps);
         else

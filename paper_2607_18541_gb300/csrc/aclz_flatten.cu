@@ -377,8 +377,10 @@ extern "C" int aclz_flatten(aclz_handle *h, void *stream) {
     h->mean_deferred_len = (double)def_bytes / (double)np;
     h->flat = true;
     h->by_level = false;  // the pieces are one step after the in-order levels
-    if (int rc = aclz_set_range_bytes(h, h->range_bytes, stream)) return rc;
-    return build_steps(h, stream);
+    // the steps first: those there are point into the worklist freed above,
+    // and the ranges may not fit
+    if (int rc = build_steps(h, stream)) return rc;
+    return aclz_set_range_bytes(h, h->range_bytes, stream);
 }
 
 // ------------------------------------------------------------- reshape

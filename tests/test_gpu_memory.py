@@ -1,4 +1,4 @@
-"""Uploads with little device memory left: an upload that does not fit
+"""Uploads and flattening with little device memory left: an upload that does not fit
 reports it, one that fits without the level list decodes by waves and the
 walk, and every upload that succeeds decodes to the input."""
 import pytest
@@ -51,3 +51,44 @@ def test_upload_as_memory_runs_out():
             aclz.aclz_free(h)
     assert walked and refused, (walked, refused)
     assert plan == full  # enough memory at the end
+
+
+def test_flatten_as_memory_runs_out():
+    # however far a flattening comes, the handle decodes in every mode after
+    # it, and flattens once there is memory
+    sw = synth.copy_sweep(128 * MIB, 32 << 10, 16, seed=12)
+    c = aclz.aclz_pack(sw.total, sw.block_size, (4, 4, 4, 4), sw.blk_ntok, sw.lit_len, sw.match_len, sw.src, sw.literals)
+    s = torch.cuda.current_stream()
+    want = torch.from_numpy(oracle.decode(c)).cuda()
+    out = torch.empty(sw.total, dtype=torch.uint8, device="cuda")
+    refused = 0
+    for left in range(128, 1000, 48):
+        h = aclz.aclz_upload(c, s)
+        try:
+            torch.cuda.empty_cache()
+            free, _ = torch.cuda.mem_get_info()
+            fill = torch.empty(max(0, free - left * MIB), dtype=torch.uint8, device="cuda")
+            try:
+                aclz.aclz_flatten(h, s)
+                ok = True
+            except aclz.AclzError as e:
+                assert e.code == aclz.ACLZ_E_NOMEM
+                refused += 1
+                ok = False
+            del fill
+            for mode, flags in ((aclz.ACLZ_MODE_AUTO, 0), (aclz.ACLZ_MODE_WAVES, 0), (aclz.ACLZ_MODE_PERSISTENT, 0),
+                                (aclz.ACLZ_MODE_PERSISTENT, aclz.ACLZ_FLAG_STAGED)):
+                out.zero_()
+                aclz.aclz_decode_all(h, out, mode=mode, flags=flags, stream=s)
+                assert aclz.aclz_device_status(h, s) == 0
+                assert torch.equal(out, want), (left, ok, mode, flags)
+            if not ok:
+                torch.cuda.empty_cache()
+                aclz.aclz_flatten(h, s)
+                assert aclz.aclz_handle_info(h).n_waves == 2
+                out.zero_()
+                aclz.aclz_decode_all(h, out, stream=s)
+                assert torch.equal(out, want)
+        finally:
+            aclz.aclz_free(h)
+    assert refused
