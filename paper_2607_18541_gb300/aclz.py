@@ -211,12 +211,22 @@ def aclz_encode_gpu(src, params: aclz_encode_params, block_min_match=None, strea
         bmm = np.ascontiguousarray(block_min_match, dtype=np.uint8)
     size = ctypes.c_uint64(0)
     bp = _hptr(bmm) if bmm is not None else None
-    # room for any container, so that the parse runs once (untouched pages of
-    # it are never backed)
-    out = np.empty(max(1, aclz_encode_bound(x.size, params.block_size)), dtype=np.uint8)
-    _ck(lib().aclz_encode_gpu(_hptr(x), x.size, ctypes.byref(params), bp, _stream(stream), _hptr(out), out.size,
-                              ctypes.byref(size)), "aclz_encode_gpu")
-    return out[:size.value]
+
+    def call(out, cap):
+        _ck(lib().aclz_encode_gpu(_hptr(x), x.size, ctypes.byref(params), bp, _stream(stream),
+                                  None if out is None else _hptr(out), cap, ctypes.byref(size)), "aclz_encode_gpu")
+
+    try:
+        # room for any container (about five times the input), so that the
+        # parse runs once; untouched pages of it are never backed
+        out = np.empty(max(1, aclz_encode_bound(x.size, params.block_size)), dtype=np.uint8)
+    except MemoryError:
+        # no address space for that: the size first
+        call(None, 0)
+        out = np.empty(max(1, size.value), dtype=np.uint8)
+    call(out, out.size)
+    out.resize(size.value, refcheck=False)  # gives the rest back
+    return out
 
 
 def aclz_pack_bytes(total_len: int, block_size: int, n_tokens: int, n_literals: int) -> int:
