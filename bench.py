@@ -150,11 +150,12 @@ def kernel_sources_sha() -> str:
     return h.hexdigest()[:16]
 
 
-def recorded_traffic(workload: str):
+def recorded_traffic(workload: str, kernel: str, launch: dict, root: str = ROOT):
     """DRAM bytes per launch of the dominant kernel from the committed ncu
     summary (profiles/traffic_k_levels_persistent_<workload>.txt, lines "key: value"),
-    if it was taken on the current kernel sources; else None."""
-    p = os.path.join(ROOT, "profiles", f"traffic_k_levels_persistent_{workload}.txt")
+    if it was taken of this kernel, on the current kernel sources and with
+    this launch (G, block_size, ctas_per_sm); else None."""
+    p = os.path.join(root, "profiles", f"traffic_k_levels_persistent_{workload}.txt")
     if not os.path.exists(p):
         return None
     d = {}
@@ -163,7 +164,9 @@ def recorded_traffic(workload: str):
             if ":" in line and not line.startswith("#"):
                 k, v = line.split(":", 1)
                 d[k.strip()] = v.strip()
-    if d.get("kernel_sources_sha") != kernel_sources_sha():
+    if d.get("kernel_sources_sha") != kernel_sources_sha() or not kernel.startswith("k_levels_persistent"):
+        return None
+    if any(d.get(k) != str(v) for k, v in launch.items()):
         return None
     try:
         return int(d["dram_bytes_read"]) + int(d["dram_bytes_write"])
@@ -305,7 +308,22 @@ def workload_config(args, extra):
 
 MODE = {"auto": 2, "waves": 0, "persistent": 1}
 LIB_RANGE_BYTES = 20480  # the work-range size an upload picks
-KERNEL = {0: "k_wave_copy (one launch per wave >= 1)", 1: "k_levels_persistent (every level in one launch)"}
+STAGED = 1
+
+
+def timed_mode(mode: int, mean: float) -> int:
+    """The mode a decode with an event between its phases takes for this mode
+    (automatic: by the mean bytes of a deferred match)."""
+    return mode if mode != MODE["auto"] else int(mean >= 192)
+
+
+def deferred_kernel(plan: dict) -> str:
+    """Label of the kernel that copies the deferred matches."""
+    if plan["mode"] == 0:
+        return "k_wave_copy (one launch per wave >= 1)"
+    if plan["flags"] & STAGED:
+        return "k_levels_persistent (every level in one launch)"
+    return "k_ranges (work ranges, register copies, in one launch)"
 
 
 def sweep_leg(args, dev, st, peak):
@@ -433,8 +451,10 @@ def run_ours(args):
         aclz.aclz_set_range_bytes(h, args.range_bytes, st)
     info = aclz.aclz_handle_info(h)
     cfg = dict(G=args.G, mode=MODE[args.mode], ctas_per_sm=args.ctas_per_sm)
-    plan, launches_per_step = aclz.aclz_decode_plan(h, **cfg)
     w0_bytes, def_bytes, n_def = phase_bytes(sw, aclz.aclz_tags(h))
+    # def_bytes: sources and targets
+    plan, launches_per_step = aclz.aclz_decode_plan(
+        h, **{**cfg, "mode": timed_mode(cfg["mode"], def_bytes / 2 / n_def if n_def else 0.0)})
     out = torch.empty(((sw.total + 15) // 16) * 16, dtype=torch.uint8, device=dev)
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
     starts = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
@@ -476,14 +496,14 @@ def run_ours(args):
     peak, peak_kind = peaks()
     w0_ms, d_ms = statistics.mean(ms_w0), statistics.mean(ms_def)
     if d_ms >= w0_ms and n_def:
-        kern, kbytes, kms = KERNEL[plan["mode"]], def_bytes, d_ms
+        kern, kbytes, kms = deferred_kernel(plan), def_bytes, d_ms
         klaunch = launches_per_step - 1
     else:
         kern, kbytes, kms = "k_lits (literals)", w0_bytes, w0_ms
         klaunch = 1
     achieved = kbytes / (kms * 1e-3) / 1e9
     workload = workload_config(args, None)["workload"]
-    traffic = recorded_traffic(workload)
+    traffic = recorded_traffic(workload, kern, dict(G=args.G, block_size=args.block_size, ctas_per_sm=args.ctas_per_sm))
 
     # end to end through the C ABI from pinned host memory: the container as
     # written once with its wave tags (aclz_export), so each upload checks
