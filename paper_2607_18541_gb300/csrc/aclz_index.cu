@@ -51,13 +51,17 @@ __global__ void __launch_bounds__(256) k_index_scan(const uint4 *__restrict__ to
                                                     uint32_t log2bs, uint64_t total, int has_tags,
                                                     uint32_t *err, unsigned long long *first_bad,
                                                     long long *near_matches, uint32_t *crosses) {
+    __shared__ int cta_near;  // of the CTA's blocks: one atomic on global memory for all
+    __shared__ uint32_t cta_cross;
     Group<32> g;
+    if (threadIdx.x == 0) cta_near = 0, cta_cross = 0;
+    __syncthreads();
     const uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (b >= nb) return;
+    const bool on = b < nb;
     if (b == 0 && g.lane == 0) cell[n_cells] = (uint32_t)nt;
-    const uint64_t t0 = blk_tok[b], t1 = blk_tok[b + 1];
+    const uint64_t t0 = on ? blk_tok[b] : 0, t1 = on ? blk_tok[b + 1] : 0;
     const uint64_t bstart = (uint64_t)b << log2bs;
-    const uint64_t blen = min((uint64_t)1 << log2bs, total - bstart);
+    const uint64_t blen = on ? min((uint64_t)1 << log2bs, total - bstart) : 0;
     uint64_t carry = 0, lcarry = 0;
     int near = 0;  // matches that read the match before them, less the others (of 31 in 32)
     bool bad = false, cross = false;  // cross: a source starts in another block
@@ -71,7 +75,7 @@ __global__ void __launch_bounds__(256) k_index_scan(const uint4 *__restrict__ to
         const uint64_t incl = g.scan_incl(tot);
         const uint64_t rel = carry + incl - tot;
         const uint64_t lsum = g.scan_incl(lit);
-        const uint64_t m1 = g.shfl_up(rel + lit, 1);  // where the match before starts
+        const uint32_t m1 = g.shfl_up((uint32_t)(rel + lit), 1);  // where the match before starts
         cross = cross || (v && ml && (sw & kSrcMask) < bstart);
         if (v && ml && g.lane)
             near += (sw & kSrcMask) + ml > bstart + m1 && (sw & kSrcMask) < bstart + rel ? 1 : -1;
@@ -101,11 +105,19 @@ __global__ void __launch_bounds__(256) k_index_scan(const uint4 *__restrict__ to
         carry += g.shfl(incl, 31);
         lcarry += g.shfl(lsum, 31);
     }
-    if (g.lane == 0 && (carry != blen || blk_lit[b] + lcarry != blk_lit[b + 1])) bad = true;
+    if (g.lane == 0 && on && (carry != blen || blk_lit[b] + lcarry != blk_lit[b + 1])) bad = true;
     if (g.ballot(bad) && g.lane == 0) atomicOr(err, kErrCorrupt);
-    if (g.ballot(cross) && g.lane == 0) *crosses = 1u;
+    const unsigned anycross = g.ballot(cross);
     near = __reduce_add_sync(0xffffffffu, near);
-    if (g.lane == 0 && near) atomicAdd((unsigned long long *)near_matches, (unsigned long long)(long long)near);
+    if (g.lane == 0) {
+        if (near) atomicAdd(&cta_near, near);
+        if (anycross) cta_cross = 1u;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (cta_near) atomicAdd((unsigned long long *)near_matches, (unsigned long long)(long long)cta_near);
+        if (cta_cross) *crosses = 1u;
+    }
 }
 
 // Requirement of match i under the current tags: max over the tokens its
