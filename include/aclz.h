@@ -102,13 +102,13 @@ int aclz_encode(const void *host_src, uint64_t n, const aclz_encode_params *p,
  * program and makes no speed claim, Sec. VI): the same container, byte for
  * byte, from the same arguments.  Every candidate chain of the greedy parse
  * is an ordered run of positions with one 4-byte prefix, so the device sorts
- * the positions by (prefix, position), then parses every LZ block with one
- * warp whose lanes score up to 32 candidates at a time, and lays the
- * container out by scans.  host_src: n input bytes (host); n < 2^32 - 64
+ * the positions by (prefix, position), scores every position's candidates at
+ * once, one thread a position, then walks every LZ block with one warp from
+ * match to match, and lays the container out by scans.  host_src: n input bytes (host); n < 2^32 - 64
  * (else ACLZ_E_UNSUPPORTED).  With host_out NULL only *out_size is set (the
  * parse still runs); otherwise cap must hold *out_size bytes
  * (ACLZ_E_CAPACITY).  Allocates device memory of about 25 bytes per input
- * byte for the call (sorted prefixes, ranks, per-block token slots) and
+ * byte for the call (sorted prefixes, best matches, per-block token slots) and
  * frees it before returning; synchronizes the stream. */
 int aclz_encode_gpu(const void *host_src, uint64_t n, const aclz_encode_params *p,
                     const uint8_t *block_min_match, void *stream, void *host_out, uint64_t cap,

@@ -1,6 +1,6 @@
 """Autotuner for the decode: picks the cooperation width G, the encode-time
-block size and the lanes per SM (resident CTAs per SM of the persistent
-launch, and the size of its work ranges).
+block size and, for streams that AUTO decodes in one persistent launch, the
+lanes per SM (its resident CTAs per SM, and the size of its work ranges).
 
 The paper's effective-workload law (Sec. III-A, Table I) ties throughput
 to lanes = G x N_blocks: starved below ~32K lanes, about half of saturated
@@ -80,8 +80,10 @@ def tune(build, total: int, block_sizes=(8192, 16384, 32768, 65536, 131072), Gs=
             if out is None or out.numel() < need:
                 out = torch.empty(need, dtype=torch.uint8, device="cuda")
             for G2 in sorted({G, 32}):
-                for cps in ctas:
-                    for rb in range_bytes:
+                # a decode by levels or waves reads neither of the two
+                read = aclz.aclz_decode_plan(h, G=G2)[0]["mode"] == aclz.ACLZ_MODE_PERSISTENT
+                for cps in ctas if read else ctas[:1]:
+                    for rb in range_bytes if read else range_bytes[:1]:
                         aclz.aclz_set_range_bytes(h, rb, st)
                         ms = measure(h, out, reps=reps, stream=st, G=G2, ctas_per_sm=cps)
                         trials.append(dict(block_size=bs, G=G2, ctas_per_sm=cps, range_bytes=rb,

@@ -1,10 +1,10 @@
-"""Batched decode of many independent compressed streams in one launch.
+"""Batched decode of many independent compressed streams in one graph launch.
 
 Streams are merged into one container whose stream i starts on a block
 boundary (``aclz_batch_merge``: sources rebased, streams never reference one
-another), so the persistent decode schedules the (stream, block, wave) work of
-every stream in one wave-major list and one cooperative launch, captured in a
-CUDA graph.  The lanes law of Sec. III-A is why this pays: a small stream alone
+another), so one decode schedules the work of every stream together: by
+dependency level, one kernel per level of all streams, or in one cooperative
+launch when matches are long, captured in a CUDA graph.  The lanes law of Sec. III-A is why this pays: a small stream alone
 has too few G-lane groups to fill the GPU, thousands of them together do.
 
 The comparison point is the same streams decoded one at a time with the
@@ -190,7 +190,7 @@ def main():
         exact = 0
         for i, x in enumerate(streams):
             exact += bool(torch.equal(dec.stream_output(i), torch.from_numpy(x).to("cuda", non_blocking=True)))
-        row_b = dict(form="batched: one persistent graph-captured launch", streams=len(streams), bytes=total,
+        row_b = dict(form="batched: one graph-captured decode", streams=len(streams), bytes=total,
                      blocks=info.n_blocks, waves=info.n_waves, lanes=best["G"] * info.n_blocks,
                      ms=round(ms_b, 3), gbs=round(total / ms_b / 1e6, 1), exact_streams=exact, **cfg,
                      block_size=best["block_size"], range_bytes=best["range_bytes"])

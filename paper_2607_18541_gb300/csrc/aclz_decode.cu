@@ -15,13 +15,14 @@
 //  - ACLZ_MODE_WAVES: one kernel per wave (k_wave_copy), kernel boundaries
 //    as the wave barrier.  Where ACLZ_MODE_AUTO takes this schedule it goes
 //    by levels instead of waves when the upload found them, one kernel per
-//    level (k_level): every match of a level is independent of the others,
-//    so no chain is left inside a step;
+//    level (k_level; runs of narrow levels together, k_level_run): every match
+//    of a level is independent of the others, so no chain is left inside a step;
 //  - ACLZ_MODE_PERSISTENT: one cooperative launch.  With staged copies it
 //    runs the levels, with a bounded grid barrier between them
 //    (k_levels_persistent); with register copies, or when the upload found no
-//    levels (chains too deep), ranges of consecutive (block, wave) segments
-//    in wave-major order (k_ranges), with bounded waits on per-block
+//    levels (chains too deep) or mostly narrow ones, ranges of consecutive
+//    (block, wave) segments in wave-major order (k_ranges), with bounded waits
+//    on per-block
 //    completed-wave bits instead of barriers, so a match is copied as soon as
 //    the blocks it reads have finished the waves below its own.
 //

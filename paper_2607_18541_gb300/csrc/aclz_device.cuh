@@ -14,7 +14,6 @@ namespace aclz {
 // device status bits latched in a handle's error word
 constexpr uint32_t kErrTimeout = 1u;
 constexpr uint32_t kErrCorrupt = 2u;
-constexpr uint32_t kErrBounds = 4u;
 
 // most polls of any bounded wait
 constexpr uint32_t kSpinLimitMax = 1u << 26;
