@@ -22,9 +22,8 @@
 //    (k_levels_persistent); with register copies, or when the upload found no
 //    levels (chains too deep) or mostly narrow ones, ranges of consecutive
 //    (block, wave) segments in wave-major order (k_ranges), with bounded waits
-//    on per-block
-//    completed-wave bits instead of barriers, so a match is copied as soon as
-//    the blocks it reads have finished the waves below its own.
+//    on per-block completed-wave bits instead of barriers, so a match is copied
+//    as soon as the blocks it reads have finished the waves below its own.
 //
 // All copies are 16-byte vectorised with every lane owning aligned output
 // chunks, so short matches from several tokens share one pass instead of
@@ -722,7 +721,8 @@ uint32_t level_launches(const std::vector<Step> &levels, uint32_t count, const v
     return n;
 }
 
-// Levels: one kernel each (runs of narrow ones one kernel together), fewer matches per group in the small ones, whose
+// Levels: one kernel each (a run of narrow ones one kernel together), fewer
+// matches per group in the small ones, whose
 // groups are all resident at once and take as long as their own window.  Up
 // to kLevelOne (about the warps resident at a time) a group takes one match:
 // 64 MiB copy sweep at L = 900 137 -> 115 us, 256 KiB of Markov bytes 38.5 ->

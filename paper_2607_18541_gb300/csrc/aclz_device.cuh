@@ -300,8 +300,8 @@ __device__ __forceinline__ void group_copy(const Group<G> &g, uint8_t *out, uint
 // a single job (lane j's) is dealt to the lanes by its chunks at once, without
 // the search for every chunk's job.  A step of a chain of 64-byte matches
 // takes 0.38 us instead of 0.80 us (0.59 us with a packed copy that found every
-// chunk's job by shuffles): 1 MiB of zeros in one block 13.2 -> 6.3 ms, 256 KiB in 16
-// KiB blocks by waves 3.11 -> 1.57 ms, by ranges 3.55 -> 1.88 ms.
+// chunk's job by shuffles): 1 MiB of zeros in one block 13.2 -> 6.3 ms, 256 KiB
+// in 16 KiB blocks by waves 3.11 -> 1.57 ms, by ranges 3.55 -> 1.88 ms.
 template <int G, int U, Source SRC = kFromL2>
 __device__ __forceinline__ void group_copy_batch(const Group<G> &g, uint8_t *out, uint64_t d, const uint8_t *s,
                                                  uint32_t n) {

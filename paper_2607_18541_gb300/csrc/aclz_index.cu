@@ -10,10 +10,12 @@
 //                    sources are ordered within the block) and its level
 //                    (the length of the longest chain of matches that ends
 //                    in it).
-//     k_tags_min     the tags of streams whose chains are too deep for the
-//                    passes, in one launch: blocks are taken in increasing
-//                    order and a block waits (bounded) for the earlier
-//                    blocks its sources lie in.
+//     k_tags_relax   the tags of streams whose chains inside blocks are too
+//                    deep for those passes, by passes over blocks.
+//     k_tags_min     the tags of streams whose chains are too deep for either,
+//                    in one launch: blocks are taken in increasing order and
+//                    a block waits (bounded) for the earlier blocks its
+//                    sources lie in.
 //     k_tags_check   legality of tags supplied by the container.
 //  3. k_wave_hist, an exclusive scan and k_slots: the wave-major, block-
 //     ordered worklist slot of every deferred match.
@@ -903,7 +905,8 @@ int relax_levels(aclz_handle *h, unsigned long long *d_val, uint32_t *d_out, cud
     if (cudaMemsetAsync(d_out, 0, 12, st) != cudaSuccess ||
         cudaMemsetAsync(d_val, 0, 8 * (nt ? nt : 1), st) != cudaSuccess)
         return ACLZ_E_CUDA;
-    if (state.alloc(4 * kRelaxState, st) != cudaSuccess || cover.alloc(16 * (nt ? nt : 1), st) != cudaSuccess) return ACLZ_OK;
+    if (state.alloc(4 * kRelaxState, st) != cudaSuccess || cover.alloc(16 * (nt ? nt : 1), st) != cudaSuccess)
+        return ACLZ_OK;
     if (cudaMemsetAsync(state.p, 0, 4 * kRelaxState, st) != cudaSuccess) return ACLZ_E_CUDA;
     k_cover<<<(nb + 7) / 8, 256, 0, st>>>((const uint4 *)h->d_tok, h->d_blk_tok, h->d_tokdst, nb, h->log2_bs, nt,
                                            (uint4 *)cover.p);
@@ -940,10 +943,11 @@ int relax_levels(aclz_handle *h, unsigned long long *d_val, uint32_t *d_out, cud
 // chain, this about one for every wave; the ordered pass (k_tags_min) takes
 // the blocks one after another.  128 MiB of word text at 6/8/10/12 in blocks of
 // 1 MiB (128 waves, over 512 levels) uploads in 1.03 s by these passes alone,
-// in 4.26 s by k_relax and the ordered pass and in 0.20 s by k_relax and these.  A stream of few tokens takes
-// the ordered pass at once (4096 matches in one chain, 16 blocks: 19 ms by
-// these passes and then it, 9 ms by it), and so does one whose chains mostly
-// go from block to block, for which these passes are as many as k_relax's.
+// in 4.26 s by k_relax and the ordered pass and in 0.20 s by k_relax and these.
+// A stream of few tokens takes the ordered pass at once (4096 matches in one
+// chain, 16 blocks: 19 ms by these passes and then it, 9 ms by it), and so does
+// one whose chains mostly go from block to block, for which these passes are as
+// many as k_relax's.
 constexpr uint32_t kBlockBatch = 8, kBlockPasses = 512;
 constexpr uint64_t kOrderedTokens = 1u << 17;
 int relax_blocks(aclz_handle *h, uint32_t *d_tags, uint32_t *d_maxtag, bool *reached, cudaStream_t st) {

@@ -10,8 +10,8 @@
 //    level l and below.  The matches of one level are independent of each
 //    other, in every block at once.  The list holds the in-order matches
 //    (tag 0: every source byte is a literal or an in-order match byte of the
-//    same block), for every schedule; for streams that are decoded as waves
-//    it holds the deferred ones too and is a schedule of its own: the fewest
+//    same block), for every schedule; where the levels of all matches are
+//    known it holds the deferred ones too and is a schedule of its own: the fewest
 //    dependent steps there are (a wave hides its chains within a block:
 //    4 MiB of FASTQ-like text at 12/16/24/32 has 9 waves with chains adding
 //    up to 42 steps, and 14 levels).
