@@ -124,8 +124,10 @@ __device__ __forceinline__ unsigned long long pack_piece(uint64_t a, uint32_t n,
 // loads) times the depth of the chain, so the lanes of a warp each follow a
 // chain of their own, 32 tokens' pieces at a time.  Against one chain per
 // warp, started from 256 output bytes and found by a search of the block's
-// tokens, on flattened word text at 12/16/24/32: one 16 KiB range 93 ->
-// 21 us, 64 ranges of 16 KiB to 4 MiB (50 MB) 1.9-2.6 ms -> 0.21 ms.  6 CTAs
+// tokens, on flattened word text at 12/16/24/32 (the depth of the chains
+// differs from text to text, both sides on the same): one 16 KiB range 54 to
+// 103 -> 16 to 23 us, 64 ranges of 16 KiB to 4 MiB (50 MB) 1.3 to 3.4 ms ->
+// 0.17 to 0.26 ms.  6 CTAs
 // per SM (80 registers): 5 and 7 were 2% slower; units up to 8 KiB: with 1
 // KiB units and no windows 0.31 ms.
 __global__ void __launch_bounds__(kSeekThreads, 6) k_seek(const SeekReq *__restrict__ reqs, SeekReq one,
