@@ -12,6 +12,18 @@ pytestmark = pytest.mark.gpu
 MIB = 1 << 20
 
 
+def _fill(left):
+    """All device memory but about `left` MiB."""
+    torch.cuda.empty_cache()
+    for spare in (0, 64, 256, 1024):
+        free, _ = torch.cuda.mem_get_info()
+        try:
+            return torch.empty(max(1, free - (left + spare) * MIB), dtype=torch.uint8, device="cuda")
+        except torch.OutOfMemoryError:
+            torch.cuda.empty_cache()
+    raise AssertionError("no allocation near the free memory succeeds")
+
+
 def test_upload_as_memory_runs_out():
     # 20 million matches in some 40 levels; the library keeps up to 512 MiB of
     # what it freed, which an upload uses first
@@ -26,9 +38,7 @@ def test_upload_as_memory_runs_out():
     aclz.aclz_free(h)
     walked, refused = 0, 0
     for left in range(128, 2900, 128):
-        torch.cuda.empty_cache()
-        free, _ = torch.cuda.mem_get_info()
-        fill = torch.empty(max(0, free - left * MIB), dtype=torch.uint8, device="cuda")
+        fill = _fill(left)
         try:
             h = aclz.aclz_upload(c, s)
         except aclz.AclzError as e:
@@ -65,9 +75,7 @@ def test_flatten_as_memory_runs_out():
     for left in range(128, 1000, 48):
         h = aclz.aclz_upload(c, s)
         try:
-            torch.cuda.empty_cache()
-            free, _ = torch.cuda.mem_get_info()
-            fill = torch.empty(max(0, free - left * MIB), dtype=torch.uint8, device="cuda")
+            fill = _fill(left)
             try:
                 aclz.aclz_flatten(h, s)
                 ok = True
